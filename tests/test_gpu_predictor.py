@@ -83,6 +83,38 @@ def test_sgd_step_with_clipping_matches_oracle(tera, clip):
     ctx.close()
 
 
+@pytest.mark.parametrize("n,batch", [(1, 1), (40, 31), (40, 33), (700, 64), (90, 200),
+                                     (6000, 4864), (6000, 4865), (300, 10000)])
+def test_training_steps_at_tile_edges(tera, n, batch):
+    # three steps against the float64 oracle: batches below, at and beyond the
+    # kernel's 32-sample tiles and one tile per SM, wrapping round fewer valid
+    # samples (more than once in the last case)
+    rng = np.random.default_rng(n + batch)
+    X = rng.standard_normal((n, 8)).astype(np.float32)
+    Y = rng.standard_normal((n, 3)).astype(np.float32)
+    flag = (rng.random(n) < 0.9).astype(np.float32)
+    flag[0] = 1.0
+    samples = np.concatenate([X, Y, flag[:, None]], axis=1).astype(np.float32)
+    p0 = (rng.standard_normal(4931) * 0.2).astype(np.float32)
+    ctx = tera.Context((0, 0, 0), (10, 10, 10), (1, 1, 1), 1.0)
+    pt = torch.from_numpy(p0.copy()).cuda()
+    lr, clip, steps = 0.02, 1.0, 3
+    nv = ctx.mlp_train(torch.from_numpy(samples).cuda(), pt, steps, batch, lr, clip)
+    Xv, Yv = X[flag != 0].astype(np.float64), Y[flag != 0].astype(np.float64)
+    assert nv == len(Xv)
+    want, tol = p0.astype(np.float64), 0.0
+    for k in range(steps):
+        at = (k * batch + np.arange(batch)) % nv
+        _, g = oracle.mlp_loss_grad(want, Xv[at], Yv[at])
+        want = oracle.mlp_sgd_clip(want, g, float(np.float32(lr)), clip)
+        c = min(1.0, clip / np.linalg.norm(g))
+        # per step as for one clipped step, twice over for what a step's
+        # difference does to the gradients after it
+        tol += 2 * (lr * c * 1e-3 * np.abs(g).max() + 4e-7 * np.abs(p0).max())
+    assert np.abs(pt.cpu().numpy().astype(np.float64) - want).max() <= tol
+    ctx.close()
+
+
 def run_pred_chain(tera, wl, params, path, tune=None):
     gen = Generator(wl, device="cuda")
     states = list(gen.series(wl.iterations))
