@@ -140,6 +140,13 @@ struct DecArgs {
   PredArgs pr{};
 };
 
+// codec_tiles.cu: steps a3-a5 of every pair (no explicit schedule).  E and D as
+// the entry point filled them; with the predictor, each side's predictions are
+// made.  The lists' bounds for cap records of P pairs.
+tera_status launch_tiles(tera_ctx* ctx, const EncArgs& E, const DecArgs& D, bool pr, int mode,
+                         u64 wire_cap, u64 recv_cap, cudaStream_t s);
+void tile_list_bounds(u64 cap, u64 P, u64 warps, u64* units, u64* items, u64* bigs);
+
 __device__ __forceinline__ u32 rec_code(const Rec& d, u32* bytes) {
   u32 code = 0, b = 0;
 #pragma unroll

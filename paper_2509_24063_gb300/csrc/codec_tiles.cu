@@ -1,0 +1,1309 @@
+// Batched codec over tiles: steps a3-a5 (paper Sec. 2.3, steps B, C and D) for
+// every pair of one iteration, as launches over tiles of kT entries that know
+// nothing of the pairs' sizes:
+//
+//   setup   (two launches) per-pair facts, wire slabs and the lists of tiles
+//   match   one block per pair: the message record of every reference slot
+//           (ids in shared memory), the matches before each tile and the list
+//           of the records no slot took; pairs of more than kTableMax records
+//           index their ids in global hash segments here, a tile each, and are
+//           matched by
+//   bigmatch  (tiles of such pairs; does nothing without them)
+//   sizes   predictor only: the payload of the XOR and of the residual form
+//   encode  one tile of slots or new records: difference, code, new-reference
+//           records, and the payload, packed, into the tile's own part of the
+//           receive buffer (a tile's payload never exceeds its records)
+//   wire    one tile: its payload's place in the message, from the counts of
+//           the tiles before it, and the payload copied there
+//   decode  one tile of entries from the wire and the receiver's reference
+//
+// Only the payload's place depends on other tiles' contents, and the payload
+// is a small part of the bytes moved (11 of some 330 per record), so writing
+// it twice costs less than any order among the tiles: no tile waits for
+// another.
+//
+// Why tiles: a block that carries a pair through all steps on its own (the
+// persistent launch of batched.cu, used for an explicit schedule) pays every
+// step's memory latency once per tile of every pair, one after the other, and
+// the largest pair is the launch's length.  Measured, whole codec: uniform 100
+// M agents (16.6 M records) 1.98 -> 1.54 ms, of which encode 683 us (3.65 GB,
+// 79 % of the measured copy rate), decode 464 us (2.4 GB), match 264, wire 88,
+// setup 32; 16 M agents kept box by box 0.93 -> 0.78 ms; a pair of 1.1 M
+// records among 6.5 M: 3.3 -> 1.2 ms; 6.3 K records in 12 pairs: 92 -> 60 us.
+// A look-back over the tiles in place of the second copy of the payload
+// (tiles claimed in order, sums published) left encode and decode at 1.16 ms
+// each; a block a tile with barriers between its steps at 0.86 and 0.74.
+#include "codec_tile.cuh"
+
+using namespace tera;
+
+namespace {
+
+constexpr int kT = 256;           // threads of a block
+constexpr int kPerSm = 4;         // resident blocks per SM (64 registers a thread)
+constexpr int kEncPerSm = 4, kDecPerSm = 3;  // (the decode's shared memory: 65 KB a block)
+constexpr u32 kBigTile = kT * kIlp;  // ids of a tile of a pair matched through global memory
+// Entries of a tile: 32 << 0 .. 3, the most that still gives every resident
+// warp kTilesPerWarp tiles; a warp takes a tile's entries 32 at a time, so a small
+// iteration's tiles are a single step (uniform 4 thousand agents: encode 23 ->
+// 10 us) and a large one's are not all set-up.
+constexpr u32 kMinShift = 5, kMaxShift = 8;
+constexpr u64 kTilesPerWarp = 8;
+// new-record tiles of a pair beyond the m - r records that must be new: one
+// per kNewShare tiles of records, so that a pair whose records all changed is
+// still spread over many warps, while a usual pair has one
+constexpr u32 kNewShare = 16;
+// Pairs of at most this many slots and records are matched by one warp, so
+// that the thousands of edge and corner pairs of a large grid are in flight at
+// once (13,824 pairs, 100 M agents: match 297 -> 264 us).  A grid with few
+// pairs for the GPU's blocks gives all but the smallest a block (1 M agents,
+// 936 pairs: 39 us with the higher limit, 32 with the lower).
+constexpr u32 kWarpPair = 512, kWarpPairFew = 64;
+
+// Per-pair facts, one 64-byte line.
+struct __align__(16) TilePair {
+  u64 g_lo;   // first record of the message (pair_off)
+  u64 ro;     // first slot of the sender reference (ref_off)
+  u64 w_off;  // the message's slab
+  u32 r, m;   // slots (0 when sent raw), records
+  u32 unit0;  // first tile of the pair
+  u32 nst, nnu;  // slot tiles, new-record units
+  u32 item0;  // first match item
+  u32 big0;   // first bigmatch item
+  u32 nbig;   // bigmatch items
+  u32 mode;   // XOR or raw
+  u32 fits;   // the receiver's reference has the slots the message refers to
+};
+static_assert(sizeof(TilePair) == 64, "one line per pair");
+
+// Device scalars of one call.
+enum { TS_UNITS = 0, TS_ITEMS, TS_BIG, TS_SMALL, TS_SHIFT, TS_TICKET_MATCH, TS_TICKET_BIG,
+       TS_COUNT };
+
+struct TileArgs {
+  EncArgs E;
+  DecArgs D;
+  TilePair* pair;
+  u32* unit_pair;       // pair of each tile
+  u32* item_pair;       // pair of each match item
+  u32* big_pair;        // pair of each bigmatch item
+  u32* small_pair;      // pairs matched by one warp
+  u32 warps;            // resident warps of a launch
+  u32 warp_pair;        // slots and records of a pair matched by one warp, at most
+  u32* before;          // matched slots before each slot tile (bigmatch: first, in it)
+  u32* bytes;           // payload bytes of each tile
+  u64* place;           // payload bytes of the pair before each tile
+  u64* tot;             // [P * PT_COUNT] matched records, XOR and residual bytes
+  u32* done;            // [P] bigmatch items finished
+  u32* bits;            // taken records of big pairs: word (g_lo >> 5) + p of pair p
+  u32* new_idx;         // new records of each pair in message order, from g_lo
+  u32* scal;            // TS_*
+  u64 P;
+};
+
+enum { PT_MATCHED = 0, PT_XOR = 1, PT_RES = 2, PT_COUNT = 4 };
+
+// ---------------- setup ----------------
+
+struct Facts {
+  u64 r, m, rr, r_full, slab;
+  bool raw;
+  u64 units, items, big, small;
+};
+
+// log2 of the tiles' entries.
+__device__ __forceinline__ u32 tile_shift(const TileArgs& A) {
+  const u64 E = A.E.pair_off[A.P], R = A.E.ref_off ? A.E.ref_off[A.P] : 0;
+  const u64 most = E > R ? E : R;
+  u32 s = kMaxShift;
+  while (s > kMinShift && (most >> s) < kTilesPerWarp * (u64)A.warps) --s;
+  return s;
+}
+
+__device__ __forceinline__ u64 tiles(u64 entries, u32 shift) {
+  return (entries + (1ull << shift) - 1ull) >> shift;
+}
+
+__device__ __forceinline__ Facts facts_of(const TileArgs& A, u64 p, int mode, u32 shift) {
+  Facts f;
+  f.m = A.E.pair_off[p + 1] - A.E.pair_off[p];
+  f.r_full = A.E.ref_off ? A.E.ref_off[p + 1] - A.E.ref_off[p] : 0;
+  f.raw = mode == TERA_MODE_RAW || A.E.reset[p];
+  f.r = f.raw ? 0 : f.r_full;
+  f.rr = A.D.ref_off ? A.D.ref_off[p + 1] - A.D.ref_off[p] : 0;
+  f.slab = round16((u64)kHdrBytes + 4 * (f.r_full + f.m) + (u64)kRecBytes * f.m);
+  const u64 sure = f.m > f.r ? f.m - f.r : 0;
+  u64 nnu = tiles(sure, shift) + ceil_div(tiles(f.m, shift), kNewShare);
+  // a pair without entries whose receiver holds a reference still goes
+  // through the decode's header check
+  if (f.r == 0 && f.m == 0 && f.rr != 0) nnu = 1;
+  f.units = tiles(f.r, shift) + nnu;
+  const bool big = f.m > kTableMax;
+  f.small = f.r + f.m != 0 && f.r <= A.warp_pair && f.m <= A.warp_pair;
+  f.items = big ? ceil_div(f.m, kBigTile) : (f.r + f.m != 0 && !f.small ? 1 : 0);
+  f.big = big ? ceil_div(f.r, kBigTile) : 0;
+  return f;
+}
+
+constexpr int kSetupT = 1024;
+
+// First launch: kSetupT pairs per block, the block's sums of (slab bytes,
+// tiles) and (match items and pairs matched by a warp in the two halves of a
+// word, bigmatch items).
+__global__ void __launch_bounds__(kSetupT) tiles_sums_kernel(TileArgs A, int mode,
+                                                             U64x2* __restrict__ part) {
+  __shared__ u64 sm[4][32];
+  const u64 p = (u64)blockIdx.x * kSetupT + threadIdx.x;
+  u64 v[4] = {0, 0, 0, 0};
+  if (p < A.P) {
+    const Facts f = facts_of(A, p, mode, tile_shift(A));
+    v[0] = f.slab;
+    v[1] = f.units;
+    v[2] = f.items | (f.small << 32);
+    v[3] = f.big;
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) v[i] = warp_sum(v[i]);
+  if ((threadIdx.x & 31) == 0)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) sm[i][threadIdx.x >> 5] = v[i];
+  __syncthreads();
+  if (threadIdx.x < 32) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) v[i] = warp_sum(sm[i][threadIdx.x]);
+    if (threadIdx.x == 0) {
+      part[2 * blockIdx.x] = U64x2{v[0], v[1]};
+      part[2 * blockIdx.x + 1] = U64x2{v[2], v[3]};
+    }
+  }
+}
+
+// out[i] = pair of item i for the items [lo, lo + n) of the block's pairs,
+// first[k] (k < np) the first item of pair p0 + k counted from lo (first[np] = n).
+__device__ __forceinline__ void fill_map(u32* __restrict__ out, u64 lo, u32 n, const u32* first,
+                                         u32 np, u32 p0) {
+  for (u32 i = threadIdx.x; i < n; i += kSetupT)
+    out[lo + i] = p0 + upper_pair(first, 0u, np, (u64)i);
+}
+
+// Second launch (the same blocks): offsets from the first launch's sums, the
+// per-pair facts and the maps.  Pairs without entries on
+// either side are finished here.
+__global__ void __launch_bounds__(kSetupT)
+    tiles_place_kernel(TileArgs A, int mode, u64* __restrict__ wire_off, u64 wire_cap, u64 rec_cap,
+                       u64 recv_cap, u64 unit_cap, u64 item_cap, u64 big_cap, u32* epoch,
+                       const U64x2* __restrict__ part) {
+  __shared__ U64x2 sm2[33];
+  __shared__ u32 first[4][kSetupT];
+  const u32 shift = tile_shift(A);
+  U64x2 ca{0, 0}, cb{0, 0}, qa{0, 0}, qb{0, 0};
+  for (u32 i = threadIdx.x; i < gridDim.x; i += kSetupT) {
+    const U64x2 a = part[2 * i], b = part[2 * i + 1];
+    if (i < blockIdx.x) {
+      ca += a;
+      cb += b;
+    }
+    qa += a;
+    qb += b;
+  }
+  U64x2 carry_a, carry_b, tot_a, tot_b;
+  block_excl_scan2(ca, sm2, &carry_a);
+  block_excl_scan2(cb, sm2, &carry_b);
+  block_excl_scan2(qa, sm2, &tot_a);
+  block_excl_scan2(qb, sm2, &tot_b);
+  const u64 P = A.P, E = A.E.pair_off[P];
+  const u64 rmax = A.E.ref_off ? A.E.ref_off[P] : 0, dmax = A.D.ref_off ? A.D.ref_off[P] : 0;
+  const u64 big = E > rmax ? (E > dmax ? E : dmax) : (rmax > dmax ? rmax : dmax);
+  const u64 n_items = tot_b.a & 0xFFFFFFFFull, n_small = tot_b.a >> 32;
+  const bool fits = tot_a.b <= unit_cap && n_items <= item_cap && tot_b.b <= big_cap;
+  const bool abort = tot_a.a > wire_cap || big > rec_cap || E + P > recv_cap || !fits;
+  const u64 p = (u64)blockIdx.x * kSetupT + threadIdx.x;
+  Facts f{};
+  if (p < P) f = facts_of(A, p, mode, shift);
+  U64x2 ta, tb;
+  const U64x2 ea = block_excl_scan2(U64x2{f.slab, f.units}, sm2, &ta);
+  const U64x2 eb = block_excl_scan2(U64x2{f.items | (f.small << 32), f.big}, sm2, &tb);
+  first[0][threadIdx.x] = (u32)ea.b;
+  first[1][threadIdx.x] = (u32)eb.a;
+  first[2][threadIdx.x] = (u32)eb.b;
+  first[3][threadIdx.x] = (u32)(eb.a >> 32);
+  u64 empties = 0;
+  if (p < P) {
+    const u64 w = carry_a.a + ea.a, g_lo = A.E.pair_off[p];
+    wire_off[p] = w;
+    A.D.recv_off[p] = g_lo;
+    if (!abort) {
+      TilePair x;
+      x.g_lo = g_lo;
+      x.ro = A.E.ref_off ? A.E.ref_off[p] : 0;
+      x.w_off = w;
+      x.r = (u32)f.r;
+      x.m = (u32)f.m;
+      x.unit0 = (u32)(carry_a.b + ea.b);
+      x.nst = (u32)tiles(f.r, shift);
+      x.nnu = (u32)f.units - x.nst;
+      x.item0 = (u32)carry_b.a + (u32)eb.a;
+      x.big0 = (u32)(carry_b.b + eb.b);
+      x.nbig = (u32)f.big;
+      x.mode = f.raw ? TERA_MODE_RAW : TERA_MODE_XOR;
+      x.fits = f.raw || f.r == (A.D.ref ? f.rr : 0) ? 1u : 0u;
+      A.pair[p] = x;
+      ulonglong2* tot = reinterpret_cast<ulonglong2*>(A.tot + p * PT_COUNT);
+      tot[0] = make_ulonglong2(0, 0);
+      tot[1] = make_ulonglong2(0, 0);
+      A.done[p] = 0;
+      if (f.units == 0) {  // no slots, no records: headers alone
+        ulonglong2* h = reinterpret_cast<ulonglong2*>(A.E.wire + w);
+        h[0] = make_ulonglong2((u64)kWireMagic | ((u64)kVersion << 32) | ((u64)kRecBytes << 48),
+                               (u64)A.E.class_id | ((u64)x.mode << 32));
+        h[1] = make_ulonglong2(0, 0);
+        h[2] = make_ulonglong2(0, 0);
+        h[3] = make_ulonglong2(p, kHdrBytes);
+        A.E.wire_len[p] = kHdrBytes;
+        write_taio_header(A.E.ref_next + (g_lo + p) * kRecBytes, A.E.class_id, (u32)p, 0);
+        write_taio_header(A.D.recv + (g_lo + p) * kRecBytes, A.D.class_id, (u32)p, 0);
+        A.E.reset[p] = 0;
+        empties = 1;
+        if (x.mode != TERA_MODE_RAW && A.D.ref) {  // as the decode's header check
+          const u64* rh =
+              reinterpret_cast<const u64*>(A.D.ref + (A.D.ref_off[p] + p) * kRecBytes);
+          if ((u32)rh[0] != kTaioMagic || (u32)rh[1] != A.D.class_id ||
+              (u32)(rh[1] >> 32) != (u32)p || rh[2] != 0)
+            latch(A.D.st, TERA_ECORRUPT);
+        }
+      }
+    }
+  }
+  __syncthreads();
+  if (!abort) {
+    const u64 left = P - (u64)blockIdx.x * kSetupT;
+    const u32 np = (u32)(left < (u64)kSetupT ? left : (u64)kSetupT), p0 = blockIdx.x * kSetupT;
+    fill_map(A.unit_pair, carry_a.b, (u32)ta.b, first[0], np, p0);
+    fill_map(A.item_pair, carry_b.a & 0xFFFFFFFFull, (u32)tb.a, first[1], np, p0);
+    fill_map(A.small_pair, carry_b.a >> 32, (u32)(tb.a >> 32), first[3], np, p0);
+    fill_map(A.big_pair, carry_b.b, (u32)tb.b, first[2], np, p0);
+    const u64 n = warp_sum(empties);
+    if ((threadIdx.x & 31) == 0 && n) atomicAdd(&A.E.stats->wire_bytes, n * kHdrBytes);
+  }
+  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
+    const u32 ep = *epoch + 1u;
+    *epoch = ep == 0u ? 1u : ep;
+    wire_off[P] = tot_a.a;
+    A.D.recv_off[P] = E;
+    if (tot_a.a > wire_cap) {
+      latch(A.E.st, TERA_ECAPACITY);
+      need(A.E.st, tot_a.a);
+    }
+    if (big > rec_cap) {
+      latch(A.E.st, TERA_ECAPACITY);
+      need(A.E.st, big);
+    }
+    if (E + P > recv_cap) {
+      latch(A.E.st, TERA_ECAPACITY);
+      need(A.E.st, E + P);
+    }
+    if (!fits) latch(A.E.st, TERA_ECAPACITY);  // cannot happen: the lists are sized for it
+    A.scal[TS_UNITS] = abort ? 0u : (u32)tot_a.b;
+    A.scal[TS_ITEMS] = abort ? 0u : (u32)n_items;
+    A.scal[TS_SMALL] = abort ? 0u : (u32)n_small;
+    A.scal[TS_SHIFT] = shift;
+    A.scal[TS_BIG] = abort ? 0u : (u32)tot_b.b;
+    for (int i = TS_TICKET_MATCH; i < TS_COUNT; ++i) A.scal[i] = 0u;
+  }
+}
+
+// ---------------- match ----------------
+
+// The next item of a list, claimed in order: thread 0 claims, every thread
+// gets it (~0u when the list is done).  Ends with a block barrier; the caller
+// passes another one before the next claim.
+__device__ __forceinline__ u32 claim(u32* ticket, u32 n, u32* s_next) {
+  if (threadIdx.x == 0) {
+    const u32 t = atomicAdd(ticket, 1u);
+    *s_next = t < n ? t : ~0u;
+  }
+  __syncthreads();
+  return *s_next;
+}
+
+// Word k / 32 of the taken bits of pair p's message (global, big pairs).
+__device__ __forceinline__ u32* big_bits(const TileArgs& A, const TilePair& x, u32 p) {
+  return A.bits + (x.g_lo >> 5) + p;
+}
+
+// The records of pair p whose bit is not set, in message order, into
+// new_idx[g_lo ..]; words of 32 records, `bits` in shared (or, G, global) memory.
+template <int T, bool G>
+__device__ __forceinline__ void new_list(const TileArgs& A, const TilePair& x, const u32* bits,
+                                         u32* sm32) {
+  const u32 words = (x.m + 31u) / 32u;
+  u64 run = 0;
+  for (u32 w0 = 0; w0 < words; w0 += T) {  // group-uniform
+    const u32 w = w0 + group_thread<T>();
+    u32 free = 0;
+    if (w < words) {
+      const u32 b = G ? __ldcg(bits + w) : bits[w];
+      free = ~b & ((w + 1u) * 32u <= x.m ? 0xFFFFFFFFu : (1u << (x.m & 31u)) - 1u);
+    }
+    u32 tot, pos;
+    if constexpr (T == 32) {
+      const u32 c = (u32)__popc(free), inc = warp_incl_scan<u32>(c);
+      pos = inc - c;
+      tot = __shfl_sync(0xFFFFFFFFu, inc, 31);
+    } else {
+      pos = block_excl_scan<u32>((u32)__popc(free), sm32, &tot);
+    }
+    u32* out = A.new_idx + x.g_lo + run + pos;
+    for (; free; free &= free - 1u) *out++ = w * 32u + (u32)__ffs(free) - 1u;
+    run += tot;
+  }
+}
+
+// before[unit0 + t] from the matches of each of the pair's nst slot tiles
+// (counts in the same places): their exclusive sums.
+template <int T>
+__device__ __forceinline__ void sum_tiles(const TileArgs& A, const TilePair& x, u32* sm32) {
+  u32 run = 0;
+  for (u32 t0 = 0; t0 < x.nst; t0 += T) {  // group-uniform
+    const u32 t = t0 + group_thread<T>();
+    const u32 c = t < x.nst ? __ldcg(A.before + x.unit0 + t) : 0u;
+    u32 tot, ex;
+    if constexpr (T == 32) {
+      const u32 inc = warp_incl_scan<u32>(c);
+      ex = inc - c;
+      tot = __shfl_sync(0xFFFFFFFFu, inc, 31);
+    } else {
+      ex = block_excl_scan<u32>(c, sm32, &tot);
+    }
+    if (t < x.nst) A.before[x.unit0 + t] = run + ex;
+    run += tot;
+  }
+}
+
+// The matches of each slot tile of a pair whose slot_src this group wrote, a
+// tile per warp.
+template <int T>
+__device__ __forceinline__ void count_tiles(const TileArgs& A, const TilePair& x, u32 shift) {
+  for (u32 t = group_thread<T>() >> 5; t < x.nst; t += T / 32) {
+    u32 c = 0;
+    for (u32 i = threadIdx.x & 31; i < (1u << shift); i += 32) {
+      const u32 j = (t << shift) + i;
+      c += j < x.r && __ldcg(A.E.slot_src + x.ro + j) != kNoMatch;
+    }
+    c = warp_sum(c);
+    if ((threadIdx.x & 31) == 0) A.before[x.unit0 + t] = c;
+  }
+}
+
+// One tile of message ids of a big pair into its hash segment (as the
+// persistent launch does), its taken bits cleared.
+__device__ __forceinline__ void big_build(const TileArgs& A, const TilePair& x, u32 p, u32 tile,
+                                          u32 epoch) {
+  const EncArgs& E = A.E;
+  const u64 base = seg_base(x.g_lo, p), size = seg_size(x.m);
+  const u32 k0 = tile * kBigTile;
+  if (threadIdx.x < kBigTile / 32) {
+    const u32 w = k0 / 32 + threadIdx.x;
+    if (w < (x.m + 31u) / 32u) big_bits(A, x, p)[w] = 0u;
+  }
+  u64 id[kIlp], at[kIlp], cur[kIlp], prev[kIlp];
+  bool live[kIlp];
+#pragma unroll
+  for (u32 i = 0; i < kIlp; ++i) {
+    const u32 k = k0 + i * kT + threadIdx.x;
+    live[i] = k < x.m;
+    id[i] = live[i] ? msg_id(E, p, x.g_lo + k) : 0;
+  }
+#pragma unroll
+  for (u32 i = 0; i < kIlp; ++i) {
+    at[i] = seg_start(id[i], size);
+    cur[i] = live[i] ? __ldcg(&E.seg[base + at[i]].a) : 0;
+  }
+#pragma unroll
+  for (u32 i = 0; i < kIlp; ++i) {
+    const u32 k = k0 + i * kT + threadIdx.x;
+    const bool empty = live[i] && (u32)(cur[i] >> 32) != epoch;
+    prev[i] = empty ? atomicCAS(&E.seg[base + at[i]].a, cur[i], ((u64)epoch << 32) | k) : ~0ull;
+  }
+#pragma unroll
+  for (u32 i = 0; i < kIlp; ++i) {
+    if (!live[i]) continue;
+    const u32 k = k0 + i * kT + threadIdx.x;
+    if ((u32)(cur[i] >> 32) != epoch && prev[i] == cur[i]) {
+      E.seg[base + at[i]].b = id[i];
+    } else {  // taken in this iteration: continue along the probe sequence
+      seg_insert_from<true>(E.seg, base, size, id[i], ((u64)epoch << 32) | k, epoch,
+                            at[i] + 1 == size ? 0 : at[i] + 1);
+    }
+  }
+}
+
+// The matches of a pair that fits shared memory, by a group of T threads:
+// slot_src, the new records, the matches before each slot tile and in all.
+template <int T>
+__device__ __forceinline__ void match_pair(const TileArgs& A, const TilePair& x, u32 p, u32 shift,
+                                           SmemTable& tb, u64* window, u32* s_cnt, u32* sm32) {
+  if (group_thread<T>() == 0) *s_cnt = 0;
+  u32 size = 32;
+  while (size < 2 * x.m) size <<= 1;
+  tb.mask = size - 1;
+  u32 c = 0;
+  group_sync<T>();
+  if (ids_ascending<T>(A.E, p, x.m)) {
+    if (x.r) c = sorted_match<T>(A.E, p, x.m, x.r, tb, window);
+  } else {
+    smem_build<T>(A.E, p, x.m, tb);  // also finds an id that occurs twice
+    group_sync<T>();
+    if (x.r) c = smem_match<T>(A.E, p, x.r, tb);
+  }
+  if (x.r == 0) return;
+  c = warp_sum(c);
+  if ((threadIdx.x & 31) == 0 && c) atomicAdd(s_cnt, c);
+  group_sync<T>();
+  const u32 matched = *s_cnt;
+  if (group_thread<T>() == 0) A.tot[(u64)p * PT_COUNT + PT_MATCHED] = matched;
+  if (matched < x.m) new_list<T, false>(A, x, tb.bits, sm32);
+  if (x.nst == 1) {
+    if (group_thread<T>() == 0) A.before[x.unit0] = 0u;
+  } else {
+    __threadfence_block();
+    group_sync<T>();
+    count_tiles<T>(A, x, shift);
+    __threadfence_block();
+    group_sync<T>();
+    sum_tiles<T>(A, x, sm32);
+  }
+}
+
+// Shared memory of the match: the table (or the id window of an ascending
+// message) and the taken bits; then, a warp's share of it each, those of the
+// pairs matched by one warp.
+constexpr u32 kMatchTable = 4 * (kTableMax + 1);
+constexpr size_t kMatchSmem = kMatchTable + (kTableMax + 1) / 8 + 16;
+constexpr u32 kWarpTable = 3072 + 512;  // the window of 32 threads, or 1024 table entries
+constexpr u32 kWarpShare = kWarpTable + kWarpPair / 8;
+static_assert(kMatchTable >= 8 * (2 * kIlp * kT + 2 * kWinSlack), "the id window fits");
+static_assert(kWarpTable >= 8 * (2 * kIlp * 32 + 2 * kWinSlack) && kWarpTable >= 4 * kWarpPair,
+              "a warp's window and table fit");
+static_assert(8 * kWarpShare <= kMatchSmem, "eight warps' shares fit");
+
+// The pairs of the match list, a block each, claimed one by one; then the
+// small ones, a warp each.
+__global__ void __launch_bounds__(kT, kPerSm) codec_match_kernel(TileArgs A) {
+  extern __shared__ __align__(16) uint8_t dyn[];
+  __shared__ u32 sm32[33];
+  __shared__ u32 s_next, s_cnt[kT / 32];
+  const u32 n = A.scal[TS_ITEMS], n_small = A.scal[TS_SMALL], shift = A.scal[TS_SHIFT];
+  const u32 epoch = *A.E.epoch;
+  if (n) {
+    SmemTable tb;
+    tb.tbl = reinterpret_cast<unsigned short*>(dyn);
+    tb.bits = reinterpret_cast<u32*>(dyn + kMatchTable);
+    for (;;) {
+      const u32 it = claim(A.scal + TS_TICKET_MATCH, n, &s_next);
+      if (it == ~0u) break;
+      const u32 p = A.item_pair[it];
+      const TilePair x = A.pair[p];
+      if (x.m > kTableMax) big_build(A, x, p, it - x.item0, epoch);
+      else match_pair<kT>(A, x, p, shift, tb, reinterpret_cast<u64*>(dyn), s_cnt, sm32);
+      __syncthreads();
+    }
+  }
+  const u32 warp = threadIdx.x >> 5;
+  uint8_t* share = dyn + warp * kWarpShare;
+  SmemTable tb;
+  tb.tbl = reinterpret_cast<unsigned short*>(share);
+  tb.bits = reinterpret_cast<u32*>(share + kWarpTable);
+  for (u32 i = blockIdx.x * (kT / 32) + warp; i < n_small; i += gridDim.x * (kT / 32)) {
+    const u32 p = A.small_pair[i];
+    const TilePair x = A.pair[p];
+    match_pair<32>(A, x, p, shift, tb, reinterpret_cast<u64*>(share), s_cnt + warp, nullptr);
+    __syncwarp();
+  }
+}
+
+// Slots of the big pairs: ids looked up in the pair's hash segment, the taken
+// records marked; the block that finishes a pair's last tile lists its new
+// records.
+__global__ void __launch_bounds__(kT) codec_bigmatch_kernel(TileArgs A) {
+  __shared__ u32 sm32[33];
+  __shared__ u32 s_next, s_last, s_hits[kBigTile / 32];
+  static_assert(kBigTile == 1024, "one warp adds an item's hits up");
+  const u32 n = A.scal[TS_BIG];
+  if (n == 0) return;
+  const u32 shift = A.scal[TS_SHIFT];
+  const EncArgs& E = A.E;
+  const u32 epoch = *E.epoch;
+  for (;;) {
+    const u32 it = claim(A.scal + TS_TICKET_BIG, n, &s_next);
+    if (it == ~0u) return;
+    const u32 p = A.big_pair[it];
+    const TilePair x = A.pair[p];
+    const u32 j0 = (it - x.big0) * kBigTile;
+    const u64 base = seg_base(x.g_lo, p), size = seg_size(x.m);
+    u32* bits = big_bits(A, x, p);
+    u64 id[kIlp], at[kIlp];
+    U64x2 e[kIlp];
+    bool live[kIlp];
+#pragma unroll
+    for (u32 i = 0; i < kIlp; ++i) {
+      const u32 j = j0 + i * kT + threadIdx.x;
+      live[i] = j < x.r;
+      id[i] = live[i] ? ref_id(E, p, x.ro, j) : 0;
+    }
+#pragma unroll
+    for (u32 i = 0; i < kIlp; ++i) {
+      at[i] = seg_start(id[i], size);
+      e[i] = live[i] ? ldx<true>(E.seg + base + at[i]) : U64x2{0, 0};
+    }
+    u32 k[kIlp];
+#pragma unroll
+    for (u32 i = 0; i < kIlp; ++i) {
+      k[i] = kNoMatch;
+      if (!live[i] || (u32)(e[i].a >> 32) != epoch) continue;
+      if (e[i].b == id[i]) {
+        k[i] = (u32)e[i].a;
+      } else {
+        k[i] = seg_lookup_from<true>(E.seg, epoch, base, size, 0, id[i],
+                                     at[i] + 1 == size ? 0 : at[i] + 1);
+      }
+    }
+    u32 old[kIlp];
+#pragma unroll
+    for (u32 i = 0; i < kIlp; ++i)
+      old[i] = k[i] != kNoMatch ? atomicOr(bits + (k[i] >> 5), 1u << (k[i] & 31u)) : 0u;
+#pragma unroll
+    for (u32 i = 0; i < kIlp; ++i) {
+      if (!live[i]) continue;
+      if (k[i] != kNoMatch && ((old[i] >> (k[i] & 31u)) & 1u)) {
+        latch(E.st, TERA_EINVAL);  // a second slot with the same id: that slot is a hole
+        k[i] = kNoMatch;
+      }
+      E.slot_src[x.ro + j0 + i * kT + threadIdx.x] =
+          k[i] != kNoMatch ? (u32)(x.g_lo + k[i]) : kNoMatch;
+    }
+    // the matches of the slot tiles this item is made of
+#pragma unroll
+    for (u32 i = 0; i < kIlp; ++i) {
+      const u32 hits = __ballot_sync(0xFFFFFFFFu, live[i] && k[i] != kNoMatch);
+      if ((threadIdx.x & 31) == 0) s_hits[i * (kT / 32) + (threadIdx.x >> 5)] = (u32)__popc(hits);
+    }
+    __syncthreads();
+    if (threadIdx.x < kBigTile / 32) {
+      const u32 mine = s_hits[threadIdx.x], per = 1u << (shift - 5);
+      const u32 found = warp_sum(mine);
+      u32 c = 0;
+      if (threadIdx.x < kBigTile >> shift)
+        for (u32 i = 0; i < per; ++i) c += s_hits[threadIdx.x * per + i];
+      const u32 t = (j0 >> shift) + threadIdx.x;
+      if (threadIdx.x < kBigTile >> shift && t < x.nst) A.before[x.unit0 + t] = c;
+      if (threadIdx.x == 0 && found)
+        atomicAdd(A.tot + (u64)p * PT_COUNT + PT_MATCHED, (u64)found);
+    }
+    __threadfence();  // the bits before the count of finished tiles
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(A.done + p, 1u) + 1u == x.nbig;
+    __syncthreads();
+    if (s_last) {
+      __threadfence();
+      new_list<kT, true>(A, x, bits, sm32);
+      sum_tiles<kT>(A, x, sm32);
+    }
+    __syncthreads();
+  }
+}
+
+// ---------------- sizes of the predictor's forms ----------------
+
+// Predictor: the XOR and residual payload bytes of every slot tile, added up
+// per pair (they choose the message mode), and the training samples.
+__global__ void __launch_bounds__(kT, kPerSm) codec_sizes_kernel(TileArgs A) {
+  __shared__ U64x2 sm[33];
+  const EncArgs& E = A.E;
+  const u32 n = A.scal[TS_UNITS], shift = A.scal[TS_SHIFT];
+  for (u32 u = blockIdx.x; u < n; u += gridDim.x) {
+    const u32 p = A.unit_pair[u];
+    const TilePair x = A.pair[p];
+    const u32 tile = u - x.unit0;
+    if (tile >= x.nst) continue;
+    const u64 j = ((u64)tile << shift) + threadIdx.x;
+    u64 bx = 0, br = 0;
+    if (threadIdx.x < 1u << shift && j < x.r) {
+      if (E.pr.samples) E.pr.samples[(u64)kSampleFloats * (x.ro + j) + 11] = 0.0f;
+      const u32 g = E.slot_src[x.ro + j];
+      if (g != kNoMatch) {
+        const Rec R = load_rec(E.ref + (x.ro + p + 1 + j) * kRecBytes);
+        const Rec M = load_rec(E.rec + ((u64)g + p + 1) * kRecBytes);
+        u32 b = 0;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) b += sig_bytes(M.w[w] ^ R.w[w]);
+        bx = b;
+        br = pred_slot<true>(E, p, j, x.r, x.mode, R, M, b);
+      }
+    }
+    U64x2 tot;
+    block_excl_scan2(U64x2{bx, br}, sm, &tot);
+    if (threadIdx.x == 0) {
+      u64* t = A.tot + (u64)p * PT_COUNT;
+      if (tot.a) atomicAdd(t + PT_XOR, tot.a);
+      if (tot.b) atomicAdd(t + PT_RES, tot.b);
+    }
+  }
+}
+
+// The new-record ranks [*lo, *hi) of unit i of a pair's nnu units.
+__device__ __forceinline__ void new_range(u32 n_new, u32 nnu, u32 i, u32 shift, u32* lo, u32* hi) {
+  u32 per = (n_new + nnu - 1u) / nnu;
+  per = (per + (1u << shift) - 1u) >> shift << shift;
+  const u64 a = (u64)per * i, b = a + per;
+  *lo = a < n_new ? (u32)a : n_new;
+  *hi = b < n_new ? (u32)b : n_new;
+}
+
+// Message record of new rank i.
+__device__ __forceinline__ u64 new_record(const TileArgs& A, const TilePair& x, u32 i) {
+  return x.r ? A.new_idx[x.g_lo + i] : i;
+}
+
+// ---------------- encode, wire, decode: one warp a tile ----------------
+//
+// A warp carries a tile in steps of 32 entries; nothing is shared between
+// warps, so there are no barriers, and a pair of a few records costs one warp
+// one step.  Four lanes hold a record, 16 bytes each, eight records at a time:
+// a load or store of the warp then covers whole cache lines (four to eight,
+// where a record a lane covers sixteen to thirty-two with every one of its four
+// loads, and the L1 is what bounds the kernel), and the lanes' order is the
+// order of the payload's words, so one scan over the lanes places them.
+
+constexpr u32 kWarps = kT / 32;
+// a warp's payload stage: up to 15 bytes carried from the step before, 32
+// records, and what the copies read or clear past the bytes
+constexpr u32 kStage = 16 + 32 * kRecBytes + 32;
+constexpr u32 kRows = 32 * kRecBytes;  // a step's reference records
+constexpr size_t kEncSmem = kWarps * (kStage + 2 * kRows);  // reference and message rows
+constexpr size_t kDecSmem = kWarps * (2 * kStage + 2 * kRows);
+
+__device__ __forceinline__ void copy16(void* dst, const void* src) {
+  const u32 d = (u32)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" : : "r"(d), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copies_commit() {
+  asm volatile("cp.async.commit_group;" : : : "memory");
+}
+template <int N>
+__device__ __forceinline__ void copies_wait() {  // all but the last N groups
+  asm volatile("cp.async.wait_group %0;" : : "n"(N) : "memory");
+}
+
+// What a tile's warp needs of its pair.
+struct Tile {
+  TilePair x;
+  u32 p, local;
+  u32 n_new;
+};
+
+__device__ __forceinline__ Tile tile_of(const TileArgs& A, u32 u, u32 p) {
+  Tile t;
+  t.p = p;
+  t.x = A.pair[p];
+  t.local = u - t.x.unit0;
+  t.n_new = t.x.m - (u32)A.tot[(u64)p * PT_COUNT + PT_MATCHED];
+  return t;
+}
+
+template <bool PR>
+__device__ __forceinline__ u64 message_mode(const TileArgs& A, const Tile& t) {
+  if constexpr (PR) {
+    const u64* tot = A.tot + (u64)t.p * PT_COUNT;
+    if (A.E.pr.params && A.E.pr.allow_residual && t.x.mode == TERA_MODE_XOR &&
+        tot[PT_RES] < tot[PT_XOR])
+      return kModeResidual;
+  }
+  return t.x.mode;
+}
+
+// Where the records of a pair lie in the receive buffer; until the decode it
+// holds the tiles' packed payload, each tile's from its first record's place.
+__device__ __forceinline__ uint8_t* payload_place(const TileArgs& A, const Tile& t, u64 record) {
+  return A.D.recv + (t.x.g_lo + t.p + 1 + record) * kRecBytes;
+}
+
+// Two words of a record, and their significant bytes.
+struct Piece {
+  u64 a, b;
+};
+__device__ __forceinline__ Piece load_piece(const uint8_t* rec, u32 q) {
+  const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(rec + 16 * q);
+  return Piece{v.x, v.y};
+}
+__device__ __forceinline__ void store_piece(uint8_t* rec, u32 q, const Piece& v) {
+  *reinterpret_cast<ulonglong2*>(rec + 16 * q) = make_ulonglong2(v.a, v.b);
+}
+
+// Exclusive offsets of four steps' lane counts (each below 2^16 in all), in
+// the order step, lane; returns the total.  Two counts a word, so two scans.
+__device__ __forceinline__ u32 scan4(const u32 c[4], u32 off[4]) {
+  const u32 lo = c[0] | (c[1] << 16), hi = c[2] | (c[3] << 16);
+  const u32 il = warp_incl_scan<u32>(lo), ih = warp_incl_scan<u32>(hi);
+  const u32 tl = __shfl_sync(0xFFFFFFFFu, il, 31), th = __shfl_sync(0xFFFFFFFFu, ih, 31);
+  const u32 t0 = tl & 0xFFFFu, t1 = t0 + (tl >> 16), t2 = t1 + (th & 0xFFFFu);
+  off[0] = (il & 0xFFFFu) - c[0];
+  off[1] = t0 + (il >> 16) - c[1];
+  off[2] = t1 + (ih & 0xFFFFu) - c[2];
+  off[3] = t2 + (ih >> 16) - c[3];
+  return t2 + (th >> 16);
+}
+
+// Payload of the warp's next 32 entries (d: this lane's entry's words, code:
+// their lengths, vb bytes in all) behind the *bytes already packed at out:
+// whole 16-byte pieces are stored, the rest stays at the start of the stage.
+// An entry a lane: neighbouring lanes' bytes are then mostly in different
+// words of the stage (with two words of a record a lane the lanes' ORs met in
+// the same words: 370 against 275 us on a blob population's 6.5 M records).
+__device__ __forceinline__ void pack_step(uint8_t* st, uint8_t* out, const Rec& d, u32 code, u32 vb,
+                                          u32* bytes) {
+  const u32 lane = threadIdx.x & 31;
+  const u32 incl = warp_incl_scan<u32>(vb);
+  const u32 total = __shfl_sync(0xFFFFFFFFu, incl, 31);
+  if (total == 0) return;
+  const u32 fill = *bytes & 15u, end = fill + total;
+  for (u32 c = 1 + lane; c < ((end + 15u) >> 4) + 1u; c += 32)
+    *reinterpret_cast<uint4*>(st + (c << 4)) = make_uint4(0u, 0u, 0u, 0u);
+  __syncwarp();
+  u32 o = fill + incl - vb;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) {
+    const u32 L = (code >> (4 * w)) & 0xFu;
+    if (__any_sync(0xFFFFFFFFu, L)) {
+      stage_or(st, o, d.w[w], L);
+      o += L;
+    }
+  }
+  __syncwarp();
+  const u32 whole = end >> 4;
+  uint8_t* to = out + (*bytes - fill);
+  for (u32 c = lane; c < whole; c += 32)
+    *reinterpret_cast<uint4*>(to + (c << 4)) = *reinterpret_cast<const uint4*>(st + (c << 4));
+  if (whole) {
+    const uint4 rest = *reinterpret_cast<const uint4*>(st + (whole << 4));
+    __syncwarp();
+    if (lane == 0) *reinterpret_cast<uint4*>(st) = rest;
+  }
+  *bytes += total;
+  __syncwarp();
+}
+
+// A step's records in shared memory: piece k (16 bytes) of record e at row e,
+// place (k + e / 2) mod 4, so that eight lanes reading piece k of eight
+// consecutive records meet no bank twice.
+__device__ __forceinline__ u32 row_at(u32 e, u32 k) { return e * kRecBytes + (((k + (e >> 1)) & 3u) << 4); }
+
+__device__ __forceinline__ Rec row_rec(const uint8_t* rows, u32 e) {
+  Rec r;
+#pragma unroll
+  for (u32 k = 0; k < 4; ++k) {
+    const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(rows + row_at(e, k));
+    r.w[2 * k] = v.x;
+    r.w[2 * k + 1] = v.y;
+  }
+  return r;
+}
+
+// The step's message records (rows) named by `hits`, in order, to the new
+// sender reference from record g on, and their ids to the id column.
+__device__ __forceinline__ void store_next(const EncArgs& E, u32 p, u64 g, const uint8_t* rows,
+                                           u32 hits, u64 id) {
+  const u32 lane = threadIdx.x & 31, q = lane & 3;
+  uint8_t* to = E.ref_next + (g + p + 1) * kRecBytes;
+#pragma unroll
+  for (int s = 0; s < 4; ++s) {
+    const u32 e = 8 * s + (lane >> 2);
+    if (!(hits >> e & 1u)) continue;
+    const u32 k = (u32)__popc(hits & ((1u << e) - 1u));
+    if (!in_bounds(E.st, g + k, E.pair_off[p], E.pair_off[p + 1])) continue;
+    *reinterpret_cast<ulonglong2*>(to + (u64)k * kRecBytes + 16 * q) =
+        *reinterpret_cast<const ulonglong2*>(rows + row_at(e, q));
+  }
+  if (E.ref_ids_next && (hits >> lane & 1u)) {
+    const u64 k = g + (u32)__popc(hits & ((1u << lane) - 1u));
+    if (in_bounds(E.st, k, E.pair_off[p], E.pair_off[p + 1])) E.ref_ids_next[k] = id;
+  }
+}
+
+template <bool PR>
+__global__ void __launch_bounds__(kT, kEncPerSm) codec_encode_kernel(TileArgs A) {
+  extern __shared__ __align__(16) uint8_t dyn[];
+  const EncArgs& E = A.E;
+  const u32 warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const u32 r8 = lane >> 2, q = lane & 3;  // this lane's record of each eight, and its piece
+  uint8_t* st = dyn + warp * (kStage + 2 * kRows);
+  uint8_t* rows = st + kStage;
+  const u32 n = A.scal[TS_UNITS], shift = A.scal[TS_SHIFT];
+  const u32 epoch = *E.epoch;
+  const u32 stride = gridDim.x * kWarps;
+  u32 u = blockIdx.x * kWarps + warp;
+  u32 p_next = u < n ? A.unit_pair[u] : 0u;
+  for (; u < n; u += stride) {
+    const Tile t = tile_of(A, u, p_next);
+    if (u + stride < n) p_next = A.unit_pair[u + stride];
+    const u32 p = t.p;
+    u32* codes = reinterpret_cast<u32*>(E.wire + t.x.w_off + kHdrBytes);
+    if (lane == 0) *reinterpret_cast<uint4*>(st) = make_uint4(0u, 0u, 0u, 0u);
+    __syncwarp();
+    u32 bytes = 0;
+    uint8_t* out;
+    if (t.local < t.x.nst) {
+      const u32 j0 = t.local << shift;
+      const u32 nj = t.x.r - j0 < (1u << shift) ? t.x.r - j0 : 1u << shift;
+      const u32* src = E.slot_src + t.x.ro + j0;
+      const uint8_t* ref = E.ref + (t.x.ro + p + 1 + j0) * kRecBytes;
+      const uint8_t* rec = E.rec + ((u64)p + 1) * kRecBytes;
+      u64 pos = A.before[u];
+      out = payload_place(A, t, pos);
+      bool residual = false;
+      if constexpr (PR) residual = message_mode<PR>(A, t) == kModeResidual;
+      // a step's records are asked for before the step before is packed, their
+      // places a step earlier still
+      const auto request = [&](u32 i0, u32 g) {
+        const u32 hits = __ballot_sync(0xFFFFFFFFu, g != kNoMatch);
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+          const u32 e = 8 * s + r8, gs = __shfl_sync(0xFFFFFFFFu, g, e);
+          if (hits >> e & 1u) {
+            copy16(rows + row_at(e, q), ref + (u64)(i0 + e) * kRecBytes + 16 * q);
+            copy16(rows + kRows + row_at(e, q), rec + (u64)gs * kRecBytes + 16 * q);
+          }
+        }
+        copies_commit();
+        return hits;
+      };
+      u32 g_next = 32 + lane < nj ? src[32 + lane] : kNoMatch;
+      u32 hits = request(0, lane < nj ? src[lane] : kNoMatch);
+      for (u32 i0 = 0; i0 < nj; i0 += 32) {
+        const u32 g_now = g_next;
+        g_next = i0 + 64 + lane < nj ? src[i0 + 64 + lane] : kNoMatch;
+        copies_wait<0>();
+        __syncwarp();
+        const bool hit = hits >> lane & 1u;
+        Rec d{};
+        u32 code = 0, vb = 0;
+        u64 id = 0;
+        if (hit) {
+          d = row_rec(rows, lane);
+          const Rec cur = row_rec(rows + kRows, lane);
+          id = cur.w[0];
+          const u64* ps = nullptr;
+          if constexpr (PR) {
+            if (E.pr.hist_next) {
+              uint8_t* hn = E.pr.hist_next +
+                            kHistBytes * (t.x.g_lo + pos + (u32)__popc(hits & ((1u << lane) - 1u)));
+              if (E.pr.hist) {
+                const Hist H = load_hist(E.pr.hist + kHistBytes * (t.x.ro + j0 + i0 + lane));
+                store_hist_next(hn, &d, &H);
+              } else {
+                store_hist_next(hn, &d, nullptr);
+              }
+            }
+            if (residual) {
+              ps = E.pr.pscr + 4 * (t.x.ro + j0 + i0 + lane);
+              if (!ps[3]) ps = nullptr;
+            }
+          }
+#pragma unroll
+          for (int w = 0; w < 8; ++w) {
+            if (PR && ps && w >= 1 && w <= 3) d.w[w] = zigzag(cur.w[w] - ps[w - 1]);
+            else d.w[w] ^= cur.w[w];
+          }
+        }
+        __syncwarp();
+        store_next(E, p, t.x.g_lo + pos, rows + kRows, hits, id);
+        __syncwarp();  // the rows are read: the next step's may come
+        u32 hits_next = 0;
+        if (i0 + 32 < nj) hits_next = request(i0 + 32, g_now);
+        if (hit) code = rec_code(d, &vb);
+        if (i0 + lane < nj && in_bounds(E.st, j0 + i0 + lane, 0, (u64)t.x.r + t.n_new))
+          codes[j0 + i0 + lane] = hit ? code : 0xFu;  // 0xF: placeholder
+        pack_step(st, out, d, code, vb, &bytes);
+        pos += (u32)__popc(hits);
+        hits = hits_next;
+      }
+    } else {
+      // new records: rank i's code and new-reference record have known places
+      const u64 matched = (u64)t.x.m - t.n_new;
+      u32 lo, hi;
+      new_range(t.n_new, t.x.nnu, t.local - t.x.nst, shift, &lo, &hi);
+      out = payload_place(A, t, matched + lo);
+      for (u32 i0 = lo; i0 < hi; i0 += 32) {
+        const u32 hits = hi - i0 >= 32 ? 0xFFFFFFFFu : (1u << (hi - i0)) - 1u;
+        const u64 k = i0 + lane < hi ? new_record(A, t.x, i0 + lane) : 0;
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+          const u32 e = 8 * s + r8;
+          const u64 ks = __shfl_sync(0xFFFFFFFFu, k, e);
+          if (i0 + e < hi)
+            copy16(rows + row_at(e, q), E.rec + (t.x.g_lo + ks + p + 1) * kRecBytes + 16 * q);
+        }
+        copies_commit();
+        copies_wait<0>();
+        __syncwarp();
+        Rec d{};
+        u32 code = 0, vb = 0;
+        if (i0 + lane < hi) {
+          d = row_rec(rows, lane);
+          // an id that occurs twice in a big pair's message: the other record is found
+          if (t.x.m > kTableMax &&
+              seg_lookup<true>(E.seg, epoch, p, t.x.g_lo, t.x.m, d.w[0]) != (u32)(t.x.g_lo + k))
+            latch(E.st, TERA_EINVAL);
+          code = rec_code(d, &vb);
+          if (in_bounds(E.st, i0 + lane, 0, t.n_new)) codes[t.x.r + i0 + lane] = code;
+          if constexpr (PR) {
+            if (E.pr.hist_next)
+              store_hist_next(E.pr.hist_next + kHistBytes * (t.x.g_lo + matched + i0 + lane),
+                              nullptr, nullptr);
+          }
+        }
+        store_next(E, p, t.x.g_lo + matched + i0, rows, hits, d.w[0]);
+        pack_step(st, out, d, code, vb, &bytes);
+        __syncwarp();
+      }
+    }
+    // the last piece may carry zeros past the bytes, still inside the records' place
+    if ((bytes & 15u) && lane == 0)
+      *reinterpret_cast<uint4*>(out + (bytes & ~15u)) = *reinterpret_cast<const uint4*>(st);
+    if (lane == 0) A.bytes[u] = bytes;
+    __syncwarp();
+  }
+}
+
+// Header, padding, iteration totals and the new reference's header of a pair,
+// by the warp that knows the pair's payload.
+__device__ __forceinline__ void finish_message(const TileArgs& A, const Tile& t, u64 payload,
+                                               u64 mode) {
+  const EncArgs& E = A.E;
+  const int lane = threadIdx.x & 31;
+  const u32 p = t.p;
+  const u64 r = t.x.r, n_new = t.n_new;
+  const u64 body = (u64)kHdrBytes + 4 * (r + n_new) + payload;
+  const u64 msg = round16(body);
+  const u64 matched = (u64)t.x.m - n_new;
+  uint8_t* w8 = E.wire + t.x.w_off;
+  if (lane == 0) {
+    // the message fits the slab reserved for it (checked after the fact)
+    (void)in_bounds(E.st, msg, 0, E.wire_off[p + 1] - t.x.w_off + 1);
+    ulonglong2* h = reinterpret_cast<ulonglong2*>(w8);
+    h[0] = make_ulonglong2((u64)kWireMagic | ((u64)kVersion << 32) | ((u64)kRecBytes << 48),
+                           (u64)E.class_id | (mode << 32));
+    h[1] = make_ulonglong2(r, n_new);
+    h[2] = make_ulonglong2(r - matched, payload);
+    h[3] = make_ulonglong2((u64)p, msg);
+    E.wire_len[p] = msg;
+    atomicAdd(&E.stats->ref_slots, r);
+    atomicAdd(&E.stats->holes, r - matched);
+    atomicAdd(&E.stats->new_records, n_new);
+    atomicAdd(&E.stats->payload_bytes, payload);
+    atomicAdd(&E.stats->wire_bytes, msg);
+    write_taio_header(E.ref_next + (t.x.g_lo + p) * kRecBytes, E.class_id, p, t.x.m);
+    E.reset[p] = 0;
+  }
+  if (body + lane < msg) w8[body + lane] = 0;  // zero padding (< 16 bytes)
+}
+
+// A tile's payload to its place in the message, behind that of the pair's
+// tiles before it (their counts added up).
+template <bool PR>
+__global__ void __launch_bounds__(kT, kPerSm) codec_wire_kernel(TileArgs A) {
+  const EncArgs& E = A.E;
+  const u32 warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const u32 n = A.scal[TS_UNITS], shift = A.scal[TS_SHIFT];
+  const u32 stride = gridDim.x * kWarps;
+  u32 u = blockIdx.x * kWarps + warp;
+  u32 p_next = u < n ? A.unit_pair[u] : 0u;
+  for (; u < n; u += stride) {
+    const Tile t = tile_of(A, u, p_next);
+    if (u + stride < n) p_next = A.unit_pair[u + stride];
+    const u32 own = A.bytes[u];
+    u64 record;
+    bool last;
+    if (t.local < t.x.nst) {
+      record = A.before[u];
+      last = t.n_new == 0 && t.local + 1 == t.x.nst;
+    } else {
+      u32 lo, hi;
+      new_range(t.n_new, t.x.nnu, t.local - t.x.nst, shift, &lo, &hi);
+      record = (u64)t.x.m - t.n_new + lo;
+      // an entryless pair's message is its header
+      last = hi == t.n_new && (lo < hi || (t.n_new == 0 && t.x.r == 0 && t.local == 0));
+    }
+    u64 pre = 0;
+    for (u32 i = lane; i < t.local; i += 32) pre += A.bytes[t.x.unit0 + i];
+    pre = warp_sum(pre);
+    if (lane == 0) A.place[u] = pre;
+    uint8_t* pay = E.wire + t.x.w_off + kHdrBytes + 4 * ((u64)t.x.r + t.n_new);
+    if (own) warp_flush(payload_place(A, t, record), pay + pre, own);
+    if (last) finish_message(A, t, pre + own, message_mode<PR>(A, t));
+  }
+}
+
+// Tiles and their places are the encode's (both sides of the call run here); a
+// tile's payload bytes, from the codes on the wire, have to come to the
+// encode's.
+template <bool PR>
+__global__ void __launch_bounds__(kT, kDecPerSm) codec_decode_kernel(TileArgs A) {
+  extern __shared__ __align__(16) uint8_t dyn[];
+  const DecArgs& D = A.D;
+  const u32 warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const u32 r8 = lane >> 2, q = lane & 3;  // this lane's record of each eight, and its piece
+  uint8_t* stages = dyn + warp * (2 * kStage + 2 * kRows);
+  uint8_t* rows = stages + 2 * kStage;
+  const u32 n_units = A.scal[TS_UNITS], shift = A.scal[TS_SHIFT];
+  const u32 stride = gridDim.x * kWarps;
+  u32 u = blockIdx.x * kWarps + warp;
+  u32 p_next = u < n_units ? A.unit_pair[u] : 0u;
+  for (; u < n_units; u += stride) {
+    const Tile t = tile_of(A, u, p_next);
+    if (u + stride < n_units) p_next = A.unit_pair[u + stride];
+    const u32 p = t.p;
+    const u64 m = t.x.m, ns = t.x.r, n = ns + t.n_new;
+    u32 lo, hi, base = 0;  // this tile's entries [lo, hi) behind the pair's entry `base`
+    u64 pos;               // records before it
+    if (t.local < t.x.nst) {
+      lo = t.local << shift;
+      hi = t.x.r - lo < (1u << shift) ? t.x.r : lo + (1u << shift);
+      pos = A.before[u];
+    } else {
+      new_range(t.n_new, t.x.nnu, t.local - t.x.nst, shift, &lo, &hi);
+      base = t.x.r;
+      pos = m - t.n_new + lo;
+    }
+    const uint8_t* w8 = D.wire + t.x.w_off;
+    u64 mode = t.x.mode;
+    bool usable = t.x.fits != 0 && lo < hi;
+    if (PR || t.local == 0) {
+      DecHdr H;
+      const u32 err = dec_read_header<false, PR>(D, p, m, &H);
+      if (t.local == 0 && lane == 0) {
+        if (err) latch(D.st, err);
+        else if (H.ns != ns || H.nn != t.n_new) latch(D.st, TERA_ECORRUPT);
+        write_taio_header(D.recv + (t.x.g_lo + p) * kRecBytes, D.class_id, p, m);
+      }
+      usable = usable && !err;
+      mode = H.mode;
+    }
+    if (!usable) continue;
+    const u32* codes = reinterpret_cast<const u32*>(w8 + kHdrBytes) + base;
+    const uint8_t* pay = w8 + kHdrBytes + 4 * n + A.place[u];
+    const u32 want = A.bytes[u];
+    const u64 ro = D.ref_off ? D.ref_off[p] : 0;
+    const uint8_t* ref = D.ref + (ro + p + 1) * kRecBytes;
+    uint8_t* recv = D.recv + (t.x.g_lo + p + 1) * kRecBytes;
+    u32 at = 0;  // payload bytes of the steps asked for
+    // a step: what its codes say, and where its payload starts in the stage
+    struct Step {
+      u32 code, hits, records, off[4], s0;
+    };
+    bool broken = false;
+    // asks for a step's payload and reference records (a step ahead of their use)
+    const auto request = [&](u32 i0, u32 code) {
+      Step x;
+      x.code = code;
+      const DecEnt c = dec_entry(D.st, code, i0 + lane < hi ? (u64)base + i0 + lane : n, n, ns);
+      x.hits = __ballot_sync(0xFFFFFFFFu, c.vn && !c.bad);
+      x.records = __ballot_sync(0xFFFFFFFFu, c.vn);
+      const bool odd = ((i0 - lo) & 32u) != 0;
+      uint8_t* row = rows + (odd ? kRows : 0);
+      u32 b[4];
+#pragma unroll
+      for (int s = 0; s < 4; ++s) {
+        const u32 e = 8 * s + r8;
+        const u32 y = __shfl_sync(0xFFFFFFFFu, code, e) >> (8 * q);
+        const bool live = x.hits >> e & 1u;
+        b[s] = live ? (y & 0xFu) + (y >> 4 & 0xFu) : 0u;
+        if (live && base == 0 && i0 + e < ns)
+          copy16(row + (s * 32 + lane) * 16, ref + (u64)(i0 + e) * kRecBytes + 16 * q);
+      }
+      const u32 total = scan4(b, x.off);
+      const uint8_t* g = pay + at;
+      x.s0 = (u32)((uintptr_t)g & 15u);
+      // inside the tile's bytes
+      if (at + total > want) broken = true;
+      else if (total) {
+        // the slab is 16-byte aligned and padded, so the rounded range stays
+        // inside the message
+        const uint8_t* g16 = g - x.s0;
+        uint8_t* st = stages + (odd ? kStage : 0);
+        for (u32 k = lane; k < ((x.s0 + total + 15u) >> 4); k += 32)
+          copy16(st + (k << 4), g16 + (k << 4));
+      }
+      at += total;
+      copies_commit();
+      return x;
+    };
+    u32 c_next = lo + 32 + lane < hi ? codes[lo + 32 + lane] : 0u;
+    Step now = request(lo, lo + lane < hi ? codes[lo + lane] : 0u);
+    for (u32 i0 = lo; i0 < hi; i0 += 32) {
+      const bool odd = ((i0 - lo) & 32u) != 0;
+      const u32 code_next = c_next;
+      c_next = i0 + 64 + lane < hi ? codes[i0 + 64 + lane] : 0u;
+      Step next = now;
+      if (i0 + 32 < hi && !broken) {
+        next = request(i0 + 32, code_next);
+        copies_wait<1>();
+      } else {
+        copies_wait<0>();
+      }
+      __syncwarp();
+      const u32 hits = now.hits, records = now.records;
+      // inside the pair's records
+      if (pos + (u32)__popc(records) > m) broken = true;
+      if (broken) break;
+      const uint8_t* st = stages + (odd ? kStage : 0);
+      const uint8_t* row = rows + (odd ? kRows : 0);
+      const u32 i = i0 + lane;
+      if constexpr (PR) {
+        if ((hits >> lane & 1u) && D.pr.hist_next) {
+          const u64 to = pos + (u32)__popc(records & ((1u << lane) - 1u));
+          uint8_t* hn = D.pr.hist_next + kHistBytes * (t.x.g_lo + to);
+          if (base == 0 && i < ns) {
+            Rec r;
+            const u64* w = reinterpret_cast<const u64*>(ref + (u64)i * kRecBytes);
+            r.w[1] = w[1];
+            r.w[2] = w[2];
+            r.w[3] = w[3];
+            Hist h;
+            if (D.pr.hist) h = load_hist(D.pr.hist + kHistBytes * (ro + i));
+            store_hist_next(hn, &r, D.pr.hist ? &h : nullptr);
+          } else {
+            store_hist_next(hn, nullptr, nullptr);
+          }
+        }
+      }
+#pragma unroll
+      for (int s = 0; s < 4; ++s) {
+        const u32 e = 8 * s + r8;
+        const u32 y = __shfl_sync(0xFFFFFFFFu, now.code, e) >> (8 * q);
+        if (!(hits >> e & 1u)) continue;
+        const u32 la = y & 0xFu, lb = y >> 4 & 0xFu;
+        const u32 o = now.s0 + now.off[s];
+        Piece v{stage_bytes_at(st, o, la), stage_bytes_at(st, o + la, lb)};
+        if (base == 0 && i0 + e < ns) {
+          const Piece R = load_piece(row + (s * 32 + r8 * 4) * 16, q);
+          bool done = false;
+          if constexpr (PR) {
+            if (D.pr.pre && mode == kModeResidual && q < 2) {
+              const u64* ps = D.pr.pscr + 4 * (ro + i0 + e);
+              if (ps[3]) {  // words 1 to 3
+                v.a = q ? ps[1] + unzigzag(v.a) : v.a ^ R.a;
+                v.b = ps[q ? 2 : 0] + unzigzag(v.b);
+                done = true;
+              }
+            }
+          }
+          if (!done) {
+            v.a ^= R.a;
+            v.b ^= R.b;
+          }
+        }
+        const u64 to = pos + (u32)__popc(records & ((1u << e) - 1u));
+        if (in_bounds(D.st, to, 0, m)) store_piece(recv + to * kRecBytes, q, v);
+      }
+      pos += (u32)__popc(records);
+      now = next;
+      __syncwarp();
+    }
+    copies_wait<0>();
+    __syncwarp();
+    if (lane == 0 && (broken || at != want)) latch(D.st, TERA_ECORRUPT);
+  }
+}
+
+}  // namespace
+
+namespace tera {
+
+tera_status launch_tiles(tera_ctx* ctx, const EncArgs& E, const DecArgs& D, bool pr, int mode,
+                         u64 wire_cap, u64 recv_cap, cudaStream_t s) {
+  const u64 P = ctx->n_pairs;
+  tera_status st;
+  const unsigned grid = (unsigned)(ctx->num_sms * kPerSm);
+  static bool configured = false;
+  if (!configured) {
+    const void* k[] = {reinterpret_cast<const void*>(codec_encode_kernel<false>),
+                       reinterpret_cast<const void*>(codec_encode_kernel<true>),
+                       reinterpret_cast<const void*>(codec_decode_kernel<false>),
+                       reinterpret_cast<const void*>(codec_decode_kernel<true>)};
+    for (int i = 0; i < 4; ++i)
+      if (cudaFuncSetAttribute(k[i], cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)(i < 2 ? kEncSmem : kDecSmem)) != cudaSuccess)
+        return TERA_ECUDA;
+    configured = true;
+  }
+  TileArgs A;
+  A.E = E;
+  A.D = D;
+  A.pair = reinterpret_cast<TilePair*>(ctx->t_pair);
+  A.unit_pair = ctx->t_unit_pair;
+  A.item_pair = ctx->t_item_pair;
+  A.big_pair = ctx->t_big_pair;
+  A.small_pair = ctx->t_small_pair;
+  A.warps = (u32)(ctx->num_sms * kPerSm * (kT / 32));
+  A.warp_pair = P > 8ull * grid ? kWarpPair : kWarpPairFew;
+  A.before = ctx->t_before;
+  A.bytes = ctx->t_bytes;
+  A.place = ctx->t_place;
+  A.tot = ctx->t_tot;
+  A.done = ctx->t_done;
+  A.bits = ctx->t_bits;
+  A.new_idx = ctx->t_new;
+  A.scal = ctx->t_scal;
+  A.P = P;
+  const unsigned setup = (unsigned)(P == 0 ? 1 : (P + kSetupT - 1) / kSetupT);
+  U64x2* part = reinterpret_cast<U64x2*>(ctx->t_part);
+  const unsigned egrid = (unsigned)(ctx->num_sms * kEncPerSm), dgrid = (unsigned)(ctx->num_sms * kDecPerSm);
+  prof_begin(ctx, s);
+  tiles_sums_kernel<<<setup, kSetupT, 0, s>>>(A, mode, part);
+  if ((st = check_launch(ctx, "tiles_sums_kernel", s)) != TERA_OK) return st;
+  prof_begin(ctx, s);
+  tiles_place_kernel<<<setup, kSetupT, 0, s>>>(A, mode, const_cast<u64*>(E.wire_off), wire_cap,
+                                               ctx->cap_records, recv_cap, ctx->t_units,
+                                               ctx->t_items, ctx->t_bigs, ctx->d_epoch, part);
+  if ((st = check_launch(ctx, "tiles_place_kernel", s)) != TERA_OK) return st;
+  prof_begin(ctx, s);
+  codec_match_kernel<<<grid, kT, kMatchSmem, s>>>(A);
+  if ((st = check_launch(ctx, "codec_match_kernel", s)) != TERA_OK) return st;
+  if (ctx->cap_records > kTableMax) {  // a big pair needs that many records
+    prof_begin(ctx, s);
+    codec_bigmatch_kernel<<<grid, kT, 0, s>>>(A);
+    if ((st = check_launch(ctx, "codec_bigmatch_kernel", s)) != TERA_OK) return st;
+  }
+  if (pr) {
+    prof_begin(ctx, s);
+    codec_sizes_kernel<<<grid, kT, 0, s>>>(A);
+    if ((st = check_launch(ctx, "codec_sizes_kernel", s)) != TERA_OK) return st;
+  }
+  prof_begin(ctx, s);
+  if (pr) codec_encode_kernel<true><<<egrid, kT, kEncSmem, s>>>(A);
+  else codec_encode_kernel<false><<<egrid, kT, kEncSmem, s>>>(A);
+  if ((st = check_launch(ctx, "codec_encode_kernel", s)) != TERA_OK) return st;
+  prof_begin(ctx, s);
+  if (pr) codec_wire_kernel<true><<<grid, kT, 0, s>>>(A);
+  else codec_wire_kernel<false><<<grid, kT, 0, s>>>(A);
+  if ((st = check_launch(ctx, "codec_wire_kernel", s)) != TERA_OK) return st;
+  prof_begin(ctx, s);
+  if (pr) codec_decode_kernel<true><<<dgrid, kT, kDecSmem, s>>>(A);
+  else codec_decode_kernel<false><<<dgrid, kT, kDecSmem, s>>>(A);
+  return check_launch(ctx, "codec_decode_kernel", s);
+}
+
+// Bounds of the lists for `cap` slots, records and pairs P (the setup's
+// counts): tiles of slots, tiles of records that must be new, shares of
+// records; match items and bigmatch items of big pairs.  Tiles below the
+// largest size come with fewer than twice kTilesPerWarp per resident warp.
+void tile_list_bounds(u64 cap, u64 P, u64 warps, u64* units, u64* items, u64* bigs) {
+  const u64 few = 2 * kTilesPerWarp * warps;
+  const u64 most = (cap >> kMaxShift) > few ? cap >> kMaxShift : few;
+  *units = 2 * most + most / kNewShare + 5 * P + 64;
+  *items = cap / kBigTile + 2 * P + 64;
+  *bigs = cap / kBigTile + P + 64;
+}
+
+}  // namespace tera

@@ -9,7 +9,7 @@
 #include <string>
 #include <vector>
 
-#include "tera_internal.cuh"
+#include "codec.cuh"
 
 using namespace tera;
 
@@ -316,6 +316,33 @@ tera_status ensure_batched(tera_ctx* ctx) {
   if ((st = alloc_dev(ctx->b_tsum, tsum)) != TERA_OK) return st;
   ctx->b_items_cap = items;
   ctx->b_tsum_cap = tsum;
+  return TERA_OK;
+}
+
+tera_status ensure_tiles(tera_ctx* ctx) {
+  if (ctx->t_cap >= ctx->cap_records && ctx->t_pair) return TERA_OK;
+  cudaDeviceSynchronize();
+  const u64 P = ctx->n_pairs, cap = ctx->cap_records;
+  tera_status st;
+  ctx->t_cap = 0;
+  if (!ctx->t_pair) {
+    if ((st = alloc_dev(ctx->t_tot, P * 4)) != TERA_OK) return st;
+    if ((st = alloc_dev(ctx->t_done, P)) != TERA_OK) return st;
+    if ((st = alloc_dev(ctx->t_scal, 8)) != TERA_OK) return st;
+    if ((st = alloc_dev(ctx->t_part, 4 * (P / 1024 + 1))) != TERA_OK) return st;
+    if ((st = alloc_dev(ctx->t_small_pair, P)) != TERA_OK) return st;
+    if ((st = alloc_dev(ctx->t_pair, P * 8)) != TERA_OK) return st;
+  }
+  tile_list_bounds(cap, P, (u64)ctx->num_sms * 32, &ctx->t_units, &ctx->t_items, &ctx->t_bigs);
+  if ((st = alloc_dev(ctx->t_unit_pair, ctx->t_units)) != TERA_OK) return st;
+  if ((st = alloc_dev(ctx->t_item_pair, ctx->t_items)) != TERA_OK) return st;
+  if ((st = alloc_dev(ctx->t_big_pair, ctx->t_bigs)) != TERA_OK) return st;
+  if ((st = alloc_dev(ctx->t_before, ctx->t_units)) != TERA_OK) return st;
+  if ((st = alloc_dev(ctx->t_bytes, ctx->t_units)) != TERA_OK) return st;
+  if ((st = alloc_dev(ctx->t_place, ctx->t_units)) != TERA_OK) return st;
+  if ((st = alloc_dev(ctx->t_bits, cap / 32 + P + 2)) != TERA_OK) return st;
+  if ((st = alloc_dev(ctx->t_new, cap)) != TERA_OK) return st;
+  ctx->t_cap = cap;
   return TERA_OK;
 }
 
@@ -712,6 +739,20 @@ tera_status tera_ctx_destroy(tera_ctx* c) {
   free_dev(c->b_tsum);
   free_dev(c->b_tbase);
   free_dev(c->b_part);
+  free_dev(c->t_pair);
+  free_dev(c->t_unit_pair);
+  free_dev(c->t_item_pair);
+  free_dev(c->t_big_pair);
+  free_dev(c->t_small_pair);
+  free_dev(c->t_before);
+  free_dev(c->t_bytes);
+  free_dev(c->t_place);
+  free_dev(c->t_tot);
+  free_dev(c->t_done);
+  free_dev(c->t_bits);
+  free_dev(c->t_new);
+  free_dev(c->t_scal);
+  free_dev(c->t_part);
   free_dev(c->m_tile_cnt);
   free_dev(c->m_tile_base);
   free_dev(c->m_from);

@@ -126,6 +126,23 @@ struct tera_ctx {
   uint64_t b_tsum_cap;
   tera::u64* b_tbase;    // [P] first tile total of each team pair
   tera::u64* b_part;     // [4 * (P / 1024 + 1)] block sums of the setup's first launch
+  // batched codec over tiles (codec_tiles.cu)
+  uint64_t t_cap;          // records the lists below are sized for (0: none)
+  tera::u64 t_units, t_items, t_bigs;  // entries of the lists
+  tera::u64* t_pair;       // [P * 8] per-pair facts
+  uint32_t* t_unit_pair;   // [t_units] pair of each tile
+  uint32_t* t_item_pair;   // [t_items] pair of each match item
+  uint32_t* t_big_pair;    // [t_bigs] pair of each tile of a big pair
+  uint32_t* t_small_pair;  // [P] pairs matched by one warp
+  uint32_t* t_before;      // [t_units] matched slots before each tile
+  uint32_t* t_bytes;       // [t_units] payload bytes of each tile
+  tera::u64* t_place;      // [t_units] payload bytes of the pair before each tile
+  tera::u64* t_tot;        // [P * 4] matched records, XOR and residual bytes
+  uint32_t* t_done;        // [P] finished tiles of a big pair
+  uint32_t* t_bits;        // taken records of big pairs
+  uint32_t* t_new;         // [t_cap] new records of each pair
+  uint32_t* t_scal;        // [8] list lengths and claim tickets
+  tera::u64* t_part;       // [4 * (P / 1024 + 1)] block sums of the setup's first launch
   // agent migration (migrate.cu)
   uint64_t m_cap_agents;   // agents the tile arrays cover
   uint64_t m_cap_leavers;  // leavers the list and sort buffers hold
@@ -164,6 +181,8 @@ tera_status launch_unit_map(tera_ctx* ctx, u32 p0, u64 npr, cudaStream_t s);
 tera_status ensure_pred(tera_ctx* ctx);
 // Scratch of the batched codec.
 tera_status ensure_batched(tera_ctx* ctx);
+// Scratch of the batched codec over tiles.
+tera_status ensure_tiles(tera_ctx* ctx);
 // Scratch of agent migration for n agents and up to `leavers` leavers.
 tera_status ensure_migrate(tera_ctx* ctx, uint64_t n, uint64_t leavers);
 
