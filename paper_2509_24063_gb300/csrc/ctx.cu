@@ -33,70 +33,62 @@ tera_status alloc_dev(T*& p, size_t count) {
   return TERA_OK;
 }
 
-// ---- generic exclusive scan of u32 values (reduce, scan partials, down-sweep) ----
-
-__global__ void scan_reduce_kernel(const u32* __restrict__ in, u64 n, u64* __restrict__ part) {
+// ---- generic exclusive scan of u32 values ----
+//
+// One launch: a block scans kScanChunk values and finds the sum before them by
+// a look-back over the chunks (state[i] of chunk i, then the claim ticket; all
+// zero at launch).  A single chunk needs neither.  Three launches before
+// (chunk sums, a block scanning them, the chunks again): 12 to 17 us of an
+// iteration's chain each time, where one is 4.
+__global__ void __launch_bounds__(kScanThreads)
+    scan_kernel(const u32* __restrict__ in, u64 n, u64* __restrict__ out64,
+                u32* __restrict__ out32, u64* __restrict__ state, DevStatus* st) {
   __shared__ u64 sm[33];
-  const u64 base = (u64)blockIdx.x * kScanChunk;
-  u64 s = 0;
-#pragma unroll
-  for (int k = 0; k < kScanPerThread; ++k) {
-    u64 i = base + (u64)k * kScanThreads + threadIdx.x;
-    if (i < n) s += in[i];
+  __shared__ u64 s_pre;
+  __shared__ u32 s_tile;
+  __shared__ int s_fine;
+  u32 tile = 0;
+  if (gridDim.x > 1) {
+    if (threadIdx.x == 0) s_tile = atomicAdd(reinterpret_cast<u32*>(state + gridDim.x), 1u);
+    __syncthreads();
+    tile = s_tile;
   }
-  s = warp_sum(s);
-  if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = s;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    u64 t = threadIdx.x < (kScanThreads / 32) ? sm[threadIdx.x] : 0;
-    t = warp_sum(t);
-    if (threadIdx.x == 0) part[blockIdx.x] = t;
-  }
-}
-
-// Single block: exclusive scan of part[0..m) in place, total to part[m].
-__global__ void scan_partials_kernel(u64* part, u64 m) {
-  __shared__ u64 sm[33];
-  u64 carry = 0;
-  for (u64 base = 0; base < m; base += kScanThreads) {
-    u64 i = base + threadIdx.x;
-    u64 v = i < m ? part[i] : 0;
-    u64 tot;
-    u64 ex = block_excl_scan<u64>(v, sm, &tot);
-    if (i < m) part[i] = carry + ex;
-    carry += tot;
-  }
-  if (threadIdx.x == 0) part[m] = carry;
-}
-
-__global__ void scan_down_kernel(const u32* __restrict__ in, u64 n, const u64* __restrict__ part,
-                                 u64* __restrict__ out64, u32* __restrict__ out32) {
-  __shared__ u64 sm[33];
-  const u64 base = (u64)blockIdx.x * kScanChunk + (u64)threadIdx.x * kScanPerThread;
+  const u64 base = (u64)tile * kScanChunk + (u64)threadIdx.x * kScanPerThread;
   u32 v[kScanPerThread];
   u64 s = 0;
 #pragma unroll
   for (int k = 0; k < kScanPerThread; ++k) {
-    u64 i = base + k;
+    const u64 i = base + k;
     v[k] = i < n ? in[i] : 0u;
     s += v[k];
   }
   u64 tot;
-  u64 ex = block_excl_scan<u64>(s, sm, &tot);
-  u64 run = part[blockIdx.x] + ex;
+  u64 run = block_excl_scan<u64>(s, sm, &tot);
+  if (gridDim.x > 1) {
+    if (threadIdx.x < 32) {
+      u64 pre;
+      const bool fine = lb_warp_sum(state, tile, tot, st, &pre);
+      if (threadIdx.x == 0) {
+        s_pre = pre;
+        s_fine = fine;
+      }
+    }
+    __syncthreads();
+    if (!s_fine) return;  // the abort flag is set: nothing reads the result
+    run += s_pre;
+  }
 #pragma unroll
   for (int k = 0; k < kScanPerThread; ++k) {
-    u64 i = base + k;
+    const u64 i = base + k;
     if (i < n) {
       if (out64) out64[i] = run;
       if (out32) out32[i] = (u32)run;
     }
     run += v[k];
   }
-  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
-    u64 total = part[gridDim.x];
-    if (out64) out64[n] = total;
-    if (out32) out32[n] = (u32)total;
+  if (tile == gridDim.x - 1 && threadIdx.x == kScanThreads - 1) {
+    if (out64) out64[n] = run;
+    if (out32) out32[n] = (u32)run;
   }
 }
 
@@ -217,23 +209,11 @@ tera_status scan_u32(tera_ctx* ctx, const u32* in, u64* out64, u32* out32, u64 n
   if (st != TERA_OK) return st;
   u64 chunks = (n + kScanChunk - 1) / kScanChunk;
   if (chunks == 0) chunks = 1;
-  if (chunks == 1) {
-    cudaMemsetAsync(ctx->scan_part, 0, sizeof(u64), s);
-    // part[1] = total is written by the down kernel through part[gridDim.x]; compute it
-    prof_begin(ctx, s);
-    scan_reduce_kernel<<<1, kScanThreads, 0, s>>>(in, n, ctx->scan_part + 1);
-    if ((st = check_launch(ctx, "scan_reduce_kernel", s)) != TERA_OK) return st;
-  } else {
-    prof_begin(ctx, s);
-    scan_reduce_kernel<<<(unsigned)chunks, kScanThreads, 0, s>>>(in, n, ctx->scan_part);
-    if ((st = check_launch(ctx, "scan_reduce_kernel", s)) != TERA_OK) return st;
-    prof_begin(ctx, s);
-    scan_partials_kernel<<<1, kScanThreads, 0, s>>>(ctx->scan_part, chunks);
-    if ((st = check_launch(ctx, "scan_partials_kernel", s)) != TERA_OK) return st;
-  }
+  if (chunks > 1) cudaMemsetAsync(ctx->scan_part, 0, sizeof(u64) * (chunks + 1), s);
   prof_begin(ctx, s);
-  scan_down_kernel<<<(unsigned)chunks, kScanThreads, 0, s>>>(in, n, ctx->scan_part, out64, out32);
-  return check_launch(ctx, "scan_down_kernel", s);
+  scan_kernel<<<(unsigned)chunks, kScanThreads, 0, s>>>(in, n, out64, out32, ctx->scan_part,
+                                                        ctx->d_status);
+  return check_launch(ctx, "scan_kernel", s);
 }
 
 tera_status ensure_agents(tera_ctx* ctx, int64_t n, cudaStream_t s) {
@@ -264,8 +244,7 @@ tera_status ensure_records(tera_ctx* ctx, uint64_t cap, cudaStream_t s) {
   if ((st = alloc_dev(ctx->vals_c, c)) != TERA_OK) return st;
   if ((st = alloc_dev(ctx->agents_b, c)) != TERA_OK) return st;
   if ((st = alloc_dev(ctx->agents_c, c)) != TERA_OK) return st;
-  u64 tiles = (c + kSortTile - 1) / kSortTile;
-  if ((st = alloc_dev(ctx->rs_hist, (u64)kRadix * tiles + 1)) != TERA_OK) return st;
+  if ((st = alloc_dev(ctx->rs_hist, sort_scratch(c, ctx->n_pairs))) != TERA_OK) return st;
   if ((st = alloc_dev(ctx->matched, c)) != TERA_OK) return st;
   if ((st = alloc_dev(ctx->slot_src, c)) != TERA_OK) return st;
   if ((st = alloc_dev(ctx->seg, 2 * c + 2 * ctx->n_pairs)) != TERA_OK) return st;
@@ -273,7 +252,7 @@ tera_status ensure_records(tera_ctx* ctx, uint64_t cap, cudaStream_t s) {
   cudaMemset(ctx->seg, 0, sizeof(U64x2) * (2 * c + 2 * ctx->n_pairs));
   cudaMemset(ctx->matched, 0, sizeof(u32) * c);
   ctx->cap_records = c;
-  return ensure_scan_part(ctx, (u64)kRadix * tiles + 1);
+  return TERA_OK;
 }
 
 tera_status ensure_units(tera_ctx* ctx, uint64_t cap, cudaStream_t s) {
@@ -376,9 +355,7 @@ tera_status ensure_migrate(tera_ctx* ctx, uint64_t n, uint64_t leavers) {
     if ((st = alloc_dev(ctx->m_vals_c, c)) != TERA_OK) return st;
     if ((st = alloc_dev(ctx->m_agents_b, c)) != TERA_OK) return st;
     if ((st = alloc_dev(ctx->m_agents_c, c)) != TERA_OK) return st;
-    u64 tiles = (c + kSortTile - 1) / kSortTile;
-    if ((st = alloc_dev(ctx->m_hist, (u64)kRadix * tiles + 1)) != TERA_OK) return st;
-    if ((st = ensure_scan_part(ctx, (u64)kRadix * tiles + 1)) != TERA_OK) return st;
+    if ((st = alloc_dev(ctx->m_hist, sort_scratch(c, ctx->n_pairs))) != TERA_OK) return st;
     ctx->m_cap_leavers = c;
   }
   return TERA_OK;

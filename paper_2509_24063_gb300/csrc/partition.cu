@@ -12,10 +12,13 @@
 //                    scans inside a run, run bases from a scan)
 //   rs_hist_kernel / rs_scatter_kernel
 //                    stable LSD radix sort of the entry indices by pair
-//                    index, so each pair's list keeps ascending agent order
-//                    (tiles staged into shared memory by cp.async); the last
-//                    pass writes the agent of every record and the record
-//                    index of every entry (pack reads in agent order)
+//                    index, so each pair's list keeps ascending agent order:
+//                    the digit counts of every pass in one read of the keys,
+//                    then a launch a pass, whose tiles (staged into shared
+//                    memory by cp.async) find the digits' places by a
+//                    look-back over the tiles before them; the last pass
+//                    writes the agent of every record and the record index of
+//                    every entry (pack reads in agent order)
 //   pair_off_kernel  per-pair counts and offsets from the sorted keys
 #include "classify.cuh"
 #include "tera_internal.cuh"
@@ -81,12 +84,17 @@ __global__ void __launch_bounds__(kClassifyThreads, 6)
                     const u64* __restrict__ z, u64 n, const GridTables* __restrict__ g,
                     const AxisBuckets* __restrict__ bk, u64 n_tiles, int* __restrict__ owner,
                     u32* __restrict__ mask, u32* __restrict__ run_cnt, u64 n_runs, DevStatus* st,
-                    DevStats* stats) {
+                    DevStats* stats, u64* __restrict__ sort_head) {
   __shared__ SmemGrid sg;
   __shared__ float s_flo[3], s_fs[3];
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    stats->iterations += 1;
-    stats->agents += n;
+  if (blockIdx.x == 0) {  // what the launches after this one find zero
+    for (u32 i = threadIdx.x; i < kSortHead; i += blockDim.x) sort_head[i] = 0;
+    if (threadIdx.x == 0) {
+      stats->iterations += 1;
+      stats->agents += n;
+      st->abort = 0;
+      if (n == 0) run_cnt[0] = 0;
+    }
   }
   // the tables follow the grid rows (a multiple of 32 bytes) in dynamic shared memory
   uint8_t* tab = reinterpret_cast<uint8_t*>(grid_rows() + (g->n[0] + g->n[1] + g->n[2]));
@@ -160,6 +168,7 @@ __global__ void __launch_bounds__(kClassifyThreads)
     emit_kernel(const int* __restrict__ owner, const u32* __restrict__ mask, u64 n,
                 const u64* __restrict__ run_base, u64 n_runs, u32* __restrict__ keys,
                 u32* __restrict__ vals, u64 cap, DevStatus* st) {
+  if (*reinterpret_cast<const volatile u32*>(&st->abort)) return;  // the scan gave up
   const u64 total = run_base[n_runs];
   const u64 n_entries = total;  // (a warp's own count below is also called total)
   if (total > cap) {
@@ -222,32 +231,65 @@ __global__ void __launch_bounds__(kClassifyThreads)
   }
 }
 
-__device__ __forceinline__ u64 live_entries(const u64* total_ptr, u64 cap) {
+// Entries to sort: none when they exceed the capacity or the call was aborted.
+__device__ __forceinline__ u64 live_entries(const u64* total_ptr, u64 cap, const DevStatus* st) {
+  if (*reinterpret_cast<const volatile u32*>(&st->abort)) return 0;
   u64 t = *total_ptr;
   return t > cap ? 0 : t;
 }
 
-// Digit histogram of one sort tile; hist is digit-major: hist[d * n_tiles + t].
-__global__ void __launch_bounds__(kSortThreads)
-    rs_hist_kernel(const u32* __restrict__ keys, const u64* __restrict__ total_ptr, u64 cap,
-                   u32 shift, u32 radix, u32* __restrict__ hist, u32 n_tiles) {
-  __shared__ u32 cnt[kRadix];
-  const u64 E = live_entries(total_ptr, cap);
-  for (u32 d = threadIdx.x; d < radix; d += blockDim.x) cnt[d] = 0;
-  __syncthreads();
-  const u64 t0 = (u64)blockIdx.x * kSortTile;
-  if (t0 < E) {
-#pragma unroll 4
-    for (int k = 0; k < kSortPerThread; ++k) {
-      u64 i = t0 + (u64)k * kSortThreads + threadIdx.x;
-      if (i < E) atomicAdd(&cnt[(keys[i] >> shift) & (radix - 1)], 1u);
-    }
-  }
-  __syncthreads();
-  for (u32 d = threadIdx.x; d < radix; d += blockDim.x) hist[(u64)d * n_tiles + blockIdx.x] = cnt[d];
+// Scratch of a sort (SortBufs::hist): counts[pass * kRadix + d] of digit d,
+// then a claim ticket per pass, then the look-back states of each pass's
+// tiles, state[(pass * tiles + tile) * radix + d].
+__device__ __forceinline__ u64* sort_states(u64* head, u32 pass, u64 tiles, u32 radix) {
+  return head + kSortHead + (u64)pass * tiles * radix;
 }
 
-// Stable scatter of one sort tile of kSortTile entries.  The tile's input
+// Digit counts of every pass from one read of the keys, and the cleared
+// look-back states of the tiles that hold entries.  Resident blocks only, each
+// counting in shared memory, so that the counts cost the blocks' atomics and
+// not the tiles'.
+__global__ void __launch_bounds__(kSortThreads)
+    rs_hist_kernel(const u32* __restrict__ keys, const u64* __restrict__ total_ptr, u64 cap,
+                   u32 passes, u32 dbits, u64 tiles, u64* __restrict__ head, const DevStatus* st) {
+  __shared__ u32 cnt[4 * kRadix];
+  const u64 E = live_entries(total_ptr, cap, st);
+  const u32 radix = 1u << dbits;
+  for (u32 d = threadIdx.x; d < passes * kRadix; d += blockDim.x) cnt[d] = 0;
+  __syncthreads();
+  const u64 step = (u64)gridDim.x * blockDim.x;
+  const u64 tid = (u64)blockIdx.x * blockDim.x + threadIdx.x;
+  const bool wide = (reinterpret_cast<uintptr_t>(keys) & 15u) == 0;
+  const u64 quads = wide ? E / 4 : 0;
+  for (u64 i = tid; i < quads; i += step) {
+    const uint4 k = reinterpret_cast<const uint4*>(keys)[i];
+    for (u32 p = 0; p < passes; ++p) {
+      const u32 sh = p * dbits;
+      atomicAdd(&cnt[p * kRadix + ((k.x >> sh) & (radix - 1))], 1u);
+      atomicAdd(&cnt[p * kRadix + ((k.y >> sh) & (radix - 1))], 1u);
+      atomicAdd(&cnt[p * kRadix + ((k.z >> sh) & (radix - 1))], 1u);
+      atomicAdd(&cnt[p * kRadix + ((k.w >> sh) & (radix - 1))], 1u);
+    }
+  }
+  for (u64 i = 4 * quads + tid; i < E; i += step)
+    for (u32 p = 0; p < passes; ++p)
+      atomicAdd(&cnt[p * kRadix + ((keys[i] >> (p * dbits)) & (radix - 1))], 1u);
+  const u64 live = (E + kSortTile - 1) / kSortTile * radix;
+  for (u32 p = 0; p < passes; ++p) {
+    u64* s = sort_states(head, p, tiles, radix);
+    for (u64 i = tid; i < live; i += step) s[i] = 0;
+  }
+  __syncthreads();
+  for (u32 d = threadIdx.x; d < passes * kRadix; d += blockDim.x)
+    if (cnt[d]) atomicAdd(head + d, (u64)cnt[d]);
+}
+
+// Stable scatter of sort tiles of kSortTile entries, claimed one after the
+// other by resident blocks.  A tile counts its digits, publishes the counts,
+// and while its entries are ranked the tiles before it publish theirs; thread
+// d then walks back over digit d's counts (eight tiles' in flight) to the
+// nearest inclusive sum.  A histogram launch and a scan of three per pass did
+// this before: 178 + 58 us a pass at 16.6 M entries.  The tile's input
 // (keys, entry indices when given, agents) is first copied into shared memory
 // in input order by cp.async in 16-byte pieces (a ragged end, or unaligned
 // arrays, by plain loads), so the tile pays the latency of its global loads
@@ -283,7 +325,7 @@ __global__ void __launch_bounds__(kSortThreads)
                       const u32* __restrict__ agents_in, u32* __restrict__ keys_out,
                       u32* __restrict__ vals_out, u32* __restrict__ agents_out,
                       u32* __restrict__ dest, int last, const u64* __restrict__ total_ptr, u64 cap,
-                      u32 shift, u32 radix, const u32* __restrict__ hist_scan, u32 n_tiles,
+                      u32 pass, u32 shift, u32 radix, u64* __restrict__ head, u64 n_tiles,
                       DevStatus* st) {
   constexpr int kWarps = kSortThreads / 32;
   constexpr int kRoundEntries = kSortThreads * kSortSub;
@@ -297,19 +339,34 @@ __global__ void __launch_bounds__(kSortThreads)
   __shared__ u32 run[kR];     // entries of each digit placed in earlier rounds
   __shared__ u32 wcnt[kWarps][kR];
   __shared__ u32 sm[33];
-  const u64 E = live_entries(total_ptr, cap);
-  const u64 t0 = (u64)blockIdx.x * kSortTile;
-  if (t0 >= E) return;
-  const u32 tile_n = (u32)(E - t0 < (u64)kSortTile ? E - t0 : (u64)kSortTile);
+  __shared__ u32 s_tile;
+  const u64 E = live_entries(total_ptr, cap, st);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const u32 lt = (1u << lane) - 1u;
+  u64* states = sort_states(head, pass, n_tiles, radix);
+  // global start of this thread's digit
+  u32 dstart;
+  {
+    u32 tot;
+    dstart = block_excl_scan<u32>(
+        threadIdx.x < radix ? (u32)head[pass * kRadix + threadIdx.x] : 0u, sm, &tot);
+  }
+  for (;;) {
+  if (threadIdx.x == 0) s_tile = (u32)atomicAdd(head + 4 * kRadix + pass, 1ull);
+  for (u32 d = threadIdx.x; d < radix; d += blockDim.x) run[d] = 0;
+  __syncthreads();
+  const u64 tile = s_tile;
+  const u64 t0 = tile * kSortTile;
+  if (t0 >= E) return;
+  const u32 tile_n = (u32)(E - t0 < (u64)kSortTile ? E - t0 : (u64)kSortTile);
   {
     const uintptr_t al = reinterpret_cast<uintptr_t>(keys_in) |
                          reinterpret_cast<uintptr_t>(agents_in) |
                          reinterpret_cast<uintptr_t>(vals_in);
     const u32 n4 = (al & 15u) == 0 ? tile_n / 4 : 0;  // t0 is a multiple of 4 entries
+    for (u32 c = threadIdx.x; c < n4; c += blockDim.x) cp_async16(rkey + 4 * c, keys_in + t0 + 4 * c);
+    asm volatile("cp.async.commit_group;" : : : "memory");
     for (u32 c = threadIdx.x; c < n4; c += blockDim.x) {
-      cp_async16(rkey + 4 * c, keys_in + t0 + 4 * c);
       cp_async16(ragt + 4 * c, agents_in + t0 + 4 * c);
       if (vals_in) cp_async16(rval + 4 * c, vals_in + t0 + 4 * c);
     }
@@ -320,18 +377,21 @@ __global__ void __launch_bounds__(kSortThreads)
       if (vals_in) rval[li] = vals_in[t0 + li];
     }
   }
+  asm volatile("cp.async.wait_group 1;" : : : "memory");
+  __syncthreads();
+  for (u32 li = threadIdx.x; li < tile_n; li += blockDim.x)
+    atomicAdd(&run[(rkey[li] >> shift) & (radix - 1)], 1u);
+  __syncthreads();
+  const u32 mine = threadIdx.x < radix ? run[threadIdx.x] : 0u;  // this thread's digit's entries
+  if (threadIdx.x < radix)
+    lb_put(states + tile * radix + threadIdx.x, mine, tile ? kLbOwn : kLbSum);
   {
-    const u32 d = threadIdx.x;
-    u32 c = 0;
-    if (d < radix) {
-      const u64 at = (u64)d * n_tiles + blockIdx.x;
-      base[d] = hist_scan[at];
-      c = hist_scan[at + 1] - hist_scan[at];
-      run[d] = 0;
-    }
     u32 tot;
-    const u32 ex = block_excl_scan<u32>(c, sm, &tot);
-    if (d < radix) lstart[d] = ex;
+    const u32 ex = block_excl_scan<u32>(mine, sm, &tot);
+    if (threadIdx.x < radix) {
+      lstart[threadIdx.x] = ex;
+      run[threadIdx.x] = 0;
+    }
   }
   asm volatile("cp.async.wait_all;" : : : "memory");
   __syncthreads();
@@ -370,6 +430,38 @@ __global__ void __launch_bounds__(kSortThreads)
     }
     __syncthreads();
   }
+  bool gone = false;
+  if (threadIdx.x < radix) {
+    constexpr int kFlight = 8;
+    u64 pre = 0;
+    bool done = tile == 0;
+    LbWait wait;
+    for (long long at = (long long)tile - 1; !done && !gone;) {
+      u64 v[kFlight];
+#pragma unroll
+      for (int i = 0; i < kFlight; ++i)
+        v[i] = at - i >= 0 ? lb_get(states + (u64)(at - i) * radix + threadIdx.x) : 0ull;
+      int taken = 0;
+#pragma unroll
+      for (int i = 0; i < kFlight; ++i) {
+        const u64 state = v[i] >> kLbShift;
+        if (done || gone || taken < i || state == 0) continue;
+        if (state == kLbGone) {
+          gone = true;
+          continue;
+        }
+        pre += v[i] & kLbMask;
+        ++taken;
+        done = state == kLbSum;
+      }
+      at -= taken;
+      if (taken == 0 && !done && !gone && wait.over(st)) gone = true;
+    }
+    lb_put(states + tile * radix + threadIdx.x, gone ? 0ull : pre + mine, gone ? kLbGone : kLbSum);
+    base[threadIdx.x] = dstart + (u32)pre;
+  }
+  // (a tile that was given up sets the call's abort flag: nothing reads the lists)
+  if (__syncthreads_or(gone)) return;
   for (u32 lp = threadIdx.x; lp < tile_n; lp += blockDim.x) {
     const u32 src = inv[lp];
     const u32 key = rkey[src], a = ragt[src];
@@ -386,29 +478,44 @@ __global__ void __launch_bounds__(kSortThreads)
       agents_out[pos] = a;
     }
   }
-}
-
-__device__ __forceinline__ u64 lower_bound_u32(const u32* a, u64 n, u32 v) {
-  u64 lo = 0, hi = n;
-  while (lo < hi) {
-    u64 mid = (lo + hi) >> 1;
-    if (a[mid] < v) lo = mid + 1;
-    else hi = mid;
+  __syncthreads();  // the tile's shared memory is used again
   }
-  return lo;
 }
 
-__global__ void pair_off_kernel(const u32* __restrict__ sorted_keys,
-                                const u64* __restrict__ total_ptr, u64 cap, u64 n_pairs,
-                                u64* __restrict__ pair_off, u64* __restrict__ pair_count,
-                                DevStats* stats) {
-  const u64 E = live_entries(total_ptr, cap);
+// One probe step of a warp's search for the first of a[0, *hi) that is not
+// below v, 32 probes at a time: [*lo, *hi) shrinks to a 32nd.
+__device__ __forceinline__ void warp_probe(bool less, u64 len, u64* lo, u64* hi) {
+  const u32 bal = __ballot_sync(0xFFFFFFFFu, less);
+  const u32 c = (u32)__popc(bal);  // the probes are ascending, so these are the first
+  const u64 base = *lo;
+  if (c < 32u) *hi = base + len * c / 32;
+  if (c > 0u) *lo = base + len * (c - 1u) / 32 + 1;
+}
+
+// Offsets and counts of the pairs: a warp finds where pair p's and pair p + 1's
+// entries begin, both searches a step at a time (five steps of 32 probes for
+// 16 M entries; a thread's bisection took 24 dependent loads twice over, 15 us).
+__global__ void __launch_bounds__(256)
+    pair_off_kernel(const u32* __restrict__ sorted_keys, const u64* __restrict__ total_ptr, u64 cap,
+                    u64 n_pairs, u64* __restrict__ pair_off, u64* __restrict__ pair_count,
+                    DevStats* stats, const DevStatus* st) {
+  const u64 E = live_entries(total_ptr, cap, st);
   if (blockIdx.x == 0 && threadIdx.x == 0) stats->records += E;
-  for (u64 p = (u64)blockIdx.x * blockDim.x + threadIdx.x; p <= n_pairs;
-       p += (u64)gridDim.x * blockDim.x) {
-    u64 a = lower_bound_u32(sorted_keys, E, (u32)p);
-    pair_off[p] = a;
-    if (p < n_pairs) pair_count[p] = lower_bound_u32(sorted_keys, E, (u32)(p + 1)) - a;
+  const u32 lane = threadIdx.x & 31;
+  const u64 warps = (u64)gridDim.x * (blockDim.x / 32);
+  for (u64 p = (u64)blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5); p <= n_pairs; p += warps) {
+    u64 lo0 = 0, hi0 = E, lo1 = 0, hi1 = E;
+    while (lo0 < hi0 || lo1 < hi1) {  // warp-uniform
+      const u64 len0 = hi0 - lo0, len1 = hi1 - lo1;
+      const u64 m0 = lo0 + len0 * lane / 32, m1 = lo1 + len1 * lane / 32;
+      const u32 k0 = len0 ? sorted_keys[m0] : 0u, k1 = len1 ? sorted_keys[m1] : 0u;
+      if (len0) warp_probe(k0 < (u32)p, len0, &lo0, &hi0);
+      if (len1) warp_probe(k1 < (u32)(p + 1), len1, &lo1, &hi1);
+    }
+    if (lane == 0) {
+      pair_off[p] = lo0;
+      if (p < n_pairs) pair_count[p] = lo1 - lo0;
+    }
   }
 }
 
@@ -423,15 +530,27 @@ namespace tera {
 // writes the sorted keys to the buffer it does not read, vals_final[pos] =
 // agent[e] for the entry e sorted to pos, and dest[e] = pos (dest may be null).
 // The agents travel with the entries (read in order on every pass).
-tera_status radix_sort_entries(tera_ctx* ctx, const SortBufs& b, const u32* keys_in,
-                               const u32* agent, u32* dest, u32* vals_final, const u64* total_ptr,
-                               u64 cap, u64 key_limit, const u32** sorted_keys, cudaStream_t s) {
+static void sort_shape(u64 key_limit, int* passes, int* dbits) {
   int bits = 1;
   while ((1ull << bits) < key_limit) ++bits;
-  const int passes = (bits + kRadixBits - 1) / kRadixBits;
-  const int dbits = (bits + passes - 1) / passes;
+  *passes = (bits + kRadixBits - 1) / kRadixBits;
+  *dbits = (bits + *passes - 1) / *passes;
+}
+
+u64 sort_scratch(u64 cap, u64 key_limit) {
+  int passes, dbits;
+  sort_shape(key_limit, &passes, &dbits);
+  return kSortHead + (((u64)passes * ((cap + kSortTile - 1) / kSortTile)) << dbits);
+}
+
+tera_status radix_sort_entries(tera_ctx* ctx, const SortBufs& b, const u32* keys_in,
+                               const u32* agent, u32* dest, u32* vals_final, const u64* total_ptr,
+                               u64 cap, u64 key_limit, const u32** sorted_keys, cudaStream_t s,
+                               bool zeroed) {
+  int passes, dbits;
+  sort_shape(key_limit, &passes, &dbits);
   const u32 radix = 1u << dbits;
-  const u64 sort_tiles = cap == 0 ? 1 : (cap + kSortTile - 1) / kSortTile;
+  const u64 tiles = cap == 0 ? 1 : (cap + kSortTile - 1) / kSortTile;
   const u32* kin = keys_in;
   const u32* vin = nullptr;
   const u32* ain = agent;
@@ -445,28 +564,33 @@ tera_status radix_sort_entries(tera_ctx* ctx, const SortBufs& b, const u32* keys
                          (int)sort_smem_bytes(true));
     smem_set = true;
   }
+  if (cap > 0) {
+    if (!zeroed) cudaMemsetAsync(b.hist, 0, sizeof(u64) * kSortHead, s);
+    const u64 hgrid = (u64)grid_for(ctx, 4);
+    prof_begin(ctx, s);
+    rs_hist_kernel<<<(unsigned)(tiles < hgrid ? tiles : hgrid), kSortThreads, 0, s>>>(
+        keys_in, total_ptr, cap, (u32)passes, (u32)dbits, tiles, b.hist, ctx->d_status);
+    if ((st = check_launch(ctx, "rs_hist_kernel", s)) != TERA_OK) return st;
+  }
   for (int pass = 0; pass < passes && cap > 0; ++pass) {
     const u32 shift = (u32)(pass * dbits);
     const bool last = pass + 1 == passes;
     u32* kout = last ? kfinal : ((pass & 1) ? b.keys_c : b.keys_b);
     u32* vout = last ? vals_final : ((pass & 1) ? b.vals_c : b.vals_b);
     u32* aout = last ? nullptr : ((pass & 1) ? b.agents_c : b.agents_b);
-    prof_begin(ctx, s);
-    rs_hist_kernel<<<(unsigned)sort_tiles, kSortThreads, 0, s>>>(kin, total_ptr, cap, shift, radix,
-                                                                 b.hist, (u32)sort_tiles);
-    if ((st = check_launch(ctx, "rs_hist_kernel", s)) != TERA_OK) return st;
-    if ((st = scan_u32(ctx, b.hist, nullptr, b.hist, (u64)radix * sort_tiles, s)) != TERA_OK)
-      return st;
-    prof_begin(ctx, s);
     const size_t smem = sort_smem_bytes(vin != nullptr);
+    // resident blocks: six per SM on the first pass (no entry indices staged), four after it
+    const u64 res = (u64)grid_for(ctx, vin ? 4 : 6);
+    const unsigned grid = (unsigned)(tiles < res ? tiles : res);
+    prof_begin(ctx, s);
     if (radix <= 128)
-      rs_scatter_kernel<128><<<(unsigned)sort_tiles, kSortThreads, smem, s>>>(
+      rs_scatter_kernel<128><<<grid, kSortThreads, smem, s>>>(
           kin, vin, ain, kout, vout, aout, last ? dest : nullptr, last ? 1 : 0, total_ptr, cap,
-          shift, radix, b.hist, (u32)sort_tiles, ctx->d_status);
+          (u32)pass, shift, radix, b.hist, tiles, ctx->d_status);
     else
-      rs_scatter_kernel<kRadix><<<(unsigned)sort_tiles, kSortThreads, smem, s>>>(
+      rs_scatter_kernel<kRadix><<<grid, kSortThreads, smem, s>>>(
           kin, vin, ain, kout, vout, aout, last ? dest : nullptr, last ? 1 : 0, total_ptr, cap,
-          shift, radix, b.hist, (u32)sort_tiles, ctx->d_status);
+          (u32)pass, shift, radix, b.hist, tiles, ctx->d_status);
     if ((st = check_launch(ctx, "rs_scatter_kernel", s)) != TERA_OK) return st;
     kin = kout;
     vin = vout;
@@ -499,10 +623,8 @@ extern "C" tera_status tera_partition(tera_ctx* ctx, const tera_soa* soa, tera_p
   if (!ctx->tile_cnt || !ctx->tile_base) return TERA_ENOMEM;
   if ((st = ensure_records(ctx, out->idx_capacity, s)) != TERA_OK) return st;
   ctx->iterations += 1;
-  cudaMemsetAsync(&ctx->d_status->abort, 0, sizeof(u32), s);
   const u64 blocks = n == 0 ? 1 : (n + kClassifyTile - 1) / kClassifyTile;
   const u64 runs = n == 0 ? 1 : (n + kRunAgents - 1) / kRunAgents;
-  if (n == 0) cudaMemsetAsync(ctx->tile_cnt, 0, sizeof(u32), s);
   // resident blocks only (6 per SM): each copies the tables into shared memory once
   const size_t csmem =
       grid_smem_bytes(ctx->grid) + (ctx->d_buckets ? 3 * (size_t)kAxisBuckets : 0);
@@ -517,7 +639,7 @@ extern "C" tera_status tera_partition(tera_ctx* ctx, const tera_soa* soa, tera_p
   classify_kernel<<<(unsigned)cgrid, kClassifyThreads, csmem, s>>>(
       reinterpret_cast<const u64*>(soa->x), reinterpret_cast<const u64*>(soa->y),
       reinterpret_cast<const u64*>(soa->z), n, ctx->d_grid, ctx->d_buckets, blocks, out->owner,
-      out->mask, ctx->tile_cnt, runs, ctx->d_status, ctx->d_stats);
+      out->mask, ctx->tile_cnt, runs, ctx->d_status, ctx->d_stats, ctx->rs_hist);
   if ((st = check_launch(ctx, "classify_kernel", s)) != TERA_OK) return st;
   if ((st = scan_u32(ctx, ctx->tile_cnt, ctx->tile_base, nullptr, runs, s)) != TERA_OK)
     return st;
@@ -536,13 +658,13 @@ extern "C" tera_status tera_partition(tera_ctx* ctx, const tera_soa* soa, tera_p
                       ctx->agents_b, ctx->agents_c, ctx->rs_hist};
   const u32* sorted = nullptr;
   if ((st = radix_sort_entries(ctx, bufs, ctx->keys_a, ctx->ent_agent, ctx->ent_dest, out->pair_idx,
-                               total_ptr, cap, P, &sorted, s)) != TERA_OK)
+                               total_ptr, cap, P, &sorted, s, true)) != TERA_OK)
     return st;
   ctx->rec_pair = const_cast<u32*>(sorted);
   ctx->pack_n = soa->n;
   prof_begin(ctx, s);
-  pair_off_kernel<<<(unsigned)((P + 256) / 256), 256, 0, s>>>(
+  pair_off_kernel<<<(unsigned)(P / 8 + 1), 256, 0, s>>>(
       sorted, total_ptr, cap, P, reinterpret_cast<u64*>(out->pair_off),
-      reinterpret_cast<u64*>(out->pair_count), ctx->d_stats);
+      reinterpret_cast<u64*>(out->pair_count), ctx->d_stats, ctx->d_status);
   return check_launch(ctx, "pair_off_kernel", s);
 }

@@ -182,6 +182,87 @@ __device__ __forceinline__ T block_excl_scan(T v, T* smem, T* total) {
   return res;
 }
 
+// ---- decoupled look-back ----
+// A tile of a chain publishes its own value as soon as it knows it, sums its
+// predecessors' and publishes the inclusive sum: one 64-bit word per tile, the
+// state in its top two bits (zero: nothing yet), written and read whole.
+// Tiles are claimed in order and publish before they wait, so a tile only
+// waits for running blocks; a wait gives up after a second all the same.
+constexpr int kLbShift = 62;
+constexpr u64 kLbOwn = 1, kLbSum = 2, kLbGone = 3;
+constexpr u64 kLbMask = (1ull << kLbShift) - 1ull;
+constexpr u64 kLbLimitNs = 1000000000ull;
+
+__device__ __forceinline__ void lb_put(u64* s, u64 v, u64 state) {
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" : : "l"(s), "l"(v | (state << kLbShift))
+               : "memory");
+}
+__device__ __forceinline__ u64 lb_get(const u64* s) {
+  u64 v;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(s) : "memory");
+  return v;
+}
+__device__ __forceinline__ u64 lb_now() {
+  u64 t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
+}
+// Counts polls of one wait; true when it has taken too long (TERA_ETIMEOUT and
+// the call's abort flag set).
+struct LbWait {
+  u64 t0 = 0;
+  u32 polls = 0;
+  __device__ __forceinline__ bool over(DevStatus* st) {
+    if ((++polls & 63u) != 0u) return false;
+    const u64 now = lb_now();
+    if (t0 == 0) t0 = now;
+    if (now - t0 <= kLbLimitNs && polls < (1u << 30)) return false;
+    latch(st, TERA_ETIMEOUT);
+    atomicExch(&st->abort, 1u);
+    return true;
+  }
+};
+
+// One warp: the sum of the tiles before `tile` of a chain whose tile i publishes
+// at state[i], this tile's value `own` published first.  False (the tile is
+// given up, and so is every tile after it) when the wait was cut short.
+__device__ __forceinline__ bool lb_warp_sum(u64* state, u64 tile, u64 own, DevStatus* st,
+                                            u64* before) {
+  const int lane = threadIdx.x & 31;
+  u64 pre = 0;
+  bool fine = true;
+  if (tile > 0) {
+    if (lane == 0) lb_put(state + tile, own, kLbOwn);
+    LbWait wait;
+    for (long long at = (long long)tile - 1; fine; at -= 32) {
+      const long long i = at - lane;
+      u64 v;
+      u32 first;
+      for (;;) {
+        v = i >= 0 ? lb_get(state + i) : kLbSum << kLbShift;
+        const u32 done = __ballot_sync(0xFFFFFFFFu, (v >> kLbShift) >= kLbSum);
+        const u32 none = __ballot_sync(0xFFFFFFFFu, (v >> kLbShift) == 0);
+        first = done ? (u32)__ffs(done) - 1u : 32u;
+        if (!(none & (first < 32u ? (1u << first) - 1u : 0xFFFFFFFFu))) break;
+        if (__any_sync(0xFFFFFFFFu, wait.over(st))) {
+          fine = false;
+          break;
+        }
+      }
+      if (!fine) break;
+      if (__any_sync(0xFFFFFFFFu, (v >> kLbShift) == kLbGone && (u32)lane <= first)) {
+        fine = false;
+        break;
+      }
+      pre += warp_sum((u32)lane <= first ? v & kLbMask : 0ull);
+      if (first < 32u) break;
+    }
+  }
+  if (lane == 0) lb_put(state + tile, fine ? pre + own : 0ull, fine ? kLbSum : kLbGone);
+  *before = pre;
+  return fine;
+}
+
 // Pair scan of two counters at once.
 struct U64x2 {
   u64 a, b;

@@ -79,7 +79,7 @@ struct tera_ctx {
   uint32_t* agents_c;
   uint32_t* rec_pair;      // pair of each record of the last partition (sorted keys)
   int64_t pack_n;          // agents of the last partition (its runs cover them)
-  uint32_t* rs_hist;       // [kRadix * sort tiles]
+  tera::u64* rs_hist;      // [sort_scratch] digit counts and look-back states of the sort
   tera::u64* scan_part;     // partials of the generic scan
   uint64_t scan_part_cap;
   tera::u64* d_total;       // [4] scalars: total records, ...
@@ -161,7 +161,7 @@ struct tera_ctx {
   uint32_t* m_vals_c;
   uint32_t* m_agents_b;
   uint32_t* m_agents_c;
-  uint32_t* m_hist;
+  tera::u64* m_hist;       // as rs_hist
 };
 
 namespace tera {
@@ -194,9 +194,14 @@ struct SortBufs {
   u32* vals_c;
   u32* agents_b;  // agents carried with the entries between passes
   u32* agents_c;
-  u32* hist;  // [kRadix * sort tiles + 1]
+  u64* hist;  // [sort_scratch]
 };
+// Words of SortBufs::hist for `cap` entries with keys below key_limit.
+u64 sort_scratch(u64 cap, u64 key_limit);
+// Words of it that are zero when a sort begins.
+constexpr u64 kSortHead = 4 * kRadix + 4;
 tera_status radix_sort_entries(tera_ctx* ctx, const SortBufs& b, const u32* keys_in,
                                const u32* agent, u32* dest, u32* vals_final, const u64* total_ptr,
-                               u64 cap, u64 key_limit, const u32** sorted_keys, cudaStream_t s);
+                               u64 cap, u64 key_limit, const u32** sorted_keys, cudaStream_t s,
+                               bool zeroed = false);
 }  // namespace tera
