@@ -85,6 +85,9 @@ struct TileArgs {
   DecArgs D;
   TilePair* pair;
   u32* unit_pair;       // pair of each tile
+  u32* unit_first;      // [P] first tile of each pair
+  u64* setup_state;     // look-back states of the setup (zero between calls)
+  u32* setup_ticket;
   u32* item_pair;       // pair of each match item
   u32* big_pair;        // pair of each bigmatch item
   u32* small_pair;      // pairs matched by one warp
@@ -147,86 +150,64 @@ __device__ __forceinline__ Facts facts_of(const TileArgs& A, u64 p, int mode, u3
 
 constexpr int kSetupT = 1024;
 
-// First launch: kSetupT pairs per block, the block's sums of (slab bytes,
-// tiles) and (match items and pairs matched by a warp in the two halves of a
-// word, bigmatch items).
-__global__ void __launch_bounds__(kSetupT) tiles_sums_kernel(TileArgs A, int mode,
-                                                             U64x2* __restrict__ part) {
-  __shared__ u64 sm[4][32];
-  const u64 p = (u64)blockIdx.x * kSetupT + threadIdx.x;
-  u64 v[4] = {0, 0, 0, 0};
-  if (p < A.P) {
-    const Facts f = facts_of(A, p, mode, tile_shift(A));
-    v[0] = f.slab;
-    v[1] = f.units;
-    v[2] = f.items | (f.small << 32);
-    v[3] = f.big;
-  }
-#pragma unroll
-  for (int i = 0; i < 4; ++i) v[i] = warp_sum(v[i]);
-  if ((threadIdx.x & 31) == 0)
-#pragma unroll
-    for (int i = 0; i < 4; ++i) sm[i][threadIdx.x >> 5] = v[i];
-  __syncthreads();
-  if (threadIdx.x < 32) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) v[i] = warp_sum(sm[i][threadIdx.x]);
-    if (threadIdx.x == 0) {
-      part[2 * blockIdx.x] = U64x2{v[0], v[1]};
-      part[2 * blockIdx.x + 1] = U64x2{v[2], v[3]};
-    }
-  }
-}
-
 // out[i] = pair of item i for the items [lo, lo + n) of the block's pairs,
 // first[k] (k < np) the first item of pair p0 + k counted from lo (first[np] = n).
-__device__ __forceinline__ void fill_map(u32* __restrict__ out, u64 lo, u32 n, const u32* first,
-                                         u32 np, u32 p0) {
-  for (u32 i = threadIdx.x; i < n; i += kSetupT)
+__device__ __forceinline__ void fill_map(u32* __restrict__ out, u64 lo, u32 n, u64 cap,
+                                         const u32* first, u32 np, u32 p0) {
+  for (u32 i = threadIdx.x; i < n && lo + i < cap; i += kSetupT)
     out[lo + i] = p0 + upper_pair(first, 0u, np, (u64)i);
 }
 
-// Second launch (the same blocks): offsets from the first launch's sums, the
-// per-pair facts and the maps.  Pairs without entries on
-// either side are finished here.
+// One launch, kSetupT pairs a block: the pairs' facts, then their places in the
+// slabs and lists by a block scan and a look-back over the blocks (four chains:
+// slab bytes, tiles, match items and warp pairs in the halves of a word, items
+// of big pairs).  Pairs without entries on either side are finished here.  The
+// last block writes the totals and checks the capacities; until then a block
+// knows all but the slabs' total, so it writes to the wire only inside its
+// capacity.
 __global__ void __launch_bounds__(kSetupT)
-    tiles_place_kernel(TileArgs A, int mode, u64* __restrict__ wire_off, u64 wire_cap, u64 rec_cap,
-                       u64 recv_cap, u64 unit_cap, u64 item_cap, u64 big_cap, u32* epoch,
-                       const U64x2* __restrict__ part) {
+    tiles_setup_kernel(TileArgs A, int mode, u64* __restrict__ wire_off, u64 wire_cap, u64 rec_cap,
+                       u64 recv_cap, u64 unit_cap, u64 item_cap, u64 big_cap, u32* epoch) {
   __shared__ U64x2 sm2[33];
-  __shared__ u32 first[4][kSetupT];
-  const u32 shift = tile_shift(A);
-  U64x2 ca{0, 0}, cb{0, 0}, qa{0, 0}, qb{0, 0};
-  for (u32 i = threadIdx.x; i < gridDim.x; i += kSetupT) {
-    const U64x2 a = part[2 * i], b = part[2 * i + 1];
-    if (i < blockIdx.x) {
-      ca += a;
-      cb += b;
-    }
-    qa += a;
-    qb += b;
+  __shared__ u32 first[3][kSetupT];
+  __shared__ u64 s_pre[4];
+  __shared__ u32 s_block, s_fine;
+  if (threadIdx.x == 0) {
+    s_block = gridDim.x > 1 ? atomicAdd(A.setup_ticket, 1u) : 0u;
+    s_fine = 1;
   }
-  U64x2 carry_a, carry_b, tot_a, tot_b;
-  block_excl_scan2(ca, sm2, &carry_a);
-  block_excl_scan2(cb, sm2, &carry_b);
-  block_excl_scan2(qa, sm2, &tot_a);
-  block_excl_scan2(qb, sm2, &tot_b);
+  const u32 shift = tile_shift(A);
   const u64 P = A.P, E = A.E.pair_off[P];
   const u64 rmax = A.E.ref_off ? A.E.ref_off[P] : 0, dmax = A.D.ref_off ? A.D.ref_off[P] : 0;
   const u64 big = E > rmax ? (E > dmax ? E : dmax) : (rmax > dmax ? rmax : dmax);
-  const u64 n_items = tot_b.a & 0xFFFFFFFFull, n_small = tot_b.a >> 32;
-  const bool fits = tot_a.b <= unit_cap && n_items <= item_cap && tot_b.b <= big_cap;
-  const bool abort = tot_a.a > wire_cap || big > rec_cap || E + P > recv_cap || !fits;
-  const u64 p = (u64)blockIdx.x * kSetupT + threadIdx.x;
+  const bool abort = big > rec_cap || E + P > recv_cap;
+  __syncthreads();
+  const u32 block = s_block;
+  const u64 p = (u64)block * kSetupT + threadIdx.x;
   Facts f{};
   if (p < P) f = facts_of(A, p, mode, shift);
   U64x2 ta, tb;
   const U64x2 ea = block_excl_scan2(U64x2{f.slab, f.units}, sm2, &ta);
   const U64x2 eb = block_excl_scan2(U64x2{f.items | (f.small << 32), f.big}, sm2, &tb);
-  first[0][threadIdx.x] = (u32)ea.b;
-  first[1][threadIdx.x] = (u32)eb.a;
+  first[0][threadIdx.x] = (u32)eb.a;
+  first[1][threadIdx.x] = (u32)(eb.a >> 32);
   first[2][threadIdx.x] = (u32)eb.b;
-  first[3][threadIdx.x] = (u32)(eb.a >> 32);
+  if (threadIdx.x < 128) {  // a warp a chain
+    const u32 c = threadIdx.x >> 5;
+    const u64 own = c == 0 ? ta.a : (c == 1 ? ta.b : (c == 2 ? tb.a : tb.b));
+    u64 pre = 0;
+    if (gridDim.x > 1 && !lb_warp_sum(A.setup_state + (u64)c * gridDim.x, block, own, A.E.st, &pre) &&
+        (threadIdx.x & 31) == 0)
+      s_fine = 0;
+    if ((threadIdx.x & 31) == 0) s_pre[c] = pre;
+  }
+  __syncthreads();
+  const bool last = block == gridDim.x - 1;
+  if (!s_fine) {  // (the timeout is latched) no tile of this call runs
+    if (last && threadIdx.x < TS_COUNT) A.scal[threadIdx.x] = 0u;
+    return;
+  }
+  const U64x2 carry_a{s_pre[0], s_pre[1]}, carry_b{s_pre[2], s_pre[3]};
   u64 empties = 0;
   if (p < P) {
     const u64 w = carry_a.a + ea.a, g_lo = A.E.pair_off[p];
@@ -252,7 +233,8 @@ __global__ void __launch_bounds__(kSetupT)
       tot[0] = make_ulonglong2(0, 0);
       tot[1] = make_ulonglong2(0, 0);
       A.done[p] = 0;
-      if (f.units == 0) {  // no slots, no records: headers alone
+      A.unit_first[p] = x.unit0;
+      if (f.units == 0 && w + kHdrBytes <= wire_cap) {  // no slots, no records: headers alone
         ulonglong2* h = reinterpret_cast<ulonglong2*>(A.E.wire + w);
         h[0] = make_ulonglong2((u64)kWireMagic | ((u64)kVersion << 32) | ((u64)kRecBytes << 48),
                                (u64)A.E.class_id | ((u64)x.mode << 32));
@@ -276,23 +258,26 @@ __global__ void __launch_bounds__(kSetupT)
   }
   __syncthreads();
   if (!abort) {
-    const u64 left = P - (u64)blockIdx.x * kSetupT;
-    const u32 np = (u32)(left < (u64)kSetupT ? left : (u64)kSetupT), p0 = blockIdx.x * kSetupT;
-    fill_map(A.unit_pair, carry_a.b, (u32)ta.b, first[0], np, p0);
-    fill_map(A.item_pair, carry_b.a & 0xFFFFFFFFull, (u32)tb.a, first[1], np, p0);
-    fill_map(A.small_pair, carry_b.a >> 32, (u32)(tb.a >> 32), first[3], np, p0);
-    fill_map(A.big_pair, carry_b.b, (u32)tb.b, first[2], np, p0);
+    const u64 left = P - (u64)block * kSetupT;
+    const u32 np = (u32)(left < (u64)kSetupT ? left : (u64)kSetupT), p0 = block * kSetupT;
+    fill_map(A.item_pair, carry_b.a & 0xFFFFFFFFull, (u32)tb.a, item_cap, first[0], np, p0);
+    fill_map(A.small_pair, carry_b.a >> 32, (u32)(tb.a >> 32), P, first[1], np, p0);
+    fill_map(A.big_pair, carry_b.b, (u32)tb.b, big_cap, first[2], np, p0);
     const u64 n = warp_sum(empties);
     if ((threadIdx.x & 31) == 0 && n) atomicAdd(&A.E.stats->wire_bytes, n * kHdrBytes);
   }
-  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
+  if (last && threadIdx.x == 0) {
     const u32 ep = *epoch + 1u;
     *epoch = ep == 0u ? 1u : ep;
-    wire_off[P] = tot_a.a;
+    const U64x2 all_a = carry_a + ta, all_b = carry_b + tb;
+    const u64 n_items = all_b.a & 0xFFFFFFFFull, n_small = all_b.a >> 32;
+    wire_off[P] = all_a.a;
     A.D.recv_off[P] = E;
-    if (tot_a.a > wire_cap) {
+    bool none = abort;
+    if (all_a.a > wire_cap) {
       latch(A.E.st, TERA_ECAPACITY);
-      need(A.E.st, tot_a.a);
+      need(A.E.st, all_a.a);
+      none = true;
     }
     if (big > rec_cap) {
       latch(A.E.st, TERA_ECAPACITY);
@@ -302,12 +287,15 @@ __global__ void __launch_bounds__(kSetupT)
       latch(A.E.st, TERA_ECAPACITY);
       need(A.E.st, E + P);
     }
-    if (!fits) latch(A.E.st, TERA_ECAPACITY);  // cannot happen: the lists are sized for it
-    A.scal[TS_UNITS] = abort ? 0u : (u32)tot_a.b;
-    A.scal[TS_ITEMS] = abort ? 0u : (u32)n_items;
-    A.scal[TS_SMALL] = abort ? 0u : (u32)n_small;
+    if (all_a.b > unit_cap || n_items > item_cap || all_b.b > big_cap) {
+      latch(A.E.st, TERA_ECAPACITY);  // cannot happen: the lists are sized for it
+      none = true;
+    }
+    A.scal[TS_UNITS] = none ? 0u : (u32)all_a.b;
+    A.scal[TS_ITEMS] = none ? 0u : (u32)n_items;
+    A.scal[TS_SMALL] = none ? 0u : (u32)n_small;
     A.scal[TS_SHIFT] = shift;
-    A.scal[TS_BIG] = abort ? 0u : (u32)tot_b.b;
+    A.scal[TS_BIG] = none ? 0u : (u32)all_b.b;
     for (int i = TS_TICKET_MATCH; i < TS_COUNT; ++i) A.scal[i] = 0u;
   }
 }
@@ -487,6 +475,34 @@ static_assert(kWarpTable >= 8 * (2 * kIlp * 32 + 2 * kWinSlack) && kWarpTable >=
               "a warp's window and table fit");
 static_assert(8 * kWarpShare <= kMatchSmem, "eight warps' shares fit");
 
+// The pair of every tile (unit_pair), which the launches after this one read:
+// each warp of the launch takes a run of tiles, finds the first one's pair and
+// walks on from it.
+__device__ __forceinline__ void map_tiles(const TileArgs& A) {
+  const u32 lane = threadIdx.x & 31;
+  const u64 units = A.scal[TS_UNITS], warps = (u64)gridDim.x * (kT / 32);
+  const u64 run = (ceil_div(units, warps) + 31) & ~31ull;
+  const u64 a = ((u64)blockIdx.x * (kT / 32) + (threadIdx.x >> 5)) * run;
+  const u64 b = a + run < units ? a + run : units;
+  if (a >= b) return;
+  // the last pair whose first tile is a or before it, 32 probes at a time
+  u32 lo = 0, hi = (u32)A.P - 1;
+  while (lo < hi) {
+    const u32 step = (hi - lo + 32) / 32, at = lo + lane * step;
+    const u32 bal = __ballot_sync(0xFFFFFFFFu, at <= hi && A.unit_first[at] <= a);
+    const u32 k = 31u - (u32)__clz(bal | 1u);
+    const u32 next = lo + k * step;
+    hi = next + step - 1u < hi ? next + step - 1u : hi;
+    lo = next;
+    if (step == 1u) break;
+  }
+  u32 p = lo;
+  for (u64 u = a + lane; u < b; u += 32) {
+    while (p + 1 < (u32)A.P && A.unit_first[p + 1] <= u) ++p;
+    A.unit_pair[u] = p;
+  }
+}
+
 // The pairs of the match list, a block each, claimed one by one; then the
 // small ones, a warp each.
 __global__ void __launch_bounds__(kT, kPerSm) codec_match_kernel(TileArgs A) {
@@ -495,6 +511,12 @@ __global__ void __launch_bounds__(kT, kPerSm) codec_match_kernel(TileArgs A) {
   __shared__ u32 s_next, s_cnt[kT / 32];
   const u32 n = A.scal[TS_ITEMS], n_small = A.scal[TS_SMALL], shift = A.scal[TS_SHIFT];
   const u32 epoch = *A.E.epoch;
+  if (blockIdx.x == 0) {  // the setup's states, zero for the next call
+    const u32 blocks = (u32)((A.P + kSetupT - 1) / kSetupT);
+    for (u32 i = threadIdx.x; i < 4 * blocks; i += kT) A.setup_state[i] = 0;
+    if (threadIdx.x == 0) *A.setup_ticket = 0;
+  }
+  map_tiles(A);
   if (n) {
     SmemTable tb;
     tb.tbl = reinterpret_cast<unsigned short*>(dyn);
@@ -1242,6 +1264,8 @@ tera_status launch_tiles(tera_ctx* ctx, const EncArgs& E, const DecArgs& D, bool
   A.D = D;
   A.pair = reinterpret_cast<TilePair*>(ctx->t_pair);
   A.unit_pair = ctx->t_unit_pair;
+  A.unit_first = ctx->t_unit_first;
+  A.setup_state = ctx->t_part;
   A.item_pair = ctx->t_item_pair;
   A.big_pair = ctx->t_big_pair;
   A.small_pair = ctx->t_small_pair;
@@ -1257,16 +1281,13 @@ tera_status launch_tiles(tera_ctx* ctx, const EncArgs& E, const DecArgs& D, bool
   A.scal = ctx->t_scal;
   A.P = P;
   const unsigned setup = (unsigned)(P == 0 ? 1 : (P + kSetupT - 1) / kSetupT);
-  U64x2* part = reinterpret_cast<U64x2*>(ctx->t_part);
   const unsigned egrid = (unsigned)(ctx->num_sms * kEncPerSm), dgrid = (unsigned)(ctx->num_sms * kDecPerSm);
+  A.setup_ticket = reinterpret_cast<u32*>(ctx->t_part + 4 * (u64)setup);
   prof_begin(ctx, s);
-  tiles_sums_kernel<<<setup, kSetupT, 0, s>>>(A, mode, part);
-  if ((st = check_launch(ctx, "tiles_sums_kernel", s)) != TERA_OK) return st;
-  prof_begin(ctx, s);
-  tiles_place_kernel<<<setup, kSetupT, 0, s>>>(A, mode, const_cast<u64*>(E.wire_off), wire_cap,
+  tiles_setup_kernel<<<setup, kSetupT, 0, s>>>(A, mode, const_cast<u64*>(E.wire_off), wire_cap,
                                                ctx->cap_records, recv_cap, ctx->t_units,
-                                               ctx->t_items, ctx->t_bigs, ctx->d_epoch, part);
-  if ((st = check_launch(ctx, "tiles_place_kernel", s)) != TERA_OK) return st;
+                                               ctx->t_items, ctx->t_bigs, ctx->d_epoch);
+  if ((st = check_launch(ctx, "tiles_setup_kernel", s)) != TERA_OK) return st;
   prof_begin(ctx, s);
   codec_match_kernel<<<grid, kT, kMatchSmem, s>>>(A);
   if ((st = check_launch(ctx, "codec_match_kernel", s)) != TERA_OK) return st;

@@ -308,7 +308,9 @@ tera_status ensure_tiles(tera_ctx* ctx) {
     if ((st = alloc_dev(ctx->t_tot, P * 4)) != TERA_OK) return st;
     if ((st = alloc_dev(ctx->t_done, P)) != TERA_OK) return st;
     if ((st = alloc_dev(ctx->t_scal, 8)) != TERA_OK) return st;
-    if ((st = alloc_dev(ctx->t_part, 4 * (P / 1024 + 1))) != TERA_OK) return st;
+    if ((st = alloc_dev(ctx->t_part, 4 * (P / 1024 + 1) + 1)) != TERA_OK) return st;
+    cudaMemset(ctx->t_part, 0, sizeof(u64) * (4 * (P / 1024 + 1) + 1));
+    if ((st = alloc_dev(ctx->t_unit_first, P)) != TERA_OK) return st;
     if ((st = alloc_dev(ctx->t_small_pair, P)) != TERA_OK) return st;
     if ((st = alloc_dev(ctx->t_pair, P * 8)) != TERA_OK) return st;
   }
@@ -718,6 +720,7 @@ tera_status tera_ctx_destroy(tera_ctx* c) {
   free_dev(c->b_part);
   free_dev(c->t_pair);
   free_dev(c->t_unit_pair);
+  free_dev(c->t_unit_first);
   free_dev(c->t_item_pair);
   free_dev(c->t_big_pair);
   free_dev(c->t_small_pair);

@@ -142,7 +142,8 @@ struct tera_ctx {
   uint32_t* t_bits;        // taken records of big pairs
   uint32_t* t_new;         // [t_cap] new records of each pair
   uint32_t* t_scal;        // [8] list lengths and claim tickets
-  tera::u64* t_part;       // [4 * (P / 1024 + 1)] block sums of the setup's first launch
+  uint32_t* t_unit_first;  // [P] first tile of each pair
+  tera::u64* t_part;       // [4 * (P / 1024 + 1) + 1] look-back states of the setup, its ticket
   // agent migration (migrate.cu)
   uint64_t m_cap_agents;   // agents the tile arrays cover
   uint64_t m_cap_leavers;  // leavers the list and sort buffers hold
