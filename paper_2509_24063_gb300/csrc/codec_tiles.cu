@@ -5,10 +5,12 @@
 //   setup   (two launches) per-pair facts, wire slabs and the lists of tiles
 //   match   one block per pair: the message record of every reference slot
 //           (ids in shared memory), the matches before each tile and the list
-//           of the records no slot took; pairs of more than kTableMax records
-//           index their ids in global hash segments here, a tile each, and are
+//           of the records no slot took; a pair of more than kTableMax records
+//           is only asked here, a tile each, whether its ids ascend, and
 //           matched by
-//   bigmatch  (tiles of such pairs; does nothing without them)
+//   bigmatch  (tiles of such pairs; does nothing without them): by bisection
+//           over ascending ids, else in a global hash segment that its tiles
+//           index first
 //   sizes   predictor only: the payload of the XOR and of the residual form
 //   encode  one tile of slots or new records: difference, code, new-reference
 //           records, and the payload, packed, into the tile's own part of the
@@ -97,7 +99,9 @@ struct TileArgs {
   u32* bytes;           // payload bytes of each tile
   u64* place;           // payload bytes of the pair before each tile
   u64* tot;             // [P * PT_COUNT] matched records, XOR and residual bytes
-  u32* done;            // [P] bigmatch items finished
+  u32* done;            // [P] matched tiles of a big pair
+  u32* built;           // [P] indexed tiles of a big pair
+  u32* unsorted;        // [P] a big pair whose message ids do not ascend
   u32* bits;            // taken records of big pairs: word (g_lo >> 5) + p of pair p
   u32* new_idx;         // new records of each pair in message order, from g_lo
   u32* scal;            // TS_*
@@ -144,7 +148,7 @@ __device__ __forceinline__ Facts facts_of(const TileArgs& A, u64 p, int mode, u3
   const bool big = f.m > kTableMax;
   f.small = f.r + f.m != 0 && f.r <= A.warp_pair && f.m <= A.warp_pair;
   f.items = big ? ceil_div(f.m, kBigTile) : (f.r + f.m != 0 && !f.small ? 1 : 0);
-  f.big = big ? ceil_div(f.r, kBigTile) : 0;
+  f.big = big ? ceil_div(f.m, kBigTile) + ceil_div(f.r, kBigTile) : 0;
   return f;
 }
 
@@ -233,6 +237,8 @@ __global__ void __launch_bounds__(kSetupT)
       tot[0] = make_ulonglong2(0, 0);
       tot[1] = make_ulonglong2(0, 0);
       A.done[p] = 0;
+      A.built[p] = 0;
+      A.unsorted[p] = 0;
       A.unit_first[p] = x.unit0;
       if (f.units == 0 && w + kHdrBytes <= wire_cap) {  // no slots, no records: headers alone
         ulonglong2* h = reinterpret_cast<ulonglong2*>(A.E.wire + w);
@@ -383,17 +389,34 @@ __device__ __forceinline__ void count_tiles(const TileArgs& A, const TilePair& x
   }
 }
 
-// One tile of message ids of a big pair into its hash segment (as the
-// persistent launch does), its taken bits cleared.
-__device__ __forceinline__ void big_build(const TileArgs& A, const TilePair& x, u32 p, u32 tile,
-                                          u32 epoch) {
-  const EncArgs& E = A.E;
-  const u64 base = seg_base(x.g_lo, p), size = seg_size(x.m);
+// One tile of a big pair's message: whether its ids ascend (up to the next
+// tile's first), and its taken bits cleared.
+__device__ __forceinline__ void big_check(const TileArgs& A, const TilePair& x, u32 p, u32 tile) {
   const u32 k0 = tile * kBigTile;
   if (threadIdx.x < kBigTile / 32) {
     const u32 w = k0 / 32 + threadIdx.x;
     if (w < (x.m + 31u) / 32u) big_bits(A, x, p)[w] = 0u;
   }
+  u64 a[kIlp], b[kIlp];
+#pragma unroll
+  for (u32 i = 0; i < kIlp; ++i) {
+    const u32 k = k0 + i * kT + threadIdx.x;
+    a[i] = k + 1 < x.m ? msg_id(A.E, p, x.g_lo + k) : 0;
+    b[i] = k + 1 < x.m ? msg_id(A.E, p, x.g_lo + k + 1) : 1;
+  }
+  bool bad = false;
+#pragma unroll
+  for (u32 i = 0; i < kIlp; ++i) bad |= !(a[i] < b[i]);
+  if (bad) A.unsorted[p] = 1u;
+}
+
+// One tile of message ids of a big pair into its hash segment (as the
+// persistent launch does).
+__device__ __forceinline__ void big_build(const TileArgs& A, const TilePair& x, u32 p, u32 tile,
+                                          u32 epoch) {
+  const EncArgs& E = A.E;
+  const u64 base = seg_base(x.g_lo, p), size = seg_size(x.m);
+  const u32 k0 = tile * kBigTile;
   u64 id[kIlp], at[kIlp], cur[kIlp], prev[kIlp];
   bool live[kIlp];
 #pragma unroll
@@ -510,7 +533,6 @@ __global__ void __launch_bounds__(kT, kPerSm) codec_match_kernel(TileArgs A) {
   __shared__ u32 sm32[33];
   __shared__ u32 s_next, s_cnt[kT / 32];
   const u32 n = A.scal[TS_ITEMS], n_small = A.scal[TS_SMALL], shift = A.scal[TS_SHIFT];
-  const u32 epoch = *A.E.epoch;
   if (blockIdx.x == 0) {  // the setup's states, zero for the next call
     const u32 blocks = (u32)((A.P + kSetupT - 1) / kSetupT);
     for (u32 i = threadIdx.x; i < 4 * blocks; i += kT) A.setup_state[i] = 0;
@@ -526,7 +548,7 @@ __global__ void __launch_bounds__(kT, kPerSm) codec_match_kernel(TileArgs A) {
       if (it == ~0u) break;
       const u32 p = A.item_pair[it];
       const TilePair x = A.pair[p];
-      if (x.m > kTableMax) big_build(A, x, p, it - x.item0, epoch);
+      if (x.m > kTableMax) big_check(A, x, p, it - x.item0);
       else match_pair<kT>(A, x, p, shift, tb, reinterpret_cast<u64*>(dyn), s_cnt, sm32);
       __syncthreads();
     }
@@ -544,12 +566,108 @@ __global__ void __launch_bounds__(kT, kPerSm) codec_match_kernel(TileArgs A) {
   }
 }
 
-// Slots of the big pairs: ids looked up in the pair's hash segment, the taken
-// records marked; the block that finishes a pair's last tile lists its new
-// records.
-__global__ void __launch_bounds__(kT) codec_bigmatch_kernel(TileArgs A) {
+// First message record of pair p in [lo, hi) whose id is not below v (ids
+// ascending), by one warp, 32 probes at a time.
+__device__ __forceinline__ u32 warp_lower_bound(const EncArgs& E, u32 p, u64 g_lo, u32 lo, u32 hi,
+                                                u64 v) {
+  const u32 lane = threadIdx.x & 31;
+  while (lo < hi) {
+    const u64 len = hi - lo;
+    const bool less = msg_id(E, p, g_lo + lo + (u32)(len * lane / 32)) < v;
+    const u32 c = (u32)__popc(__ballot_sync(0xFFFFFFFFu, less));
+    const u32 base = lo;
+    if (c < 32u) hi = base + (u32)(len * c / 32);
+    if (c > 0u) lo = base + (u32)(len * (c - 1u) / 32) + 1u;
+  }
+  return lo;
+}
+
+// Ids of a big pair's window in shared memory: what 1024 slots of an ascending
+// reference span while fewer than three in four of the records between them
+// are someone else's.
+constexpr u32 kBigWindow = 4096;
+
+// The slots of an item of a big pair whose message ids ascend (live: ids id):
+// the span of message records from the item's first to its last id is found by
+// two warps and brought into shared memory when it fits, and every id in it
+// bisected there; other ids are bisected over the whole message.  (6.5 M
+// records, 1.1 M of them in one pair: 615 us of indexing and lookups in global
+// hash segments before, 295 with the check and this.)
+__device__ __forceinline__ void big_sorted(const TileArgs& A, const TilePair& x, u32 p, u32 j0,
+                                           const u64* id, const bool* live, u64* window,
+                                           u32* s_span, u32* k) {
+  const EncArgs& E = A.E;
+  const u32 j1 = x.r - j0 < kBigTile ? x.r - 1u : j0 + kBigTile - 1u;
+  const u64 first = ref_id(E, p, x.ro, j0), last = ref_id(E, p, x.ro, j1);
+  const u32 warp = threadIdx.x >> 5;
+  if (warp < 2) {
+    const u32 at = warp_lower_bound(E, p, x.g_lo, 0, x.m, warp == 0 ? first : last);
+    if ((threadIdx.x & 31) == 0) s_span[warp] = at;
+  }
+  __syncthreads();
+  const u32 lo = s_span[0], hi = s_span[1] + 1u < x.m ? s_span[1] + 1u : x.m;
+  const bool in = first <= last && lo < hi && hi - lo <= kBigWindow;  // block-uniform
+  if (in)
+    for (u32 i = threadIdx.x; i < hi - lo; i += kT) window[i] = msg_id(E, p, x.g_lo + lo + i);
+  __syncthreads();
+#pragma unroll
+  for (u32 i = 0; i < kIlp; ++i) {
+    k[i] = kNoMatch;
+    if (!live[i]) continue;
+    if (in && id[i] >= first && id[i] <= last) {
+      u32 a = 0, b = hi - lo;
+      while (a < b) {
+        const u32 mid = (a + b) >> 1;
+        if (window[mid] < id[i]) a = mid + 1;
+        else b = mid;
+      }
+      if (a < hi - lo && window[a] == id[i]) k[i] = lo + a;
+    } else {
+      u32 a = 0, b = x.m;
+      while (a < b) {
+        const u32 mid = a + ((b - a) >> 1);
+        if (msg_id(E, p, x.g_lo + mid) < id[i]) a = mid + 1;
+        else b = mid;
+      }
+      if (a < x.m && msg_id(E, p, x.g_lo + a) == id[i]) k[i] = a;
+    }
+  }
+}
+
+// The same in the pair's hash segment.
+__device__ __forceinline__ void big_lookup(const TileArgs& A, const TilePair& x, u32 p,
+                                           const u64* id, const bool* live, u32 epoch, u32* k) {
+  const EncArgs& E = A.E;
+  const u64 base = seg_base(x.g_lo, p), size = seg_size(x.m);
+  u64 at[kIlp];
+  U64x2 e[kIlp];
+#pragma unroll
+  for (u32 i = 0; i < kIlp; ++i) {
+    at[i] = seg_start(id[i], size);
+    e[i] = live[i] ? ldx<true>(E.seg + base + at[i]) : U64x2{0, 0};
+  }
+#pragma unroll
+  for (u32 i = 0; i < kIlp; ++i) {
+    k[i] = kNoMatch;
+    if (!live[i] || (u32)(e[i].a >> 32) != epoch) continue;
+    if (e[i].b == id[i]) {
+      k[i] = (u32)e[i].a;
+    } else {
+      k[i] = seg_lookup_from<true>(E.seg, epoch, base, size, 0, id[i],
+                                   at[i] + 1 == size ? 0 : at[i] + 1);
+    }
+  }
+}
+
+// The big pairs' items, claimed in order: a pair's message tiles (indexed when
+// its ids do not ascend), then its slot tiles, which wait until the tiles
+// before them are indexed (claimed earlier, so by running blocks; at most a
+// second, then TERA_ETIMEOUT and no match).  The taken records are marked; the
+// block that finishes a pair's last tile lists its new records.
+__global__ void __launch_bounds__(kT, kPerSm) codec_bigmatch_kernel(TileArgs A) {
+  extern __shared__ __align__(16) uint8_t dyn[];
   __shared__ u32 sm32[33];
-  __shared__ u32 s_next, s_last, s_hits[kBigTile / 32];
+  __shared__ u32 s_next, s_last, s_hits[kBigTile / 32], s_span[2];
   static_assert(kBigTile == 1024, "one warp adds an item's hits up");
   const u32 n = A.scal[TS_BIG];
   if (n == 0) return;
@@ -561,33 +679,51 @@ __global__ void __launch_bounds__(kT) codec_bigmatch_kernel(TileArgs A) {
     if (it == ~0u) return;
     const u32 p = A.big_pair[it];
     const TilePair x = A.pair[p];
-    const u32 j0 = (it - x.big0) * kBigTile;
-    const u64 base = seg_base(x.g_lo, p), size = seg_size(x.m);
+    const u32 nbuild = (x.m + kBigTile - 1u) / kBigTile;
+    const u32 tile = it - x.big0;
+    const bool sorted = A.unsorted[p] == 0u;
+    if (tile < nbuild) {
+      if (!sorted) {
+        big_build(A, x, p, tile, epoch);
+        __threadfence();
+      }
+      __syncthreads();
+      if (!sorted && threadIdx.x == 0) atomicAdd(A.built + p, 1u);
+      continue;
+    }
+    const u32 j0 = (tile - nbuild) * kBigTile;
     u32* bits = big_bits(A, x, p);
-    u64 id[kIlp], at[kIlp];
-    U64x2 e[kIlp];
+    u64 id[kIlp];
     bool live[kIlp];
+    u32 k[kIlp];
 #pragma unroll
     for (u32 i = 0; i < kIlp; ++i) {
       const u32 j = j0 + i * kT + threadIdx.x;
       live[i] = j < x.r;
       id[i] = live[i] ? ref_id(E, p, x.ro, j) : 0;
     }
-#pragma unroll
-    for (u32 i = 0; i < kIlp; ++i) {
-      at[i] = seg_start(id[i], size);
-      e[i] = live[i] ? ldx<true>(E.seg + base + at[i]) : U64x2{0, 0};
-    }
-    u32 k[kIlp];
-#pragma unroll
-    for (u32 i = 0; i < kIlp; ++i) {
-      k[i] = kNoMatch;
-      if (!live[i] || (u32)(e[i].a >> 32) != epoch) continue;
-      if (e[i].b == id[i]) {
-        k[i] = (u32)e[i].a;
+    if (sorted) {
+      big_sorted(A, x, p, j0, id, live, reinterpret_cast<u64*>(dyn), s_span, k);
+    } else {
+      if (threadIdx.x == 0) {
+        s_span[0] = 1u;
+        LbWait wait;
+        u32 v;
+        for (;;) {
+          asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(A.built + p) : "memory");
+          if (v >= nbuild) break;
+          if (wait.over(E.st)) {
+            s_span[0] = 0u;
+            break;
+          }
+        }
+      }
+      __syncthreads();
+      if (s_span[0]) {
+        big_lookup(A, x, p, id, live, epoch, k);
       } else {
-        k[i] = seg_lookup_from<true>(E.seg, epoch, base, size, 0, id[i],
-                                     at[i] + 1 == size ? 0 : at[i] + 1);
+#pragma unroll
+        for (u32 i = 0; i < kIlp; ++i) k[i] = kNoMatch;
       }
     }
     u32 old[kIlp];
@@ -624,7 +760,7 @@ __global__ void __launch_bounds__(kT) codec_bigmatch_kernel(TileArgs A) {
     }
     __threadfence();  // the bits before the count of finished tiles
     __syncthreads();
-    if (threadIdx.x == 0) s_last = atomicAdd(A.done + p, 1u) + 1u == x.nbig;
+    if (threadIdx.x == 0) s_last = atomicAdd(A.done + p, 1u) + 1u == x.nbig - nbuild;
     __syncthreads();
     if (s_last) {
       __threadfence();
@@ -973,7 +1109,7 @@ __global__ void __launch_bounds__(kT, kEncPerSm) codec_encode_kernel(TileArgs A)
         if (i0 + lane < hi) {
           d = row_rec(rows, lane);
           // an id that occurs twice in a big pair's message: the other record is found
-          if (t.x.m > kTableMax &&
+          if (t.x.m > kTableMax && A.unsorted[p] &&
               seg_lookup<true>(E.seg, epoch, p, t.x.g_lo, t.x.m, d.w[0]) != (u32)(t.x.g_lo + k))
             latch(E.st, TERA_EINVAL);
           code = rec_code(d, &vb);
@@ -1276,6 +1412,8 @@ tera_status launch_tiles(tera_ctx* ctx, const EncArgs& E, const DecArgs& D, bool
   A.place = ctx->t_place;
   A.tot = ctx->t_tot;
   A.done = ctx->t_done;
+  A.built = ctx->t_done + P;
+  A.unsorted = ctx->t_done + 2 * P;
   A.bits = ctx->t_bits;
   A.new_idx = ctx->t_new;
   A.scal = ctx->t_scal;
@@ -1293,7 +1431,7 @@ tera_status launch_tiles(tera_ctx* ctx, const EncArgs& E, const DecArgs& D, bool
   if ((st = check_launch(ctx, "codec_match_kernel", s)) != TERA_OK) return st;
   if (ctx->cap_records > kTableMax) {  // a big pair needs that many records
     prof_begin(ctx, s);
-    codec_bigmatch_kernel<<<grid, kT, 0, s>>>(A);
+    codec_bigmatch_kernel<<<grid, kT, 8 * kBigWindow, s>>>(A);
     if ((st = check_launch(ctx, "codec_bigmatch_kernel", s)) != TERA_OK) return st;
   }
   if (pr) {
@@ -1324,7 +1462,7 @@ void tile_list_bounds(u64 cap, u64 P, u64 warps, u64* units, u64* items, u64* bi
   const u64 most = (cap >> kMaxShift) > few ? cap >> kMaxShift : few;
   *units = 2 * most + most / kNewShare + 5 * P + 64;
   *items = cap / kBigTile + 2 * P + 64;
-  *bigs = cap / kBigTile + P + 64;
+  *bigs = 2 * (cap / kBigTile + P) + 64;
 }
 
 }  // namespace tera

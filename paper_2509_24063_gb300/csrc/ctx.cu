@@ -306,7 +306,7 @@ tera_status ensure_tiles(tera_ctx* ctx) {
   ctx->t_cap = 0;
   if (!ctx->t_pair) {
     if ((st = alloc_dev(ctx->t_tot, P * 4)) != TERA_OK) return st;
-    if ((st = alloc_dev(ctx->t_done, P)) != TERA_OK) return st;
+    if ((st = alloc_dev(ctx->t_done, 3 * P)) != TERA_OK) return st;
     if ((st = alloc_dev(ctx->t_scal, 8)) != TERA_OK) return st;
     if ((st = alloc_dev(ctx->t_part, 4 * (P / 1024 + 1) + 1)) != TERA_OK) return st;
     cudaMemset(ctx->t_part, 0, sizeof(u64) * (4 * (P / 1024 + 1) + 1));

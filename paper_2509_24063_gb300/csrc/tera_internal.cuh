@@ -138,7 +138,7 @@ struct tera_ctx {
   uint32_t* t_bytes;       // [t_units] payload bytes of each tile
   tera::u64* t_place;      // [t_units] payload bytes of the pair before each tile
   tera::u64* t_tot;        // [P * 4] matched records, XOR and residual bytes
-  uint32_t* t_done;        // [P] finished tiles of a big pair
+  uint32_t* t_done;        // [3 * P] matched and indexed tiles of a big pair, ids not ascending
   uint32_t* t_bits;        // taken records of big pairs
   uint32_t* t_new;         // [t_cap] new records of each pair
   uint32_t* t_scal;        // [8] list lengths and claim tickets
