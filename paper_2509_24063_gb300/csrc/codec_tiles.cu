@@ -172,6 +172,7 @@ __device__ __forceinline__ void fill_map(u32* __restrict__ out, u64 lo, u32 n, u
 __global__ void __launch_bounds__(kSetupT)
     tiles_setup_kernel(TileArgs A, int mode, u64* __restrict__ wire_off, u64 wire_cap, u64 rec_cap,
                        u64 recv_cap, u64 unit_cap, u64 item_cap, u64 big_cap, u32* epoch) {
+  chain_begin();
   __shared__ U64x2 sm2[33];
   __shared__ u32 first[3][kSetupT];
   __shared__ u64 s_pre[4];
@@ -330,25 +331,36 @@ __device__ __forceinline__ u32* big_bits(const TileArgs& A, const TilePair& x, u
 template <int T, bool G>
 __device__ __forceinline__ void new_list(const TileArgs& A, const TilePair& x, const u32* bits,
                                          u32* sm32) {
+  // eight words a thread and round in global memory: one block lists a big
+  // pair's records, and a round is two barriers
+  constexpr u32 kV = G ? 8 : 1;
   const u32 words = (x.m + 31u) / 32u;
   u64 run = 0;
-  for (u32 w0 = 0; w0 < words; w0 += T) {  // group-uniform
-    const u32 w = w0 + group_thread<T>();
-    u32 free = 0;
-    if (w < words) {
-      const u32 b = G ? __ldcg(bits + w) : bits[w];
-      free = ~b & ((w + 1u) * 32u <= x.m ? 0xFFFFFFFFu : (1u << (x.m & 31u)) - 1u);
+  for (u32 w0 = 0; w0 < words; w0 += T * kV) {  // group-uniform
+    const u32 w = w0 + group_thread<T>() * kV;
+    u32 free[kV], c = 0;
+#pragma unroll
+    for (u32 v = 0; v < kV; ++v) {
+      free[v] = 0;
+      if (w + v < words) {
+        const u32 b = G ? __ldcg(bits + w + v) : bits[w + v];
+        free[v] = ~b & ((w + v + 1u) * 32u <= x.m ? 0xFFFFFFFFu : (1u << (x.m & 31u)) - 1u);
+      }
     }
+#pragma unroll
+    for (u32 v = 0; v < kV; ++v) c += (u32)__popc(free[v]);
     u32 tot, pos;
     if constexpr (T == 32) {
-      const u32 c = (u32)__popc(free), inc = warp_incl_scan<u32>(c);
+      const u32 inc = warp_incl_scan<u32>(c);
       pos = inc - c;
       tot = __shfl_sync(0xFFFFFFFFu, inc, 31);
     } else {
-      pos = block_excl_scan<u32>((u32)__popc(free), sm32, &tot);
+      pos = block_excl_scan<u32>(c, sm32, &tot);
     }
     u32* out = A.new_idx + x.g_lo + run + pos;
-    for (; free; free &= free - 1u) *out++ = w * 32u + (u32)__ffs(free) - 1u;
+#pragma unroll
+    for (u32 v = 0; v < kV; ++v)
+      for (u32 f = free[v]; f; f &= f - 1u) *out++ = (w + v) * 32u + (u32)__ffs(f) - 1u;
     run += tot;
   }
 }
@@ -357,19 +369,28 @@ __device__ __forceinline__ void new_list(const TileArgs& A, const TilePair& x, c
 // (counts in the same places): their exclusive sums.
 template <int T>
 __device__ __forceinline__ void sum_tiles(const TileArgs& A, const TilePair& x, u32* sm32) {
+  constexpr u32 kV = T == 32 ? 1 : 8;
   u32 run = 0;
-  for (u32 t0 = 0; t0 < x.nst; t0 += T) {  // group-uniform
-    const u32 t = t0 + group_thread<T>();
-    const u32 c = t < x.nst ? __ldcg(A.before + x.unit0 + t) : 0u;
+  for (u32 t0 = 0; t0 < x.nst; t0 += T * kV) {  // group-uniform
+    const u32 t = t0 + group_thread<T>() * kV;
+    u32 c[kV], sum = 0;
+#pragma unroll
+    for (u32 v = 0; v < kV; ++v) c[v] = t + v < x.nst ? __ldcg(A.before + x.unit0 + t + v) : 0u;
+#pragma unroll
+    for (u32 v = 0; v < kV; ++v) sum += c[v];
     u32 tot, ex;
     if constexpr (T == 32) {
-      const u32 inc = warp_incl_scan<u32>(c);
-      ex = inc - c;
+      const u32 inc = warp_incl_scan<u32>(sum);
+      ex = inc - sum;
       tot = __shfl_sync(0xFFFFFFFFu, inc, 31);
     } else {
-      ex = block_excl_scan<u32>(c, sm32, &tot);
+      ex = block_excl_scan<u32>(sum, sm32, &tot);
     }
-    if (t < x.nst) A.before[x.unit0 + t] = run + ex;
+#pragma unroll
+    for (u32 v = 0; v < kV; ++v) {
+      if (t + v < x.nst) A.before[x.unit0 + t + v] = run + ex;
+      ex += c[v];
+    }
     run += tot;
   }
 }
@@ -529,6 +550,7 @@ __device__ __forceinline__ void map_tiles(const TileArgs& A) {
 // The pairs of the match list, a block each, claimed one by one; then the
 // small ones, a warp each.
 __global__ void __launch_bounds__(kT, kPerSm) codec_match_kernel(TileArgs A) {
+  chain_begin();
   extern __shared__ __align__(16) uint8_t dyn[];
   __shared__ u32 sm32[33];
   __shared__ u32 s_next, s_cnt[kT / 32];
@@ -665,6 +687,7 @@ __device__ __forceinline__ void big_lookup(const TileArgs& A, const TilePair& x,
 // second, then TERA_ETIMEOUT and no match).  The taken records are marked; the
 // block that finishes a pair's last tile lists its new records.
 __global__ void __launch_bounds__(kT, kPerSm) codec_bigmatch_kernel(TileArgs A) {
+  chain_begin();
   extern __shared__ __align__(16) uint8_t dyn[];
   __shared__ u32 sm32[33];
   __shared__ u32 s_next, s_last, s_hits[kBigTile / 32], s_span[2];
@@ -776,6 +799,7 @@ __global__ void __launch_bounds__(kT, kPerSm) codec_bigmatch_kernel(TileArgs A) 
 // Predictor: the XOR and residual payload bytes of every slot tile, added up
 // per pair (they choose the message mode), and the training samples.
 __global__ void __launch_bounds__(kT, kPerSm) codec_sizes_kernel(TileArgs A) {
+  chain_begin();
   __shared__ U64x2 sm[33];
   const EncArgs& E = A.E;
   const u32 n = A.scal[TS_UNITS], shift = A.scal[TS_SHIFT];
@@ -990,6 +1014,7 @@ __device__ __forceinline__ void store_next(const EncArgs& E, u32 p, u64 g, const
 
 template <bool PR>
 __global__ void __launch_bounds__(kT, kEncPerSm) codec_encode_kernel(TileArgs A) {
+  chain_begin();
   extern __shared__ __align__(16) uint8_t dyn[];
   const EncArgs& E = A.E;
   const u32 warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1170,6 +1195,7 @@ __device__ __forceinline__ void finish_message(const TileArgs& A, const Tile& t,
 // tiles before it (their counts added up).
 template <bool PR>
 __global__ void __launch_bounds__(kT, kPerSm) codec_wire_kernel(TileArgs A) {
+  chain_begin();
   const EncArgs& E = A.E;
   const u32 warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const u32 n = A.scal[TS_UNITS], shift = A.scal[TS_SHIFT];
@@ -1207,6 +1233,7 @@ __global__ void __launch_bounds__(kT, kPerSm) codec_wire_kernel(TileArgs A) {
 // encode's.
 template <bool PR>
 __global__ void __launch_bounds__(kT, kDecPerSm) codec_decode_kernel(TileArgs A) {
+  chain_begin();
   extern __shared__ __align__(16) uint8_t dyn[];
   const DecArgs& D = A.D;
   const u32 warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1422,34 +1449,34 @@ tera_status launch_tiles(tera_ctx* ctx, const EncArgs& E, const DecArgs& D, bool
   const unsigned egrid = (unsigned)(ctx->num_sms * kEncPerSm), dgrid = (unsigned)(ctx->num_sms * kDecPerSm);
   A.setup_ticket = reinterpret_cast<u32*>(ctx->t_part + 4 * (u64)setup);
   prof_begin(ctx, s);
-  tiles_setup_kernel<<<setup, kSetupT, 0, s>>>(A, mode, const_cast<u64*>(E.wire_off), wire_cap,
+  launch_chained(tiles_setup_kernel, setup, kSetupT, 0, s, A, mode, const_cast<u64*>(E.wire_off), wire_cap,
                                                ctx->cap_records, recv_cap, ctx->t_units,
                                                ctx->t_items, ctx->t_bigs, ctx->d_epoch);
   if ((st = check_launch(ctx, "tiles_setup_kernel", s)) != TERA_OK) return st;
   prof_begin(ctx, s);
-  codec_match_kernel<<<grid, kT, kMatchSmem, s>>>(A);
+  launch_chained(codec_match_kernel, grid, kT, kMatchSmem, s, A);
   if ((st = check_launch(ctx, "codec_match_kernel", s)) != TERA_OK) return st;
   if (ctx->cap_records > kTableMax) {  // a big pair needs that many records
     prof_begin(ctx, s);
-    codec_bigmatch_kernel<<<grid, kT, 8 * kBigWindow, s>>>(A);
+    launch_chained(codec_bigmatch_kernel, grid, kT, 8 * kBigWindow, s, A);
     if ((st = check_launch(ctx, "codec_bigmatch_kernel", s)) != TERA_OK) return st;
   }
   if (pr) {
     prof_begin(ctx, s);
-    codec_sizes_kernel<<<grid, kT, 0, s>>>(A);
+    launch_chained(codec_sizes_kernel, grid, kT, 0, s, A);
     if ((st = check_launch(ctx, "codec_sizes_kernel", s)) != TERA_OK) return st;
   }
   prof_begin(ctx, s);
-  if (pr) codec_encode_kernel<true><<<egrid, kT, kEncSmem, s>>>(A);
-  else codec_encode_kernel<false><<<egrid, kT, kEncSmem, s>>>(A);
+  if (pr) launch_chained(codec_encode_kernel<true>, egrid, kT, kEncSmem, s, A);
+  else launch_chained(codec_encode_kernel<false>, egrid, kT, kEncSmem, s, A);
   if ((st = check_launch(ctx, "codec_encode_kernel", s)) != TERA_OK) return st;
   prof_begin(ctx, s);
-  if (pr) codec_wire_kernel<true><<<grid, kT, 0, s>>>(A);
-  else codec_wire_kernel<false><<<grid, kT, 0, s>>>(A);
+  if (pr) launch_chained(codec_wire_kernel<true>, grid, kT, 0, s, A);
+  else launch_chained(codec_wire_kernel<false>, grid, kT, 0, s, A);
   if ((st = check_launch(ctx, "codec_wire_kernel", s)) != TERA_OK) return st;
   prof_begin(ctx, s);
-  if (pr) codec_decode_kernel<true><<<dgrid, kT, kDecSmem, s>>>(A);
-  else codec_decode_kernel<false><<<dgrid, kT, kDecSmem, s>>>(A);
+  if (pr) launch_chained(codec_decode_kernel<true>, dgrid, kT, kDecSmem, s, A);
+  else launch_chained(codec_decode_kernel<false>, dgrid, kT, kDecSmem, s, A);
   return check_launch(ctx, "codec_decode_kernel", s);
 }
 

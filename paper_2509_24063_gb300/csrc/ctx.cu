@@ -43,6 +43,7 @@ tera_status alloc_dev(T*& p, size_t count) {
 __global__ void __launch_bounds__(kScanThreads)
     scan_kernel(const u32* __restrict__ in, u64 n, u64* __restrict__ out64,
                 u32* __restrict__ out32, u64* __restrict__ state, DevStatus* st) {
+  chain_begin();
   __shared__ u64 sm[33];
   __shared__ u64 s_pre;
   __shared__ u32 s_tile;
@@ -211,7 +212,7 @@ tera_status scan_u32(tera_ctx* ctx, const u32* in, u64* out64, u32* out32, u64 n
   if (chunks == 0) chunks = 1;
   if (chunks > 1) cudaMemsetAsync(ctx->scan_part, 0, sizeof(u64) * (chunks + 1), s);
   prof_begin(ctx, s);
-  scan_kernel<<<(unsigned)chunks, kScanThreads, 0, s>>>(in, n, out64, out32, ctx->scan_part,
+  launch_chained(scan_kernel, (unsigned)chunks, kScanThreads, 0, s, in, n, out64, out32, ctx->scan_part,
                                                         ctx->d_status);
   return check_launch(ctx, "scan_kernel", s);
 }
@@ -924,6 +925,7 @@ namespace {
 __global__ void __launch_bounds__(256)
     wire_to_host_kernel(const uint4* __restrict__ wire, const u64* __restrict__ wire_off, u64 P,
                         uint4* __restrict__ dst, u64 cap, u64* count, DevStatus* st) {
+  chain_begin();
   const u64 n = wire_off[P];
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     *count = n;
@@ -952,7 +954,7 @@ extern "C" tera_status tera_wire_to_host(tera_ctx* ctx, const uint8_t* wire,
   cudaSetDevice(ctx->device);
   cudaStream_t s = (cudaStream_t)stream;
   prof_begin(ctx, s);
-  wire_to_host_kernel<<<(unsigned)grid_for(ctx, 8), 256, 0, s>>>(
+  launch_chained(wire_to_host_kernel, (unsigned)grid_for(ctx, 8), 256, 0, s, 
       reinterpret_cast<const uint4*>(wire), reinterpret_cast<const u64*>(wire_off),
       ctx->n_pairs, reinterpret_cast<uint4*>(host_dst), host_capacity,
       reinterpret_cast<u64*>(host_count), ctx->d_status);

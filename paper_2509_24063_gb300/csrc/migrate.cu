@@ -159,6 +159,7 @@ __global__ void __launch_bounds__(kClassifyThreads, 5)
                      const u64* __restrict__ z, u64 n, const u64* __restrict__ box_off,
                      u32 n_boxes, const GridTables* __restrict__ g, u32* __restrict__ tile_cnt,
                      u64 n_wtiles, u64* __restrict__ from, u64* __restrict__ cnt, DevStatus* st) {
+  chain_begin();
   __shared__ SmemGrid sg;
   load_grid(sg, g);
   const int lane = threadIdx.x & 31;
@@ -231,6 +232,7 @@ __global__ void __launch_bounds__(1024)
                     const u64* __restrict__ from, const u64* __restrict__ cnt, u64 arena_units,
                     u64 lv_cap, u64* __restrict__ inbox_off, u64* __restrict__ box_off_next,
                     u64* __restrict__ before, DevStatus* st) {
+  chain_begin();
   __shared__ u64 sm[33];
   __shared__ u32 bad;
   const u64 Q = (u64)n_boxes * 27u;
@@ -296,6 +298,7 @@ __global__ void __launch_bounds__(kClassifyThreads, 4)
                     const u64* __restrict__ box_off_next, const u64* __restrict__ before,
                     ColsOut next, u32* __restrict__ lv_key, u32* __restrict__ lv_agent, u64 lv_cap,
                     const DevStatus* st) {
+  chain_begin();
   __shared__ SmemGrid sg;
   if (aborted(st)) return;
   load_grid(sg, g);
@@ -389,6 +392,7 @@ __global__ void __launch_bounds__(256)
                     const u32* __restrict__ lv_key, const u32* __restrict__ lv_agent,
                     const u32* __restrict__ lv_dest, u32 class_id, uint8_t* __restrict__ arena,
                     const DevStatus* st) {
+  chain_begin();
   if (aborted(st)) return;
   const u64 L = inbox_off[Q];
   const u64 total = Q + 4 * L;
@@ -430,6 +434,7 @@ __global__ void __launch_bounds__(256)
     mig_unpack_kernel(const uint8_t* __restrict__ arena, u64 arena_units,
                       const u64* __restrict__ inbox_off, u64 Q, const u64* __restrict__ box_off_next,
                       u32 class_id, ColsOut next, u64 n_next, DevStatus* st) {
+  chain_begin();
   if (aborted(st)) return;
   const u64 L = inbox_off[Q];
   if (L > arena_units || L + Q > arena_units) {  // more records than the arena holds
@@ -540,19 +545,19 @@ extern "C" tera_status tera_migrate_send(tera_ctx* ctx, const tera_soa* prev,
   const u64 blocks = n == 0 ? 1 : (n + kBlockAgents - 1) / kBlockAgents;
   const u64 wtiles = n == 0 ? 1 : (n + kWarpAgents - 1) / kWarpAgents;
   prof_begin(ctx, s);
-  mig_count_kernel<<<(unsigned)blocks, kClassifyThreads, grid_smem_bytes(ctx->grid), s>>>(
+  launch_chained(mig_count_kernel, (unsigned)blocks, kClassifyThreads, grid_smem_bytes(ctx->grid), s, 
       cp.c[1], cp.c[2], cp.c[3], n, off_prev, (u32)B, ctx->d_grid, ctx->m_tile_cnt, wtiles,
       ctx->m_from, ctx->m_cnt, ctx->d_status);
   if ((st = check_launch(ctx, "mig_count_kernel", s)) != TERA_OK) return st;
   if ((st = scan_u32(ctx, ctx->m_tile_cnt, ctx->m_tile_base, nullptr, wtiles, s)) != TERA_OK)
     return st;
   prof_begin(ctx, s);
-  mig_scan_kernel<<<1, 1024, 0, s>>>(off_prev, n, (u32)B, ctx->m_from, ctx->m_cnt, arena_units,
+  launch_chained(mig_scan_kernel, 1, 1024, 0, s, off_prev, n, (u32)B, ctx->m_from, ctx->m_cnt, arena_units,
                                      lv_cap, inbox, off_next, ctx->m_before, ctx->d_status);
   if ((st = check_launch(ctx, "mig_scan_kernel", s)) != TERA_OK) return st;
   if (n > 0) {
     prof_begin(ctx, s);
-    mig_move_kernel<<<(unsigned)blocks, kClassifyThreads, grid_smem_bytes(ctx->grid), s>>>(
+    launch_chained(mig_move_kernel, (unsigned)blocks, kClassifyThreads, grid_smem_bytes(ctx->grid), s, 
         cp, n, off_prev, (u32)B, ctx->d_grid, ctx->m_tile_base, off_next, ctx->m_before, cn,
         ctx->m_key, ctx->m_agent, lv_cap, ctx->d_status);
     if ((st = check_launch(ctx, "mig_move_kernel", s)) != TERA_OK) return st;
@@ -566,7 +571,7 @@ extern "C" tera_status tera_migrate_send(tera_ctx* ctx, const tera_soa* prev,
                                inbox + Q, lv_cap, Q, &sorted, s)) != TERA_OK)
     return st;
   prof_begin(ctx, s);
-  mig_pack_kernel<<<(unsigned)grid_for(ctx, 4), 256, 0, s>>>(cp, inbox, Q, ctx->m_key,
+  launch_chained(mig_pack_kernel, (unsigned)grid_for(ctx, 4), 256, 0, s, cp, inbox, Q, ctx->m_key,
                                                              ctx->m_agent, ctx->m_dest,
                                                              ctx->class_id, arena, ctx->d_status);
   return check_launch(ctx, "mig_pack_kernel", s);
@@ -584,7 +589,7 @@ extern "C" tera_status tera_migrate_recv(tera_ctx* ctx, const uint8_t* arena, ui
   cudaSetDevice(ctx->device);
   cudaStream_t s = (cudaStream_t)stream;
   prof_begin(ctx, s);
-  mig_unpack_kernel<<<(unsigned)grid_for(ctx, 4), 256, 0, s>>>(
+  launch_chained(mig_unpack_kernel, (unsigned)grid_for(ctx, 4), 256, 0, s, 
       arena, arena_units, reinterpret_cast<const u64*>(inbox_off), ctx->n_pairs,
       reinterpret_cast<const u64*>(box_off_next), ctx->class_id, cn, (u64)next->n,
       ctx->d_status);

@@ -120,6 +120,7 @@ __global__ void __launch_bounds__(kClassifyThreads)
                      const u32* __restrict__ ent_dest, const u64* __restrict__ pair_off, u64 P,
                      uint8_t* __restrict__ arena, u64 arena_units, u32 class_id, DevStatus* st,
                      u64* __restrict__ rec_ids) {
+  chain_begin();
   const u64 E = pair_off[P];
   if (E + P > arena_units) {
     if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -232,7 +233,7 @@ static tera_status pack_impl(tera_ctx* ctx, const tera_soa* soa, const tera_part
     const u64 blocks = n == 0 ? 1 : (n + kClassifyTile - 1) / kClassifyTile;
     const u64 runs = n == 0 ? 1 : (n + kRunAgents - 1) / kRunAgents;
     prof_begin(ctx, s);
-    pack_runs_kernel<<<(unsigned)blocks, kClassifyThreads, 0, s>>>(
+    launch_chained(pack_runs_kernel, (unsigned)blocks, kClassifyThreads, 0, s, 
         p, n, part->owner, part->mask, ctx->tile_base, runs, ctx->ent_dest,
         reinterpret_cast<const u64*>(part->pair_off), ctx->n_pairs, rec_arena, arena_units,
         ctx->class_id, ctx->d_status, reinterpret_cast<u64*>(rec_ids));

@@ -87,15 +87,6 @@ __global__ void __launch_bounds__(kClassifyThreads, 6)
                     DevStats* stats, u64* __restrict__ sort_head) {
   __shared__ SmemGrid sg;
   __shared__ float s_flo[3], s_fs[3];
-  if (blockIdx.x == 0) {  // what the launches after this one find zero
-    for (u32 i = threadIdx.x; i < kSortHead; i += blockDim.x) sort_head[i] = 0;
-    if (threadIdx.x == 0) {
-      stats->iterations += 1;
-      stats->agents += n;
-      st->abort = 0;
-      if (n == 0) run_cnt[0] = 0;
-    }
-  }
   // the tables follow the grid rows (a multiple of 32 bytes) in dynamic shared memory
   uint8_t* tab = reinterpret_cast<uint8_t*>(grid_rows() + (g->n[0] + g->n[1] + g->n[2]));
   if (bk) {
@@ -108,6 +99,16 @@ __global__ void __launch_bounds__(kClassifyThreads, 6)
     }
   }
   load_grid(sg, g);  // ends with a block barrier
+  chain_begin();  // (the tables are the context's: written when it was made)
+  if (blockIdx.x == 0) {  // what the launches after this one find zero
+    for (u32 i = threadIdx.x; i < kSortHead; i += blockDim.x) sort_head[i] = 0;
+    if (threadIdx.x == 0) {
+      stats->iterations += 1;
+      stats->agents += n;
+      st->abort = 0;
+      if (n == 0) run_cnt[0] = 0;
+    }
+  }
   const int lane = threadIdx.x & 31;
   bool bad = false;
   for (u64 tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
@@ -168,6 +169,7 @@ __global__ void __launch_bounds__(kClassifyThreads)
     emit_kernel(const int* __restrict__ owner, const u32* __restrict__ mask, u64 n,
                 const u64* __restrict__ run_base, u64 n_runs, u32* __restrict__ keys,
                 u32* __restrict__ vals, u64 cap, DevStatus* st) {
+  chain_begin();
   if (*reinterpret_cast<const volatile u32*>(&st->abort)) return;  // the scan gave up
   const u64 total = run_base[n_runs];
   const u64 n_entries = total;  // (a warp's own count below is also called total)
@@ -252,6 +254,7 @@ __device__ __forceinline__ u64* sort_states(u64* head, u32 pass, u64 tiles, u32 
 __global__ void __launch_bounds__(kSortThreads)
     rs_hist_kernel(const u32* __restrict__ keys, const u64* __restrict__ total_ptr, u64 cap,
                    u32 passes, u32 dbits, u64 tiles, u64* __restrict__ head, const DevStatus* st) {
+  chain_begin();
   __shared__ u32 cnt[4 * kRadix];
   const u64 E = live_entries(total_ptr, cap, st);
   const u32 radix = 1u << dbits;
@@ -327,6 +330,7 @@ __global__ void __launch_bounds__(kSortThreads)
                       u32* __restrict__ dest, int last, const u64* __restrict__ total_ptr, u64 cap,
                       u32 pass, u32 shift, u32 radix, u64* __restrict__ head, u64 n_tiles,
                       DevStatus* st) {
+  chain_begin();
   constexpr int kWarps = kSortThreads / 32;
   constexpr int kRoundEntries = kSortThreads * kSortSub;
   extern __shared__ __align__(16) u32 sort_stage[];
@@ -499,6 +503,7 @@ __global__ void __launch_bounds__(256)
     pair_off_kernel(const u32* __restrict__ sorted_keys, const u64* __restrict__ total_ptr, u64 cap,
                     u64 n_pairs, u64* __restrict__ pair_off, u64* __restrict__ pair_count,
                     DevStats* stats, const DevStatus* st) {
+  chain_begin();
   const u64 E = live_entries(total_ptr, cap, st);
   if (blockIdx.x == 0 && threadIdx.x == 0) stats->records += E;
   const u32 lane = threadIdx.x & 31;
@@ -568,7 +573,7 @@ tera_status radix_sort_entries(tera_ctx* ctx, const SortBufs& b, const u32* keys
     if (!zeroed) cudaMemsetAsync(b.hist, 0, sizeof(u64) * kSortHead, s);
     const u64 hgrid = (u64)grid_for(ctx, 4);
     prof_begin(ctx, s);
-    rs_hist_kernel<<<(unsigned)(tiles < hgrid ? tiles : hgrid), kSortThreads, 0, s>>>(
+    launch_chained(rs_hist_kernel, (unsigned)(tiles < hgrid ? tiles : hgrid), kSortThreads, 0, s, 
         keys_in, total_ptr, cap, (u32)passes, (u32)dbits, tiles, b.hist, ctx->d_status);
     if ((st = check_launch(ctx, "rs_hist_kernel", s)) != TERA_OK) return st;
   }
@@ -584,11 +589,11 @@ tera_status radix_sort_entries(tera_ctx* ctx, const SortBufs& b, const u32* keys
     const unsigned grid = (unsigned)(tiles < res ? tiles : res);
     prof_begin(ctx, s);
     if (radix <= 128)
-      rs_scatter_kernel<128><<<grid, kSortThreads, smem, s>>>(
+      launch_chained(rs_scatter_kernel<128>, grid, kSortThreads, smem, s, 
           kin, vin, ain, kout, vout, aout, last ? dest : nullptr, last ? 1 : 0, total_ptr, cap,
           (u32)pass, shift, radix, b.hist, tiles, ctx->d_status);
     else
-      rs_scatter_kernel<kRadix><<<grid, kSortThreads, smem, s>>>(
+      launch_chained(rs_scatter_kernel<kRadix>, grid, kSortThreads, smem, s, 
           kin, vin, ain, kout, vout, aout, last ? dest : nullptr, last ? 1 : 0, total_ptr, cap,
           (u32)pass, shift, radix, b.hist, tiles, ctx->d_status);
     if ((st = check_launch(ctx, "rs_scatter_kernel", s)) != TERA_OK) return st;
@@ -636,7 +641,7 @@ extern "C" tera_status tera_partition(tera_ctx* ctx, const tera_soa* soa, tera_p
   }
   const u64 cgrid = blocks < (u64)ctx->num_sms * 6 ? blocks : (u64)ctx->num_sms * 6;
   prof_begin(ctx, s);
-  classify_kernel<<<(unsigned)cgrid, kClassifyThreads, csmem, s>>>(
+  launch_chained(classify_kernel, (unsigned)cgrid, kClassifyThreads, csmem, s, 
       reinterpret_cast<const u64*>(soa->x), reinterpret_cast<const u64*>(soa->y),
       reinterpret_cast<const u64*>(soa->z), n, ctx->d_grid, ctx->d_buckets, blocks, out->owner,
       out->mask, ctx->tile_cnt, runs, ctx->d_status, ctx->d_stats, ctx->rs_hist);
@@ -649,7 +654,7 @@ extern "C" tera_status tera_partition(tera_ctx* ctx, const tera_soa* soa, tera_p
   const u64* total_ptr = ctx->tile_base + runs;
   if (cap > 0 || n > 0) {
     prof_begin(ctx, s);
-    emit_kernel<<<(unsigned)blocks, kClassifyThreads, 0, s>>>(
+    launch_chained(emit_kernel, (unsigned)blocks, kClassifyThreads, 0, s, 
         out->owner, out->mask, n, ctx->tile_base, runs, ctx->keys_a, ctx->ent_agent, cap,
         ctx->d_status);
     if ((st = check_launch(ctx, "emit_kernel", s)) != TERA_OK) return st;
@@ -663,7 +668,7 @@ extern "C" tera_status tera_partition(tera_ctx* ctx, const tera_soa* soa, tera_p
   ctx->rec_pair = const_cast<u32*>(sorted);
   ctx->pack_n = soa->n;
   prof_begin(ctx, s);
-  pair_off_kernel<<<(unsigned)(P / 8 + 1), 256, 0, s>>>(
+  launch_chained(pair_off_kernel, (unsigned)(P / 8 + 1), 256, 0, s, 
       sorted, total_ptr, cap, P, reinterpret_cast<u64*>(out->pair_off),
       reinterpret_cast<u64*>(out->pair_count), ctx->d_stats, ctx->d_status);
   return check_launch(ctx, "pair_off_kernel", s);

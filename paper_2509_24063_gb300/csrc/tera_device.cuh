@@ -99,6 +99,17 @@ struct DevStats {
 __device__ __forceinline__ void latch(DevStatus* s, u32 code) { atomicCAS(&s->code, 0u, code); }
 __device__ __forceinline__ void need(DevStatus* s, u64 req) { atomicMax(&s->required, req); }
 
+// Chained launches (launch_chained): a kernel may be started before the memory
+// of the one before it in the stream is flushed.  chain_begin() comes before a
+// kernel's first access to memory that an earlier launch may write or read, and
+// waits for the earlier launches.  No kernel lets the next one start early: its
+// blocks would take the registers and shared memory of blocks still at work
+// (griddepcontrol.launch_dependents at each kernel's start: 100 M agents 4.10
+// -> 4.75 ms).
+__device__ __forceinline__ void chain_begin() {
+  asm volatile("griddepcontrol.wait;" : : : "memory");
+}
+
 // Bounds check of the debug build (compiled with TERA_DEBUG_BOUNDS): true
 // when lo <= i < hi; otherwise TERA_EBOUNDS is latched and the caller skips
 // its write.  Other builds check nothing (always true, no code).

@@ -166,6 +166,26 @@ struct tera_ctx {
 };
 
 namespace tera {
+// Launch of a kernel that calls chain_begin() before it touches memory other
+// launches use: it is set up while the launch before it ends, so that a chain
+// of launches does not pay each one's start-up (1 M agents, 15 launches: 251 ->
+// 218 us; 16 M kept box by box 1.35 -> 1.31 ms).
+template <typename... P, typename... A>
+inline void launch_chained(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem,
+                           cudaStream_t s, A... args) {
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = dim3(grid);
+  c.blockDim = dim3(block);
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  c.attrs = &attr;
+  c.numAttrs = 1;
+  cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+}
+
 // ctx.cu
 void prof_begin(tera_ctx* ctx, cudaStream_t s);
 tera_status check_launch(tera_ctx* ctx, const char* name, cudaStream_t s);
