@@ -142,7 +142,8 @@ struct DecArgs {
 
 // codec_tiles.cu: steps a3-a5 of every pair (no explicit schedule).  E and D as
 // the entry point filled them; with the predictor, each side's predictions are
-// made.  The lists' bounds for cap records of P pairs.
+// made.  D.recv null: steps a3 and a4 alone (the payload is packed in the
+// context's scratch).  The lists' bounds for cap records of P pairs.
 tera_status launch_tiles(tera_ctx* ctx, const EncArgs& E, const DecArgs& D, bool pr, int mode,
                          u64 wire_cap, u64 recv_cap, cudaStream_t s);
 void tile_list_bounds(u64 cap, u64 P, u64 warps, u64* units, u64* items, u64* bigs);

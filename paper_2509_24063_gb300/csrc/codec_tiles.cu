@@ -104,6 +104,7 @@ struct TileArgs {
   u32* unsorted;        // [P] a big pair whose message ids do not ascend
   u32* bits;            // taken records of big pairs: word (g_lo >> 5) + p of pair p
   u32* new_idx;         // new records of each pair in message order, from g_lo
+  uint8_t* scratch;     // arena for the packed payload
   u32* scal;            // TS_*
   u64 P;
 };
@@ -217,7 +218,7 @@ __global__ void __launch_bounds__(kSetupT)
   if (p < P) {
     const u64 w = carry_a.a + ea.a, g_lo = A.E.pair_off[p];
     wire_off[p] = w;
-    A.D.recv_off[p] = g_lo;
+    if (A.D.recv_off) A.D.recv_off[p] = g_lo;  // receive buffers sized by the record counts
     if (!abort) {
       TilePair x;
       x.g_lo = g_lo;
@@ -250,7 +251,8 @@ __global__ void __launch_bounds__(kSetupT)
         h[3] = make_ulonglong2(p, kHdrBytes);
         A.E.wire_len[p] = kHdrBytes;
         write_taio_header(A.E.ref_next + (g_lo + p) * kRecBytes, A.E.class_id, (u32)p, 0);
-        write_taio_header(A.D.recv + (g_lo + p) * kRecBytes, A.D.class_id, (u32)p, 0);
+        if (A.D.recv)
+          write_taio_header(A.D.recv + (g_lo + p) * kRecBytes, A.D.class_id, (u32)p, 0);
         A.E.reset[p] = 0;
         empties = 1;
         if (x.mode != TERA_MODE_RAW && A.D.ref) {  // as the decode's header check
@@ -279,7 +281,7 @@ __global__ void __launch_bounds__(kSetupT)
     const U64x2 all_a = carry_a + ta, all_b = carry_b + tb;
     const u64 n_items = all_b.a & 0xFFFFFFFFull, n_small = all_b.a >> 32;
     wire_off[P] = all_a.a;
-    A.D.recv_off[P] = E;
+    if (A.D.recv_off) A.D.recv_off[P] = E;
     bool none = abort;
     if (all_a.a > wire_cap) {
       latch(A.E.st, TERA_ECAPACITY);
@@ -904,10 +906,12 @@ __device__ __forceinline__ u64 message_mode(const TileArgs& A, const Tile& t) {
   return t.x.mode;
 }
 
-// Where the records of a pair lie in the receive buffer; until the decode it
-// holds the tiles' packed payload, each tile's from its first record's place.
+// Where the records of a pair lie in an arena the size of the receive buffer
+// (the receive buffer itself, which holds the payload until the decode, or the
+// context's when there is no decode): the tiles' packed payload, each tile's
+// from its first record's place.
 __device__ __forceinline__ uint8_t* payload_place(const TileArgs& A, const Tile& t, u64 record) {
-  return A.D.recv + (t.x.g_lo + t.p + 1 + record) * kRecBytes;
+  return A.scratch + (t.x.g_lo + t.p + 1 + record) * kRecBytes;
 }
 
 // Two words of a record, and their significant bytes.
@@ -1408,6 +1412,7 @@ namespace tera {
 tera_status launch_tiles(tera_ctx* ctx, const EncArgs& E, const DecArgs& D, bool pr, int mode,
                          u64 wire_cap, u64 recv_cap, cudaStream_t s) {
   const u64 P = ctx->n_pairs;
+  const bool encode_only = D.recv == nullptr;
   tera_status st;
   const unsigned grid = (unsigned)(ctx->num_sms * kPerSm);
   static bool configured = false;
@@ -1443,6 +1448,7 @@ tera_status launch_tiles(tera_ctx* ctx, const EncArgs& E, const DecArgs& D, bool
   A.unsorted = ctx->t_done + 2 * P;
   A.bits = ctx->t_bits;
   A.new_idx = ctx->t_new;
+  A.scratch = encode_only ? ctx->t_scratch : D.recv;
   A.scal = ctx->t_scal;
   A.P = P;
   const unsigned setup = (unsigned)(P == 0 ? 1 : (P + kSetupT - 1) / kSetupT);
@@ -1474,6 +1480,7 @@ tera_status launch_tiles(tera_ctx* ctx, const EncArgs& E, const DecArgs& D, bool
   if (pr) launch_chained(codec_wire_kernel<true>, grid, kT, 0, s, A);
   else launch_chained(codec_wire_kernel<false>, grid, kT, 0, s, A);
   if ((st = check_launch(ctx, "codec_wire_kernel", s)) != TERA_OK) return st;
+  if (encode_only) return TERA_OK;
   prof_begin(ctx, s);
   if (pr) launch_chained(codec_decode_kernel<true>, dgrid, kT, kDecSmem, s, A);
   else launch_chained(codec_decode_kernel<false>, dgrid, kT, kDecSmem, s, A);

@@ -7,6 +7,7 @@
 #include <cstring>
 #include <new>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "codec.cuh"
@@ -299,33 +300,60 @@ tera_status ensure_batched(tera_ctx* ctx) {
   return TERA_OK;
 }
 
+// One allocation holds every list, so that a first call pays for one.
 tera_status ensure_tiles(tera_ctx* ctx) {
-  if (ctx->t_cap >= ctx->cap_records && ctx->t_pair) return TERA_OK;
+  if (ctx->t_cap >= ctx->cap_records && ctx->t_block) return TERA_OK;
   cudaDeviceSynchronize();
   const u64 P = ctx->n_pairs, cap = ctx->cap_records;
-  tera_status st;
   ctx->t_cap = 0;
-  if (!ctx->t_pair) {
-    if ((st = alloc_dev(ctx->t_tot, P * 4)) != TERA_OK) return st;
-    if ((st = alloc_dev(ctx->t_done, 3 * P)) != TERA_OK) return st;
-    if ((st = alloc_dev(ctx->t_scal, 8)) != TERA_OK) return st;
-    if ((st = alloc_dev(ctx->t_part, 4 * (P / 1024 + 1) + 1)) != TERA_OK) return st;
-    cudaMemset(ctx->t_part, 0, sizeof(u64) * (4 * (P / 1024 + 1) + 1));
-    if ((st = alloc_dev(ctx->t_unit_first, P)) != TERA_OK) return st;
-    if ((st = alloc_dev(ctx->t_small_pair, P)) != TERA_OK) return st;
-    if ((st = alloc_dev(ctx->t_pair, P * 8)) != TERA_OK) return st;
-  }
   tile_list_bounds(cap, P, (u64)ctx->num_sms * 32, &ctx->t_units, &ctx->t_items, &ctx->t_bigs);
-  if ((st = alloc_dev(ctx->t_unit_pair, ctx->t_units)) != TERA_OK) return st;
-  if ((st = alloc_dev(ctx->t_item_pair, ctx->t_items)) != TERA_OK) return st;
-  if ((st = alloc_dev(ctx->t_big_pair, ctx->t_bigs)) != TERA_OK) return st;
-  if ((st = alloc_dev(ctx->t_before, ctx->t_units)) != TERA_OK) return st;
-  if ((st = alloc_dev(ctx->t_bytes, ctx->t_units)) != TERA_OK) return st;
-  if ((st = alloc_dev(ctx->t_place, ctx->t_units)) != TERA_OK) return st;
-  if ((st = alloc_dev(ctx->t_bits, cap / 32 + P + 2)) != TERA_OK) return st;
-  if ((st = alloc_dev(ctx->t_new, cap)) != TERA_OK) return st;
+  uint8_t* base = nullptr;
+  size_t at = 0;
+  auto take = [&](auto*& p, u64 count) {  // 64-byte aligned; placed once the block exists
+    if (base) p = reinterpret_cast<std::remove_reference_t<decltype(p)>>(base + at);
+    at += (sizeof(*p) * count + 63) & ~(size_t)63;
+  };
+  auto lay = [&]() {
+    at = 0;
+    take(ctx->t_part, 4 * (P / 1024 + 1) + 1);
+    take(ctx->t_pair, P * 8);
+    take(ctx->t_tot, P * 4);
+    take(ctx->t_done, 3 * P);
+    take(ctx->t_scal, 8);
+    take(ctx->t_unit_first, P);
+    take(ctx->t_small_pair, P);
+    take(ctx->t_unit_pair, ctx->t_units);
+    take(ctx->t_item_pair, ctx->t_items);
+    take(ctx->t_big_pair, ctx->t_bigs);
+    take(ctx->t_before, ctx->t_units);
+    take(ctx->t_bytes, ctx->t_units);
+    take(ctx->t_place, ctx->t_units);
+    take(ctx->t_bits, cap / 32 + P + 2);
+    take(ctx->t_new, cap);
+  };
+  lay();
+  tera_status st = alloc_dev(ctx->t_block, at);
+  if (st != TERA_OK) return st;
+  base = ctx->t_block;
+  lay();
+  cudaMemset(ctx->t_part, 0, sizeof(u64) * (4 * (P / 1024 + 1) + 1));
   ctx->t_cap = cap;
   return TERA_OK;
+}
+
+bool encode_tiles_ready(tera_ctx* ctx, cudaStream_t s) {
+  const bool have = ctx->t_block && ctx->t_cap >= ctx->cap_records && ctx->t_scratch &&
+                    ctx->t_scratch_cap >= ctx->cap_records;
+  if (have) return true;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) return false;
+  if (ensure_tiles(ctx) != TERA_OK) return false;
+  cudaDeviceSynchronize();
+  ctx->t_scratch_cap = 0;
+  if (alloc_dev(ctx->t_scratch, (ctx->cap_records + ctx->n_pairs + 1) * (u64)kRecBytes) != TERA_OK)
+    return false;
+  ctx->t_scratch_cap = ctx->cap_records;
+  return true;
 }
 
 tera_status ensure_migrate(tera_ctx* ctx, uint64_t n, uint64_t leavers) {
@@ -719,21 +747,8 @@ tera_status tera_ctx_destroy(tera_ctx* c) {
   free_dev(c->b_tsum);
   free_dev(c->b_tbase);
   free_dev(c->b_part);
-  free_dev(c->t_pair);
-  free_dev(c->t_unit_pair);
-  free_dev(c->t_unit_first);
-  free_dev(c->t_item_pair);
-  free_dev(c->t_big_pair);
-  free_dev(c->t_small_pair);
-  free_dev(c->t_before);
-  free_dev(c->t_bytes);
-  free_dev(c->t_place);
-  free_dev(c->t_tot);
-  free_dev(c->t_done);
-  free_dev(c->t_bits);
-  free_dev(c->t_new);
-  free_dev(c->t_scal);
-  free_dev(c->t_part);
+  free_dev(c->t_block);
+  free_dev(c->t_scratch);
   free_dev(c->m_tile_cnt);
   free_dev(c->m_tile_base);
   free_dev(c->m_from);

@@ -1,4 +1,5 @@
-"""The batched codec over tiles (no explicit schedule) at the sizes where its
+"""The codec over tiles (batched without an explicit schedule, and the encode
+of every pair) at the sizes where its
 steps, tiles and ways of matching change, byte for byte against the oracle."""
 import numpy as np
 import pytest
@@ -17,10 +18,10 @@ def tera():
     return t
 
 
-def run_states(tera, states, lo, hi, grid, w, id_columns=True):
+def run_states(tera, states, lo, hi, grid, w, id_columns=True, path="batched"):
     ctx = tera.Context(lo, hi, grid, w)
     nmax = max(int(s["x"].shape[0]) for s in states)
-    ex = tera.AuraExchange(ctx, max_agents=nmax, max_records=3 * nmax + 1024, path="batched",
+    ex = tera.AuraExchange(ctx, max_agents=nmax, max_records=3 * nmax + 1024, path=path,
                            id_columns=id_columns)
     g = oracle.make_grid(lo, hi, grid, w)
     ref = recv_ref = None
@@ -70,10 +71,12 @@ def two_pairs(a, b, seed):
     return [st, second, third]
 
 
+@pytest.mark.parametrize("path", ["batched", "all_pairs"])
 @pytest.mark.parametrize("order", ["ascending", "shuffled"])
 @pytest.mark.parametrize("a,b", [(0, 0), (1, 0), (31, 33), (32, 64), (63, 65), (255, 257),
-                                 (511, 513), (2047, 4097), (8191, 8192), (8193, 70000)])
-def test_pair_sizes_at_the_edges(tera, a, b, order):
+                                 (511, 513), (3136, 3137), (2047, 4097), (6272, 6273), (8191, 8192),
+                                 (8193, 70000)])
+def test_pair_sizes_at_the_edges(tera, a, b, order, path):
     states = two_pairs(a, b, 7 * a + b)
     if order == "shuffled":  # a message's ids in no order: the hash tables match them
         g = torch.Generator(device="cuda")
@@ -81,7 +84,7 @@ def test_pair_sizes_at_the_edges(tera, a, b, order):
         for k, st in enumerate(states):
             perm = torch.randperm(st["x"].shape[0], generator=g, device="cuda")
             states[k] = {f: v[perm].contiguous() for f, v in st.items()}
-    run_states(tera, states, (0.0,) * 3, (200.0, 100.0, 100.0), (2, 1, 1), 20.0)
+    run_states(tera, states, (0.0,) * 3, (200.0, 100.0, 100.0), (2, 1, 1), 20.0, path=path)
 
 
 @pytest.mark.parametrize("id_columns", [True, False])
