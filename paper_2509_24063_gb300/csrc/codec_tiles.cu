@@ -60,7 +60,7 @@ constexpr u32 kNewShare = 16;
 // once (13,824 pairs, 100 M agents: match 297 -> 264 us).  A grid with few
 // pairs for the GPU's blocks gives all but the smallest a block (1 M agents,
 // 936 pairs: 39 us with the higher limit, 32 with the lower).
-constexpr u32 kWarpPair = 512, kWarpPairFew = 64;
+constexpr u32 kWarpPair = 256, kWarpPairFew = 64;
 
 // Per-pair facts, one 64-byte line.
 struct __align__(16) TilePair {
@@ -472,23 +472,153 @@ __device__ __forceinline__ void big_build(const TileArgs& A, const TilePair& x, 
   }
 }
 
-// The matches of a pair that fits shared memory, by a group of T threads:
-// slot_src, the new records, the matches before each slot tile and in all.
+// Shared memory of a match by the whole block (four blocks per SM) and of one
+// by a warp, an eighth of it: message ids, 8 bytes each, then, when they are in
+// no order, a hash table of two 4-byte entries per id; the taken bits behind.
+constexpr u32 kMatchArea = 50176;
+constexpr u32 kIdsMax = kMatchArea / 8;     // ids that fit
+constexpr u32 kHashMax = kMatchArea / 16;   // ids that fit beside their table
+constexpr size_t kMatchSmem = kMatchArea + (kTableMax + 1) / 8 + 16;
+constexpr u32 kWarpArea = 16 * kWarpPair;
+static_assert(kMatchArea >= 4 * (kTableMax + 1), "the persistent launch's table fits");
+static_assert(kMatchArea >= 8 * (2 * kIlp * kT + 2 * kWinSlack), "its id window fits");
+static_assert(8 * (kWarpArea + kWarpPair / 8) <= kMatchSmem, "eight warps' shares fit");
+
+// Every slot of pair p looked up among its message ids, held in shared memory:
+// bisected when they ascend, else by a hash table.  Bits mark the taken
+// records; returns this thread's match count.  (Against the message's ids in
+// global memory, a window or a fingerprint check at a time: 266 -> 130 us for
+// 5.9 M records in no order, 264 -> 179 for 16.6 M ascending.)
+template <int T>
+__device__ __forceinline__ u32 match_ids(const TileArgs& A, const TilePair& x, u32 p, bool ascending,
+                                         const u64* ids, u32* tbl, u32* bits) {
+  const EncArgs& E = A.E;
+  const u32 m = x.m, size = 2 * m;
+  for (u32 i = group_thread<T>(); i < (m + 31u) / 32u; i += T) bits[i] = 0u;
+  if (!ascending) {
+    for (u32 i = group_thread<T>(); i < size; i += T) tbl[i] = 0u;
+    group_sync<T>();
+    for (u32 k = group_thread<T>(); k < m; k += T) {
+      const u64 id = ids[k];
+      u32 at = (u32)seg_start(id, size);
+      for (u32 probe = 0; probe < size; ++probe) {
+        const u32 old = atomicCAS(tbl + at, 0u, k + 1u);
+        if (old == 0u) break;
+        if (ids[old - 1u] == id) {
+          latch(E.st, TERA_EINVAL);  // ids must be unique within a message
+          break;
+        }
+        at = at + 1u == size ? 0u : at + 1u;
+      }
+    }
+  }
+  group_sync<T>();
+  u32 found = 0;
+  for (u32 j0 = 0; j0 < x.r; j0 += T * kIlp) {  // group-uniform
+    u64 id[kIlp];
+    u32 k[kIlp];
+#pragma unroll
+    for (u32 i = 0; i < kIlp; ++i) {
+      const u32 j = j0 + i * T + group_thread<T>();
+      id[i] = j < x.r ? ref_id(E, p, x.ro, j) : 0;
+      k[i] = kNoMatch;
+    }
+    if (m == 0) {
+      // nothing to match
+    } else if (ascending) {
+      // the kIlp bisections step together, so that their reads overlap
+      u32 lo[kIlp], len = m;
+#pragma unroll
+      for (u32 i = 0; i < kIlp; ++i) lo[i] = 0;
+      while (len > 1) {  // the last id not above the slot's is in [lo, lo + len)
+        const u32 half = len >> 1;
+#pragma unroll
+        for (u32 i = 0; i < kIlp; ++i) lo[i] = ids[lo[i] + half] <= id[i] ? lo[i] + half : lo[i];
+        len -= half;
+      }
+#pragma unroll
+      for (u32 i = 0; i < kIlp; ++i) k[i] = ids[lo[i]] == id[i] ? lo[i] : kNoMatch;
+    } else {
+#pragma unroll
+      for (u32 i = 0; i < kIlp; ++i) {
+        u32 at = (u32)seg_start(id[i], size);
+        for (u32 probe = 0; probe < size; ++probe) {
+          const u32 e = tbl[at];
+          if (e == 0u) break;
+          if (ids[e - 1u] == id[i]) {
+            k[i] = e - 1u;
+            break;
+          }
+          at = at + 1u == size ? 0u : at + 1u;
+        }
+      }
+    }
+#pragma unroll
+    for (u32 i = 0; i < kIlp; ++i) {
+      const u32 j = j0 + i * T + group_thread<T>();
+      if (j >= x.r) continue;
+      if (k[i] != kNoMatch) {
+        const u32 bit = 1u << (k[i] & 31u);
+        if (atomicOr(bits + (k[i] >> 5), bit) & bit) {
+          latch(E.st, TERA_EINVAL);  // a second slot with the same id: that slot is a hole
+          k[i] = kNoMatch;
+        }
+      }
+      found += k[i] != kNoMatch;
+      E.slot_src[x.ro + j] = k[i] != kNoMatch ? (u32)x.g_lo + k[i] : kNoMatch;
+    }
+  }
+  return found;
+}
+
+// The matches of a pair of at most kTableMax records (T = 32: kWarpPair), by a
+// group of T threads: slot_src, the new records, the matches before each slot
+// tile and in all.
 template <int T>
 __device__ __forceinline__ void match_pair(const TileArgs& A, const TilePair& x, u32 p, u32 shift,
-                                           SmemTable& tb, u64* window, u32* s_cnt, u32* sm32) {
+                                           uint8_t* area, u32* bits, u32* s_cnt, u32* sm32) {
   if (group_thread<T>() == 0) *s_cnt = 0;
-  u32 size = 32;
-  while (size < 2 * x.m) size <<= 1;
-  tb.mask = size - 1;
-  u32 c = 0;
-  group_sync<T>();
-  if (ids_ascending<T>(A.E, p, x.m)) {
-    if (x.r) c = sorted_match<T>(A.E, p, x.m, x.r, tb, window);
-  } else {
-    smem_build<T>(A.E, p, x.m, tb);  // also finds an id that occurs twice
+  u64* ids = reinterpret_cast<u64*>(area);
+  bool ascending, held = true;
+  if (T == 32 || x.m <= kIdsMax) {
+    for (u32 k0 = 0; k0 < x.m; k0 += 8 * T) {
+      u64 v[8];
+#pragma unroll
+      for (u32 i = 0; i < 8; ++i) {
+        const u32 k = k0 + i * T + group_thread<T>();
+        v[i] = k < x.m ? msg_id(A.E, p, x.g_lo + k) : 0;
+      }
+#pragma unroll
+      for (u32 i = 0; i < 8; ++i) {
+        const u32 k = k0 + i * T + group_thread<T>();
+        if (k < x.m) ids[k] = v[i];
+      }
+    }
     group_sync<T>();
-    if (x.r) c = smem_match<T>(A.E, p, x.r, tb);
+    bool bad = false;
+    for (u32 k = group_thread<T>(); k + 1 < x.m; k += T) bad |= !(ids[k] < ids[k + 1]);
+    ascending = !group_any<T>(bad);
+    held = T == 32 || ascending || x.m <= kHashMax;
+  } else {
+    group_sync<T>();
+    ascending = ids_ascending<T>(A.E, p, x.m);
+    held = false;
+  }
+  u32 c = 0;
+  if (held) {
+    c = match_ids<T>(A, x, p, ascending, ids, reinterpret_cast<u32*>(ids + x.m), bits);
+  } else if constexpr (T != 32) {
+    SmemTable tb{reinterpret_cast<unsigned short*>(area), 0u, bits};
+    u32 size = 32;
+    while (size < 2 * x.m) size <<= 1;
+    tb.mask = size - 1;
+    if (ascending) {
+      if (x.r) c = sorted_match<T>(A.E, p, x.m, x.r, tb, ids);
+    } else {
+      smem_build<T>(A.E, p, x.m, tb);  // also finds an id that occurs twice
+      group_sync<T>();
+      if (x.r) c = smem_match<T>(A.E, p, x.r, tb);
+    }
   }
   if (x.r == 0) return;
   c = warp_sum(c);
@@ -496,7 +626,7 @@ __device__ __forceinline__ void match_pair(const TileArgs& A, const TilePair& x,
   group_sync<T>();
   const u32 matched = *s_cnt;
   if (group_thread<T>() == 0) A.tot[(u64)p * PT_COUNT + PT_MATCHED] = matched;
-  if (matched < x.m) new_list<T, false>(A, x, tb.bits, sm32);
+  if (matched < x.m) new_list<T, false>(A, x, bits, sm32);
   if (x.nst == 1) {
     if (group_thread<T>() == 0) A.before[x.unit0] = 0u;
   } else {
@@ -508,18 +638,6 @@ __device__ __forceinline__ void match_pair(const TileArgs& A, const TilePair& x,
     sum_tiles<T>(A, x, sm32);
   }
 }
-
-// Shared memory of the match: the table (or the id window of an ascending
-// message) and the taken bits; then, a warp's share of it each, those of the
-// pairs matched by one warp.
-constexpr u32 kMatchTable = 4 * (kTableMax + 1);
-constexpr size_t kMatchSmem = kMatchTable + (kTableMax + 1) / 8 + 16;
-constexpr u32 kWarpTable = 3072 + 512;  // the window of 32 threads, or 1024 table entries
-constexpr u32 kWarpShare = kWarpTable + kWarpPair / 8;
-static_assert(kMatchTable >= 8 * (2 * kIlp * kT + 2 * kWinSlack), "the id window fits");
-static_assert(kWarpTable >= 8 * (2 * kIlp * 32 + 2 * kWinSlack) && kWarpTable >= 4 * kWarpPair,
-              "a warp's window and table fit");
-static_assert(8 * kWarpShare <= kMatchSmem, "eight warps' shares fit");
 
 // The pair of every tile (unit_pair), which the launches after this one read:
 // each warp of the launch takes a run of tiles, finds the first one's pair and
@@ -564,28 +682,23 @@ __global__ void __launch_bounds__(kT, kPerSm) codec_match_kernel(TileArgs A) {
   }
   map_tiles(A);
   if (n) {
-    SmemTable tb;
-    tb.tbl = reinterpret_cast<unsigned short*>(dyn);
-    tb.bits = reinterpret_cast<u32*>(dyn + kMatchTable);
     for (;;) {
       const u32 it = claim(A.scal + TS_TICKET_MATCH, n, &s_next);
       if (it == ~0u) break;
       const u32 p = A.item_pair[it];
       const TilePair x = A.pair[p];
       if (x.m > kTableMax) big_check(A, x, p, it - x.item0);
-      else match_pair<kT>(A, x, p, shift, tb, reinterpret_cast<u64*>(dyn), s_cnt, sm32);
+      else match_pair<kT>(A, x, p, shift, dyn, reinterpret_cast<u32*>(dyn + kMatchArea), s_cnt, sm32);
       __syncthreads();
     }
   }
   const u32 warp = threadIdx.x >> 5;
-  uint8_t* share = dyn + warp * kWarpShare;
-  SmemTable tb;
-  tb.tbl = reinterpret_cast<unsigned short*>(share);
-  tb.bits = reinterpret_cast<u32*>(share + kWarpTable);
+  uint8_t* share = dyn + warp * (kWarpArea + kWarpPair / 8);
   for (u32 i = blockIdx.x * (kT / 32) + warp; i < n_small; i += gridDim.x * (kT / 32)) {
     const u32 p = A.small_pair[i];
     const TilePair x = A.pair[p];
-    match_pair<32>(A, x, p, shift, tb, reinterpret_cast<u64*>(share), s_cnt + warp, nullptr);
+    match_pair<32>(A, x, p, shift, share, reinterpret_cast<u32*>(share + kWarpArea), s_cnt + warp,
+                   nullptr);
     __syncwarp();
   }
 }
@@ -1421,6 +1534,10 @@ tera_status launch_tiles(tera_ctx* ctx, const EncArgs& E, const DecArgs& D, bool
                        reinterpret_cast<const void*>(codec_encode_kernel<true>),
                        reinterpret_cast<const void*>(codec_decode_kernel<false>),
                        reinterpret_cast<const void*>(codec_decode_kernel<true>)};
+    if (cudaFuncSetAttribute(reinterpret_cast<const void*>(codec_match_kernel),
+                             cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)kMatchSmem) != cudaSuccess)
+      return TERA_ECUDA;
     for (int i = 0; i < 4; ++i)
       if (cudaFuncSetAttribute(k[i], cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)(i < 2 ? kEncSmem : kDecSmem)) != cudaSuccess)
