@@ -27,48 +27,39 @@ using namespace tera;
 
 namespace {
 
-// One axis by the bucket table when the coordinate's bucket holds an answer,
-// else by the exact key comparisons.  The estimate is taken only for
-// magnitudes in the float normal range (2^-126 <= |v| < 2^128, which also
-// sends NaN and infinities to the exact path).
-__device__ __forceinline__ u32 classify_axis_table(u64 bits, int a, const SmemGrid& s,
-                                                   const uint8_t* tab, float flo, float fs,
-                                                   int* idx) {
+// One axis by the exact comparisons, out of line (few coordinates come here,
+// and inlined into every round of the kernel it pushed the rounds' code out of
+// the instruction cache): (box index << 2) | aura offsets (bit 0: -1, bit 1:
+// +1), or ~0 outside the domain.
+__device__ __noinline__ u32 axis_exact(u64 bits, int a, const SmemGrid& s) {
+  int i;
+  const u32 o = classify_axis(bits, a, s, &i);
+  return o ? ((u32)i << 2) | (o & 1u) | ((o & 4u) >> 1) : ~0u;
+}
+
+// The same by the bucket table when the coordinate's bucket holds an answer.
+// The estimate is taken only for magnitudes in the float normal range (2^-126
+// <= |v| < 2^128, which also sends NaN and infinities to the exact path).
+__device__ __forceinline__ u32 axis_entry(u64 bits, int a, const SmemGrid& s, const uint8_t* tab,
+                                          float flo, float fs) {
   const u32 hi = (u32)(bits >> 32);
   const u32 ha = hi & 0x7FFFFFFFu;
+  u32 e = kBucketExact;
   if (ha - 0x38100000u < 0x0FE00000u) {
     const float af = __uint_as_float((hi & 0x80000000u) | ((ha - 0x38000000u) << 3));
     const int j = __float2int_rz((af - flo) * fs);
-    if ((u32)j < (u32)kAxisBuckets) {
-      const u32 e = tab[j];
-      if (!(e & kBucketExact)) {
-        *idx = (int)(e >> 2);
-        return 2u | (e & 1u) | ((e & 2u) << 1);
-      }
-    }
+    if ((u32)j < (u32)kAxisBuckets) e = tab[j];
   }
-  return classify_axis(bits, a, s, idx);
+  return e & kBucketExact ? axis_exact(bits, a, s) : e;
 }
 
-// classify_agent with the bucket tables in shared memory (tab: three axes of
-// kAxisBuckets entries).
-__device__ __forceinline__ void classify_agent_table(u64 bx, u64 by, u64 bz, const SmemGrid& s,
-                                                     const uint8_t* tab, const float* flo,
-                                                     const float* fs, int* owner, u32* mask,
-                                                     bool* ok) {
-  int ix, iy, iz;
-  const u32 ox = classify_axis_table(bx, 0, s, tab, flo[0], fs[0], &ix);
-  const u32 oy = classify_axis_table(by, 1, s, tab + kAxisBuckets, flo[1], fs[1], &iy);
-  const u32 oz = classify_axis_table(bz, 2, s, tab + 2 * kAxisBuckets, flo[2], fs[2], &iz);
-  *ok = ox && oy && oz;
-  if (!*ok) {
-    *owner = -1;
-    *mask = 0;
-    return;
-  }
-  *owner = ix + s.n[0] * (iy + s.n[1] * iz);
-  const u32 m = ox * spread3(oy, 3) * spread3(oz, 9);
-  *mask = m & ~(1u << 13);
+// Owner and aura mask of one agent from its three axes; lut: the mask of every
+// combination of the axes' offsets (bit pairs x, y, z).
+__device__ __forceinline__ void agent_entry(u32 ex, u32 ey, u32 ez, int n0, int n1, const u32* lut,
+                                            int* owner, u32* mask, bool* ok) {
+  *ok = ex != ~0u && ey != ~0u && ez != ~0u;
+  *owner = *ok ? (int)(ex >> 2) + n0 * ((int)(ey >> 2) + n1 * (int)(ez >> 2)) : -1;
+  *mask = *ok ? lut[(ex & 3u) | ((ey & 3u) << 2) | ((ez & 3u) << 4)] : 0u;
 }
 
 // Each block classifies tiles of kClassifyTile agents (tile blockIdx.x, then
@@ -78,7 +69,15 @@ __device__ __forceinline__ void classify_agent_table(u64 bx, u64 by, u64 bz, con
 // 16-byte load per coordinate), so every warp load is fully coalesced, and
 // each warp covers a run of kRunAgents consecutive agents per round; the
 // number of (agent, pair) entries of every run is written (runs are in agent
-// order).  bk == nullptr: every agent takes the exact key comparisons.
+// order).  TAB: with bucket tables (bk); else every agent takes the exact key
+// comparisons.
+//
+// Bound: issue and HBM about equally.  338 warp instructions per 64 agents and
+// the exact comparisons inlined 24 times over (3.3 stall cycles an issue on
+// instruction fetches) took 689 us for 100 M agents; with the masks looked up
+// and the exact path out of line 537.  (Fewer resident blocks for more
+// registers: 5 per SM 752 us, 4 per SM 725; two rounds unrolled 654.)
+template <bool TAB>
 __global__ void __launch_bounds__(kClassifyThreads, 6)
     classify_kernel(const u64* __restrict__ x, const u64* __restrict__ y,
                     const u64* __restrict__ z, u64 n, const GridTables* __restrict__ g,
@@ -87,9 +86,20 @@ __global__ void __launch_bounds__(kClassifyThreads, 6)
                     DevStats* stats, u64* __restrict__ sort_head) {
   __shared__ SmemGrid sg;
   __shared__ float s_flo[3], s_fs[3];
+  __shared__ u32 s_lut[64];
   // the tables follow the grid rows (a multiple of 32 bytes) in dynamic shared memory
   uint8_t* tab = reinterpret_cast<uint8_t*>(grid_rows() + (g->n[0] + g->n[1] + g->n[2]));
-  if (bk) {
+  if constexpr (TAB) {
+    if (threadIdx.x < 64) {
+      const u32 q = threadIdx.x;
+      u32 o[3];
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        const u32 b = q >> (2 * a) & 3u;
+        o[a] = 2u | (b & 1u) | ((b & 2u) << 1);
+      }
+      s_lut[q] = o[0] * spread3(o[1], 3) * spread3(o[2], 9) & ~(1u << 13);
+    }
     const uint4* src = reinterpret_cast<const uint4*>(bk->tab);
     uint4* dst = reinterpret_cast<uint4*>(tab);
     for (int i = threadIdx.x; i < 3 * kAxisBuckets / 16; i += blockDim.x) dst[i] = src[i];
@@ -110,6 +120,7 @@ __global__ void __launch_bounds__(kClassifyThreads, 6)
     }
   }
   const int lane = threadIdx.x & 31;
+  const int n0 = sg.n[0], n1 = sg.n[1];
   bool bad = false;
   for (u64 tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
     const u64 tile0 = tile * kClassifyTile;
@@ -138,8 +149,11 @@ __global__ void __launch_bounds__(kClassifyThreads, 6)
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
         bool ok;
-        if (bk)
-          classify_agent_table(vx[q], vy[q], vz[q], sg, tab, s_flo, s_fs, &o[q], &m[q], &ok);
+        if constexpr (TAB)
+          agent_entry(axis_entry(vx[q], 0, sg, tab, s_flo[0], s_fs[0]),
+                      axis_entry(vy[q], 1, sg, tab + kAxisBuckets, s_flo[1], s_fs[1]),
+                      axis_entry(vz[q], 2, sg, tab + 2 * kAxisBuckets, s_flo[2], s_fs[2]), n0, n1,
+                      s_lut, &o[q], &m[q], &ok);
         else
           classify_agent(vx[q], vy[q], vz[q], sg, &o[q], &m[q], &ok);
         if (a0 + q < n) {
@@ -635,13 +649,15 @@ extern "C" tera_status tera_partition(tera_ctx* ctx, const tera_soa* soa, tera_p
       grid_smem_bytes(ctx->grid) + (ctx->d_buckets ? 3 * (size_t)kAxisBuckets : 0);
   static bool csmem_set = false;
   if (!csmem_set) {
-    cudaFuncSetAttribute(classify_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaFuncSetAttribute(classify_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)(sizeof(BoxKeys) * 3 * kMaxAxis + 3 * (size_t)kAxisBuckets));
+    cudaFuncSetAttribute(classify_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)(sizeof(BoxKeys) * 3 * kMaxAxis));
     csmem_set = true;
   }
   const u64 cgrid = blocks < (u64)ctx->num_sms * 6 ? blocks : (u64)ctx->num_sms * 6;
   prof_begin(ctx, s);
-  launch_chained(classify_kernel, (unsigned)cgrid, kClassifyThreads, csmem, s, 
+  launch_chained(ctx->d_buckets ? classify_kernel<true> : classify_kernel<false>, (unsigned)cgrid, kClassifyThreads, csmem, s, 
       reinterpret_cast<const u64*>(soa->x), reinterpret_cast<const u64*>(soa->y),
       reinterpret_cast<const u64*>(soa->z), n, ctx->d_grid, ctx->d_buckets, blocks, out->owner,
       out->mask, ctx->tile_cnt, runs, ctx->d_status, ctx->d_stats, ctx->rs_hist);
