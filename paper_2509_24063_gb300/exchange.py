@@ -98,9 +98,10 @@ class AuraExchange:
         """Buffer of iteration t's outputs."""
         return self.schedule(t)[0]
 
-    def _launch(self, state: dict, t: int, stream=None):
+    def _launch(self, state: dict, t: int, stream=None, columns_ready=None):
         """Enqueue iteration t on the stream (outputs and references in the
-        buffers tera_ref_schedule names)."""
+        buffers tera_ref_schedule names).  columns_ready: an event the stream
+        waits for before it reads any column but x, y and z."""
         ctx = self.ctx
         first = t == 0
         cur, prv, _ = self.schedule(t)
@@ -110,6 +111,8 @@ class AuraExchange:
         pair_off = self.pair_off[cur]
         part.pair_off = pair_off  # this iteration's offsets become the next one's reference layout
         ctx.partition(state, part, stream)
+        if columns_ready is not None:
+            (stream or torch.cuda.current_stream()).wait_event(columns_ready)
         ref_prev = None if first else self.ref[prv]
         ref_off_prev = None if first else self.pair_off[prv]
         recv_prev = None if first else self.recv[prv]
@@ -165,9 +168,13 @@ class AuraExchange:
                              ref_next=self.ref_ids[cur])
         return args, kw
 
-    def step(self, state: dict, stream=None):
-        """Classify, pack, encode and decode every pair for one iteration."""
-        self._launch(state, self.t, stream)
+    def step(self, state: dict, stream=None, columns_ready=None):
+        """Classify, pack, encode and decode every pair for one iteration.
+
+        columns_ready: an event after which the columns other than x, y and z
+        hold the state (they may still be being copied when step is called);
+        the partition, which reads positions only, does not wait for it."""
+        self._launch(state, self.t, stream, columns_ready)
         self.t += 1
         return self.last
 
