@@ -13,6 +13,7 @@
 // order, then its inboxes in ascending side.
 //
 // tera_migrate_send
+//   mig_begin_kernel   counters and abort flag zeroed
 //   mig_count_kernel   one pass over x, y, z: owner box of every agent; leavers
 //                      per warp tile, per source box and per inbox
 //   scan of the warp-tile counts (leavers before every warp tile)
@@ -149,6 +150,18 @@ __device__ __forceinline__ void warp_boxes(const u64* __restrict__ box_off, u32 
                                            u64 w_end, u32* lo, u32* hi) {
   *lo = warp_box_search(box_off, 0, n_boxes - 1, w0);
   *hi = warp_box_search(box_off, *lo, n_boxes - 1, w_end - 1);
+}
+
+// Zeroes the counters and the abort flag in one launch (three memsets took
+// three, and the count kernel could not be set up behind a memset).
+__global__ void __launch_bounds__(256)
+    mig_begin_kernel(u64* __restrict__ from, u64 n_boxes, u64* __restrict__ cnt, u64 Q,
+                     DevStatus* st) {
+  chain_begin();
+  const u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i == 0) st->abort = 0;
+  if (i < n_boxes) from[i] = 0;
+  if (i < Q) cnt[i] = 0;
 }
 
 constexpr int kCountBlocks = 4;  // resident blocks per SM of mig_count_kernel
@@ -617,9 +630,10 @@ extern "C" tera_status tera_migrate_send(tera_ctx* ctx, const tera_soa* prev,
   const u64 lv_cap = arena_units > Q ? (arena_units - Q < n ? arena_units - Q : n) : 0;
   tera_status st;
   if ((st = ensure_migrate(ctx, n, lv_cap)) != TERA_OK) return st;
-  cudaMemsetAsync(&ctx->d_status->abort, 0, sizeof(u32), s);
-  cudaMemsetAsync(ctx->m_from, 0, sizeof(u64) * B, s);
-  cudaMemsetAsync(ctx->m_cnt, 0, sizeof(u64) * Q, s);
+  prof_begin(ctx, s);
+  launch_chained(mig_begin_kernel, (unsigned)((Q + 255) / 256), 256, 0, s, ctx->m_from, B, ctx->m_cnt,
+                 Q, ctx->d_status);
+  if ((st = check_launch(ctx, "mig_begin_kernel", s)) != TERA_OK) return st;
   const u64 blocks = n == 0 ? 1 : (n + kBlockAgents - 1) / kBlockAgents;
   const u64 wtiles = n == 0 ? 1 : (n + kWarpAgents - 1) / kWarpAgents;
   prof_begin(ctx, s);
