@@ -1274,9 +1274,9 @@ __device__ __noinline__ void team_pair(const EncArgs& E, const DecArgs& D, const
 // the cell counts of its pair's reference, not on the message: each side makes
 // the predictions of its own reference before the codec runs, over every slot
 // of every pair at once: the cell counts, the features (one thread per slot,
-// few registers, so that many loads are in flight), then the network (two
-// slots per thread, in a kernel with room for both slots' accumulators).  The
-// codec then reads them.
+// few registers, so that many loads are in flight), then the network (64 slots
+// per warp, in a kernel with room for their accumulators).  The codec then
+// reads them.
 
 // The pair of slot g of an arena laid out with off[0..P] (off[p] <= g < off[p+1]).
 __device__ __forceinline__ u32 pair_of_slot(const u64* __restrict__ off, u32 P, u64 g) {
@@ -1326,13 +1326,35 @@ __global__ void __launch_bounds__(256) pred_cells_kernel(PredArgs pr, const uint
   }
 }
 
-// The network's weights in shared memory with layer 2 stored by columns: the
-// weights of hidden input k for neurons 0 .. 63 at kMlpW2 + 64 k (the other
-// arrays as in the parameter vector).
+// The network over tiles of 64 slots, one warp a tile, each layer an outer
+// product over its inputs: lane (vg, ng) = (lane & 7, lane >> 3) holds the
+// accumulators of 8 slots (4 vg .. and 32 + 4 vg ..) by 16 neurons (16 ng ..),
+// and an input costs it two 16-byte loads of the slots' values and four of the
+// weights for 128 fused multiply-adds.  Every neuron still starts at its bias
+// and adds its inputs in ascending order with the same fused multiply-adds as
+// mlp_infer, so the bits are the same.
+//
+// Bound: FP32 issue and shared-memory reads about equally.  A thread that runs
+// whole vectors reads each weight for itself, and even with two vectors a
+// thread the loads of the weights (all lanes the same, but 512 bytes into
+// registers each) took twice the time of the arithmetic: 1408 us for 6.4 M
+// slots, now 1175 (70 % of the FP32 rate; with two multiply-adds per instruction,
+// one at a time 1285.  12 warps per SM spill: 1730).
+constexpr int kNetThreads = 256;
+constexpr int kNetTile = 64;
+constexpr int kNetWeights = (kMlpParams + 3) & ~3;
+constexpr int kNetWarpFloats = (kMlpH + kMlpIn) * kNetTile;  // layer outputs, features
+constexpr size_t kNetSmem =
+    sizeof(float) * (kNetWeights + (kNetThreads / 32) * (size_t)kNetWarpFloats);
+
+// The parameter vector into shared memory, layers 1 and 2 by columns: the
+// weights of input k for neurons 0 .. 63 at kMlpW1 + 64 k and kMlpW2 + 64 k.
 __device__ __forceinline__ void load_mlp_cols(float* sW, const float* __restrict__ params) {
   for (int i = threadIdx.x; i < kMlpParams; i += blockDim.x) {
     int d = i;
-    if (i >= kMlpW2 && i < kMlpW2 + kMlpH * kMlpH) {
+    if (i < kMlpB1) {
+      d = kMlpW1 + i % kMlpIn * kMlpH + i / kMlpIn;
+    } else if (i >= kMlpW2 && i < kMlpB2) {
       const int j = (i - kMlpW2) / kMlpH, k = (i - kMlpW2) % kMlpH;
       d = kMlpW2 + k * kMlpH + j;
     }
@@ -1341,70 +1363,118 @@ __device__ __forceinline__ void load_mlp_cols(float* sW, const float* __restrict
   __syncthreads();
 }
 
-// First-layer neuron k of one feature vector: its bias, then the inputs in
-// ascending order, then ReLU (as mlp_infer).
-__device__ __forceinline__ float hidden1(const float4 wa, const float4 wb, float bias,
-                                         const float* f) {
-  float h = bias;
-  h = __fmaf_rn(wa.x, f[0], h);
-  h = __fmaf_rn(wa.y, f[1], h);
-  h = __fmaf_rn(wa.z, f[2], h);
-  h = __fmaf_rn(wa.w, f[3], h);
-  h = __fmaf_rn(wb.x, f[4], h);
-  h = __fmaf_rn(wb.y, f[5], h);
-  h = __fmaf_rn(wb.z, f[6], h);
-  h = __fmaf_rn(wb.w, f[7], h);
-  return h > 0.0f ? h : 0.0f;
+// Two binary32 values in one register pair, and two fused multiply-adds in one
+// instruction, each rounded as __fmaf_rn rounds it.
+__device__ __forceinline__ u64 pack2(float a, float b) {
+  u64 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(u64 v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ u64 fma2(u64 a, u64 b, u64 c) {
+  u64 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
 }
 
-// The network on two feature vectors A and B with the same fused
-// multiply-adds, in the same order per neuron, as mlp_infer (so the same
-// bits), each weight read from shared memory once for both vectors.  The
-// second layer runs in two halves of 32 neurons (the first layer is made
-// again for each half, one neuron k at a time, and its output enters the
-// half's 32 accumulators of both vectors); each second-layer neuron adds its
-// inputs k = 0 .. 63 in ascending order, and each output adds j = 0 .. 63 in
-// ascending order across the halves.
-__device__ __forceinline__ void mlp_infer_pair(const float* __restrict__ sW, const float* fA,
-                                               const float* fB, float* oA, float* oB) {
-  const float4* W4 = reinterpret_cast<const float4*>(sW);
+// One layer of K inputs X[k][slot] with weights W[k][neuron], ReLU, into
+// Y[neuron][slot] (Y may be X: every lane has read X before the first store).
+template <int K>
+__device__ __forceinline__ void net_layer(const float* __restrict__ W, const float* bias,
+                                          const float* X, float* Y) {
+  const int lane = threadIdx.x & 31, v0 = 4 * (lane & 7), n0 = 16 * (lane >> 3);
+  u64 acc2[8][8];
 #pragma unroll
-  for (int a = 0; a < kMlpOut; ++a) oA[a] = oB[a] = sW[kMlpB3 + a];
-#pragma unroll 1
-  for (int hf = 0; hf < 2; ++hf) {
-    float accA[32], accB[32];
+  for (int n = 0; n < 8; ++n) {
+    const u64 b = *reinterpret_cast<const u64*>(bias + n0 + 2 * n);
 #pragma unroll
-    for (int j = 0; j < 32; ++j) accA[j] = accB[j] = sW[kMlpB2 + 32 * hf + j];
-#pragma unroll 1
-    for (int k = 0; k < kMlpH; ++k) {
-      const float4 wa = W4[(kMlpW1 + k * kMlpIn) / 4], wb = W4[(kMlpW1 + k * kMlpIn) / 4 + 1];
-      const float bias = sW[kMlpB1 + k];
-      const float hA = hidden1(wa, wb, bias, fA), hB = hidden1(wa, wb, bias, fB);
-      const float4* col = W4 + (kMlpW2 + k * kMlpH + 32 * hf) / 4;
+    for (int v = 0; v < 8; ++v) acc2[v][n] = b;
+  }
+#pragma unroll 2
+  for (int k = 0; k < K; ++k) {
+    float x[8];
+    ulonglong2 w[4];
+    *reinterpret_cast<float4*>(x) = *reinterpret_cast<const float4*>(X + kNetTile * k + v0);
+    *reinterpret_cast<float4*>(x + 4) =
+        *reinterpret_cast<const float4*>(X + kNetTile * k + 32 + v0);
 #pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const float4 w = col[q];
-        accA[4 * q] = __fmaf_rn(w.x, hA, accA[4 * q]);
-        accB[4 * q] = __fmaf_rn(w.x, hB, accB[4 * q]);
-        accA[4 * q + 1] = __fmaf_rn(w.y, hA, accA[4 * q + 1]);
-        accB[4 * q + 1] = __fmaf_rn(w.y, hB, accB[4 * q + 1]);
-        accA[4 * q + 2] = __fmaf_rn(w.z, hA, accA[4 * q + 2]);
-        accB[4 * q + 2] = __fmaf_rn(w.z, hB, accB[4 * q + 2]);
-        accA[4 * q + 3] = __fmaf_rn(w.w, hA, accA[4 * q + 3]);
-        accB[4 * q + 3] = __fmaf_rn(w.w, hB, accB[4 * q + 3]);
-      }
-    }
+    for (int q = 0; q < 4; ++q)
+      w[q] = *reinterpret_cast<const ulonglong2*>(W + kMlpH * k + n0 + 4 * q);
 #pragma unroll
-    for (int j = 0; j < 32; ++j) {
-      const float h2A = accA[j] > 0.0f ? accA[j] : 0.0f, h2B = accB[j] > 0.0f ? accB[j] : 0.0f;
+    for (int v = 0; v < 8; ++v) {
+      const u64 xx = pack2(x[v], x[v]);
 #pragma unroll
-      for (int a = 0; a < kMlpOut; ++a) {
-        const float w = sW[kMlpW3 + a * kMlpH + 32 * hf + j];
-        oA[a] = __fmaf_rn(w, h2A, oA[a]);
-        oB[a] = __fmaf_rn(w, h2B, oB[a]);
+      for (int q = 0; q < 4; ++q) {
+        acc2[v][2 * q] = fma2(w[q].x, xx, acc2[v][2 * q]);
+        acc2[v][2 * q + 1] = fma2(w[q].y, xx, acc2[v][2 * q + 1]);
       }
     }
   }
+  float acc[8][16];
+#pragma unroll
+  for (int v = 0; v < 8; ++v)
+#pragma unroll
+    for (int n = 0; n < 8; ++n) {
+      const float2 t = unpack2(acc2[v][n]);
+      acc[v][2 * n] = t.x;
+      acc[v][2 * n + 1] = t.y;
+    }
+  __syncwarp();
+#pragma unroll
+  for (int n = 0; n < 16; ++n) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      float r[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float a = acc[4 * h + i][n];
+        r[i] = a > 0.0f ? a : 0.0f;
+      }
+      *reinterpret_cast<float4*>(Y + kNetTile * (n0 + n) + 32 * h + v0) =
+          make_float4(r[0], r[1], r[2], r[3]);
+    }
+  }
+  __syncwarp();
+}
+
+// The network on the warp's tile: lane's slots are lane (fA, oA) and lane + 32
+// (fB, oB).  buf: kNetWarpFloats floats of the warp.
+__device__ __forceinline__ void net_tile(const float* __restrict__ sW, float* buf, const float* fA,
+                                         const float* fB, float* oA, float* oB) {
+  const int lane = threadIdx.x & 31;
+  float* F = buf + kMlpH * kNetTile;
+#pragma unroll
+  for (int i = 0; i < kMlpIn; ++i) {
+    F[kNetTile * i + lane] = fA[i];
+    F[kNetTile * i + 32 + lane] = fB[i];
+  }
+  __syncwarp();
+  net_layer<kMlpIn>(sW + kMlpW1, sW + kMlpB1, F, buf);
+  net_layer<kMlpH>(sW + kMlpW2, sW + kMlpB2, buf, buf);
+#pragma unroll
+  for (int a = 0; a < kMlpOut; ++a) oA[a] = oB[a] = sW[kMlpB3 + a];
+#pragma unroll 4
+  for (int j = 0; j < kMlpH; j += 4) {
+    float4 w[kMlpOut];
+#pragma unroll
+    for (int a = 0; a < kMlpOut; ++a)
+      w[a] = *reinterpret_cast<const float4*>(sW + kMlpW3 + a * kMlpH + j);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float hA = buf[kNetTile * (j + i) + lane], hB = buf[kNetTile * (j + i) + 32 + lane];
+#pragma unroll
+      for (int a = 0; a < kMlpOut; ++a) {
+        const float wi = i == 0 ? w[a].x : i == 1 ? w[a].y : i == 2 ? w[a].z : w[a].w;
+        oA[a] = __fmaf_rn(wi, hA, oA[a]);
+        oB[a] = __fmaf_rn(wi, hB, oB[a]);
+      }
+    }
+  }
+  __syncwarp();
 }
 
 // Every reference slot's features into out[4 g .. 4 g + 3] (8 floats), the
@@ -1469,34 +1539,36 @@ __device__ __forceinline__ void store_pred(const uint8_t* __restrict__ ref, u32 
 }
 
 // Every reference slot's prediction from its features (in out[4 g .. 4 g +
-// 3], replaced).  A thread takes two slots of its warp's run at a time (gA
-// and gA + 32) and runs the network on both at once.
-__global__ void __launch_bounds__(256, 2) pred_slots_kernel(PredArgs pr,
-                                                            const uint8_t* __restrict__ ref,
-                                                            const u64* __restrict__ off, u32 P,
-                                                            u64 cap, u64* __restrict__ out) {
-  __shared__ __align__(16) float sW[(kMlpParams + 3) & ~3];
-  load_mlp_cols(sW, pr.params);
+// 3], replaced): each warp takes its run 64 slots at a time.
+__global__ void __launch_bounds__(kNetThreads, 1)
+    pred_slots_kernel(PredArgs pr, const uint8_t* __restrict__ ref, const u64* __restrict__ off,
+                      u32 P, u64 cap, u64* __restrict__ out) {
+  extern __shared__ __align__(16) float net_smem[];
+  load_mlp_cols(net_smem, pr.params);
+  float* buf = net_smem + kNetWeights + (threadIdx.x >> 5) * kNetWarpFloats;
   u64 g0, g1;
   warp_run(prepass_slots(off, P, cap), &g0, &g1);
   if (g0 >= g1) return;
-  u32 pA = pair_of_slot(off, P, g0), pB = pA;
-  for (u64 gA = g0 + (threadIdx.x & 31); gA < g1; gA += 64) {
-    const bool liveB = gA + 32 < g1;
-    const u64 gB = liveB ? gA + 32 : gA;
-    float fA[kMlpIn], fB[kMlpIn];
-    const bool okA = load_features(out, gA, fA);
-    const bool okB = liveB && load_features(out, gB, fB);
-    if (!liveB)
-      for (int i = 0; i < kMlpIn; ++i) fB[i] = 0.0f;
-    float yA[kMlpOut] = {0.0f, 0.0f, 0.0f}, yB[kMlpOut] = {0.0f, 0.0f, 0.0f};
-    if (__any_sync(__activemask(), okA || okB)) mlp_infer_pair(sW, fA, fB, yA, yB);
-    while (__ldg(off + pA + 1) <= gA) ++pA;
-    store_pred(ref, pA, out, gA, yA, okA);
-    if (liveB) {
-      if (pB < pA) pB = pA;
-      while (__ldg(off + pB + 1) <= gB) ++pB;
-      store_pred(ref, pB, out, gB, yB, okB);
+  u32 p = pair_of_slot(off, P, g0);
+  for (u64 t0 = g0; t0 < g1; t0 += kNetTile) {
+    const u64 g[2] = {t0 + (threadIdx.x & 31), t0 + 32 + (threadIdx.x & 31)};
+    float f[2][kMlpIn], y[2][kMlpOut];
+    bool ok[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+#pragma unroll
+      for (int i = 0; i < kMlpIn; ++i) f[q][i] = 0.0f;
+#pragma unroll
+      for (int a = 0; a < kMlpOut; ++a) y[q][a] = 0.0f;
+      ok[q] = g[q] < g1 && load_features(out, g[q], f[q]);
+    }
+    if (__any_sync(0xFFFFFFFFu, ok[0] || ok[1])) net_tile(net_smem, buf, f[0], f[1], y[0], y[1]);
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      if (g[q] < g1) {
+        while (__ldg(off + p + 1) <= g[q]) ++p;
+        store_pred(ref, p, out, g[q], y[q], ok[q]);
+      }
     }
   }
 }
@@ -1536,7 +1608,14 @@ static tera_status pred_prepass(tera_ctx* ctx, const PredArgs& pr, const uint8_t
                                                                    (u32)ctx->n_pairs, cap, out);
   if ((st = check_launch(ctx, "pred_features_kernel", s)) != TERA_OK) return st;
   prof_begin(ctx, s);
-  pred_slots_kernel<<<grid, 256, 0, s>>>(pr, ref, off, (u32)ctx->n_pairs, cap, out);
+  static bool net_set = false;
+  if (!net_set) {
+    cudaFuncSetAttribute(pred_slots_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)kNetSmem);
+    net_set = true;
+  }
+  pred_slots_kernel<<<(unsigned)ctx->num_sms, kNetThreads, kNetSmem, s>>>(
+      pr, ref, off, (u32)ctx->n_pairs, cap, out);
   return check_launch(ctx, "pred_slots_kernel", s);
 }
 
