@@ -191,8 +191,9 @@ __device__ __forceinline__ u64 cell_key(const Rec& R, const PredArgs& pr) {
   return c[0] + pr.ncell[0] * (c[1] + pr.ncell[1] * c[2]);
 }
 
-// Count one reference record in its cell (segment of pair p, zeroed before).
-__device__ __forceinline__ void cell_insert(u64* cseg, u64 base, u64 size, u64 key) {
+// Count n reference records in their cell (segment of pair p, zeroed before).
+__device__ __forceinline__ void cell_insert(u64* cseg, u64 base, u64 size, u64 key,
+                                            u64 n = 1) {
   u64 i = seg_start(key, size);
   for (u64 probe = 0; probe < size; ++probe) {
     u64* e = cseg + 2 * (base + i);
@@ -200,11 +201,11 @@ __device__ __forceinline__ void cell_insert(u64* cseg, u64 base, u64 size, u64 k
     if (k0 == 0) {
       const u64 prev = atomicCAS(e, 0ull, key + 1);
       if (prev == 0 || prev == key + 1) {
-        atomicAdd(e + 1, 1ull);
+        atomicAdd(e + 1, n);
         return;
       }
     } else if (k0 == key + 1) {
-      atomicAdd(e + 1, 1ull);
+      atomicAdd(e + 1, n);
       return;
     }
     i = (i + 1 == size) ? 0 : i + 1;
