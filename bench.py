@@ -51,6 +51,13 @@ def kernel_bytes(name, t):
         # (message, reference, new reference and wire on the sender; wire,
         # reference and receive buffers on the receiver)
         "codec_persistent_kernel": 64 * (3 * E + 2 * R) + 2 * t["wire_bytes"],
+        # the same over tiles: ids and matches; message and reference in, new
+        # reference, codes and payload out; payload moved to its place; codes,
+        # payload and reference in, receive buffer out
+        "codec_match_kernel": 8 * (E + R) + 4 * R,
+        "codec_encode_kernel": 64 * (E + R - t["holes"]) + 64 * E + 4 * (R + A) + Y,
+        "codec_wire_kernel": 2 * Y,
+        "codec_decode_kernel": 4 * (R + A) + Y + 64 * (R - t["holes"]) + 64 * M,
         # migration (N agents per step, L leavers): positions read to find the
         # owners; every record read and written once by the stable regroup;
         # leavers serialized (gather + arena write) and deserialized
@@ -594,7 +601,7 @@ def main():
             from paper_2509_24063_gb300 import autotune
             # tuned afresh on this workload (untimed warm-up), not from the cache
             tune, table = autotune.tune_batched(ex, states[t], use_cache=False)
-            tune_info = {"tune": list(tune), "candidates": len(table)}
+            tune_info = {"tune": list(tune) if tune else None, "candidates": len(table)}
         else:
             ex.step(states[t])
     ctx.status()  # raises on any device-side error
@@ -642,7 +649,7 @@ def main():
         stats["payload_bytes"]
     codec_bytes = kernel_bytes("pack_kernel", stats) + kernel_bytes("codec_persistent_kernel", stats)
     codec_ms = sum(prof.get(k, (0, 0.0))[1] for k in prof
-                   if k.startswith(("pack", "enc_", "dec_", "bat_", "codec_", "unit_map")))
+                   if k.startswith(("pack", "enc_", "dec_", "bat_", "codec_", "tiles_", "unit_map")))
     peaks, peak_kind = measured_peaks()
     hbm = float(peaks.get("hbm_gbs", 6800.0))
     codec_gbs = codec_bytes / (codec_ms / 1e3) / 1e9 if codec_ms > 0 else None
@@ -894,8 +901,8 @@ def run_predictor(args):
 def run_compare_paths(args):
     """The three paths of the exchange on the same states: one launch per
     sending box (per_subdomain), one launch per step for all pairs
-    (all_pairs), and the persistent batched codec replayed from CUDA graphs
-    (batched, schedule tuned at warm-up).  Each path runs W warm-up and K timed
+    (all_pairs), and the batched codec replayed from CUDA graphs (batched,
+    schedule tuned at warm-up).  Each path runs W warm-up and K timed
     iterations of the same chain; the bytes produced are the same on every
     path (the parity tests check it), so only the time differs."""
     import torch

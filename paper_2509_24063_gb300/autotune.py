@@ -1,6 +1,7 @@
-"""Autotuner of the batched codec's schedule (tile/block size and resident
-blocks per SM; each block's shared-memory match table takes what its share of
-the SM's shared memory allows).
+"""Autotuner of the batched codec's schedule: no schedule (None: the codec over
+warp tiles, several launches that size themselves), or the persistent launch
+with a tile/block size and resident blocks per SM (each block's shared-memory
+match table takes what its share of the SM's shared memory allows).
 
 The schedule never changes the bytes produced, only the time.  Candidates are
 timed on the real data of one iteration: after partition + pack, the batched
@@ -17,9 +18,10 @@ import os
 
 import torch
 
-# (threads per block, blocks per SM, table records (0: what fits), team blocks (0: by load))
-CANDIDATES = [(b, c, 0, 0) for b in (128, 256, 512, 1024) for c in (1, 2, 4, 8, 16)
-              if b * c <= 2048]
+# None (over tiles), or (threads per block, blocks per SM, table records (0: what
+# fits), team blocks (0: by load))
+CANDIDATES = [None] + [(b, c, 0, 0) for b in (128, 256, 512, 1024) for c in (1, 2, 4, 8, 16)
+                       if b * c <= 2048]
 
 
 def cache_path() -> str:
@@ -31,16 +33,23 @@ def cache_path() -> str:
 def _key(ctx, records: int) -> str:
     name = torch.cuda.get_device_name(ctx.device)
     bucket = 0 if records <= 0 else int(round(math.log2(records)))
-    return f"{name}|P={ctx.n_pairs}|E~2^{bucket}"
+    # "tiles": choices made before the codec over tiles was a candidate are not taken
+    return f"{name}|tiles|P={ctx.n_pairs}|E~2^{bucket}"
+
+
+def _cached(ctx, records: int):
+    """(found, tune) of the cache on disk."""
+    try:
+        with open(cache_path()) as f:
+            v = json.load(f)[_key(ctx, records)]["tune"]
+        return True, None if v is None else tuple(v)
+    except Exception:
+        return False, None
 
 
 def load_cached(ctx, records: int):
-    try:
-        with open(cache_path()) as f:
-            v = json.load(f).get(_key(ctx, records))
-        return tuple(v["tune"]) if v else None
-    except Exception:
-        return None
+    """The cached choice: a schedule, or None (no schedule, or nothing cached)."""
+    return _cached(ctx, records)[1]
 
 
 def store(ctx, records: int, tune, ms: float, table):
@@ -52,8 +61,9 @@ def store(ctx, records: int, tune, ms: float, table):
                 data = json.load(f)
         except Exception:
             data = {}
-        data[_key(ctx, records)] = {"tune": list(tune), "ms": ms,
-                                    "candidates": {",".join(map(str, k)): v for k, v in table}}
+        names = {("none" if k is None else ",".join(map(str, k))): v for k, v in table}
+        data[_key(ctx, records)] = {"tune": None if tune is None else list(tune), "ms": ms,
+                                    "candidates": names}
         with open(path + ".tmp", "w") as f:
             json.dump(data, f, indent=1)
         os.replace(path + ".tmp", path)
@@ -74,8 +84,8 @@ def tune_batched(ex, state: dict, reps: int = 2, candidates=None, use_cache: boo
     torch.cuda.synchronize()
     records = int(ex.pair_off[ex.slot_of(t)][-1].item())
     if use_cache:
-        cached = load_cached(ctx, records)
-        if cached is not None:
+        found, cached = _cached(ctx, records)
+        if found:
             ex.tune = cached
             return cached, {}
     args, kw = ex.codec_args(t)
