@@ -20,7 +20,7 @@ namespace tera {
 enum { PI_R = 0, PI_M = 1, PI_NST = 2, PI_MODE = 3, PI_MATCHED = 4, PI_NEW = 5, PI_SLOTPAY = 6,
        PI_PAY = 7 };
 // Per-pair facts of the decode (stride 8 per pair).
-enum { DI_NS = 0, DI_NN = 1, DI_NH = 2, DI_PAY = 3, DI_OK = 4, DI_MODE = 5, DI_NT = 6 };
+enum { DI_NS = 0, DI_NN = 1, DI_NH = 2, DI_PAY = 3, DI_OK = 4, DI_MODE = 5, DI_NT = 6, DI_ERR = 7 };
 
 template <bool CG, typename T>
 __device__ __forceinline__ T ldx(const T* p) {

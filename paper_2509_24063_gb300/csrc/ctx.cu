@@ -96,6 +96,7 @@ __global__ void __launch_bounds__(kScanThreads)
 
 __global__ void unit_map_kernel(const u64* __restrict__ unit_off, u64 npr, u32 p0,
                                 u32* __restrict__ unit_pair, const u64* __restrict__ units_total) {
+  chain_begin();
   if (units_total[1]) return;
   const int lane = threadIdx.x & 31;
   const u64 warp = ((u64)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -189,8 +190,8 @@ int grid_for(tera_ctx* ctx, int blocks_per_sm) { return ctx->num_sms * blocks_pe
 tera_status launch_unit_map(tera_ctx* ctx, u32 p0, u64 npr, cudaStream_t s) {
   if (npr == 0) return TERA_OK;
   prof_begin(ctx, s);
-  unit_map_kernel<<<(unsigned)((npr + 7) / 8), 256, 0, s>>>(ctx->unit_off, npr, p0, ctx->unit_pair,
-                                                            ctx->d_units_total);
+  launch_chained(unit_map_kernel, (unsigned)((npr + 7) / 8), 256, 0, s, ctx->unit_off, npr, p0,
+                 ctx->unit_pair, ctx->d_units_total);
   return check_launch(ctx, "unit_map_kernel", s);
 }
 

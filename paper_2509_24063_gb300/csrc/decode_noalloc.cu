@@ -125,8 +125,11 @@ extern "C" tera_status tera_delta_decode_noalloc(const uint8_t* wire, const uint
   int sms = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
   if (sms <= 0) sms = 148;
-  dec_setup_kernel<false><<<1, 1024, 0, s>>>(A, n_pairs, recv_capacity_units, units_total,
-                                             kStaticMaxUnits);
+  dec_headers_kernel<false>
+      <<<(unsigned)((n_pairs + kHeaderThreads - 1) / kHeaderThreads), kHeaderThreads, 0, s>>>(
+          A, n_pairs);
+  dec_layout_kernel<<<1, 1024, 0, s>>>(A, n_pairs, recv_capacity_units, units_total,
+                                       kStaticMaxUnits);
   static_unit_map_kernel<<<(unsigned)((n_pairs + 7) / 8), 256, 0, s>>>(
       A.unit_off, n_pairs, reinterpret_cast<u32*>(base + kOffUnitPair), units_total);
   const unsigned g = (unsigned)sms * 8u;
