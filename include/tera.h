@@ -194,7 +194,9 @@ tera_status tera_pack_ids(tera_ctx* ctx, const tera_soa* soa, const tera_partiti
  *  - writes the new sender reference ref_next, laid out with pair_off
  *    (matched records in slot order, then new records in message order).
  * mode TERA_MODE_XOR or TERA_MODE_RAW (raw: the reference is ignored).  A
- * pair marked by tera_reset_reference is sent raw once.  wire_capacity is in
+ * pair marked by tera_reset_reference is sent raw once.  A range of every
+ * pair runs over tiles as tera_codec_batched without a tune does, when the
+ * context has or can get the scratch for it.  wire_capacity is in
  * bytes; too small latches TERA_ECAPACITY with the required size. */
 tera_status tera_delta_encode(tera_ctx* ctx, const uint8_t* rec_arena, const uint64_t* pair_off,
                               const uint8_t* ref_prev, const uint64_t* ref_off_prev,
@@ -310,8 +312,9 @@ tera_status tera_mlp_train(tera_ctx* ctx, const float* samples, uint64_t n, floa
                            int steps, int batch, float lr, float clip, uint64_t* n_valid,
                            void* stream);
 
-/* Schedule of the batched codec (picked by the autotuner; outputs do not
- * depend on it): threads per block = entries per tile (128, 256, 512 or
+/* Schedule of the batched codec's persistent launch (picked by the autotuner;
+ * outputs do not depend on it; no schedule, a NULL tune, runs the codec over
+ * warp tiles instead, see tera_codec_batched): threads per block = entries per tile (128, 256, 512 or
  * 1024), blocks per SM of the persistent launch (1..16, block x blocks <=
  * 2048), and the largest message (records) matched in a block's shared-memory
  * hash table: 0 = as large as the shared memory left to the block allows, else
@@ -335,10 +338,12 @@ typedef struct {
   int reserved;
 } tera_tune;
 
-/* Steps a3-a5 for EVERY pair of one iteration in one persistent launch
- * (batching of uneven subdomain buffers; not in the paper, which batches
- * only large messages, Sec. 2.4 "Communication").  Each block carries whole
- * pairs, one at a time, through encode and decode.  Produces exactly the bytes
+/* Steps a3-a5 for EVERY pair of one iteration in one call (batching of uneven
+ * subdomain buffers; not in the paper, which batches only large messages,
+ * Sec. 2.4 "Communication").  tune == NULL: a few launches over tiles of the
+ * pairs' entries, which size themselves (the fast form at most sizes).  With a
+ * tune: one persistent launch, each block carrying whole pairs, one at a time,
+ * through encode and decode.  Either way produces exactly the bytes
  * of tera_delta_encode + tera_delta_decode over all pairs: wire_off, the wire
  * messages, wire_len, the new sender reference ref_next (laid out with
  * pair_off) and the receive buffers recv with recv_off.  The receive layout
@@ -346,9 +351,9 @@ typedef struct {
  * record count is checked against it (TERA_ECORRUPT otherwise).  The sender
  * reference is ref_prev/ref_off_prev, the receiver's recv_prev/recv_off_prev
  * (NULL pairs = empty references).  rec_arena is any packed arena laid out
- * with pair_off (record ids are read from the records).  tune == NULL uses
- * {256, 4, 0, 0, 0, 0}.  Asynchronous, no host synchronization (graph-capturable once
- * scratch is reserved); device errors are latched in the status word.  Small
+ * with pair_off (record ids are read from the records).  Asynchronous, no host synchronization (graph-capturable once
+ * scratch is reserved; a call of either form reserves it for both); device
+ * errors are latched in the status word.  With a tune, small
  * pairs (at most 512 slots, records and receiver slots) are carried by a
  * second launch on a stream the context owns, forked from `stream` after the
  * call's first kernel and joined back into it before the call returns (CUDA

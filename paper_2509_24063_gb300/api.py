@@ -253,8 +253,9 @@ class Context:
     def codec_batched(self, rec_arena, pair_off, ref_prev, ref_off_prev, ref_next, wire, wire_off,
                       wire_len, recv_prev, recv_off_prev, recv, recv_off, mode=_lib.MODE_XOR,
                       tune=None, stream=None, ids=None):
-        """Encode + decode of every pair in one persistent launch (tera_codec_batched;
-        with ids = dict(msg, ref_prev, ref_next) of id columns, tera_codec_batched_ids)."""
+        """Encode + decode of every pair in one call (tera_codec_batched: over warp
+        tiles, with a tune in one persistent launch; with ids = dict(msg, ref_prev,
+        ref_next) of id columns, tera_codec_batched_ids)."""
         t = _tune(tune)
         if ids is not None:
             c = _lib.Ids(_ptr(ids["msg"]).value,

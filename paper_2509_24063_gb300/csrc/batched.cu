@@ -1,7 +1,10 @@
 // Batched codec: steps a3-a5 (paper Sec. 2.3, steps B, C and D) for every
-// pair of one iteration in ONE persistent launch (on the plain path the small
-// pairs run in a second launch of one-warp blocks beside it), after a setup
-// of two short launches that lays out the wire slabs and the work list.
+// pair of one iteration.  Without a schedule the call runs over warp tiles
+// (codec_tiles.cu).  With one, ONE persistent launch (on the plain path the
+// small pairs run in a second launch of one-warp blocks beside it), after a
+// setup of two short launches that lays out the wire slabs and the work list;
+// this file holds that launch, the predictor's pre-pass of both forms, and the
+// entry points.
 //
 // Each block takes whole pairs (an atomic ticket over the work list, claimed
 // whenever the block is free) and carries a pair through every step on its

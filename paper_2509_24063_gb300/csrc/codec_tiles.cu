@@ -2,9 +2,9 @@
 // every pair of one iteration, as launches over tiles of kT entries that know
 // nothing of the pairs' sizes:
 //
-//   setup   (two launches) per-pair facts, wire slabs and the lists of tiles
-//   match   one block per pair: the message record of every reference slot
-//           (ids in shared memory), the matches before each tile and the list
+//   setup   per-pair facts, wire slabs and the lists of tiles
+//   match   one block (a warp for a small pair) per pair: the message record of
+//           every reference slot (ids in shared memory), the matches before each tile and the list
 //           of the records no slot took; a pair of more than kTableMax records
 //           is only asked here, a tile each, whether its ids ascend, and
 //           matched by
@@ -28,10 +28,10 @@
 // persistent launch of batched.cu, used for an explicit schedule) pays every
 // step's memory latency once per tile of every pair, one after the other, and
 // the largest pair is the launch's length.  Measured, whole codec: uniform 100
-// M agents (16.6 M records) 1.98 -> 1.54 ms, of which encode 683 us (3.65 GB,
-// 79 % of the measured copy rate), decode 464 us (2.4 GB), match 264, wire 88,
-// setup 32; 16 M agents kept box by box 0.93 -> 0.78 ms; a pair of 1.1 M
-// records among 6.5 M: 3.3 -> 1.2 ms; 6.3 K records in 12 pairs: 92 -> 60 us.
+// M agents (16.6 M records) 1.98 -> 1.43 ms, of which encode 675 us (3.65 GB,
+// 80 % of the measured copy rate), decode 465 us (2.4 GB), match 179, wire 88,
+// setup 19; 16 M agents kept box by box 0.93 -> 0.62 ms; a pair of 1.1 M
+// records among 6.5 M: 3.3 -> 0.8 ms; 6.3 K records in 12 pairs: 92 -> 60 us.
 // A look-back over the tiles in place of the second copy of the payload
 // (tiles claimed in order, sums published) left encode and decode at 1.16 ms
 // each; a block a tile with barriers between its steps at 0.86 and 0.74.
@@ -57,7 +57,8 @@ constexpr u64 kTilesPerWarp = 8;
 constexpr u32 kNewShare = 16;
 // Pairs of at most this many slots and records are matched by one warp, so
 // that the thousands of edge and corner pairs of a large grid are in flight at
-// once (13,824 pairs, 100 M agents: match 297 -> 264 us).  A grid with few
+// once (13,824 pairs, 100 M agents: match 297 -> 264 us, before the ids were held
+// in shared memory; now 179).  A grid with few
 // pairs for the GPU's blocks gives all but the smallest a block (1 M agents,
 // 936 pairs: 39 us with the higher limit, 32 with the lower).
 constexpr u32 kWarpPair = 256, kWarpPairFew = 64;

@@ -5,8 +5,9 @@ pair stores the same reference and updates it every iteration here).
 Paths (all produce the same bytes):
   "per_subdomain"  pack / encode / decode launched once per sending box
   "all_pairs"      pack / encode / decode launched once for all pairs
-  "batched"        pack, then encode + decode of all pairs in one persistent
-                   launch (tera_codec_batched); capturable in a CUDA graph
+  "batched"        pack, then encode + decode of all pairs in one call
+                   (tera_codec_batched): over warp tiles, or with a tune in
+                   one persistent launch; capturable in a CUDA graph
 
 Buffers are allocated once for a maximum agent count and record count; the
 sender and receiver references are double-buffered (previous / next).
