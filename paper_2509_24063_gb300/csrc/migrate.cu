@@ -152,13 +152,15 @@ __device__ __forceinline__ void warp_boxes(const u64* __restrict__ box_off, u32 
   *hi = warp_box_search(box_off, *lo, n_boxes - 1, w_end - 1);
 }
 
-// Zeroes the counters and the abort flag in one launch (three memsets took
-// three, and the count kernel could not be set up behind a memset).
+// Zeroes the counters, the head of the leavers' sort and the abort flag in one
+// launch (memsets took four, and no kernel can be set up behind a memset).
 __global__ void __launch_bounds__(256)
     mig_begin_kernel(u64* __restrict__ from, u64 n_boxes, u64* __restrict__ cnt, u64 Q,
-                     DevStatus* st) {
+                     u64* __restrict__ sort_head, DevStatus* st) {
   chain_begin();
   const u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x;
+  if (blockIdx.x == 0)
+    for (u32 h = threadIdx.x; h < kSortHead; h += blockDim.x) sort_head[h] = 0;
   if (i == 0) st->abort = 0;
   if (i < n_boxes) from[i] = 0;
   if (i < Q) cnt[i] = 0;
@@ -632,7 +634,7 @@ extern "C" tera_status tera_migrate_send(tera_ctx* ctx, const tera_soa* prev,
   if ((st = ensure_migrate(ctx, n, lv_cap)) != TERA_OK) return st;
   prof_begin(ctx, s);
   launch_chained(mig_begin_kernel, (unsigned)((Q + 255) / 256), 256, 0, s, ctx->m_from, B, ctx->m_cnt,
-                 Q, ctx->d_status);
+                 Q, ctx->m_hist, ctx->d_status);
   if ((st = check_launch(ctx, "mig_begin_kernel", s)) != TERA_OK) return st;
   const u64 blocks = n == 0 ? 1 : (n + kBlockAgents - 1) / kBlockAgents;
   const u64 wtiles = n == 0 ? 1 : (n + kWarpAgents - 1) / kWarpAgents;

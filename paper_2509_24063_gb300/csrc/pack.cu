@@ -125,6 +125,7 @@ __device__ __forceinline__ ulonglong2 load_pair(const u64* p) {
 // stores each agent's record once per entry, at the record index the
 // partition's sort gave the entry; the entries of a run are numbered from
 // run_base[run] in agent order.
+template <int R>
 __global__ void __launch_bounds__(kClassifyThreads)
     pack_runs_kernel(SoaPtrs soa, u64 n, const int* __restrict__ owner,
                      const u32* __restrict__ mask, const u64* __restrict__ run_base, u64 n_runs,
@@ -149,8 +150,8 @@ __global__ void __launch_bounds__(kClassifyThreads)
   // a partition that overflowed its capacity left no record indices
   if (run_base[n_runs] != E) return;
   const int lane = threadIdx.x & 31;
-  const u64 tile0 = (u64)blockIdx.x * kClassifyTile;
-  for (int k = 0; k < kClassifyPerThread / 2; ++k) {
+  const u64 tile0 = (u64)blockIdx.x * (2 * kClassifyThreads * R);
+  for (int k = 0; k < R; ++k) {
     const u64 a0 = tile0 + (u64)k * (2 * kClassifyThreads) + 2u * threadIdx.x;
     const u64 first = a0 - 2u * lane;
     if (first >= n) break;  // warp-uniform
@@ -241,10 +242,12 @@ static tera_status pack_impl(tera_ctx* ctx, const tera_soa* soa, const tera_part
   for (int w = 0; w < 8; ++w) aligned = aligned && ((uintptr_t)p.col[w] & 15u) == 0;
   if (pair_begin == 0 && pair_end == ctx->n_pairs && aligned && ctx->pack_n == soa->n) {
     const u64 n = (u64)soa->n;
-    const u64 blocks = n == 0 ? 1 : (n + kClassifyTile - 1) / kClassifyTile;
+    const int rounds = agent_rounds(ctx, n);
+    const u64 per = 2ull * kClassifyThreads * rounds;
+    const u64 blocks = n == 0 ? 1 : (n + per - 1) / per;
     const u64 runs = n == 0 ? 1 : (n + kRunAgents - 1) / kRunAgents;
     prof_begin(ctx, s);
-    launch_chained(pack_runs_kernel, (unsigned)blocks, kClassifyThreads, 0, s, 
+    launch_chained(rounds == 1 ? pack_runs_kernel<1> : pack_runs_kernel<kAgentRounds>, (unsigned)blocks, kClassifyThreads, 0, s, 
         p, n, part->owner, part->mask, ctx->tile_base, runs, ctx->ent_dest,
         reinterpret_cast<const u64*>(part->pair_off), ctx->n_pairs, rec_arena, arena_units,
         ctx->class_id, ctx->d_status, reinterpret_cast<u64*>(rec_ids));

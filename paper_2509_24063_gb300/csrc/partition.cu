@@ -62,7 +62,7 @@ __device__ __forceinline__ void agent_entry(u32 ex, u32 ey, u32 ez, int n0, int 
   *mask = *ok ? lut[(ex & 3u) | ((ey & 3u) << 2) | ((ez & 3u) << 4)] : 0u;
 }
 
-// Each block classifies tiles of kClassifyTile agents (tile blockIdx.x, then
+// Each block classifies tiles of R rounds of 512 agents (tile blockIdx.x, then
 // every gridDim.x-th: the grid holds the blocks resident at once, so the grid
 // rows and the bucket tables are copied into shared memory once per block).
 // In round k of a tile, thread t holds agents 512k + 2t and 512k + 2t + 1 (one
@@ -77,7 +77,7 @@ __device__ __forceinline__ void agent_entry(u32 ex, u32 ey, u32 ez, int n0, int 
 // instruction fetches) took 689 us for 100 M agents; with the masks looked up
 // and the exact path out of line 537.  (Fewer resident blocks for more
 // registers: 5 per SM 752 us, 4 per SM 725; two rounds unrolled 654.)
-template <bool TAB>
+template <bool TAB, int R>
 __global__ void __launch_bounds__(kClassifyThreads, 6)
     classify_kernel(const u64* __restrict__ x, const u64* __restrict__ y,
                     const u64* __restrict__ z, u64 n, const GridTables* __restrict__ g,
@@ -123,9 +123,9 @@ __global__ void __launch_bounds__(kClassifyThreads, 6)
   const int n0 = sg.n[0], n1 = sg.n[1];
   bool bad = false;
   for (u64 tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-    const u64 tile0 = tile * kClassifyTile;
+    const u64 tile0 = tile * (2 * kClassifyThreads * R);
 #pragma unroll
-    for (int k = 0; k < kClassifyPerThread / 2; ++k) {
+    for (int k = 0; k < R; ++k) {
       const u64 a0 = tile0 + (u64)k * (2 * kClassifyThreads) + 2u * threadIdx.x;
       u64 vx[2], vy[2], vz[2];
       if (a0 + 1 < n) {
@@ -179,6 +179,7 @@ __global__ void __launch_bounds__(kClassifyThreads, 6)
 // Emit (pair, agent) entries in agent order, with the rounds and runs of
 // classify_kernel: run r writes its entries from run_base[r]; within a run,
 // lanes are ranked by a warp scan.
+template <int R>
 __global__ void __launch_bounds__(kClassifyThreads)
     emit_kernel(const int* __restrict__ owner, const u32* __restrict__ mask, u64 n,
                 const u64* __restrict__ run_base, u64 n_runs, u32* __restrict__ keys,
@@ -196,8 +197,8 @@ __global__ void __launch_bounds__(kClassifyThreads)
     return;
   }
   const int lane = threadIdx.x & 31;
-  const u64 tile0 = (u64)blockIdx.x * kClassifyTile;
-  for (int k = 0; k < kClassifyPerThread / 2; ++k) {
+  const u64 tile0 = (u64)blockIdx.x * (2 * kClassifyThreads * R);
+  for (int k = 0; k < R; ++k) {
     const u64 a0 = tile0 + (u64)k * (2 * kClassifyThreads) + 2u * threadIdx.x;
     const u64 first = a0 - 2u * lane;
     if (first >= n) break;  // warp-uniform
@@ -254,11 +255,32 @@ __device__ __forceinline__ u64 live_entries(const u64* total_ptr, u64 cap, const
   return t > cap ? 0 : t;
 }
 
+constexpr int kSortSub = 4;  // sub-steps of 32 entries per warp and round of a tile
+constexpr int kSortRound = kSortThreads * kSortSub;
+static_assert(kSortTile % kSortRound == 0, "whole rounds");
+
 // Scratch of a sort (SortBufs::hist): counts[pass * kRadix + d] of digit d,
 // then a claim ticket per pass, then the look-back states of each pass's
 // tiles, state[(pass * tiles + tile) * radix + d].
 __device__ __forceinline__ u64* sort_states(u64* head, u32 pass, u64 tiles, u32 radix) {
   return head + kSortHead + (u64)pass * tiles * radix;
+}
+
+// Entries of a tile: kSortTile, or a single round of it while such tiles are
+// at most two per SM, so that a short list is still spread over the SMs (100
+// thousand agents, 70 K entries: 103 -> 98 us per iteration.  Up to four per SM
+// 1 M agents, whose tiles then wait for one another longer, lose what they
+// gain: 306 -> 308).
+constexpr u64 kSortFew = 300ull * kSortRound;
+__host__ __device__ constexpr u32 sort_tile(u64 entries) {
+  return entries <= kSortFew ? kSortRound : kSortTile;
+}
+
+// Tiles of up to cap entries, at most.
+constexpr u64 sort_tiles(u64 cap) {
+  const u64 few = ((cap < kSortFew ? cap : kSortFew) + kSortRound - 1) / kSortRound;
+  const u64 many = (cap + kSortTile - 1) / kSortTile;
+  return few > many ? few : many;
 }
 
 // Digit counts of every pass from one read of the keys, and the cleared
@@ -291,7 +313,8 @@ __global__ void __launch_bounds__(kSortThreads)
   for (u64 i = 4 * quads + tid; i < E; i += step)
     for (u32 p = 0; p < passes; ++p)
       atomicAdd(&cnt[p * kRadix + ((keys[i] >> (p * dbits)) & (radix - 1))], 1u);
-  const u64 live = (E + kSortTile - 1) / kSortTile * radix;
+  const u32 tile = sort_tile(E);
+  const u64 live = (E + tile - 1) / tile * radix;
   for (u32 p = 0; p < passes; ++p) {
     u64* s = sort_states(head, p, tiles, radix);
     for (u64 i = tid; i < live; i += step) s[i] = 0;
@@ -301,7 +324,7 @@ __global__ void __launch_bounds__(kSortThreads)
     if (cnt[d]) atomicAdd(head + d, (u64)cnt[d]);
 }
 
-// Stable scatter of sort tiles of kSortTile entries, claimed one after the
+// Stable scatter of sort tiles (sort_tile entries), claimed one after the
 // other by resident blocks.  A tile counts its digits, publishes the counts,
 // and while its entries are ranked the tiles before it publish theirs; thread
 // d then walks back over digit d's counts (eight tiles' in flight) to the
@@ -323,7 +346,6 @@ __global__ void __launch_bounds__(kSortThreads)
 // the last writes the agent as the value (vals_out[pos] = agent) and, when
 // dest is given, the entry's record index (dest[e] = pos).  kR bounds the
 // radix (digit arrays in shared memory).
-constexpr int kSortSub = 4;  // sub-steps of 32 entries per warp and round
 
 // Dynamic shared memory of a scatter: raw keys and agents, the sorted-position
 // index, and the raw entry indices when the pass reads them.
@@ -346,7 +368,7 @@ __global__ void __launch_bounds__(kSortThreads)
                       DevStatus* st) {
   chain_begin();
   constexpr int kWarps = kSortThreads / 32;
-  constexpr int kRoundEntries = kSortThreads * kSortSub;
+  constexpr int kRoundEntries = kSortRound;
   extern __shared__ __align__(16) u32 sort_stage[];
   u32* rkey = sort_stage;
   u32* ragt = sort_stage + kSortTile;
@@ -359,6 +381,7 @@ __global__ void __launch_bounds__(kSortThreads)
   __shared__ u32 sm[33];
   __shared__ u32 s_tile;
   const u64 E = live_entries(total_ptr, cap, st);
+  const u32 tile_cap = sort_tile(E);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const u32 lt = (1u << lane) - 1u;
   u64* states = sort_states(head, pass, n_tiles, radix);
@@ -374,9 +397,9 @@ __global__ void __launch_bounds__(kSortThreads)
   for (u32 d = threadIdx.x; d < radix; d += blockDim.x) run[d] = 0;
   __syncthreads();
   const u64 tile = s_tile;
-  const u64 t0 = tile * kSortTile;
+  const u64 t0 = tile * tile_cap;
   if (t0 >= E) return;
-  const u32 tile_n = (u32)(E - t0 < (u64)kSortTile ? E - t0 : (u64)kSortTile);
+  const u32 tile_n = (u32)(E - t0 < (u64)tile_cap ? E - t0 : (u64)tile_cap);
   {
     const uintptr_t al = reinterpret_cast<uintptr_t>(keys_in) |
                          reinterpret_cast<uintptr_t>(agents_in) |
@@ -559,17 +582,16 @@ static void sort_shape(u64 key_limit, int* passes, int* dbits) {
 u64 sort_scratch(u64 cap, u64 key_limit) {
   int passes, dbits;
   sort_shape(key_limit, &passes, &dbits);
-  return kSortHead + (((u64)passes * ((cap + kSortTile - 1) / kSortTile)) << dbits);
+  return kSortHead + (((u64)passes * sort_tiles(cap)) << dbits);
 }
 
 tera_status radix_sort_entries(tera_ctx* ctx, const SortBufs& b, const u32* keys_in,
                                const u32* agent, u32* dest, u32* vals_final, const u64* total_ptr,
-                               u64 cap, u64 key_limit, const u32** sorted_keys, cudaStream_t s,
-                               bool zeroed) {
+                               u64 cap, u64 key_limit, const u32** sorted_keys, cudaStream_t s) {
   int passes, dbits;
   sort_shape(key_limit, &passes, &dbits);
   const u32 radix = 1u << dbits;
-  const u64 tiles = cap == 0 ? 1 : (cap + kSortTile - 1) / kSortTile;
+  const u64 tiles = cap == 0 ? 1 : sort_tiles(cap);
   const u32* kin = keys_in;
   const u32* vin = nullptr;
   const u32* ain = agent;
@@ -584,7 +606,6 @@ tera_status radix_sort_entries(tera_ctx* ctx, const SortBufs& b, const u32* keys
     smem_set = true;
   }
   if (cap > 0) {
-    if (!zeroed) cudaMemsetAsync(b.hist, 0, sizeof(u64) * kSortHead, s);
     const u64 hgrid = (u64)grid_for(ctx, 4);
     prof_begin(ctx, s);
     launch_chained(rs_hist_kernel, (unsigned)(tiles < hgrid ? tiles : hgrid), kSortThreads, 0, s, 
@@ -642,22 +663,30 @@ extern "C" tera_status tera_partition(tera_ctx* ctx, const tera_soa* soa, tera_p
   if (!ctx->tile_cnt || !ctx->tile_base) return TERA_ENOMEM;
   if ((st = ensure_records(ctx, out->idx_capacity, s)) != TERA_OK) return st;
   ctx->iterations += 1;
-  const u64 blocks = n == 0 ? 1 : (n + kClassifyTile - 1) / kClassifyTile;
+  const int rounds = agent_rounds(ctx, n);
+  const u64 per = 2ull * kClassifyThreads * rounds;
+  const u64 blocks = n == 0 ? 1 : (n + per - 1) / per;
   const u64 runs = n == 0 ? 1 : (n + kRunAgents - 1) / kRunAgents;
   // resident blocks only (6 per SM): each copies the tables into shared memory once
   const size_t csmem =
       grid_smem_bytes(ctx->grid) + (ctx->d_buckets ? 3 * (size_t)kAxisBuckets : 0);
   static bool csmem_set = false;
   if (!csmem_set) {
-    cudaFuncSetAttribute(classify_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)(sizeof(BoxKeys) * 3 * kMaxAxis + 3 * (size_t)kAxisBuckets));
-    cudaFuncSetAttribute(classify_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)(sizeof(BoxKeys) * 3 * kMaxAxis));
+    const int rows = (int)(sizeof(BoxKeys) * 3 * kMaxAxis), tabs = rows + 3 * kAxisBuckets;
+    const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    cudaFuncSetAttribute(classify_kernel<true, kAgentRounds>, attr, tabs);
+    cudaFuncSetAttribute(classify_kernel<true, 1>, attr, tabs);
+    cudaFuncSetAttribute(classify_kernel<false, kAgentRounds>, attr, rows);
+    cudaFuncSetAttribute(classify_kernel<false, 1>, attr, rows);
     csmem_set = true;
   }
   const u64 cgrid = blocks < (u64)ctx->num_sms * 6 ? blocks : (u64)ctx->num_sms * 6;
   prof_begin(ctx, s);
-  launch_chained(ctx->d_buckets ? classify_kernel<true> : classify_kernel<false>, (unsigned)cgrid, kClassifyThreads, csmem, s, 
+  const auto classify = rounds == 1
+                            ? (ctx->d_buckets ? classify_kernel<true, 1> : classify_kernel<false, 1>)
+                            : (ctx->d_buckets ? classify_kernel<true, kAgentRounds>
+                                              : classify_kernel<false, kAgentRounds>);
+  launch_chained(classify, (unsigned)cgrid, kClassifyThreads, csmem, s,
       reinterpret_cast<const u64*>(soa->x), reinterpret_cast<const u64*>(soa->y),
       reinterpret_cast<const u64*>(soa->z), n, ctx->d_grid, ctx->d_buckets, blocks, out->owner,
       out->mask, ctx->tile_cnt, runs, ctx->d_status, ctx->d_stats, ctx->rs_hist);
@@ -670,7 +699,7 @@ extern "C" tera_status tera_partition(tera_ctx* ctx, const tera_soa* soa, tera_p
   const u64* total_ptr = ctx->tile_base + runs;
   if (cap > 0 || n > 0) {
     prof_begin(ctx, s);
-    launch_chained(emit_kernel, (unsigned)blocks, kClassifyThreads, 0, s, 
+    launch_chained(rounds == 1 ? emit_kernel<1> : emit_kernel<kAgentRounds>, (unsigned)blocks, kClassifyThreads, 0, s, 
         out->owner, out->mask, n, ctx->tile_base, runs, ctx->keys_a, ctx->ent_agent, cap,
         ctx->d_status);
     if ((st = check_launch(ctx, "emit_kernel", s)) != TERA_OK) return st;
@@ -679,7 +708,7 @@ extern "C" tera_status tera_partition(tera_ctx* ctx, const tera_soa* soa, tera_p
                       ctx->agents_b, ctx->agents_c, ctx->rs_hist};
   const u32* sorted = nullptr;
   if ((st = radix_sort_entries(ctx, bufs, ctx->keys_a, ctx->ent_agent, ctx->ent_dest, out->pair_idx,
-                               total_ptr, cap, P, &sorted, s, true)) != TERA_OK)
+                               total_ptr, cap, P, &sorted, s)) != TERA_OK)
     return st;
   ctx->rec_pair = const_cast<u32*>(sorted);
   ctx->pack_n = soa->n;

@@ -189,6 +189,18 @@ inline void launch_chained(void (*kernel)(P...), unsigned grid, unsigned block, 
   cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
 }
 
+// Rounds of 512 agents a block of the agent passes (classify, emit, pack)
+// takes: four, or one when the blocks of four would be fewer than four per SM
+// (a round is a chain of dependent loads, and a block's rounds come one after
+// the other.  100 thousand agents, 49 -> 196 blocks: classify, emit and pack 33
+// -> 18 us together, 118 -> 102 per iteration; 1 M agents 212 -> 209, with the
+// line at two per SM 213).
+constexpr int kAgentBlocks = 4;
+constexpr int kAgentRounds = kClassifyPerThread / 2;
+inline int agent_rounds(const tera_ctx* ctx, u64 n) {
+  return n < (u64)ctx->num_sms * kAgentBlocks * kClassifyTile ? 1 : kAgentRounds;
+}
+
 // ctx.cu
 void prof_begin(tera_ctx* ctx, cudaStream_t s);
 tera_status check_launch(tera_ctx* ctx, const char* name, cudaStream_t s);
@@ -225,10 +237,9 @@ struct SortBufs {
 };
 // Words of SortBufs::hist for `cap` entries with keys below key_limit.
 u64 sort_scratch(u64 cap, u64 key_limit);
-// Words of it that are zero when a sort begins.
+// Words of it that the caller has zeroed when a sort begins.
 constexpr u64 kSortHead = 4 * kRadix + 4;
 tera_status radix_sort_entries(tera_ctx* ctx, const SortBufs& b, const u32* keys_in,
                                const u32* agent, u32* dest, u32* vals_final, const u64* total_ptr,
-                               u64 cap, u64 key_limit, const u32** sorted_keys, cudaStream_t s,
-                               bool zeroed = false);
+                               u64 cap, u64 key_limit, const u32** sorted_keys, cudaStream_t s);
 }  // namespace tera
