@@ -73,6 +73,9 @@ def kernel_bytes(name, t):
 # the full-size run recorded in profiles/; used only while the kernel's sources
 # are the ones the capture was taken with (their digest is recorded beside it).
 KERNEL_SOURCES = {"codec_persistent_kernel": ("batched.cu", "codec.cuh", "tera_device.cuh"),
+                  "codec_encode_kernel": ("codec_tiles.cu", "codec_tile.cuh", "codec.cuh",
+                                          "tera_device.cuh"),
+                  "pack_runs_kernel": ("pack.cu", "tera_device.cuh"),
                   "mig_move_kernel": ("migrate.cu", "classify.cuh", "tera_device.cuh")}
 
 
