@@ -1622,11 +1622,11 @@ static tera_status pred_prepass(tera_ctx* ctx, const PredArgs& pr, const uint8_t
                                                                    (u32)ctx->n_pairs, cap, out);
   if ((st = check_launch(ctx, "pred_features_kernel", s)) != TERA_OK) return st;
   prof_begin(ctx, s);
-  static bool net_set = false;
-  if (!net_set) {
+  static PerDevice net_set;
+  if (net_set.needed(ctx->device)) {
     cudaFuncSetAttribute(pred_slots_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)kNetSmem);
-    net_set = true;
+    net_set.done(ctx->device);
   }
   pred_slots_kernel<<<(unsigned)ctx->num_sms, kNetThreads, kNetSmem, s>>>(
       pr, ref, off, (u32)ctx->n_pairs, cap, out);

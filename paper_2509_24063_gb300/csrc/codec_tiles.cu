@@ -1536,8 +1536,8 @@ tera_status launch_tiles(tera_ctx* ctx, const EncArgs& E, const DecArgs& D, bool
   const bool encode_only = D.recv == nullptr;
   tera_status st;
   const unsigned grid = (unsigned)(ctx->num_sms * kPerSm);
-  static bool configured = false;
-  if (!configured) {
+  static PerDevice configured;
+  if (configured.needed(ctx->device)) {
     const void* k[] = {reinterpret_cast<const void*>(codec_encode_kernel<false>),
                        reinterpret_cast<const void*>(codec_encode_kernel<true>),
                        reinterpret_cast<const void*>(codec_decode_kernel<false>),
@@ -1550,7 +1550,7 @@ tera_status launch_tiles(tera_ctx* ctx, const EncArgs& E, const DecArgs& D, bool
       if (cudaFuncSetAttribute(k[i], cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)(i < 2 ? kEncSmem : kDecSmem)) != cudaSuccess)
         return TERA_ECUDA;
-    configured = true;
+    configured.done(ctx->device);
   }
   TileArgs A;
   A.E = E;

@@ -597,13 +597,13 @@ tera_status radix_sort_entries(tera_ctx* ctx, const SortBufs& b, const u32* keys
   const u32* ain = agent;
   u32* kfinal = (passes & 1) ? b.keys_b : b.keys_c;
   tera_status st;
-  static bool smem_set = false;
-  if (!smem_set) {
+  static PerDevice smem_set;
+  if (smem_set.needed(ctx->device)) {
     cudaFuncSetAttribute(rs_scatter_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)sort_smem_bytes(true));
     cudaFuncSetAttribute(rs_scatter_kernel<kRadix>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)sort_smem_bytes(true));
-    smem_set = true;
+    smem_set.done(ctx->device);
   }
   if (cap > 0) {
     const u64 hgrid = (u64)grid_for(ctx, 4);
@@ -670,15 +670,15 @@ extern "C" tera_status tera_partition(tera_ctx* ctx, const tera_soa* soa, tera_p
   // resident blocks only (6 per SM): each copies the tables into shared memory once
   const size_t csmem =
       grid_smem_bytes(ctx->grid) + (ctx->d_buckets ? 3 * (size_t)kAxisBuckets : 0);
-  static bool csmem_set = false;
-  if (!csmem_set) {
+  static PerDevice csmem_set;
+  if (csmem_set.needed(ctx->device)) {
     const int rows = (int)(sizeof(BoxKeys) * 3 * kMaxAxis), tabs = rows + 3 * kAxisBuckets;
     const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
     cudaFuncSetAttribute(classify_kernel<true, kAgentRounds>, attr, tabs);
     cudaFuncSetAttribute(classify_kernel<true, 1>, attr, tabs);
     cudaFuncSetAttribute(classify_kernel<false, kAgentRounds>, attr, rows);
     cudaFuncSetAttribute(classify_kernel<false, 1>, attr, rows);
-    csmem_set = true;
+    csmem_set.done(ctx->device);
   }
   const u64 cgrid = blocks < (u64)ctx->num_sms * 6 ? blocks : (u64)ctx->num_sms * 6;
   prof_begin(ctx, s);

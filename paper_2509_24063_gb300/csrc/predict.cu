@@ -563,14 +563,14 @@ tera_status compact(tera_ctx* ctx, const float* samples, u64 n, float* dense, u3
 tera_status train_steps(tera_ctx* ctx, const TrainScratch& t, u64 nv, u64 batch, int steps,
                         const float* params_in, float* params, float* grad, float lr, float clip,
                         cudaStream_t s) {
-  static bool configured = false;
-  if (!configured) {
+  static PerDevice configured;
+  if (configured.needed(ctx->device)) {
     if (cudaFuncSetAttribute(mlp_steps_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)sizeof(TrainSmem<1>)) != cudaSuccess ||
         cudaFuncSetAttribute(mlp_steps_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)sizeof(TrainSmem<2>)) != cudaSuccess)
       return TERA_ECUDA;
-    configured = true;
+    configured.done(ctx->device);
   }
   TrainArgs A;
   A.dense = t.dense;

@@ -2,6 +2,7 @@
 // device-side helpers (tera_device.cuh) and the host-side context.
 #pragma once
 
+#include <atomic>
 #include <cstddef>
 
 #include <nvtx3/nvToolsExt.h>
@@ -188,6 +189,19 @@ inline void launch_chained(void (*kernel)(P...), unsigned grid, unsigned block, 
   c.numAttrs = 1;
   cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
 }
+
+// What a kernel needs set once per device (its shared-memory limit): needed()
+// until done() has been called for the device, from any thread; setting twice
+// does no harm.
+struct PerDevice {
+  std::atomic<uint64_t> set{0};
+  bool needed(int device) const {
+    return device >= 64 || !(set.load(std::memory_order_acquire) >> device & 1u);
+  }
+  void done(int device) {
+    if (device < 64) set.fetch_or(1ull << device, std::memory_order_release);
+  }
+};
 
 // Rounds of 512 agents a block of the agent passes (classify, emit, pack)
 // takes: four, or one when the blocks of four would be fewer than four per SM
