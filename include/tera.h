@@ -156,6 +156,15 @@ uint64_t tera_n_pairs(const tera_ctx* ctx);
  * lazy growth synchronizes the device, so call this before graph capture). */
 tera_status tera_ctx_reserve(tera_ctx* ctx, int64_t max_agents, uint64_t max_records);
 
+/* Limit, in microseconds (0 .. 60000000; 1000000 when the context is made), of a
+ * wait inside one of the context's kernels for another block of the same launch.
+ * Such a wait ends by itself; one that takes longer is given up, latches
+ * TERA_ETIMEOUT, and the call leaves its lists empty and its messages unwritten.
+ * 0: any wait is given up.  Holds for the calls after this one (a captured graph
+ * keeps the limit it was captured with); tera_tune.wait_limit_us is that of the
+ * persistent launch. */
+tera_status tera_ctx_wait_limit(tera_ctx* ctx, int64_t limit_us);
+
 /* Step a1 (Sec. 2.1 "Aura Update"): owner box and aura mask of every agent,
  * and the per-pair stable lists.  Agent i is in the aura of neighbour box at
  * offset o when, on every axis, o = 0, or o = -1 and x < e[i] + w, or o = +1

@@ -204,6 +204,11 @@ class Context:
         check(self.lib.tera_ctx_reserve(self.h, int(max_agents), int(max_records)),
               "tera_ctx_reserve")
 
+    def wait_limit(self, limit_us: int):
+        """Limit of a wait inside a kernel of the calls after this one
+        (tera_ctx_wait_limit; 0: any wait is given up)."""
+        check(self.lib.tera_ctx_wait_limit(self.h, int(limit_us)), "tera_ctx_wait_limit")
+
     def status(self, stream=None, raise_on_error=True):
         req = C.c_uint64(0)
         st = self.lib.tera_ctx_status(self.h, C.byref(req), _stream(stream))

@@ -91,6 +91,7 @@ struct TileArgs {
   u32* unit_first;      // [P] first tile of each pair
   u64* setup_state;     // look-back states of the setup (zero between calls)
   u32* setup_ticket;
+  u64 limit_ns;         // of a wait
   u32* item_pair;       // pair of each match item
   u32* big_pair;        // pair of each bigmatch item
   u32* small_pair;      // pairs matched by one warp
@@ -168,9 +169,11 @@ __device__ __forceinline__ void fill_map(u32* __restrict__ out, u64 lo, u32 n, u
 // slabs and lists by a block scan and a look-back over the blocks (four chains:
 // slab bytes, tiles, match items and warp pairs in the halves of a word, items
 // of big pairs).  Pairs without entries on either side are finished here.  The
-// last block writes the totals and checks the capacities; until then a block
-// knows all but the slabs' total, so it writes to the wire only inside its
-// capacity.
+// last block checks the capacities and writes the lists' lengths, all zero when a
+// capacity is exceeded or any block's wait was cut short (its pairs' lines and
+// list entries are then not written, and no launch may index by them); until
+// then a block knows all but the slabs' total, so it writes to the wire only
+// inside its capacity.
 __global__ void __launch_bounds__(kSetupT)
     tiles_setup_kernel(TileArgs A, int mode, u64* __restrict__ wire_off, u64 wire_cap, u64 rec_cap,
                        u64 recv_cap, u64 unit_cap, u64 item_cap, u64 big_cap, u32* epoch) {
@@ -203,20 +206,17 @@ __global__ void __launch_bounds__(kSetupT)
     const u32 c = threadIdx.x >> 5;
     const u64 own = c == 0 ? ta.a : (c == 1 ? ta.b : (c == 2 ? tb.a : tb.b));
     u64 pre = 0;
-    if (gridDim.x > 1 && !lb_warp_sum(A.setup_state + (u64)c * gridDim.x, block, own, A.E.st, &pre) &&
+    if (gridDim.x > 1 && !lb_warp_sum(A.setup_state + (u64)c * gridDim.x, block, own, A.E.st, A.limit_ns,
+                                      &pre) &&
         (threadIdx.x & 31) == 0)
       s_fine = 0;
     if ((threadIdx.x & 31) == 0) s_pre[c] = pre;
   }
   __syncthreads();
-  const bool last = block == gridDim.x - 1;
-  if (!s_fine) {  // (the timeout is latched) no tile of this call runs
-    if (last && threadIdx.x < TS_COUNT) A.scal[threadIdx.x] = 0u;
-    return;
-  }
+  const bool fine = s_fine != 0;
   const U64x2 carry_a{s_pre[0], s_pre[1]}, carry_b{s_pre[2], s_pre[3]};
   u64 empties = 0;
-  if (p < P) {
+  if (fine && p < P) {
     const u64 w = carry_a.a + ea.a, g_lo = A.E.pair_off[p];
     wire_off[p] = w;
     if (A.D.recv_off) A.D.recv_off[p] = g_lo;  // receive buffers sized by the record counts
@@ -267,7 +267,7 @@ __global__ void __launch_bounds__(kSetupT)
     }
   }
   __syncthreads();
-  if (!abort) {
+  if (fine && !abort) {
     const u64 left = P - (u64)block * kSetupT;
     const u32 np = (u32)(left < (u64)kSetupT ? left : (u64)kSetupT), p0 = block * kSetupT;
     fill_map(A.item_pair, carry_b.a & 0xFFFFFFFFull, (u32)tb.a, item_cap, first[0], np, p0);
@@ -276,17 +276,34 @@ __global__ void __launch_bounds__(kSetupT)
     const u64 n = warp_sum(empties);
     if ((threadIdx.x & 31) == 0 && n) atomicAdd(&A.E.stats->wire_bytes, n * kHdrBytes);
   }
-  if (last && threadIdx.x == 0) {
+  if (block != gridDim.x - 1) return;
+  // the words of the blocks between the first, which never waits, and this one:
+  // a block that gave up has let the blocks after it go on
+  bool gone = !fine;
+  const u32 between = gridDim.x > 2 ? gridDim.x - 2 : 0;
+  for (u32 i = threadIdx.x; i < 4 * between; i += kSetupT) {
+    const u64* word = A.setup_state + (u64)(i / between) * gridDim.x + 1 + i % between;
+    LbWait wait{A.limit_ns};
+    u64 state;
+    while ((state = lb_get(word) >> kLbShift) < kLbSum && !wait.over(A.E.st)) {
+    }
+    gone |= state != kLbSum;
+  }
+  const bool late = __syncthreads_or(gone) != 0;
+  if (threadIdx.x == 0) {
     const u32 ep = *epoch + 1u;
     *epoch = ep == 0u ? 1u : ep;
+    for (int i = 0; i < TS_COUNT; ++i) A.scal[i] = 0u;
+    if (late) return;  // (the timeout is latched) no tile of this call runs
     const U64x2 all_a = carry_a + ta, all_b = carry_b + tb;
+    const u64 slabs = all_a.a, units = all_a.b, bigs = all_b.b;
     const u64 n_items = all_b.a & 0xFFFFFFFFull, n_small = all_b.a >> 32;
-    wire_off[P] = all_a.a;
+    wire_off[P] = slabs;
     if (A.D.recv_off) A.D.recv_off[P] = E;
     bool none = abort;
-    if (all_a.a > wire_cap) {
+    if (slabs > wire_cap) {
       latch(A.E.st, TERA_ECAPACITY);
-      need(A.E.st, all_a.a);
+      need(A.E.st, slabs);
       none = true;
     }
     if (big > rec_cap) {
@@ -297,16 +314,16 @@ __global__ void __launch_bounds__(kSetupT)
       latch(A.E.st, TERA_ECAPACITY);
       need(A.E.st, E + P);
     }
-    if (all_a.b > unit_cap || n_items > item_cap || all_b.b > big_cap) {
+    if (units > unit_cap || n_items > item_cap || bigs > big_cap) {
       latch(A.E.st, TERA_ECAPACITY);  // cannot happen: the lists are sized for it
       none = true;
     }
-    A.scal[TS_UNITS] = none ? 0u : (u32)all_a.b;
-    A.scal[TS_ITEMS] = none ? 0u : (u32)n_items;
-    A.scal[TS_SMALL] = none ? 0u : (u32)n_small;
     A.scal[TS_SHIFT] = shift;
-    A.scal[TS_BIG] = none ? 0u : (u32)all_b.b;
-    for (int i = TS_TICKET_MATCH; i < TS_COUNT; ++i) A.scal[i] = 0u;
+    if (none) return;
+    A.scal[TS_UNITS] = (u32)units;
+    A.scal[TS_ITEMS] = (u32)n_items;
+    A.scal[TS_SMALL] = (u32)n_small;
+    A.scal[TS_BIG] = (u32)bigs;
   }
 }
 
@@ -799,8 +816,8 @@ __device__ __forceinline__ void big_lookup(const TileArgs& A, const TilePair& x,
 
 // The big pairs' items, claimed in order: a pair's message tiles (indexed when
 // its ids do not ascend), then its slot tiles, which wait until the tiles
-// before them are indexed (claimed earlier, so by running blocks; at most a
-// second, then TERA_ETIMEOUT and no match).  The taken records are marked; the
+// before them are indexed (claimed earlier, so by running blocks; at most the
+// context's limit, then TERA_ETIMEOUT and no match).  The taken records are marked; the
 // block that finishes a pair's last tile lists its new records.
 __global__ void __launch_bounds__(kT, kPerSm) codec_bigmatch_kernel(TileArgs A) {
   chain_begin();
@@ -846,7 +863,7 @@ __global__ void __launch_bounds__(kT, kPerSm) codec_bigmatch_kernel(TileArgs A) 
     } else {
       if (threadIdx.x == 0) {
         s_span[0] = 1u;
-        LbWait wait;
+        LbWait wait{A.limit_ns};
         u32 v;
         for (;;) {
           asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(A.built + p) : "memory");
@@ -1579,6 +1596,7 @@ tera_status launch_tiles(tera_ctx* ctx, const EncArgs& E, const DecArgs& D, bool
   const unsigned setup = (unsigned)(P == 0 ? 1 : (P + kSetupT - 1) / kSetupT);
   const unsigned egrid = (unsigned)(ctx->num_sms * kEncPerSm), dgrid = (unsigned)(ctx->num_sms * kDecPerSm);
   A.setup_ticket = reinterpret_cast<u32*>(ctx->t_part + 4 * (u64)setup);
+  A.limit_ns = ctx->wait_ns;
   prof_begin(ctx, s);
   launch_chained(tiles_setup_kernel, setup, kSetupT, 0, s, A, mode, const_cast<u64*>(E.wire_off), wire_cap,
                                                ctx->cap_records, recv_cap, ctx->t_units,

@@ -43,7 +43,7 @@ tera_status alloc_dev(T*& p, size_t count) {
 // iteration's chain each time, where one is 4.
 __global__ void __launch_bounds__(kScanThreads)
     scan_kernel(const u32* __restrict__ in, u64 n, u64* __restrict__ out64,
-                u32* __restrict__ out32, u64* __restrict__ state, DevStatus* st) {
+                u32* __restrict__ out32, u64* __restrict__ state, u64 limit_ns, DevStatus* st) {
   chain_begin();
   __shared__ u64 sm[33];
   __shared__ u64 s_pre;
@@ -69,7 +69,7 @@ __global__ void __launch_bounds__(kScanThreads)
   if (gridDim.x > 1) {
     if (threadIdx.x < 32) {
       u64 pre;
-      const bool fine = lb_warp_sum(state, tile, tot, st, &pre);
+      const bool fine = lb_warp_sum(state, tile, tot, st, limit_ns, &pre);
       if (threadIdx.x == 0) {
         s_pre = pre;
         s_fine = fine;
@@ -215,7 +215,7 @@ tera_status scan_u32(tera_ctx* ctx, const u32* in, u64* out64, u32* out32, u64 n
   if (chunks > 1) cudaMemsetAsync(ctx->scan_part, 0, sizeof(u64) * (chunks + 1), s);
   prof_begin(ctx, s);
   launch_chained(scan_kernel, (unsigned)chunks, kScanThreads, 0, s, in, n, out64, out32, ctx->scan_part,
-                                                        ctx->d_status);
+                 ctx->wait_ns, ctx->d_status);
   return check_launch(ctx, "scan_kernel", s);
 }
 
@@ -651,6 +651,7 @@ tera_status tera_ctx_create(tera_ctx** out, const tera_grid* grid, int device, u
   memset(c, 0, sizeof(*c));
   c->device = device;
   c->class_id = class_id;
+  c->wait_ns = 1000000000ull;
   c->grid = *grid;
   c->n_boxes = (uint32_t)grid->n[0] * (uint32_t)grid->n[1] * (uint32_t)grid->n[2];
   c->n_pairs = (uint64_t)c->n_boxes * 27u;
@@ -794,6 +795,12 @@ tera_status tera_ctx_reserve(tera_ctx* ctx, int64_t max_agents, uint64_t max_rec
   st = ensure_records(ctx, max_records, 0);
   if (st != TERA_OK) return st;
   return ensure_units(ctx, 2 * (max_records / kCodecTile) + 4 * ctx->n_pairs + 16, 0);
+}
+
+tera_status tera_ctx_wait_limit(tera_ctx* ctx, int64_t limit_us) {
+  if (!ctx || limit_us < 0 || limit_us > 60000000) return TERA_EINVAL;
+  ctx->wait_ns = 1000ull * (u64)limit_us;
+  return TERA_OK;
 }
 
 tera_status tera_ctx_status(tera_ctx* ctx, uint64_t* required_capacity, void* stream) {

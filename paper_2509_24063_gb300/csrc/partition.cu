@@ -365,7 +365,7 @@ __global__ void __launch_bounds__(kSortThreads)
                       u32* __restrict__ vals_out, u32* __restrict__ agents_out,
                       u32* __restrict__ dest, int last, const u64* __restrict__ total_ptr, u64 cap,
                       u32 pass, u32 shift, u32 radix, u64* __restrict__ head, u64 n_tiles,
-                      DevStatus* st) {
+                      u64 limit_ns, DevStatus* st) {
   chain_begin();
   constexpr int kWarps = kSortThreads / 32;
   constexpr int kRoundEntries = kSortRound;
@@ -476,7 +476,7 @@ __global__ void __launch_bounds__(kSortThreads)
     constexpr int kFlight = 8;
     u64 pre = 0;
     bool done = tile == 0;
-    LbWait wait;
+    LbWait wait{limit_ns};
     for (long long at = (long long)tile - 1; !done && !gone;) {
       u64 v[kFlight];
 #pragma unroll
@@ -626,11 +626,11 @@ tera_status radix_sort_entries(tera_ctx* ctx, const SortBufs& b, const u32* keys
     if (radix <= 128)
       launch_chained(rs_scatter_kernel<128>, grid, kSortThreads, smem, s, 
           kin, vin, ain, kout, vout, aout, last ? dest : nullptr, last ? 1 : 0, total_ptr, cap,
-          (u32)pass, shift, radix, b.hist, tiles, ctx->d_status);
+          (u32)pass, shift, radix, b.hist, tiles, ctx->wait_ns, ctx->d_status);
     else
       launch_chained(rs_scatter_kernel<kRadix>, grid, kSortThreads, smem, s, 
           kin, vin, ain, kout, vout, aout, last ? dest : nullptr, last ? 1 : 0, total_ptr, cap,
-          (u32)pass, shift, radix, b.hist, tiles, ctx->d_status);
+          (u32)pass, shift, radix, b.hist, tiles, ctx->wait_ns, ctx->d_status);
     if ((st = check_launch(ctx, "rs_scatter_kernel", s)) != TERA_OK) return st;
     kin = kout;
     vin = vout;

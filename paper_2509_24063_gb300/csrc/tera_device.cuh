@@ -198,11 +198,15 @@ __device__ __forceinline__ T block_excl_scan(T v, T* smem, T* total) {
 // predecessors' and publishes the inclusive sum: one 64-bit word per tile, the
 // state in its top two bits (zero: nothing yet), written and read whole.
 // Tiles are claimed in order and publish before they wait, so a tile only
-// waits for running blocks; a wait gives up after a second all the same.
+// waits for running blocks; a wait gives up after the context's limit all the
+// same.  A tile that gives up has published its own value, so tiles after it may
+// still find their sums: whoever reads what a chain's tiles write asks a flag
+// that every tile sets when it gives up, never the last tile alone.
+// (Decoupled look-back: D. Merrill and M. Garland, "Single-pass Parallel Prefix
+// Scan with Decoupled Look-back", NVIDIA technical report NVR-2016-002.)
 constexpr int kLbShift = 62;
 constexpr u64 kLbOwn = 1, kLbSum = 2, kLbGone = 3;
 constexpr u64 kLbMask = (1ull << kLbShift) - 1ull;
-constexpr u64 kLbLimitNs = 1000000000ull;
 
 __device__ __forceinline__ void lb_put(u64* s, u64 v, u64 state) {
   asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" : : "l"(s), "l"(v | (state << kLbShift))
@@ -218,16 +222,17 @@ __device__ __forceinline__ u64 lb_now() {
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
   return t;
 }
-// Counts polls of one wait; true when it has taken too long (TERA_ETIMEOUT and
-// the call's abort flag set).
+// Counts polls of one wait; true when it has taken longer than limit_ns (0: when
+// it has to wait at all; TERA_ETIMEOUT and the call's abort flag set).
 struct LbWait {
+  u64 limit_ns;
   u64 t0 = 0;
   u32 polls = 0;
   __device__ __forceinline__ bool over(DevStatus* st) {
-    if ((++polls & 63u) != 0u) return false;
+    if ((++polls & 63u) != 0u && limit_ns != 0) return false;
     const u64 now = lb_now();
     if (t0 == 0) t0 = now;
-    if (now - t0 <= kLbLimitNs && polls < (1u << 30)) return false;
+    if (limit_ns != 0 && now - t0 <= limit_ns && polls < (1u << 30)) return false;
     latch(st, TERA_ETIMEOUT);
     atomicExch(&st->abort, 1u);
     return true;
@@ -236,15 +241,15 @@ struct LbWait {
 
 // One warp: the sum of the tiles before `tile` of a chain whose tile i publishes
 // at state[i], this tile's value `own` published first.  False (the tile is
-// given up, and so is every tile after it) when the wait was cut short.
+// given up) when the wait, or one it depends on, was cut short.
 __device__ __forceinline__ bool lb_warp_sum(u64* state, u64 tile, u64 own, DevStatus* st,
-                                            u64* before) {
+                                            u64 limit_ns, u64* before) {
   const int lane = threadIdx.x & 31;
   u64 pre = 0;
   bool fine = true;
   if (tile > 0) {
     if (lane == 0) lb_put(state + tile, own, kLbOwn);
-    LbWait wait;
+    LbWait wait{limit_ns};
     for (long long at = (long long)tile - 1; fine; at -= 32) {
       const long long i = at - lane;
       u64 v;

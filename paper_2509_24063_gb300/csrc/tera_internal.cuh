@@ -54,6 +54,7 @@ struct tera_ctx {
   int num_sms;
   uint64_t launches;
   uint64_t iterations;
+  uint64_t wait_ns;  // limit of a device-side wait of the launches (tera_ctx_wait_limit)
 
   tera::GridTables* d_grid;
   tera::AxisBuckets* d_buckets;  // null when classification has no table
