@@ -207,7 +207,7 @@ __global__ void __launch_bounds__(kSetupT)
     const u64 own = c == 0 ? ta.a : (c == 1 ? ta.b : (c == 2 ? tb.a : tb.b));
     u64 pre = 0;
     if (gridDim.x > 1 && !lb_warp_sum(A.setup_state + (u64)c * gridDim.x, block, own, A.E.st, A.limit_ns,
-                                      &pre) &&
+                                      nullptr, &pre) &&
         (threadIdx.x & 31) == 0)
       s_fine = 0;
     if ((threadIdx.x & 31) == 0) s_pre[c] = pre;
@@ -283,7 +283,7 @@ __global__ void __launch_bounds__(kSetupT)
   const u32 between = gridDim.x > 2 ? gridDim.x - 2 : 0;
   for (u32 i = threadIdx.x; i < 4 * between; i += kSetupT) {
     const u64* word = A.setup_state + (u64)(i / between) * gridDim.x + 1 + i % between;
-    LbWait wait{A.limit_ns};
+    LbWait wait{A.limit_ns, nullptr};
     u64 state;
     while ((state = lb_get(word) >> kLbShift) < kLbSum && !wait.over(A.E.st)) {
     }
@@ -863,7 +863,7 @@ __global__ void __launch_bounds__(kT, kPerSm) codec_bigmatch_kernel(TileArgs A) 
     } else {
       if (threadIdx.x == 0) {
         s_span[0] = 1u;
-        LbWait wait{A.limit_ns};
+        LbWait wait{A.limit_ns, nullptr};
         u32 v;
         for (;;) {
           asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(A.built + p) : "memory");

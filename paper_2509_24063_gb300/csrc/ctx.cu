@@ -43,7 +43,8 @@ tera_status alloc_dev(T*& p, size_t count) {
 // iteration's chain each time, where one is 4.
 __global__ void __launch_bounds__(kScanThreads)
     scan_kernel(const u32* __restrict__ in, u64 n, u64* __restrict__ out64,
-                u32* __restrict__ out32, u64* __restrict__ state, u64 limit_ns, DevStatus* st) {
+                u32* __restrict__ out32, u64* __restrict__ state, u64 limit_ns, DevStatus* st,
+                u32* flag) {
   chain_begin();
   __shared__ u64 sm[33];
   __shared__ u64 s_pre;
@@ -69,14 +70,14 @@ __global__ void __launch_bounds__(kScanThreads)
   if (gridDim.x > 1) {
     if (threadIdx.x < 32) {
       u64 pre;
-      const bool fine = lb_warp_sum(state, tile, tot, st, limit_ns, &pre);
+      const bool fine = lb_warp_sum(state, tile, tot, st, limit_ns, flag, &pre);
       if (threadIdx.x == 0) {
         s_pre = pre;
         s_fine = fine;
       }
     }
     __syncthreads();
-    if (!s_fine) return;  // the abort flag is set: nothing reads the result
+    if (!s_fine) return;  // the flag is set: the launches after this one read nothing of it
     run += s_pre;
   }
 #pragma unroll
@@ -206,8 +207,8 @@ static tera_status ensure_scan_part(tera_ctx* ctx, u64 n) {
   return TERA_OK;
 }
 
-tera_status scan_u32(tera_ctx* ctx, const u32* in, u64* out64, u32* out32, u64 n,
-                     cudaStream_t s) {
+tera_status scan_u32(tera_ctx* ctx, const u32* in, u64* out64, u32* out32, u64 n, cudaStream_t s,
+                     u32* flag) {
   tera_status st = ensure_scan_part(ctx, n);
   if (st != TERA_OK) return st;
   u64 chunks = (n + kScanChunk - 1) / kScanChunk;
@@ -215,7 +216,7 @@ tera_status scan_u32(tera_ctx* ctx, const u32* in, u64* out64, u32* out32, u64 n
   if (chunks > 1) cudaMemsetAsync(ctx->scan_part, 0, sizeof(u64) * (chunks + 1), s);
   prof_begin(ctx, s);
   launch_chained(scan_kernel, (unsigned)chunks, kScanThreads, 0, s, in, n, out64, out32, ctx->scan_part,
-                 ctx->wait_ns, ctx->d_status);
+                 ctx->wait_ns, ctx->d_status, flag ? flag : &ctx->d_status->abort);
   return check_launch(ctx, "scan_kernel", s);
 }
 

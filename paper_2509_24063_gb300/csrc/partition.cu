@@ -476,7 +476,7 @@ __global__ void __launch_bounds__(kSortThreads)
     constexpr int kFlight = 8;
     u64 pre = 0;
     bool done = tile == 0;
-    LbWait wait{limit_ns};
+    LbWait wait{limit_ns, &st->abort};
     for (long long at = (long long)tile - 1; !done && !gone;) {
       u64 v[kFlight];
 #pragma unroll

@@ -16,14 +16,19 @@ namespace {
 
 constexpr int kDense = 11;     // dense sample: 8 features + 3 targets
 
-__global__ void sample_flags_kernel(const float* __restrict__ samples, u64 n, u32* __restrict__ flags) {
+// late[0]: a wait of the scan was given up (cleared here); late[1]: valid samples.
+__global__ void sample_flags_kernel(const float* __restrict__ samples, u64 n, u32* __restrict__ flags,
+                                    u32* __restrict__ late) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) *late = 0;
   for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (u64)gridDim.x * blockDim.x)
     flags[i] = samples[i * kSampleFloats + 11] != 0.0f ? 1u : 0u;
 }
 
 __global__ void sample_compact_kernel(const float* __restrict__ samples, u64 n,
                                       const u32* __restrict__ flags, const u32* __restrict__ pos,
-                                      float* __restrict__ dense) {
+                                      float* __restrict__ dense, u32* late) {
+  if (*late) return;  // positions are missing
+  if (blockIdx.x == 0 && threadIdx.x == 0) late[1] = pos[n];
   for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (u64)gridDim.x * blockDim.x) {
     if (!flags[i]) continue;
     const float* s = samples + i * kSampleFloats;
@@ -504,11 +509,11 @@ __global__ void __launch_bounds__(kTrainThreads, kTrainPerSm) mlp_steps_kernel(T
 }
 
 // Scratch layout in ctx->mlp_scratch (floats): partial [blocks * kGradStride] |
-// grad [kGradStride] | ssq [blocks rounded up to 4] | barrier [4] (u32) | dense
+// grad [kGradStride] | ssq [blocks rounded up to 4] | barrier, late [2], spare (u32) | dense
 // [n * 11] | flags [n+1] (u32) | pos [n+1] (u32)
 struct TrainScratch {
   float *partial, *grad, *ssq, *dense;
-  u32 *barrier, *flags, *pos;
+  u32 *barrier, *late, *flags, *pos;
 };
 
 tera_status prepare(tera_ctx* ctx, u64 n, TrainScratch* t) {
@@ -531,28 +536,30 @@ tera_status prepare(tera_ctx* ctx, u64 n, TrainScratch* t) {
   t->grad = b + blocks * kGradStride;
   t->ssq = t->grad + kGradStride;
   t->barrier = reinterpret_cast<u32*>(t->ssq + ((blocks + 3) & ~3ull));
+  t->late = t->barrier + 1;
   t->dense = reinterpret_cast<float*>(t->barrier + 4);
   t->flags = reinterpret_cast<u32*>(t->dense + n * kDense);
   t->pos = t->flags + (n + 1);
   return TERA_OK;
 }
 
-tera_status compact(tera_ctx* ctx, const float* samples, u64 n, float* dense, u32* flags,
-                    u32* pos, u64* nv, cudaStream_t s) {
+tera_status compact(tera_ctx* ctx, const float* samples, u64 n, const TrainScratch& t, u64* nv,
+                    cudaStream_t s) {
   const unsigned g = (unsigned)((n + 255) / 256 < 65535 ? (n + 255) / 256 + 1 : 65535);
   prof_begin(ctx, s);
-  sample_flags_kernel<<<g, 256, 0, s>>>(samples, n, flags);
+  sample_flags_kernel<<<g, 256, 0, s>>>(samples, n, t.flags, t.late);
   tera_status st = check_launch(ctx, "sample_flags_kernel", s);
   if (st != TERA_OK) return st;
-  if ((st = scan_u32(ctx, flags, nullptr, pos, n, s)) != TERA_OK) return st;
+  if ((st = scan_u32(ctx, t.flags, nullptr, t.pos, n, s, t.late)) != TERA_OK) return st;
   prof_begin(ctx, s);
-  sample_compact_kernel<<<g, 256, 0, s>>>(samples, n, flags, pos, dense);
+  sample_compact_kernel<<<g, 256, 0, s>>>(samples, n, t.flags, t.pos, t.dense, t.late);
   if ((st = check_launch(ctx, "sample_compact_kernel", s)) != TERA_OK) return st;
-  u32 h = 0;
-  if (cudaMemcpyAsync(&h, pos + n, sizeof(u32), cudaMemcpyDeviceToHost, s) != cudaSuccess)
+  u32 h[2] = {0, 0};
+  if (cudaMemcpyAsync(h, t.late, sizeof(h), cudaMemcpyDeviceToHost, s) != cudaSuccess)
     return TERA_ECUDA;
   if (cudaStreamSynchronize(s) != cudaSuccess) return TERA_ECUDA;
-  *nv = h;
+  if (h[0]) return TERA_ETIMEOUT;
+  *nv = h[1];
   return TERA_OK;
 }
 
@@ -614,7 +621,7 @@ extern "C" tera_status tera_mlp_grad(tera_ctx* ctx, const float* samples, uint64
   tera_status st = prepare(ctx, n, &t);
   if (st != TERA_OK) return st;
   u64 nv = 0;
-  if ((st = compact(ctx, samples, n, t.dense, t.flags, t.pos, &nv, s)) != TERA_OK) return st;
+  if ((st = compact(ctx, samples, n, t, &nv, s)) != TERA_OK) return st;
   if (n_valid) *n_valid = nv;
   if (nv == 0) return TERA_EINVAL;
   return train_steps(ctx, t, nv, nv, 1, params, nullptr, grad, 0.0f, 0.0f, s);
@@ -633,7 +640,7 @@ extern "C" tera_status tera_mlp_train(tera_ctx* ctx, const float* samples, uint6
   tera_status st = prepare(ctx, n, &t);
   if (st != TERA_OK) return st;
   u64 nv = 0;
-  if ((st = compact(ctx, samples, n, t.dense, t.flags, t.pos, &nv, s)) != TERA_OK) return st;
+  if ((st = compact(ctx, samples, n, t, &nv, s)) != TERA_OK) return st;
   if (n_valid) *n_valid = nv;
   if (nv == 0) return TERA_EINVAL;
   if (steps == 0) return TERA_OK;

@@ -223,9 +223,11 @@ __device__ __forceinline__ u64 lb_now() {
   return t;
 }
 // Counts polls of one wait; true when it has taken longer than limit_ns (0: when
-// it has to wait at all; TERA_ETIMEOUT and the call's abort flag set).
+// it has to wait at all; TERA_ETIMEOUT, and *flag set where there is one: the
+// later launches of the call look at it).
 struct LbWait {
   u64 limit_ns;
+  u32* flag;
   u64 t0 = 0;
   u32 polls = 0;
   __device__ __forceinline__ bool over(DevStatus* st) {
@@ -234,7 +236,7 @@ struct LbWait {
     if (t0 == 0) t0 = now;
     if (limit_ns != 0 && now - t0 <= limit_ns && polls < (1u << 30)) return false;
     latch(st, TERA_ETIMEOUT);
-    atomicExch(&st->abort, 1u);
+    if (flag) atomicExch(flag, 1u);
     return true;
   }
 };
@@ -243,13 +245,13 @@ struct LbWait {
 // at state[i], this tile's value `own` published first.  False (the tile is
 // given up) when the wait, or one it depends on, was cut short.
 __device__ __forceinline__ bool lb_warp_sum(u64* state, u64 tile, u64 own, DevStatus* st,
-                                            u64 limit_ns, u64* before) {
+                                            u64 limit_ns, u32* flag, u64* before) {
   const int lane = threadIdx.x & 31;
   u64 pre = 0;
   bool fine = true;
   if (tile > 0) {
     if (lane == 0) lb_put(state + tile, own, kLbOwn);
-    LbWait wait{limit_ns};
+    LbWait wait{limit_ns, flag};
     for (long long at = (long long)tile - 1; fine; at -= 32) {
       const long long i = at - lane;
       u64 v;

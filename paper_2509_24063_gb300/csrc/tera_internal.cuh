@@ -222,8 +222,11 @@ tera_status check_launch(tera_ctx* ctx, const char* name, cudaStream_t s);
 tera_status ensure_agents(tera_ctx* ctx, int64_t n, cudaStream_t s);
 tera_status ensure_records(tera_ctx* ctx, uint64_t cap, cudaStream_t s);
 tera_status ensure_units(tera_ctx* ctx, uint64_t cap, cudaStream_t s);
-// Exclusive scan of n u32 values into n+1 outputs (total last), any n.
-tera_status scan_u32(tera_ctx* ctx, const u32* in, u64* out64, u32* out32, u64 n, cudaStream_t s);
+// Exclusive scan of n u32 values into n+1 outputs (total last), any n.  *flag (on
+// the device; null: the status word's abort flag) is set when a wait of it was
+// given up: outputs are then missing, and no later launch may use any.
+tera_status scan_u32(tera_ctx* ctx, const u32* in, u64* out64, u32* out32, u64 n, cudaStream_t s,
+                     u32* flag = nullptr);
 int grid_for(tera_ctx* ctx, int blocks_per_sm);
 // unit_pair[u] = p0 + k for every unit u of range pair k (skipped when
 // units_total[1] flags an aborted call).

@@ -83,3 +83,36 @@ def test_setup_given_up_writes_no_message(tera, path):
     for got, want in ((ex.ref[1], res["ref_next"]), (ex.recv[1], res["recv"])):
         assert got[:units * 64].cpu().numpy().tobytes() == want[:units * 64].tobytes()
     ctx.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("grad", [False, True])
+def test_training_given_up_changes_nothing(tera, grad):
+    # 1 M samples: 256 chunks of the scan that finds the valid ones' places
+    g = torch.Generator(device="cuda")
+    g.manual_seed(3)
+    samples = torch.randn(1 << 20, 12, generator=g, device="cuda")
+    samples[:, 11] = (samples[:, 11] > 0).float()
+    samples = samples.reshape(-1)
+    params = 0.05 * torch.randn(4931, generator=g, device="cuda")
+    ctx = tera.Context((0.0,) * 3, (100.0, 100.0, 50.0), (2, 2, 1), 30.0)
+    out = torch.empty_like(params)
+
+    def call():
+        try:
+            ctx.mlp_grad(samples, params, out) if grad else ctx.mlp_train(samples, out, 2, 512, 0.1)
+        except tera.TeraError as e:
+            assert e.status == tera.ETIMEOUT
+            assert bool((out == params).all())
+
+    until_given_up(tera, ctx, call, lambda: out.copy_(params))
+    fresh = tera.Context((0.0,) * 3, (100.0, 100.0, 50.0), (2, 2, 1), 30.0)
+    results = []
+    for c in (ctx, fresh):
+        out.copy_(params)
+        n = c.mlp_grad(samples, params, out) if grad else c.mlp_train(samples, out, 2, 512, 0.1)
+        assert c.status(raise_on_error=False)[0] == tera.OK
+        results.append((n, out.clone()))
+    assert results[0][0] == results[1][0] and torch.equal(results[0][1], results[1][1])
+    ctx.close()
+    fresh.close()
