@@ -128,9 +128,9 @@ __device__ __forceinline__ ulonglong2 load_pair(const u64* p) {
 template <int R>
 __global__ void __launch_bounds__(kClassifyThreads)
     pack_runs_kernel(SoaPtrs soa, u64 n, const int* __restrict__ owner,
-                     const u32* __restrict__ mask, const u64* __restrict__ run_base, u64 n_runs,
-                     const u32* __restrict__ ent_dest, const u64* __restrict__ pair_off, u64 P,
-                     uint8_t* __restrict__ arena, u64 arena_units, u32 class_id, DevStatus* st,
+                     const u32* __restrict__ mask, const u64* __restrict__ run_base,
+                     const u64* __restrict__ packable, const u32* __restrict__ ent_dest,
+                     const u64* __restrict__ pair_off, u64 P, uint8_t* __restrict__ arena, u64 arena_units, u32 class_id, DevStatus* st,
                      u64* __restrict__ rec_ids) {
   chain_begin();
   const u64 E = pair_off[P];
@@ -147,8 +147,8 @@ __global__ void __launch_bounds__(kClassifyThreads)
     const u64 m = pair_off[p + 1] - pair_off[p];
     write_taio_header(arena + (pair_off[p] + p) * kRecBytes, class_id, (u32)p, m);
   }
-  // a partition that overflowed its capacity left no record indices
-  if (run_base[n_runs] != E) return;
+  // a partition that overflowed its capacity, or gave a wait up, left no record indices
+  if (*packable != E) return;
   const int lane = threadIdx.x & 31;
   const u64 tile0 = (u64)blockIdx.x * (2 * kClassifyThreads * R);
   for (int k = 0; k < R; ++k) {
@@ -245,10 +245,9 @@ static tera_status pack_impl(tera_ctx* ctx, const tera_soa* soa, const tera_part
     const int rounds = agent_rounds(ctx, n);
     const u64 per = 2ull * kClassifyThreads * rounds;
     const u64 blocks = n == 0 ? 1 : (n + per - 1) / per;
-    const u64 runs = n == 0 ? 1 : (n + kRunAgents - 1) / kRunAgents;
     prof_begin(ctx, s);
     launch_chained(rounds == 1 ? pack_runs_kernel<1> : pack_runs_kernel<kAgentRounds>, (unsigned)blocks, kClassifyThreads, 0, s, 
-        p, n, part->owner, part->mask, ctx->tile_base, runs, ctx->ent_dest,
+        p, n, part->owner, part->mask, ctx->tile_base, ctx->d_total, ctx->ent_dest,
         reinterpret_cast<const u64*>(part->pair_off), ctx->n_pairs, rec_arena, arena_units,
         ctx->class_id, ctx->d_status, reinterpret_cast<u64*>(rec_ids));
     return check_launch(ctx, "pack_runs_kernel", s);

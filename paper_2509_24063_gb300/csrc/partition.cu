@@ -539,10 +539,15 @@ __device__ __forceinline__ void warp_probe(bool less, u64 len, u64* lo, u64* hi)
 __global__ void __launch_bounds__(256)
     pair_off_kernel(const u32* __restrict__ sorted_keys, const u64* __restrict__ total_ptr, u64 cap,
                     u64 n_pairs, u64* __restrict__ pair_off, u64* __restrict__ pair_count,
-                    DevStats* stats, const DevStatus* st) {
+                    u64* __restrict__ packable, DevStats* stats, const DevStatus* st) {
   chain_begin();
   const u64 E = live_entries(total_ptr, cap, st);
-  if (blockIdx.x == 0 && threadIdx.x == 0) stats->records += E;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    stats->records += E;
+    // what pack_runs_kernel compares with the pairs' total: no total for lists
+    // that are not there (a scan that gave up leaves run_base as it was)
+    *packable = *reinterpret_cast<const volatile u32*>(&st->abort) ? ~0ull : E;
+  }
   const u32 lane = threadIdx.x & 31;
   const u64 warps = (u64)gridDim.x * (blockDim.x / 32);
   for (u64 p = (u64)blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5); p <= n_pairs; p += warps) {
@@ -715,6 +720,6 @@ extern "C" tera_status tera_partition(tera_ctx* ctx, const tera_soa* soa, tera_p
   prof_begin(ctx, s);
   launch_chained(pair_off_kernel, (unsigned)(P / 8 + 1), 256, 0, s, 
       sorted, total_ptr, cap, P, reinterpret_cast<u64*>(out->pair_off),
-      reinterpret_cast<u64*>(out->pair_count), ctx->d_stats, ctx->d_status);
+      reinterpret_cast<u64*>(out->pair_count), ctx->d_total, ctx->d_stats, ctx->d_status);
   return check_launch(ctx, "pair_off_kernel", s);
 }

@@ -84,7 +84,7 @@ struct tera_ctx {
   tera::u64* rs_hist;      // [sort_scratch] digit counts and look-back states of the sort
   tera::u64* scan_part;     // partials of the generic scan
   uint64_t scan_part_cap;
-  tera::u64* d_total;       // [4] scalars: total records, ...
+  tera::u64* d_total;       // [8] [0]: records of the last partition's lists, all ones: no lists
 
   // per-pair hash segments + codec scratch
   tera::U64x2* seg;      // [2 cap_records + 2 P] hash entries {tag, id}

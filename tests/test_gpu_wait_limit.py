@@ -116,3 +116,39 @@ def test_training_given_up_changes_nothing(tera, grad):
     assert results[0][0] == results[1][0] and torch.equal(results[0][1], results[1][1])
     ctx.close()
     fresh.close()
+
+
+@pytest.mark.gpu
+def test_partition_given_up_leaves_every_pair_empty(tera):
+    # 2 M agents: eight chunks of the scan over the runs, and a sort of many tiles
+    n = 1 << 21
+    g = torch.Generator(device="cuda")
+    g.manual_seed(9)
+    st = {f: torch.rand(n, generator=g, device="cuda", dtype=torch.float64) * 400.0
+          for f in ("x", "y", "z", "diameter", "volume", "adherence", "density")}
+    st["id"] = torch.arange(n, device="cuda")
+    space = ((0.0,) * 3, (400.0,) * 3, (4, 4, 4), 10.0)
+    ctx = tera.Context(*space)
+    cap = n
+    part = tera.PartitionBuffers.allocate(n, ctx.n_pairs, cap, "cuda")
+    rec = torch.empty((cap + ctx.n_pairs) * 64, dtype=torch.uint8, device="cuda")
+
+    def call():
+        ctx.partition(st, part)
+        ctx.pack(st, part, rec)
+
+    until_given_up(tera, ctx, call, lambda: rec.fill_(FILL))
+    assert not bool(part.pair_off.any()) and not bool(part.pair_count.any())
+    assert bool((rec[ctx.n_pairs * 64:] == FILL).all())  # headers alone
+    fresh = tera.Context(*space)
+    results = []
+    for c in (ctx, fresh):
+        rec.fill_(FILL)
+        c.partition(st, part)
+        c.pack(st, part, rec)
+        assert c.status(raise_on_error=False)[0] == tera.OK
+        results.append((part.pair_off.clone(), rec.clone()))
+    for a, b in zip(*results):
+        assert torch.equal(a, b)
+    ctx.close()
+    fresh.close()
