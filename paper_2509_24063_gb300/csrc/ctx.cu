@@ -34,6 +34,14 @@ tera_status alloc_dev(T*& p, size_t count) {
   return TERA_OK;
 }
 
+// The device has done everything the host asked for.  Work on the default stream
+// (a cudaMemset, the last part of a cudaMemcpy from pageable memory) is not
+// waited for by a caller's non-blocking stream, so what clears or fills new
+// scratch ends with this.
+tera_status settled() {
+  return cudaDeviceSynchronize() == cudaSuccess ? TERA_OK : TERA_ECUDA;
+}
+
 // ---- generic exclusive scan of u32 values ----
 //
 // One launch: a block scans kScanChunk values and finds the sum before them by
@@ -256,7 +264,7 @@ tera_status ensure_records(tera_ctx* ctx, uint64_t cap, cudaStream_t s) {
   cudaMemset(ctx->seg, 0, sizeof(U64x2) * (2 * c + 2 * ctx->n_pairs));
   cudaMemset(ctx->matched, 0, sizeof(u32) * c);
   ctx->cap_records = c;
-  return TERA_OK;
+  return settled();
 }
 
 tera_status ensure_units(tera_ctx* ctx, uint64_t cap, cudaStream_t s) {
@@ -299,7 +307,7 @@ tera_status ensure_batched(tera_ctx* ctx) {
   if ((st = alloc_dev(ctx->b_tsum, tsum)) != TERA_OK) return st;
   ctx->b_items_cap = items;
   ctx->b_tsum_cap = tsum;
-  return TERA_OK;
+  return settled();
 }
 
 // One allocation holds every list, so that a first call pays for one.
@@ -340,7 +348,7 @@ tera_status ensure_tiles(tera_ctx* ctx) {
   lay();
   cudaMemset(ctx->t_part, 0, sizeof(u64) * (4 * (P / 1024 + 1) + 1));
   ctx->t_cap = cap;
-  return TERA_OK;
+  return settled();
 }
 
 bool encode_tiles_ready(tera_ctx* ctx, cudaStream_t s) {
@@ -473,7 +481,7 @@ tera_status ensure_pred(tera_ctx* ctx) {
   if ((st = alloc_dev(ctx->unit_res, ctx->cap_units)) != TERA_OK) return st;
   ctx->pred_cap = cap;
   ctx->unit_res_cap = ctx->cap_units;
-  return TERA_OK;
+  return settled();
 }
 
 }  // namespace tera
