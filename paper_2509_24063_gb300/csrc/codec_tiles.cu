@@ -16,7 +16,8 @@
 //           records, and the payload, packed, into the tile's own part of the
 //           receive buffer (a tile's payload never exceeds its records)
 //   wire    one tile: its payload's place in the message, from the counts of
-//           the tiles before it, and the payload copied there
+//           the tiles before it, and the payload copied there; the headers of
+//           the pairs without entries
 //   decode  one tile of entries from the wire and the receiver's reference
 //
 // Only the payload's place depends on other tiles' contents, and the payload
@@ -79,9 +80,9 @@ struct __align__(16) TilePair {
 };
 static_assert(sizeof(TilePair) == 64, "one line per pair");
 
-// Device scalars of one call.
+// Device scalars of one call (TS_OK: the setup accepted it).
 enum { TS_UNITS = 0, TS_ITEMS, TS_BIG, TS_SMALL, TS_SHIFT, TS_TICKET_MATCH, TS_TICKET_BIG,
-       TS_COUNT };
+       TS_OK, TS_COUNT };
 
 struct TileArgs {
   EncArgs E;
@@ -168,12 +169,12 @@ __device__ __forceinline__ void fill_map(u32* __restrict__ out, u64 lo, u32 n, u
 // One launch, kSetupT pairs a block: the pairs' facts, then their places in the
 // slabs and lists by a block scan and a look-back over the blocks (four chains:
 // slab bytes, tiles, match items and warp pairs in the halves of a word, items
-// of big pairs).  Pairs without entries on either side are finished here.  The
-// last block checks the capacities and writes the lists' lengths, all zero when a
-// capacity is exceeded or any block's wait was cut short (its pairs' lines and
-// list entries are then not written, and no launch may index by them); until
-// then a block knows all but the slabs' total, so it writes to the wire only
-// inside its capacity.
+// of big pairs).  The last block checks the capacities and writes the lists'
+// lengths, all zero when a capacity is exceeded or any block's wait was cut short
+// (its pairs' lines and list entries are then not written, and no launch may
+// index by them).  Nothing of the caller's but the offsets is written here: the
+// verdict is known at the end only, and a refused call leaves messages,
+// references, reset marks and totals as they were.
 __global__ void __launch_bounds__(kSetupT)
     tiles_setup_kernel(TileArgs A, int mode, u64* __restrict__ wire_off, u64 wire_cap, u64 rec_cap,
                        u64 recv_cap, u64 unit_cap, u64 item_cap, u64 big_cap, u32* epoch) {
@@ -215,7 +216,6 @@ __global__ void __launch_bounds__(kSetupT)
   __syncthreads();
   const bool fine = s_fine != 0;
   const U64x2 carry_a{s_pre[0], s_pre[1]}, carry_b{s_pre[2], s_pre[3]};
-  u64 empties = 0;
   if (fine && p < P) {
     const u64 w = carry_a.a + ea.a, g_lo = A.E.pair_off[p];
     wire_off[p] = w;
@@ -243,27 +243,6 @@ __global__ void __launch_bounds__(kSetupT)
       A.built[p] = 0;
       A.unsorted[p] = 0;
       A.unit_first[p] = x.unit0;
-      if (f.units == 0 && w + kHdrBytes <= wire_cap) {  // no slots, no records: headers alone
-        ulonglong2* h = reinterpret_cast<ulonglong2*>(A.E.wire + w);
-        h[0] = make_ulonglong2((u64)kWireMagic | ((u64)kVersion << 32) | ((u64)kRecBytes << 48),
-                               (u64)A.E.class_id | ((u64)x.mode << 32));
-        h[1] = make_ulonglong2(0, 0);
-        h[2] = make_ulonglong2(0, 0);
-        h[3] = make_ulonglong2(p, kHdrBytes);
-        A.E.wire_len[p] = kHdrBytes;
-        write_taio_header(A.E.ref_next + (g_lo + p) * kRecBytes, A.E.class_id, (u32)p, 0);
-        if (A.D.recv)
-          write_taio_header(A.D.recv + (g_lo + p) * kRecBytes, A.D.class_id, (u32)p, 0);
-        A.E.reset[p] = 0;
-        empties = 1;
-        if (x.mode != TERA_MODE_RAW && A.D.ref) {  // as the decode's header check
-          const u64* rh =
-              reinterpret_cast<const u64*>(A.D.ref + (A.D.ref_off[p] + p) * kRecBytes);
-          if ((u32)rh[0] != kTaioMagic || (u32)rh[1] != A.D.class_id ||
-              (u32)(rh[1] >> 32) != (u32)p || rh[2] != 0)
-            latch(A.D.st, TERA_ECORRUPT);
-        }
-      }
     }
   }
   __syncthreads();
@@ -273,8 +252,6 @@ __global__ void __launch_bounds__(kSetupT)
     fill_map(A.item_pair, carry_b.a & 0xFFFFFFFFull, (u32)tb.a, item_cap, first[0], np, p0);
     fill_map(A.small_pair, carry_b.a >> 32, (u32)(tb.a >> 32), P, first[1], np, p0);
     fill_map(A.big_pair, carry_b.b, (u32)tb.b, big_cap, first[2], np, p0);
-    const u64 n = warp_sum(empties);
-    if ((threadIdx.x & 31) == 0 && n) atomicAdd(&A.E.stats->wire_bytes, n * kHdrBytes);
   }
   if (block != gridDim.x - 1) return;
   // the words of the blocks between the first, which never waits, and this one:
@@ -320,6 +297,7 @@ __global__ void __launch_bounds__(kSetupT)
     }
     A.scal[TS_SHIFT] = shift;
     if (none) return;
+    A.scal[TS_OK] = 1u;
     A.scal[TS_UNITS] = (u32)units;
     A.scal[TS_ITEMS] = (u32)n_items;
     A.scal[TS_SMALL] = (u32)n_small;
@@ -1333,6 +1311,38 @@ __device__ __forceinline__ void finish_message(const TileArgs& A, const Tile& t,
   if (body + lane < msg) w8[body + lane] = 0;  // zero padding (< 16 bytes)
 }
 
+// The pairs without entries on either side, a thread each: headers alone.  The
+// launch's last threads take them (on small iterations they have no tile).
+__device__ __forceinline__ void finish_empty(const TileArgs& A) {
+  const u64 threads = (u64)gridDim.x * kT;
+  u64 n = 0;
+  for (u64 p = threads - 1 - ((u64)blockIdx.x * kT + threadIdx.x); p < A.P; p += threads) {
+    const TilePair& x = A.pair[p];
+    if ((x.nst | x.nnu) != 0) continue;
+    const u64 g_lo = x.g_lo, w = x.w_off;
+    const u32 mode = x.mode;
+    ulonglong2* h = reinterpret_cast<ulonglong2*>(A.E.wire + w);
+    h[0] = make_ulonglong2((u64)kWireMagic | ((u64)kVersion << 32) | ((u64)kRecBytes << 48),
+                           (u64)A.E.class_id | ((u64)mode << 32));
+    h[1] = make_ulonglong2(0, 0);
+    h[2] = make_ulonglong2(0, 0);
+    h[3] = make_ulonglong2(p, kHdrBytes);
+    A.E.wire_len[p] = kHdrBytes;
+    write_taio_header(A.E.ref_next + (g_lo + p) * kRecBytes, A.E.class_id, (u32)p, 0);
+    if (A.D.recv) write_taio_header(A.D.recv + (g_lo + p) * kRecBytes, A.D.class_id, (u32)p, 0);
+    A.E.reset[p] = 0;
+    ++n;
+    if (mode != TERA_MODE_RAW && A.D.ref) {  // as the decode's header check
+      const u64* rh = reinterpret_cast<const u64*>(A.D.ref + (A.D.ref_off[p] + p) * kRecBytes);
+      if ((u32)rh[0] != kTaioMagic || (u32)rh[1] != A.D.class_id || (u32)(rh[1] >> 32) != (u32)p ||
+          rh[2] != 0)
+        latch(A.D.st, TERA_ECORRUPT);
+    }
+  }
+  n = warp_sum(n);
+  if ((threadIdx.x & 31) == 0 && n) atomicAdd(&A.E.stats->wire_bytes, n * kHdrBytes);
+}
+
 // A tile's payload to its place in the message, behind that of the pair's
 // tiles before it (their counts added up).
 template <bool PR>
@@ -1368,6 +1378,7 @@ __global__ void __launch_bounds__(kT, kPerSm) codec_wire_kernel(TileArgs A) {
     if (own) warp_flush(payload_place(A, t, record), pay + pre, own);
     if (last) finish_message(A, t, pre + own, message_mode<PR>(A, t));
   }
+  if (A.scal[TS_OK]) finish_empty(A);
 }
 
 // Tiles and their places are the encode's (both sides of the call run here); a

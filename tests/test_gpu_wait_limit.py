@@ -70,10 +70,15 @@ def test_setup_given_up_writes_no_message(tera, path):
         def call():
             ctx.delta_encode(*args[:8])
     ctx.status()
-    until_given_up(tera, ctx, call, lambda: ex.wire_len.fill_(FILL))
-    # no message of a pair with slots or records
-    entries = np.diff(res["pair_off"].view(np.int64)) + np.diff(res0["pair_off"].view(np.int64))
-    assert (ex.wire_len.cpu().numpy()[entries != 0] == FILL).all()
+    outputs = [ex.ref[1], ex.wire, ex.wire_len, ex.recv[1]]
+
+    def fill():
+        for t in outputs:
+            t.view(torch.uint8).fill_(FILL)
+
+    until_given_up(tera, ctx, call, fill)
+    for t in outputs:
+        assert bool((t.view(torch.uint8) == FILL).all())
     call()
     if path != "batched":
         ctx.delta_decode(ex.wire, ex.wire_off, *args[8:])
