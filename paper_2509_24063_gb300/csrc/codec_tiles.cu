@@ -76,7 +76,7 @@ struct __align__(16) TilePair {
   u32 big0;   // first bigmatch item
   u32 nbig;   // bigmatch items
   u32 mode;   // XOR or raw
-  u32 fits;   // the receiver's reference has the slots the message refers to
+  u32 fits;   // the receiver's reference is the one the message refers to (slots, header)
 };
 static_assert(sizeof(TilePair) == 64, "one line per pair");
 
@@ -156,6 +156,13 @@ __device__ __forceinline__ Facts facts_of(const TileArgs& A, u64 p, int mode, u3
   return f;
 }
 
+// The header check of the receiver's reference of pair p (rr records).
+__device__ __forceinline__ bool recv_header_ok(const DecArgs& D, u64 p, u64 rr) {
+  const u64* rh = reinterpret_cast<const u64*>(D.ref + (D.ref_off[p] + p) * kRecBytes);
+  return (u32)rh[0] == kTaioMagic && (u32)rh[1] == D.class_id && (u32)(rh[1] >> 32) == (u32)p &&
+         rh[2] == rr;
+}
+
 constexpr int kSetupT = 1024;
 
 // out[i] = pair of item i for the items [lo, lo + n) of the block's pairs,
@@ -196,7 +203,11 @@ __global__ void __launch_bounds__(kSetupT)
   const u32 block = s_block;
   const u64 p = (u64)block * kSetupT + threadIdx.x;
   Facts f{};
-  if (p < P) f = facts_of(A, p, mode, shift);
+  bool recv_ok = true;
+  if (p < P) {
+    f = facts_of(A, p, mode, shift);
+    if (!f.raw && A.D.ref && !abort) recv_ok = recv_header_ok(A.D, p, f.rr);
+  }
   U64x2 ta, tb;
   const U64x2 ea = block_excl_scan2(U64x2{f.slab, f.units}, sm2, &ta);
   const U64x2 eb = block_excl_scan2(U64x2{f.items | (f.small << 32), f.big}, sm2, &tb);
@@ -234,7 +245,7 @@ __global__ void __launch_bounds__(kSetupT)
       x.big0 = (u32)(carry_b.b + eb.b);
       x.nbig = (u32)f.big;
       x.mode = f.raw ? TERA_MODE_RAW : TERA_MODE_XOR;
-      x.fits = f.raw || f.r == (A.D.ref ? f.rr : 0) ? 1u : 0u;
+      x.fits = f.raw || (f.r == (A.D.ref ? f.rr : 0) && recv_ok) ? 1u : 0u;
       A.pair[p] = x;
       ulonglong2* tot = reinterpret_cast<ulonglong2*>(A.tot + p * PT_COUNT);
       tot[0] = make_ulonglong2(0, 0);
@@ -1332,12 +1343,7 @@ __device__ __forceinline__ void finish_empty(const TileArgs& A) {
     if (A.D.recv) write_taio_header(A.D.recv + (g_lo + p) * kRecBytes, A.D.class_id, (u32)p, 0);
     A.E.reset[p] = 0;
     ++n;
-    if (mode != TERA_MODE_RAW && A.D.ref) {  // as the decode's header check
-      const u64* rh = reinterpret_cast<const u64*>(A.D.ref + (A.D.ref_off[p] + p) * kRecBytes);
-      if ((u32)rh[0] != kTaioMagic || (u32)rh[1] != A.D.class_id || (u32)(rh[1] >> 32) != (u32)p ||
-          rh[2] != 0)
-        latch(A.D.st, TERA_ECORRUPT);
-    }
+    if (!x.fits) latch(A.D.st, TERA_ECORRUPT);  // as the decode's header check
   }
   n = warp_sum(n);
   if ((threadIdx.x & 31) == 0 && n) atomicAdd(&A.E.stats->wire_bytes, n * kHdrBytes);
@@ -1427,7 +1433,13 @@ __global__ void __launch_bounds__(kT, kDecPerSm) codec_decode_kernel(TileArgs A)
       usable = usable && !err;
       mode = H.mode;
     }
-    if (!usable) continue;
+    if (!usable) {
+      // a rejected pair's records are not decoded; the payload packed there goes
+      uint8_t* left = payload_place(A, t, pos);
+      for (u32 c = lane; lo < hi && c < ((A.bytes[u] + 15u) >> 4); c += 32)
+        *reinterpret_cast<uint4*>(left + (c << 4)) = make_uint4(0u, 0u, 0u, 0u);
+      continue;
+    }
     const u32* codes = reinterpret_cast<const u32*>(w8 + kHdrBytes) + base;
     const uint8_t* pay = w8 + kHdrBytes + 4 * n + A.place[u];
     const u32 want = A.bytes[u];

@@ -81,3 +81,34 @@ def test_reset_overflow_retry(path, gone):
         assert arena[:units * 64].cpu().numpy().tobytes() == nxt[:units * 64].tobytes()
     assert ctx.stats()["wire_bytes"] == int(wl.sum())
     ctx.close()
+
+
+@pytest.mark.parametrize("a", [200, 5000])
+@pytest.mark.parametrize("word", [0, 8, 12, 16])
+def test_rejected_receiver_reference_skips_the_whole_pair(a, word):
+    # a damaged header (magic, class, pair, count) of the receiver's reference, of a
+    # pair of one and of several tiles; the persistent launch's receive buffer
+    import paper_2509_24063_gb300 as tera
+    first, second, _ = two_pairs(a, 300, 3)
+    lo, hi, grid = (0.0,) * 3, (200.0, 100.0, 100.0), (2, 1, 1)
+    buffers = []
+    for tune in (None, (256, 4, 0, 0)):
+        ctx = tera.Context(lo, hi, grid, 20.0)
+        ex = tera.AuraExchange(ctx, max_agents=12000, max_records=30000, path="batched", tune=tune)
+        ex.step(first)
+        ctx.status()
+        off = ex.recv_off[0].cpu().numpy()
+        p = int(np.argmax(off[1:] - off[:-1] == a))
+        assert off[p + 1] - off[p] == a
+        ex.recv[0][(int(off[p]) + p) * 64 + word] ^= 1
+        ex.recv[1].zero_()
+        ex.step(second)
+        code, _ = ctx.status(raise_on_error=False)
+        assert code == tera.ECORRUPT
+        off = ex.recv_off[1].cpu().numpy()
+        units = int(off[-1]) + ctx.n_pairs
+        got = ex.recv[1][:units * 64].cpu().numpy()
+        assert not got[(int(off[p]) + p + 1) * 64:(int(off[p + 1]) + p + 1) * 64].any()
+        buffers.append(got.tobytes())
+        ctx.close()
+    assert buffers[0] == buffers[1]
