@@ -153,7 +153,12 @@ uint64_t tera_n_pairs(const tera_ctx* ctx);
 
 /* Pre-allocate scratch for up to max_agents agents and max_records records
  * per iteration (otherwise done lazily by the first call that needs it;
- * lazy growth synchronizes the device, so call this before graph capture). */
+ * lazy growth synchronizes the device, so call this before graph capture):
+ * what tera_partition, tera_pack, tera_delta_encode and tera_delta_decode need.
+ * About 100 bytes per record and, for the fast form of an encode of every
+ * pair, 68 more (its tile lists and the place its payload is packed in, 64
+ * bytes per record and pair; this place is left out when it would take more than
+ * an eighth of the device memory then free). */
 tera_status tera_ctx_reserve(tera_ctx* ctx, int64_t max_agents, uint64_t max_records);
 
 /* Limit, in microseconds (0 .. 60000000; 1000000 when the context is made), of a
@@ -205,7 +210,8 @@ tera_status tera_pack_ids(tera_ctx* ctx, const tera_soa* soa, const tera_partiti
  * mode TERA_MODE_XOR or TERA_MODE_RAW (raw: the reference is ignored).  A
  * pair marked by tera_reset_reference is sent raw once.  A range of every
  * pair runs over tiles as tera_codec_batched without a tune does, when the
- * context has or can get the scratch for it.  wire_capacity is in
+ * context has the scratch for it (tera_ctx_reserve) or, outside a stream
+ * capture, can get it; else in launches that need none of it.  wire_capacity is in
  * bytes; too small latches TERA_ECAPACITY with the required size. */
 tera_status tera_delta_encode(tera_ctx* ctx, const uint8_t* rec_arena, const uint64_t* pair_off,
                               const uint8_t* ref_prev, const uint64_t* ref_off_prev,

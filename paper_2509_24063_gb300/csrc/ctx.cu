@@ -351,19 +351,38 @@ tera_status ensure_tiles(tera_ctx* ctx) {
   return settled();
 }
 
+// The lists and the payload's place of an encode over tiles (64 bytes a record:
+// 1.06 GB for 16.6 M).  The place is only taken while it is at most an eighth of
+// the memory that is free: the launches that do without it leave a nearly full
+// device to its user.  A capacity that was refused is not asked for again on
+// every call.
+bool ensure_encode_tiles(tera_ctx* ctx) {
+  if (ctx->t_refused == ctx->cap_records) return false;
+  ctx->t_refused = ctx->cap_records;
+  if (ensure_tiles(ctx) != TERA_OK) return false;
+  if (!ctx->t_scratch || ctx->t_scratch_cap < ctx->cap_records) {
+    const u64 bytes = (ctx->cap_records + ctx->n_pairs + 1) * (u64)kRecBytes;
+    size_t free = 0, all = 0;
+    if (cudaMemGetInfo(&free, &all) != cudaSuccess || bytes > free / 8) {
+      cudaGetLastError();
+      return false;
+    }
+    cudaDeviceSynchronize();
+    ctx->t_scratch_cap = 0;
+    if (alloc_dev(ctx->t_scratch, bytes) != TERA_OK) return false;
+    ctx->t_scratch_cap = ctx->cap_records;
+  }
+  ctx->t_refused = 0;
+  return true;
+}
+
 bool encode_tiles_ready(tera_ctx* ctx, cudaStream_t s) {
   const bool have = ctx->t_block && ctx->t_cap >= ctx->cap_records && ctx->t_scratch &&
                     ctx->t_scratch_cap >= ctx->cap_records;
   if (have) return true;
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(s, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) return false;
-  if (ensure_tiles(ctx) != TERA_OK) return false;
-  cudaDeviceSynchronize();
-  ctx->t_scratch_cap = 0;
-  if (alloc_dev(ctx->t_scratch, (ctx->cap_records + ctx->n_pairs + 1) * (u64)kRecBytes) != TERA_OK)
-    return false;
-  ctx->t_scratch_cap = ctx->cap_records;
-  return true;
+  return ensure_encode_tiles(ctx);
 }
 
 tera_status ensure_migrate(tera_ctx* ctx, uint64_t n, uint64_t leavers) {
@@ -803,7 +822,11 @@ tera_status tera_ctx_reserve(tera_ctx* ctx, int64_t max_agents, uint64_t max_rec
   if (st != TERA_OK) return st;
   st = ensure_records(ctx, max_records, 0);
   if (st != TERA_OK) return st;
-  return ensure_units(ctx, 2 * (max_records / kCodecTile) + 4 * ctx->n_pairs + 16, 0);
+  st = ensure_units(ctx, 2 * (max_records / kCodecTile) + 4 * ctx->n_pairs + 16, 0);
+  if (st != TERA_OK) return st;
+  ctx->t_refused = 0;
+  (void)ensure_encode_tiles(ctx);  // an encode without it takes the launches that need none
+  return TERA_OK;
 }
 
 tera_status tera_ctx_wait_limit(tera_ctx* ctx, int64_t limit_us) {

@@ -134,6 +134,7 @@ struct tera_ctx {
   uint8_t* t_block;        // the allocation they lie in
   uint8_t* t_scratch;      // [64 * (t_scratch_cap + P)] packed payload of an encode without decode
   uint64_t t_scratch_cap;
+  uint64_t t_refused;      // record capacity whose encode scratch could not be had (0: none)
   tera::u64* t_pair;       // [P * 8] per-pair facts
   uint32_t* t_unit_pair;   // [t_units] pair of each tile
   uint32_t* t_item_pair;   // [t_items] pair of each match item
@@ -237,6 +238,9 @@ tera_status ensure_pred(tera_ctx* ctx);
 tera_status ensure_batched(tera_ctx* ctx);
 // Scratch of the batched codec over tiles.
 tera_status ensure_tiles(tera_ctx* ctx);
+// Scratch of an encode over tiles for the current record capacity; false when it
+// cannot be had.
+bool ensure_encode_tiles(tera_ctx* ctx);
 // Whether an encode call can run over tiles: its scratch exists, or could be
 // allocated now (not inside a stream capture, and there is memory for it).
 bool encode_tiles_ready(tera_ctx* ctx, cudaStream_t s);
