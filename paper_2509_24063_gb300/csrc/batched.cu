@@ -1894,10 +1894,11 @@ static tera_status batched_impl(
   const u32 T = (u32)tn.block;
   tera_status st = ensure_records(ctx, ctx->cap_records, s);
   if (st != TERA_OK) return st;
-  // both forms' scratch, so that a call with or without a schedule may be
-  // captured after an eager call of either kind
-  if ((st = ensure_batched(ctx)) != TERA_OK) return st;
-  if ((st = ensure_tiles(ctx)) != TERA_OK) return st;
+  // this form's scratch, and outside a capture the other's if it can be had, so
+  // that a call with or without a schedule may be captured after an eager call
+  // of either kind
+  if ((st = tune ? ensure_batched(ctx) : ensure_tiles(ctx)) != TERA_OK) return st;
+  if (!capturing(s)) (void)(tune ? ensure_tiles(ctx) : ensure_batched(ctx));
   if (!ctx->pair_info) return TERA_EINVAL;  // allocated with the context
 
   EncArgs E;

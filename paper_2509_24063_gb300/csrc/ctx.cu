@@ -194,6 +194,11 @@ tera_status check_launch(tera_ctx* ctx, const char* name, cudaStream_t s) {
   return TERA_OK;
 }
 
+bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  return cudaStreamIsCapturing(s, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone;
+}
+
 int grid_for(tera_ctx* ctx, int blocks_per_sm) { return ctx->num_sms * blocks_per_sm; }
 
 tera_status launch_unit_map(tera_ctx* ctx, u32 p0, u64 npr, cudaStream_t s) {
@@ -380,9 +385,7 @@ bool encode_tiles_ready(tera_ctx* ctx, cudaStream_t s) {
   const bool have = ctx->t_block && ctx->t_cap >= ctx->cap_records && ctx->t_scratch &&
                     ctx->t_scratch_cap >= ctx->cap_records;
   if (have) return true;
-  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(s, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) return false;
-  return ensure_encode_tiles(ctx);
+  return !capturing(s) && ensure_encode_tiles(ctx);
 }
 
 tera_status ensure_migrate(tera_ctx* ctx, uint64_t n, uint64_t leavers) {

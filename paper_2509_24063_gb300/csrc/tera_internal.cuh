@@ -229,6 +229,8 @@ tera_status ensure_units(tera_ctx* ctx, uint64_t cap, cudaStream_t s);
 tera_status scan_u32(tera_ctx* ctx, const u32* in, u64* out64, u32* out32, u64 n, cudaStream_t s,
                      u32* flag = nullptr);
 int grid_for(tera_ctx* ctx, int blocks_per_sm);
+// A capture of the stream is under way (or its state can't be told).
+bool capturing(cudaStream_t s);
 // unit_pair[u] = p0 + k for every unit u of range pair k (skipped when
 // units_total[1] flags an aborted call).
 tera_status launch_unit_map(tera_ctx* ctx, u32 p0, u64 npr, cudaStream_t s);

@@ -83,3 +83,29 @@ def test_captured_encode_without_the_scratch():
     assert "codec_encode_kernel" in captured_kernels(ctx, encode)
     check()
     ctx.close()
+
+
+@pytest.mark.parametrize("eager,captured", [(None, (256, 4, 0, 0)), ((256, 4, 0, 0), None)])
+def test_capture_of_the_other_form_of_the_batched_codec(eager, captured):
+    import paper_2509_24063_gb300 as tera
+    wl = Workload("t", 40000, (0.0,) * 3, (160.0,) * 3, (4, 4, 4), 12.0, 2, p_grow=0.1,
+                  p_divide=0.02, p_die=0.02, seed=14)
+    first, second = Generator(wl, device="cuda").series(2)
+    g = oracle.make_grid(wl.lo, wl.hi, wl.grid, wl.w)
+    res0 = oracle.exchange_iteration(g, to_numpy(first))
+    res = oracle.exchange_iteration(g, to_numpy(second), ref=(res0["ref_next"], res0["pair_off"]),
+                                    recv_ref=(res0["recv"], res0["recv_off"]))
+    ctx = tera.Context(wl.lo, wl.hi, wl.grid, wl.w)
+    ex = tera.AuraExchange(ctx, max_agents=60000, max_records=120000, path="batched", tune=eager)
+    ex.step(first)
+    ex.tune = captured
+    graph = ex.capture(second)
+    for _ in range(2):
+        graph.replay()
+    ex.advance()
+    assert ctx.status(raise_on_error=False)[0] == tera.OK
+    np.testing.assert_array_equal(ex.wire_len.cpu().numpy().view(np.uint64), res["wire_len"])
+    units = int(res["pair_off"][-1]) + ctx.n_pairs
+    for got, want in ((ex.sender_ref()[0], res["ref_next"]), (ex.receiver_ref()[0], res["recv"])):
+        assert got[:units * 64].cpu().numpy().tobytes() == want[:units * 64].tobytes()
+    ctx.close()
