@@ -533,9 +533,28 @@ __device__ __forceinline__ void warp_probe(bool less, u64 len, u64* lo, u64* hi)
   if (c > 0u) *lo = base + len * (c - 1u) / 32 + 1;
 }
 
-// Offsets and counts of the pairs: a warp finds where pair p's and pair p + 1's
-// entries begin, both searches a step at a time (five steps of 32 probes for
-// 16 M entries; a thread's bisection took 24 dependent loads twice over, 15 us).
+// First of keys[0, n) that is not below p.
+__device__ __forceinline__ u64 lower_bound_u32(const u32* __restrict__ keys, u64 n, u32 p) {
+  u64 lo = 0, hi = n;
+  while (lo < hi) {
+    const u64 mid = (lo + hi) >> 1;
+    if (keys[mid] < p) lo = mid + 1;
+    else hi = mid;
+  }
+  return lo;
+}
+
+// Offsets and counts of the pairs from the sorted keys.  WARP: a warp finds where
+// pair p's and pair p + 1's entries begin, both searches a step at a time (five
+// steps of 32 probes for 16 M entries); else a thread bisects for both, 24
+// dependent loads twice over.  A warp is the faster while every pair has one at
+// once; with more pairs their warps come in waves.  Launch times, warp against
+// thread, 100 thousand and 16 M agents: 1,728 pairs 7.8 / 12.4 and 10.4 / 20.3
+// us, 13,824 pairs 12.2 / 10.3 and 16.7 / 21.1 (whole partition 44 / 42 and 745 /
+// 750), 19,683 pairs 16.0 / 10.9 and 18.8 / 20.4, 216,000 pairs 98 / 14 and 120 /
+// 29.
+constexpr u64 kWarpPairs = 16384;
+template <bool WARP>
 __global__ void __launch_bounds__(256)
     pair_off_kernel(const u32* __restrict__ sorted_keys, const u64* __restrict__ total_ptr, u64 cap,
                     u64 n_pairs, u64* __restrict__ pair_off, u64* __restrict__ pair_count,
@@ -548,9 +567,17 @@ __global__ void __launch_bounds__(256)
     // that are not there (a scan that gave up leaves run_base as it was)
     *packable = *reinterpret_cast<const volatile u32*>(&st->abort) ? ~0ull : E;
   }
+  const u64 t = (u64)blockIdx.x * blockDim.x + threadIdx.x, threads = (u64)gridDim.x * blockDim.x;
+  if constexpr (!WARP) {
+    for (u64 p = t; p <= n_pairs; p += threads) {
+      const u64 at = lower_bound_u32(sorted_keys, E, (u32)p);
+      pair_off[p] = at;
+      if (p < n_pairs) pair_count[p] = lower_bound_u32(sorted_keys, E, (u32)(p + 1)) - at;
+    }
+    return;
+  }
   const u32 lane = threadIdx.x & 31;
-  const u64 warps = (u64)gridDim.x * (blockDim.x / 32);
-  for (u64 p = (u64)blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5); p <= n_pairs; p += warps) {
+  for (u64 p = t >> 5; p <= n_pairs; p += threads >> 5) {
     u64 lo0 = 0, hi0 = E, lo1 = 0, hi1 = E;
     while (lo0 < hi0 || lo1 < hi1) {  // warp-uniform
       const u64 len0 = hi0 - lo0, len1 = hi1 - lo1;
@@ -718,7 +745,9 @@ extern "C" tera_status tera_partition(tera_ctx* ctx, const tera_soa* soa, tera_p
   ctx->rec_pair = const_cast<u32*>(sorted);
   ctx->pack_n = soa->n;
   prof_begin(ctx, s);
-  launch_chained(pair_off_kernel, (unsigned)(P / 8 + 1), 256, 0, s, 
+  const bool warp = P <= kWarpPairs;
+  launch_chained(warp ? pair_off_kernel<true> : pair_off_kernel<false>,
+                 (unsigned)(P / (warp ? 8 : 256) + 1), 256, 0, s,
       sorted, total_ptr, cap, P, reinterpret_cast<u64*>(out->pair_off),
       reinterpret_cast<u64*>(out->pair_count), ctx->d_total, ctx->d_stats, ctx->d_status);
   return check_launch(ctx, "pair_off_kernel", s);
