@@ -1381,7 +1381,15 @@ __global__ void __launch_bounds__(kT, kPerSm) codec_wire_kernel(TileArgs A) {
     pre = warp_sum(pre);
     if (lane == 0) A.place[u] = pre;
     uint8_t* pay = E.wire + t.x.w_off + kHdrBytes + 4 * ((u64)t.x.r + t.n_new);
-    if (own) warp_flush(payload_place(A, t, record), pay + pre, own);
+    if (own) {
+      uint8_t* packed = payload_place(A, t, record);
+      warp_flush(packed, pay + pre, own);
+      if (!t.x.fits && A.D.recv) {  // a rejected pair's records will not be decoded over it
+        __syncwarp();
+        for (u32 c = lane; c < ((own + 15u) >> 4); c += 32)
+          *reinterpret_cast<uint4*>(packed + (c << 4)) = make_uint4(0u, 0u, 0u, 0u);
+      }
+    }
     if (last) finish_message(A, t, pre + own, message_mode<PR>(A, t));
   }
   if (A.scal[TS_OK]) finish_empty(A);
@@ -1433,13 +1441,7 @@ __global__ void __launch_bounds__(kT, kDecPerSm) codec_decode_kernel(TileArgs A)
       usable = usable && !err;
       mode = H.mode;
     }
-    if (!usable) {
-      // a rejected pair's records are not decoded; the payload packed there goes
-      uint8_t* left = payload_place(A, t, pos);
-      for (u32 c = lane; lo < hi && c < ((A.bytes[u] + 15u) >> 4); c += 32)
-        *reinterpret_cast<uint4*>(left + (c << 4)) = make_uint4(0u, 0u, 0u, 0u);
-      continue;
-    }
+    if (!usable) continue;
     const u32* codes = reinterpret_cast<const u32*>(w8 + kHdrBytes) + base;
     const uint8_t* pay = w8 + kHdrBytes + 4 * n + A.place[u];
     const u32 want = A.bytes[u];
