@@ -146,6 +146,7 @@ struct DecArgs {
 // context's scratch).  The lists' bounds for cap records of P pairs.
 tera_status launch_tiles(tera_ctx* ctx, const EncArgs& E, const DecArgs& D, bool pr, int mode,
                          u64 wire_cap, u64 recv_cap, cudaStream_t s);
+constexpr u32 kTileGroup = 128;  // tiles whose payload bytes are also added up
 void tile_list_bounds(u64 cap, u64 P, u64 warps, u64* units, u64* items, u64* bigs);
 
 __device__ __forceinline__ u32 rec_code(const Rec& d, u32* bytes) {

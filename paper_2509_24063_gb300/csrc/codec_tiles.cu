@@ -64,6 +64,13 @@ constexpr u32 kNewShare = 16;
 // 936 pairs: 39 us with the higher limit, 32 with the lower).
 constexpr u32 kWarpPair = 256, kWarpPairFew = 64;
 
+// The wire launch adds up the payload bytes of a pair's tiles before each: one by
+// one in pairs of at most kGroupMin tiles, else by the sums of kTileGroup tiles,
+// which the encode keeps for such pairs.  (One by one in every pair, the launch
+// grew with the square of a pair's tiles: two boxes of 8 M agents, 1.8 M records a
+// pair, 219 us, now 39; of 40 M agents, 9 M records a pair, 328, now 78.)
+constexpr u32 kGroupMin = 256;
+
 // Per-pair facts, one 64-byte line.
 struct __align__(16) TilePair {
   u64 g_lo;   // first record of the message (pair_off)
@@ -100,6 +107,8 @@ struct TileArgs {
   u32 warp_pair;        // slots and records of a pair matched by one warp, at most
   u32* before;          // matched slots before each slot tile (bigmatch: first, in it)
   u32* bytes;           // payload bytes of each tile
+  u32* group;           // payload bytes of each kTileGroup tiles (of pairs above kGroupMin)
+  u32 unit_cap;         // tiles there is room for
   u64* place;           // payload bytes of the pair before each tile
   u64* tot;             // [P * PT_COUNT] matched records, XOR and residual bytes
   u32* done;            // [P] matched tiles of a big pair
@@ -687,6 +696,8 @@ __global__ void __launch_bounds__(kT, kPerSm) codec_match_kernel(TileArgs A) {
     for (u32 i = threadIdx.x; i < 4 * blocks; i += kT) A.setup_state[i] = 0;
     if (threadIdx.x == 0) *A.setup_ticket = 0;
   }
+  for (u32 i = blockIdx.x * kT + threadIdx.x; i <= A.unit_cap / kTileGroup; i += gridDim.x * kT)
+    A.group[i] = 0u;
   map_tiles(A);
   if (n) {
     for (;;) {
@@ -1284,7 +1295,10 @@ __global__ void __launch_bounds__(kT, kEncPerSm) codec_encode_kernel(TileArgs A)
     // the last piece may carry zeros past the bytes, still inside the records' place
     if ((bytes & 15u) && lane == 0)
       *reinterpret_cast<uint4*>(out + (bytes & ~15u)) = *reinterpret_cast<const uint4*>(st);
-    if (lane == 0) A.bytes[u] = bytes;
+    if (lane == 0) {
+      A.bytes[u] = bytes;
+      if (t.x.nst + t.x.nnu > kGroupMin) atomicAdd(A.group + u / kTileGroup, bytes);
+    }
     __syncwarp();
   }
 }
@@ -1320,6 +1334,20 @@ __device__ __forceinline__ void finish_message(const TileArgs& A, const Tile& t,
     E.reset[p] = 0;
   }
   if (body + lane < msg) w8[body + lane] = 0;  // zero padding (< 16 bytes)
+}
+
+// This lane's share of the payload bytes of the tiles [a, b) of one pair.
+__device__ __forceinline__ u64 tile_bytes(const TileArgs& A, u32 a, u32 b) {
+  const u32 lane = threadIdx.x & 31;
+  u64 sum = 0;
+  if (b - a > kGroupMin) {
+    const u32 g0 = (a + kTileGroup - 1) / kTileGroup, g1 = b / kTileGroup;
+    for (u32 g = g0 + lane; g < g1; g += 32) sum += A.group[g];
+    for (u32 i = a + lane; i < g0 * kTileGroup; i += 32) sum += A.bytes[i];
+    a = g1 * kTileGroup;
+  }
+  for (u32 i = a + lane; i < b; i += 32) sum += A.bytes[i];
+  return sum;
 }
 
 // The pairs without entries on either side, a thread each: headers alone.  The
@@ -1376,9 +1404,7 @@ __global__ void __launch_bounds__(kT, kPerSm) codec_wire_kernel(TileArgs A) {
       // an entryless pair's message is its header
       last = hi == t.n_new && (lo < hi || (t.n_new == 0 && t.x.r == 0 && t.local == 0));
     }
-    u64 pre = 0;
-    for (u32 i = lane; i < t.local; i += 32) pre += A.bytes[t.x.unit0 + i];
-    pre = warp_sum(pre);
+    const u64 pre = warp_sum(tile_bytes(A, t.x.unit0, t.x.unit0 + t.local));
     if (lane == 0) A.place[u] = pre;
     uint8_t* pay = E.wire + t.x.w_off + kHdrBytes + 4 * ((u64)t.x.r + t.n_new);
     if (own) {
@@ -1608,6 +1634,8 @@ tera_status launch_tiles(tera_ctx* ctx, const EncArgs& E, const DecArgs& D, bool
   A.warp_pair = P > 8ull * grid ? kWarpPair : kWarpPairFew;
   A.before = ctx->t_before;
   A.bytes = ctx->t_bytes;
+  A.group = ctx->t_group;
+  A.unit_cap = (u32)(ctx->t_units < 0xFFFFFFFFull ? ctx->t_units : 0xFFFFFFFFull);
   A.place = ctx->t_place;
   A.tot = ctx->t_tot;
   A.done = ctx->t_done;

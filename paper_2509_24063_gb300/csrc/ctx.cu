@@ -343,6 +343,7 @@ tera_status ensure_tiles(tera_ctx* ctx) {
     take(ctx->t_before, ctx->t_units);
     take(ctx->t_bytes, ctx->t_units);
     take(ctx->t_place, ctx->t_units);
+    take(ctx->t_group, ctx->t_units / kTileGroup + 1);
     take(ctx->t_bits, cap / 32 + P + 2);
     take(ctx->t_new, cap);
   };

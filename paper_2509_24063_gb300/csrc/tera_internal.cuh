@@ -142,6 +142,7 @@ struct tera_ctx {
   uint32_t* t_small_pair;  // [P] pairs matched by one warp
   uint32_t* t_before;      // [t_units] matched slots before each tile
   uint32_t* t_bytes;       // [t_units] payload bytes of each tile
+  uint32_t* t_group;       // [t_units / kTileGroup + 1] payload bytes of that many tiles
   tera::u64* t_place;      // [t_units] payload bytes of the pair before each tile
   tera::u64* t_tot;        // [P * 4] matched records, XOR and residual bytes
   uint32_t* t_done;        // [3 * P] matched and indexed tiles of a big pair, ids not ascending
