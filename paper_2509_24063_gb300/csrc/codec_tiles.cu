@@ -52,10 +52,14 @@ constexpr u32 kBigTile = kT * kIlp;  // ids of a tile of a pair matched through 
 // 10 us) and a large one's are not all set-up.
 constexpr u32 kMinShift = 5, kMaxShift = 8;
 constexpr u64 kTilesPerWarp = 8;
-// new-record tiles of a pair beyond the m - r records that must be new: one
-// per kNewShare tiles of records, so that a pair whose records all changed is
-// still spread over many warps, while a usual pair has one
-constexpr u32 kNewShare = 16;
+// Tiles of new records: the setup plans those of the m - r records that must be
+// new, and one per kNewShare tiles of records for the others, which only the
+// match counts; where it finds more than kNewTiles tiles of them for each
+// planned one, it adds tiles at the end of the list until there is one each.
+// (16 M agents, 5.9 M records, all of other ids than the reference's: with the
+// planned tiles alone, each with up to sixteen tiles' records, 2573 us an
+// iteration, now 1450; three in ten of other ids, 1616 and 1360.)
+constexpr u32 kNewShare = 16, kNewTiles = 2;
 // Pairs of at most this many slots and records are matched by one warp, so
 // that the thousands of edge and corner pairs of a large grid are in flight at
 // once (13,824 pairs, 100 M agents: match 297 -> 264 us, before the ids were held
@@ -87,15 +91,17 @@ struct __align__(16) TilePair {
 };
 static_assert(sizeof(TilePair) == 64, "one line per pair");
 
-// Device scalars of one call (TS_OK: the setup accepted it).
+// Device scalars of one call (TS_OK: the setup accepted it; TS_EXTRA: tiles the
+// match added behind the TS_UNITS planned ones).
 enum { TS_UNITS = 0, TS_ITEMS, TS_BIG, TS_SMALL, TS_SHIFT, TS_TICKET_MATCH, TS_TICKET_BIG,
-       TS_OK, TS_COUNT };
+       TS_OK, TS_EXTRA, TS_COUNT };
 
 struct TileArgs {
   EncArgs E;
   DecArgs D;
   TilePair* pair;
   u32* unit_pair;       // pair of each tile
+  u32 unit_cap;         // tiles there is room for
   u32* unit_first;      // [P] first tile of each pair
   u64* setup_state;     // look-back states of the setup (zero between calls)
   u32* setup_ticket;
@@ -108,7 +114,6 @@ struct TileArgs {
   u32* before;          // matched slots before each slot tile (bigmatch: first, in it)
   u32* bytes;           // payload bytes of each tile
   u32* group;           // payload bytes of each kTileGroup tiles (of pairs above kGroupMin)
-  u32 unit_cap;         // tiles there is room for
   u64* place;           // payload bytes of the pair before each tile
   u64* tot;             // [P * PT_COUNT] matched records, XOR and residual bytes
   u32* done;            // [P] matched tiles of a big pair
@@ -121,7 +126,8 @@ struct TileArgs {
   u64 P;
 };
 
-enum { PT_MATCHED = 0, PT_XOR = 1, PT_RES = 2, PT_COUNT = 4 };
+// PT_EXTRA: first added tile (behind TS_UNITS) | their number << 32
+enum { PT_MATCHED = 0, PT_XOR = 1, PT_RES = 2, PT_EXTRA = 3, PT_COUNT = 4 };
 
 // ---------------- setup ----------------
 
@@ -428,6 +434,25 @@ __device__ __forceinline__ void count_tiles(const TileArgs& A, const TilePair& x
   }
 }
 
+// More tiles for the n_new new records of pair p when the planned ones would hold
+// many tiles' records each; s_first: a word of the group's shared memory.
+template <int T>
+__device__ __forceinline__ void add_new_tiles(const TileArgs& A, const TilePair& x, u32 p, u32 n_new,
+                                              u32 shift, u32* s_first) {
+  const u32 want = (u32)tiles(n_new, shift);
+  if (want <= kNewTiles * x.nnu) return;  // group-uniform
+  const u32 more = want - x.nnu;
+  group_sync<T>();
+  if (group_thread<T>() == 0) {
+    const u32 first = atomicAdd(A.scal + TS_EXTRA, more);
+    A.tot[(u64)p * PT_COUNT + PT_EXTRA] = (u64)first | ((u64)more << 32);
+    *s_first = first;
+  }
+  group_sync<T>();
+  const u64 at = (u64)A.scal[TS_UNITS] + *s_first;
+  for (u32 i = group_thread<T>(); i < more && at + i < A.unit_cap; i += T) A.unit_pair[at + i] = p;
+}
+
 // One tile of a big pair's message: whether its ids ascend (up to the next
 // tile's first), and its taken bits cleared.
 __device__ __forceinline__ void big_check(const TileArgs& A, const TilePair& x, u32 p, u32 tile) {
@@ -653,6 +678,7 @@ __device__ __forceinline__ void match_pair(const TileArgs& A, const TilePair& x,
     group_sync<T>();
     sum_tiles<T>(A, x, sm32);
   }
+  add_new_tiles<T>(A, x, p, x.m - matched, shift, s_cnt);
 }
 
 // The pair of every tile (unit_pair), which the launches after this one read:
@@ -922,6 +948,8 @@ __global__ void __launch_bounds__(kT, kPerSm) codec_bigmatch_kernel(TileArgs A) 
       __threadfence();
       new_list<kT, true>(A, x, bits, sm32);
       sum_tiles<kT>(A, x, sm32);
+      const u32 matched = (u32)__ldcg(A.tot + (u64)p * PT_COUNT + PT_MATCHED);
+      add_new_tiles<kT>(A, x, p, x.m - matched, shift, s_span);
     }
     __syncthreads();
   }
@@ -1017,18 +1045,32 @@ __device__ __forceinline__ void copies_wait() {  // all but the last N groups
   asm volatile("cp.async.wait_group %0;" : : "n"(N) : "memory");
 }
 
+// The tiles of the call: `planned` by the setup, the match's behind them.
+struct TileCount {
+  u32 planned, all;
+};
+__device__ __forceinline__ TileCount tile_count(const TileArgs& A) {
+  const u32 planned = A.scal[TS_UNITS], all = planned + A.scal[TS_EXTRA];
+  return TileCount{planned, all < A.unit_cap ? all : A.unit_cap};
+}
+
 // What a tile's warp needs of its pair.
 struct Tile {
   TilePair x;
   u32 p, local;
   u32 n_new;
+  u32 nnu;      // new-record tiles, the added ones among them
+  u32 added0;   // the first of those in the list
 };
 
-__device__ __forceinline__ Tile tile_of(const TileArgs& A, u32 u, u32 p) {
+__device__ __forceinline__ Tile tile_of(const TileArgs& A, const TileCount& n, u32 u, u32 p) {
   Tile t;
   t.p = p;
   t.x = A.pair[p];
-  t.local = u - t.x.unit0;
+  const u64 extra = A.tot[(u64)p * PT_COUNT + PT_EXTRA];
+  t.nnu = t.x.nnu + (u32)(extra >> 32);
+  t.added0 = n.planned + (u32)extra;
+  t.local = u < n.planned ? u - t.x.unit0 : t.x.nst + t.x.nnu + (u - t.added0);
   t.n_new = t.x.m - (u32)A.tot[(u64)p * PT_COUNT + PT_MATCHED];
   return t;
 }
@@ -1163,14 +1205,15 @@ __global__ void __launch_bounds__(kT, kEncPerSm) codec_encode_kernel(TileArgs A)
   const u32 r8 = lane >> 2, q = lane & 3;  // this lane's record of each eight, and its piece
   uint8_t* st = dyn + warp * (kStage + 2 * kRows);
   uint8_t* rows = st + kStage;
-  const u32 n = A.scal[TS_UNITS], shift = A.scal[TS_SHIFT];
+  const TileCount n = tile_count(A);
+  const u32 shift = A.scal[TS_SHIFT];
   const u32 epoch = *E.epoch;
   const u32 stride = gridDim.x * kWarps;
   u32 u = blockIdx.x * kWarps + warp;
-  u32 p_next = u < n ? A.unit_pair[u] : 0u;
-  for (; u < n; u += stride) {
-    const Tile t = tile_of(A, u, p_next);
-    if (u + stride < n) p_next = A.unit_pair[u + stride];
+  u32 p_next = u < n.all ? A.unit_pair[u] : 0u;
+  for (; u < n.all; u += stride) {
+    const Tile t = tile_of(A, n, u, p_next);
+    if (u + stride < n.all) p_next = A.unit_pair[u + stride];
     const u32 p = t.p;
     u32* codes = reinterpret_cast<u32*>(E.wire + t.x.w_off + kHdrBytes);
     if (lane == 0) *reinterpret_cast<uint4*>(st) = make_uint4(0u, 0u, 0u, 0u);
@@ -1256,7 +1299,7 @@ __global__ void __launch_bounds__(kT, kEncPerSm) codec_encode_kernel(TileArgs A)
       // new records: rank i's code and new-reference record have known places
       const u64 matched = (u64)t.x.m - t.n_new;
       u32 lo, hi;
-      new_range(t.n_new, t.x.nnu, t.local - t.x.nst, shift, &lo, &hi);
+      new_range(t.n_new, t.nnu, t.local - t.x.nst, shift, &lo, &hi);
       out = payload_place(A, t, matched + lo);
       for (u32 i0 = lo; i0 < hi; i0 += 32) {
         const u32 hits = hi - i0 >= 32 ? 0xFFFFFFFFu : (1u << (hi - i0)) - 1u;
@@ -1297,7 +1340,7 @@ __global__ void __launch_bounds__(kT, kEncPerSm) codec_encode_kernel(TileArgs A)
       *reinterpret_cast<uint4*>(out + (bytes & ~15u)) = *reinterpret_cast<const uint4*>(st);
     if (lane == 0) {
       A.bytes[u] = bytes;
-      if (t.x.nst + t.x.nnu > kGroupMin) atomicAdd(A.group + u / kTileGroup, bytes);
+      if (t.x.nst + t.nnu > kGroupMin) atomicAdd(A.group + u / kTileGroup, bytes);
     }
     __syncwarp();
   }
@@ -1384,13 +1427,14 @@ __global__ void __launch_bounds__(kT, kPerSm) codec_wire_kernel(TileArgs A) {
   chain_begin();
   const EncArgs& E = A.E;
   const u32 warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const u32 n = A.scal[TS_UNITS], shift = A.scal[TS_SHIFT];
+  const TileCount n = tile_count(A);
+  const u32 shift = A.scal[TS_SHIFT];
   const u32 stride = gridDim.x * kWarps;
   u32 u = blockIdx.x * kWarps + warp;
-  u32 p_next = u < n ? A.unit_pair[u] : 0u;
-  for (; u < n; u += stride) {
-    const Tile t = tile_of(A, u, p_next);
-    if (u + stride < n) p_next = A.unit_pair[u + stride];
+  u32 p_next = u < n.all ? A.unit_pair[u] : 0u;
+  for (; u < n.all; u += stride) {
+    const Tile t = tile_of(A, n, u, p_next);
+    if (u + stride < n.all) p_next = A.unit_pair[u + stride];
     const u32 own = A.bytes[u];
     u64 record;
     bool last;
@@ -1399,12 +1443,15 @@ __global__ void __launch_bounds__(kT, kPerSm) codec_wire_kernel(TileArgs A) {
       last = t.n_new == 0 && t.local + 1 == t.x.nst;
     } else {
       u32 lo, hi;
-      new_range(t.n_new, t.x.nnu, t.local - t.x.nst, shift, &lo, &hi);
+      new_range(t.n_new, t.nnu, t.local - t.x.nst, shift, &lo, &hi);
       record = (u64)t.x.m - t.n_new + lo;
       // an entryless pair's message is its header
       last = hi == t.n_new && (lo < hi || (t.n_new == 0 && t.x.r == 0 && t.local == 0));
     }
-    const u64 pre = warp_sum(tile_bytes(A, t.x.unit0, t.x.unit0 + t.local));
+    const u32 planned = t.x.nst + t.x.nnu, own_planned = t.local < planned ? t.local : planned;
+    u64 pre = tile_bytes(A, t.x.unit0, t.x.unit0 + own_planned);
+    if (t.local > planned) pre += tile_bytes(A, t.added0, t.added0 + (t.local - planned));
+    pre = warp_sum(pre);
     if (lane == 0) A.place[u] = pre;
     uint8_t* pay = E.wire + t.x.w_off + kHdrBytes + 4 * ((u64)t.x.r + t.n_new);
     if (own) {
@@ -1433,13 +1480,14 @@ __global__ void __launch_bounds__(kT, kDecPerSm) codec_decode_kernel(TileArgs A)
   const u32 r8 = lane >> 2, q = lane & 3;  // this lane's record of each eight, and its piece
   uint8_t* stages = dyn + warp * (2 * kStage + 2 * kRows);
   uint8_t* rows = stages + 2 * kStage;
-  const u32 n_units = A.scal[TS_UNITS], shift = A.scal[TS_SHIFT];
+  const TileCount tc = tile_count(A);
+  const u32 shift = A.scal[TS_SHIFT];
   const u32 stride = gridDim.x * kWarps;
   u32 u = blockIdx.x * kWarps + warp;
-  u32 p_next = u < n_units ? A.unit_pair[u] : 0u;
-  for (; u < n_units; u += stride) {
-    const Tile t = tile_of(A, u, p_next);
-    if (u + stride < n_units) p_next = A.unit_pair[u + stride];
+  u32 p_next = u < tc.all ? A.unit_pair[u] : 0u;
+  for (; u < tc.all; u += stride) {
+    const Tile t = tile_of(A, tc, u, p_next);
+    if (u + stride < tc.all) p_next = A.unit_pair[u + stride];
     const u32 p = t.p;
     const u64 m = t.x.m, ns = t.x.r, n = ns + t.n_new;
     u32 lo, hi, base = 0;  // this tile's entries [lo, hi) behind the pair's entry `base`
@@ -1449,7 +1497,7 @@ __global__ void __launch_bounds__(kT, kDecPerSm) codec_decode_kernel(TileArgs A)
       hi = t.x.r - lo < (1u << shift) ? t.x.r : lo + (1u << shift);
       pos = A.before[u];
     } else {
-      new_range(t.n_new, t.x.nnu, t.local - t.x.nst, shift, &lo, &hi);
+      new_range(t.n_new, t.nnu, t.local - t.x.nst, shift, &lo, &hi);
       base = t.x.r;
       pos = m - t.n_new + lo;
     }
@@ -1625,6 +1673,7 @@ tera_status launch_tiles(tera_ctx* ctx, const EncArgs& E, const DecArgs& D, bool
   A.D = D;
   A.pair = reinterpret_cast<TilePair*>(ctx->t_pair);
   A.unit_pair = ctx->t_unit_pair;
+  A.unit_cap = (u32)(ctx->t_units < 0xFFFFFFFFull ? ctx->t_units : 0xFFFFFFFFull);
   A.unit_first = ctx->t_unit_first;
   A.setup_state = ctx->t_part;
   A.item_pair = ctx->t_item_pair;
@@ -1635,7 +1684,6 @@ tera_status launch_tiles(tera_ctx* ctx, const EncArgs& E, const DecArgs& D, bool
   A.before = ctx->t_before;
   A.bytes = ctx->t_bytes;
   A.group = ctx->t_group;
-  A.unit_cap = (u32)(ctx->t_units < 0xFFFFFFFFull ? ctx->t_units : 0xFFFFFFFFull);
   A.place = ctx->t_place;
   A.tot = ctx->t_tot;
   A.done = ctx->t_done;
@@ -1685,7 +1733,8 @@ tera_status launch_tiles(tera_ctx* ctx, const EncArgs& E, const DecArgs& D, bool
 
 // Bounds of the lists for `cap` slots, records and pairs P (the setup's
 // counts): tiles of slots, tiles of records that must be new, shares of
-// records; match items and bigmatch items of big pairs.  Tiles below the
+// records (the tiles of new records after the match are at most the records' own
+// tiles and a share); match items and bigmatch items of big pairs.  Tiles below the
 // largest size come with fewer than twice kTilesPerWarp per resident warp.
 void tile_list_bounds(u64 cap, u64 P, u64 warps, u64* units, u64* items, u64* bigs) {
   const u64 few = 2 * kTilesPerWarp * warps;

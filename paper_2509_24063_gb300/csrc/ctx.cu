@@ -334,7 +334,7 @@ tera_status ensure_tiles(tera_ctx* ctx) {
     take(ctx->t_pair, P * 8);
     take(ctx->t_tot, P * 4);
     take(ctx->t_done, 3 * P);
-    take(ctx->t_scal, 8);
+    take(ctx->t_scal, 16);
     take(ctx->t_unit_first, P);
     take(ctx->t_small_pair, P);
     take(ctx->t_unit_pair, ctx->t_units);

@@ -148,7 +148,7 @@ struct tera_ctx {
   uint32_t* t_done;        // [3 * P] matched and indexed tiles of a big pair, ids not ascending
   uint32_t* t_bits;        // taken records of big pairs
   uint32_t* t_new;         // [t_cap] new records of each pair
-  uint32_t* t_scal;        // [8] list lengths and claim tickets
+  uint32_t* t_scal;        // [16] list lengths and claim tickets
   uint32_t* t_unit_first;  // [P] first tile of each pair
   tera::u64* t_part;       // [4 * (P / 1024 + 1) + 1] look-back states of the setup, its ticket
   // agent migration (migrate.cu)
