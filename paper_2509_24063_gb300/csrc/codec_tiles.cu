@@ -5,8 +5,8 @@
 //   setup   per-pair facts, wire slabs and the lists of tiles
 //   match   one block (a warp for a small pair) per pair: the message record of
 //           every reference slot (ids in shared memory), the matches before each tile and the list
-//           of the records no slot took; a pair of more than kTableMax records
-//           is only asked here, a tile each, whether its ids ascend, and
+//           of the records no slot took; a big pair (more than kTableMax records
+//           or kBlockSlots slots) is only asked here, a tile each, whether its ids ascend, and
 //           matched by
 //   bigmatch  (tiles of such pairs; does nothing without them): by bisection
 //           over ascending ids, else in a global hash segment that its tiles
@@ -74,6 +74,14 @@ constexpr u32 kWarpPair = 256, kWarpPairFew = 64;
 // grew with the square of a pair's tiles: two boxes of 8 M agents, 1.8 M records a
 // pair, 219 us, now 39; of 40 M agents, 9 M records a pair, 328, now 78.)
 constexpr u32 kGroupMin = 256;
+
+// A pair of more slots than this, and than twice a block's share of all slots, is
+// a big one whatever its message holds (a population that shrank): one block that
+// looks all of them up, 2.5 us for each 1,024, would be the launch's length.  Two
+// messages of some 5 K records against 450 K slots each: 1250 -> 104 us an
+// iteration, against 22 K slots 108 -> 81, 11 K 80 (with the line at 8,192: 84).
+// 8 M agents in 64 boxes, 26 K slots a pair, 668 (690 without the share).
+constexpr u32 kBlockSlots = 16384;
 
 // Per-pair facts, one 64-byte line.
 struct __align__(16) TilePair {
@@ -150,7 +158,8 @@ __device__ __forceinline__ u64 tiles(u64 entries, u32 shift) {
   return (entries + (1ull << shift) - 1ull) >> shift;
 }
 
-__device__ __forceinline__ Facts facts_of(const TileArgs& A, u64 p, int mode, u32 shift) {
+__device__ __forceinline__ Facts facts_of(const TileArgs& A, u64 p, int mode, u32 shift,
+                                          u64 all_slots) {
   Facts f;
   f.m = A.E.pair_off[p + 1] - A.E.pair_off[p];
   f.r_full = A.E.ref_off ? A.E.ref_off[p + 1] - A.E.ref_off[p] : 0;
@@ -164,7 +173,8 @@ __device__ __forceinline__ Facts facts_of(const TileArgs& A, u64 p, int mode, u3
   // through the decode's header check
   if (f.r == 0 && f.m == 0 && f.rr != 0) nnu = 1;
   f.units = tiles(f.r, shift) + nnu;
-  const bool big = f.m > kTableMax;
+  const bool big = f.m > kTableMax ||
+                   (f.r > kBlockSlots && f.r * (A.warps / (kT / 32)) > 2 * all_slots);
   f.small = f.r + f.m != 0 && f.r <= A.warp_pair && f.m <= A.warp_pair;
   f.items = big ? ceil_div(f.m, kBigTile) : (f.r + f.m != 0 && !f.small ? 1 : 0);
   f.big = big ? ceil_div(f.m, kBigTile) + ceil_div(f.r, kBigTile) : 0;
@@ -220,7 +230,7 @@ __global__ void __launch_bounds__(kSetupT)
   Facts f{};
   bool recv_ok = true;
   if (p < P) {
-    f = facts_of(A, p, mode, shift);
+    f = facts_of(A, p, mode, shift, rmax);
     if (!f.raw && A.D.ref && !abort) recv_ok = recv_header_ok(A.D, p, f.rr);
   }
   U64x2 ta, tb;
@@ -731,7 +741,7 @@ __global__ void __launch_bounds__(kT, kPerSm) codec_match_kernel(TileArgs A) {
       if (it == ~0u) break;
       const u32 p = A.item_pair[it];
       const TilePair x = A.pair[p];
-      if (x.m > kTableMax) big_check(A, x, p, it - x.item0);
+      if (x.nbig) big_check(A, x, p, it - x.item0);
       else match_pair<kT>(A, x, p, shift, dyn, reinterpret_cast<u32*>(dyn + kMatchArea), s_cnt, sm32);
       __syncthreads();
     }
@@ -1319,7 +1329,7 @@ __global__ void __launch_bounds__(kT, kEncPerSm) codec_encode_kernel(TileArgs A)
         if (i0 + lane < hi) {
           d = row_rec(rows, lane);
           // an id that occurs twice in a big pair's message: the other record is found
-          if (t.x.m > kTableMax && A.unsorted[p] &&
+          if (t.x.nbig && A.unsorted[p] &&
               seg_lookup<true>(E.seg, epoch, p, t.x.g_lo, t.x.m, d.w[0]) != (u32)(t.x.g_lo + k))
             latch(E.st, TERA_EINVAL);
           code = rec_code(d, &vb);

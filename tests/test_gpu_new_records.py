@@ -50,3 +50,25 @@ def test_new_records_with_histories(n, grid):
         ctx.close()
     for a, b in zip(*out):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("path", ["batched", "all_pairs"])
+@pytest.mark.parametrize("shuffle", [False, True])
+@pytest.mark.parametrize("slots,share", [(16300, 0.3), (16500, 0.3), (16500, 0.0), (60000, 0.02),
+                                         (60000, 0.2)])
+def test_many_slots_and_a_short_message(slots, share, shuffle, path):
+    # nearly every agent gone, or all: slots of a pair round the line above which
+    # they are looked up by many blocks
+    import paper_2509_24063_gb300 as tera
+    from test_gpu_tiles import two_pairs
+    first, second, _ = two_pairs(slots, 700, slots)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(slots)
+    k = second["x"].shape[0]
+    keep = torch.rand(k, generator=g, device="cuda") < share
+    states = [first, {f: v[keep].contiguous() for f, v in second.items()}]
+    if shuffle:
+        for i, st in enumerate(states):
+            perm = torch.randperm(st["x"].shape[0], generator=g, device="cuda")
+            states[i] = {f: v[perm].contiguous() for f, v in st.items()}
+    run_states(tera, states, (0.0,) * 3, (200.0, 100.0, 100.0), (2, 1, 1), 20.0, path=path)
