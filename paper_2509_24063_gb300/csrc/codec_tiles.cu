@@ -70,9 +70,10 @@ constexpr u32 kWarpPair = 256, kWarpPairFew = 64;
 
 // The wire launch adds up the payload bytes of a pair's tiles before each: one by
 // one in pairs of at most kGroupMin tiles, else by the sums of kTileGroup tiles,
-// which the encode keeps for such pairs.  (One by one in every pair, the launch
-// grew with the square of a pair's tiles: two boxes of 8 M agents, 1.8 M records a
-// pair, 219 us, now 39; of 40 M agents, 9 M records a pair, 328, now 78.)
+// which the encode keeps for such pairs (planned and added tiles apart).  (One by
+// one in every pair, the launch grew with the square of a pair's tiles: two boxes
+// of 8 M agents, 1.8 M records a pair, 219 us, now 39; of 40 M agents, 9 M records
+// a pair, 328, now 78.)
 constexpr u32 kGroupMin = 256;
 
 // A pair of more slots than this, and than twice a block's share of all slots, is
@@ -82,6 +83,12 @@ constexpr u32 kGroupMin = 256;
 // iteration, against 22 K slots 108 -> 81, 11 K 80 (with the line at 8,192: 84).
 // 8 M agents in 64 boxes, 26 K slots a pair, 668 (690 without the share).
 constexpr u32 kBlockSlots = 16384;
+
+// Bits beside the pair in a tile's word (pairs are below 2^29): of a pair whose
+// tiles' sums the encode keeps, and a tile the match added.  In the word, so that
+// the encode need not hold the pair's counts over a tile for them (34.6 against
+// 37.3 us at 1 M agents).
+constexpr u32 kLarge = 1u << 31, kAdded = 1u << 30, kPairMask = kAdded - 1u;
 
 // Per-pair facts, one 64-byte line.
 struct __align__(16) TilePair {
@@ -108,7 +115,7 @@ struct TileArgs {
   EncArgs E;
   DecArgs D;
   TilePair* pair;
-  u32* unit_pair;       // pair of each tile
+  u32* unit_pair;       // pair of each tile, and kLarge, kAdded
   u32 unit_cap;         // tiles there is room for
   u32* unit_first;      // [P] first tile of each pair
   u64* setup_state;     // look-back states of the setup (zero between calls)
@@ -460,7 +467,8 @@ __device__ __forceinline__ void add_new_tiles(const TileArgs& A, const TilePair&
   }
   group_sync<T>();
   const u64 at = (u64)A.scal[TS_UNITS] + *s_first;
-  for (u32 i = group_thread<T>(); i < more && at + i < A.unit_cap; i += T) A.unit_pair[at + i] = p;
+  for (u32 i = group_thread<T>(); i < more && at + i < A.unit_cap; i += T)
+    A.unit_pair[at + i] = p | kAdded | (more > kGroupMin ? kLarge : 0u);
 }
 
 // One tile of a big pair's message: whether its ids ascend (up to the next
@@ -714,8 +722,12 @@ __device__ __forceinline__ void map_tiles(const TileArgs& A) {
   }
   u32 p = lo;
   for (u64 u = a + lane; u < b; u += 32) {
-    while (p + 1 < (u32)A.P && A.unit_first[p + 1] <= u) ++p;
-    A.unit_pair[u] = p;
+    u32 end = (u32)units;
+    while (p + 1 < (u32)A.P && (end = A.unit_first[p + 1]) <= u) {
+      ++p;
+      end = (u32)units;
+    }
+    A.unit_pair[u] = p | (end - A.unit_first[p] > kGroupMin ? kLarge : 0u);
   }
 }
 
@@ -979,7 +991,7 @@ __global__ void __launch_bounds__(kT, kPerSm) codec_sizes_kernel(TileArgs A) {
   u32 u = blockIdx.x * (kT / 32) + (threadIdx.x >> 5);
   u32 p_next = u < n ? A.unit_pair[u] : 0u;
   for (; u < n; u += stride) {
-    const u32 p = p_next;
+    const u32 p = p_next & kPairMask;
     if (u + stride < n) p_next = A.unit_pair[u + stride];
     const TilePair x = A.pair[p];
     const u32 tile = u - x.unit0;
@@ -1055,13 +1067,10 @@ __device__ __forceinline__ void copies_wait() {  // all but the last N groups
   asm volatile("cp.async.wait_group %0;" : : "n"(N) : "memory");
 }
 
-// The tiles of the call: `planned` by the setup, the match's behind them.
-struct TileCount {
-  u32 planned, all;
-};
-__device__ __forceinline__ TileCount tile_count(const TileArgs& A) {
-  const u32 planned = A.scal[TS_UNITS], all = planned + A.scal[TS_EXTRA];
-  return TileCount{planned, all < A.unit_cap ? all : A.unit_cap};
+// The tiles of the call: those the setup planned, the match's behind them.
+__device__ __forceinline__ u32 tile_count(const TileArgs& A) {
+  const u32 all = A.scal[TS_UNITS] + A.scal[TS_EXTRA];
+  return all < A.unit_cap ? all : A.unit_cap;
 }
 
 // What a tile's warp needs of its pair.
@@ -1069,18 +1078,26 @@ struct Tile {
   TilePair x;
   u32 p, local;
   u32 n_new;
-  u32 nnu;      // new-record tiles, the added ones among them
-  u32 added0;   // the first of those in the list
 };
 
-__device__ __forceinline__ Tile tile_of(const TileArgs& A, const TileCount& n, u32 u, u32 p) {
+// A pair's added tiles: the first's place in the list, and how many.  Read where
+// they matter only: a slot tile does not wait for them.
+struct Added {
+  u32 first, n;
+};
+__device__ __forceinline__ Added added_tiles(const TileArgs& A, u32 p) {
+  const u64 extra = A.tot[(u64)p * PT_COUNT + PT_EXTRA];
+  return Added{A.scal[TS_UNITS] + (u32)extra, (u32)(extra >> 32)};
+}
+
+// word: unit_pair[u].
+__device__ __forceinline__ Tile tile_of(const TileArgs& A, u32 u, u32 word) {
+  const u32 p = word & kPairMask;
   Tile t;
   t.p = p;
   t.x = A.pair[p];
-  const u64 extra = A.tot[(u64)p * PT_COUNT + PT_EXTRA];
-  t.nnu = t.x.nnu + (u32)(extra >> 32);
-  t.added0 = n.planned + (u32)extra;
-  t.local = u < n.planned ? u - t.x.unit0 : t.x.nst + t.x.nnu + (u - t.added0);
+  t.local = u - t.x.unit0;
+  if (word & kAdded) t.local = t.x.nst + t.x.nnu + (u - added_tiles(A, p).first);
   t.n_new = t.x.m - (u32)A.tot[(u64)p * PT_COUNT + PT_MATCHED];
   return t;
 }
@@ -1215,15 +1232,16 @@ __global__ void __launch_bounds__(kT, kEncPerSm) codec_encode_kernel(TileArgs A)
   const u32 r8 = lane >> 2, q = lane & 3;  // this lane's record of each eight, and its piece
   uint8_t* st = dyn + warp * (kStage + 2 * kRows);
   uint8_t* rows = st + kStage;
-  const TileCount n = tile_count(A);
+  const u32 n = tile_count(A);
   const u32 shift = A.scal[TS_SHIFT];
   const u32 epoch = *E.epoch;
   const u32 stride = gridDim.x * kWarps;
   u32 u = blockIdx.x * kWarps + warp;
-  u32 p_next = u < n.all ? A.unit_pair[u] : 0u;
-  for (; u < n.all; u += stride) {
-    const Tile t = tile_of(A, n, u, p_next);
-    if (u + stride < n.all) p_next = A.unit_pair[u + stride];
+  u32 p_next = u < n ? A.unit_pair[u] : 0u;
+  for (; u < n; u += stride) {
+    const u32 word = p_next;
+    const Tile t = tile_of(A, u, word);
+    if (u + stride < n) p_next = A.unit_pair[u + stride];
     const u32 p = t.p;
     u32* codes = reinterpret_cast<u32*>(E.wire + t.x.w_off + kHdrBytes);
     if (lane == 0) *reinterpret_cast<uint4*>(st) = make_uint4(0u, 0u, 0u, 0u);
@@ -1309,7 +1327,7 @@ __global__ void __launch_bounds__(kT, kEncPerSm) codec_encode_kernel(TileArgs A)
       // new records: rank i's code and new-reference record have known places
       const u64 matched = (u64)t.x.m - t.n_new;
       u32 lo, hi;
-      new_range(t.n_new, t.nnu, t.local - t.x.nst, shift, &lo, &hi);
+      new_range(t.n_new, t.x.nnu + added_tiles(A, p).n, t.local - t.x.nst, shift, &lo, &hi);
       out = payload_place(A, t, matched + lo);
       for (u32 i0 = lo; i0 < hi; i0 += 32) {
         const u32 hits = hi - i0 >= 32 ? 0xFFFFFFFFu : (1u << (hi - i0)) - 1u;
@@ -1350,7 +1368,7 @@ __global__ void __launch_bounds__(kT, kEncPerSm) codec_encode_kernel(TileArgs A)
       *reinterpret_cast<uint4*>(out + (bytes & ~15u)) = *reinterpret_cast<const uint4*>(st);
     if (lane == 0) {
       A.bytes[u] = bytes;
-      if (t.x.nst + t.nnu > kGroupMin) atomicAdd(A.group + u / kTileGroup, bytes);
+      if (word & kLarge) atomicAdd(A.group + u / kTileGroup, bytes);
     }
     __syncwarp();
   }
@@ -1437,14 +1455,14 @@ __global__ void __launch_bounds__(kT, kPerSm) codec_wire_kernel(TileArgs A) {
   chain_begin();
   const EncArgs& E = A.E;
   const u32 warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const TileCount n = tile_count(A);
+  const u32 n = tile_count(A);
   const u32 shift = A.scal[TS_SHIFT];
   const u32 stride = gridDim.x * kWarps;
   u32 u = blockIdx.x * kWarps + warp;
-  u32 p_next = u < n.all ? A.unit_pair[u] : 0u;
-  for (; u < n.all; u += stride) {
-    const Tile t = tile_of(A, n, u, p_next);
-    if (u + stride < n.all) p_next = A.unit_pair[u + stride];
+  u32 p_next = u < n ? A.unit_pair[u] : 0u;
+  for (; u < n; u += stride) {
+    const Tile t = tile_of(A, u, p_next);
+    if (u + stride < n) p_next = A.unit_pair[u + stride];
     const u32 own = A.bytes[u];
     u64 record;
     bool last;
@@ -1453,14 +1471,14 @@ __global__ void __launch_bounds__(kT, kPerSm) codec_wire_kernel(TileArgs A) {
       last = t.n_new == 0 && t.local + 1 == t.x.nst;
     } else {
       u32 lo, hi;
-      new_range(t.n_new, t.nnu, t.local - t.x.nst, shift, &lo, &hi);
+      new_range(t.n_new, t.x.nnu + added_tiles(A, t.p).n, t.local - t.x.nst, shift, &lo, &hi);
       record = (u64)t.x.m - t.n_new + lo;
       // an entryless pair's message is its header
       last = hi == t.n_new && (lo < hi || (t.n_new == 0 && t.x.r == 0 && t.local == 0));
     }
     const u32 planned = t.x.nst + t.x.nnu, own_planned = t.local < planned ? t.local : planned;
     u64 pre = tile_bytes(A, t.x.unit0, t.x.unit0 + own_planned);
-    if (t.local > planned) pre += tile_bytes(A, t.added0, t.added0 + (t.local - planned));
+    if (t.local > planned) pre += tile_bytes(A, u - (t.local - planned), u);
     pre = warp_sum(pre);
     if (lane == 0) A.place[u] = pre;
     uint8_t* pay = E.wire + t.x.w_off + kHdrBytes + 4 * ((u64)t.x.r + t.n_new);
@@ -1490,14 +1508,14 @@ __global__ void __launch_bounds__(kT, kDecPerSm) codec_decode_kernel(TileArgs A)
   const u32 r8 = lane >> 2, q = lane & 3;  // this lane's record of each eight, and its piece
   uint8_t* stages = dyn + warp * (2 * kStage + 2 * kRows);
   uint8_t* rows = stages + 2 * kStage;
-  const TileCount tc = tile_count(A);
+  const u32 n_units = tile_count(A);
   const u32 shift = A.scal[TS_SHIFT];
   const u32 stride = gridDim.x * kWarps;
   u32 u = blockIdx.x * kWarps + warp;
-  u32 p_next = u < tc.all ? A.unit_pair[u] : 0u;
-  for (; u < tc.all; u += stride) {
-    const Tile t = tile_of(A, tc, u, p_next);
-    if (u + stride < tc.all) p_next = A.unit_pair[u + stride];
+  u32 p_next = u < n_units ? A.unit_pair[u] : 0u;
+  for (; u < n_units; u += stride) {
+    const Tile t = tile_of(A, u, p_next);
+    if (u + stride < n_units) p_next = A.unit_pair[u + stride];
     const u32 p = t.p;
     const u64 m = t.x.m, ns = t.x.r, n = ns + t.n_new;
     u32 lo, hi, base = 0;  // this tile's entries [lo, hi) behind the pair's entry `base`
@@ -1507,7 +1525,7 @@ __global__ void __launch_bounds__(kT, kDecPerSm) codec_decode_kernel(TileArgs A)
       hi = t.x.r - lo < (1u << shift) ? t.x.r : lo + (1u << shift);
       pos = A.before[u];
     } else {
-      new_range(t.n_new, t.nnu, t.local - t.x.nst, shift, &lo, &hi);
+      new_range(t.n_new, t.x.nnu + added_tiles(A, p).n, t.local - t.x.nst, shift, &lo, &hi);
       base = t.x.r;
       pos = m - t.n_new + lo;
     }
