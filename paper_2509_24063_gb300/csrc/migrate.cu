@@ -200,16 +200,12 @@ __device__ __forceinline__ BoxWords box_words(u32 s, const SmemGrid& g,
   return w;
 }
 
-// The exact way, out of line: the box of agent a (of boxes [s_lo, s_hi]) in
-// *s, its next box as the result (-1 outside the domain).
-__device__ __noinline__ int exact_owner(u64 bx, u64 by, u64 bz, u64 a,
-                                        const u64* __restrict__ box_off, u32 s_lo, u32 s_hi,
-                                        const SmemGrid& g, u32* s) {
-  const u32 b = box_search(box_off, s_lo, s_hi, a);
-  *s = b;
-  BoxBounds bb;
-  box_bounds(b, g, &bb);
-  return inside_box(bx, by, bz, bb) ? (int)b : locate_agent(bx, by, bz, g);
+// The exact way, out of line: the next box of an agent (-1 outside the domain).
+// Its own box is found as any other: most that come here have left it, and its
+// edges cost four divisions (16 M agents, all regrouped from one box: 560 -> 477
+// us; 100 M of which few leave: 442 -> 418, for the registers it saves).
+__device__ __noinline__ int exact_owner(u64 bx, u64 by, u64 bz, const SmemGrid& g) {
+  return locate_agent(bx, by, bz, g);
 }
 
 // The coordinates of agents a0 and a0 + 1 (zeros past the end).
@@ -241,8 +237,8 @@ __device__ __forceinline__ void load_position_pair(const u64* __restrict__ x,
 //
 // Bound: the reads of x, y and z.  With both 64-bit comparisons of every axis
 // for every agent, a block per eight warp tiles and the loads behind each
-// tile's box search it took 645 us for 100 M agents, now 444 (80 % of the
-// measured copy rate; 2, 3 and 5 blocks per SM: 467, 569 and 489).
+// tile's box search it took 645 us for 100 M agents, now 418 (85 % of the
+// measured copy rate; at 444, 2, 3 and 5 blocks per SM took 467, 569 and 489).
 __global__ void __launch_bounds__(kClassifyThreads, kCountBlocks)
     mig_count_kernel(const u64* __restrict__ x, const u64* __restrict__ y,
                      const u64* __restrict__ z, u64 n, const u64* __restrict__ box_off,
@@ -295,7 +291,8 @@ __global__ void __launch_bounds__(kClassifyThreads, kCountBlocks)
         bool leave = false;
         u32 s = 0, key = 0;
         if (exact[q]) {
-          const int d = exact_owner(v[0][q], v[1][q], v[2][q], a0 + q, box_off, s_lo, s_hi, sg, &s);
+          s = box_search(box_off, s_lo, s_hi, a0 + q);
+          const int d = exact_owner(v[0][q], v[1][q], v[2][q], sg);
           if (d < 0) {
             bad = true;  // stays in its box; TERA_EDOMAIN
           } else if ((u32)d != s) {
