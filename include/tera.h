@@ -163,9 +163,10 @@ tera_status tera_ctx_reserve(tera_ctx* ctx, int64_t max_agents, uint64_t max_rec
 
 /* Limit, in microseconds (0 .. 60000000; 1000000 when the context is made), of a
  * wait inside one of the context's kernels for another block of the same launch.
- * Such a wait ends by itself; one that takes longer is given up, latches
- * TERA_ETIMEOUT, and the call leaves its lists empty and its messages unwritten.
- * 0: any wait is given up.  Holds for the calls after this one (a captured graph
+ * Such a wait ends by itself; one that takes longer is given up and latches
+ * TERA_ETIMEOUT.  The call's outputs are then not to be used: its lists are empty,
+ * its messages unwritten or without matches (training returns TERA_ETIMEOUT before
+ * it trains); nothing outside them is touched.  0: any wait is given up.  Holds for the calls after this one (a captured graph
  * keeps the limit it was captured with); tera_tune.wait_limit_us is that of the
  * persistent launch. */
 tera_status tera_ctx_wait_limit(tera_ctx* ctx, int64_t limit_us);
@@ -312,7 +313,8 @@ tera_status tera_delta_decode_pred(tera_ctx* ctx, const uint8_t* wire, const uin
                                    uint64_t recv_capacity_units, uint64_t* recv_off,
                                    const tera_predictor* pred, void* stream);
 
-/* Training of the predictor on the GPU (float32, deterministic).
+/* Training of the predictor on the GPU (float32; deterministic on one GPU model:
+ * the order of the sums depends on the batch and on the number of SMs).
  * samples: n records of 12 floats as written by the encoder (records with a
  * zero valid flag are skipped; the valid ones are compacted in order).
  * tera_mlp_grad: gradient (4931 floats) of the mean squared error

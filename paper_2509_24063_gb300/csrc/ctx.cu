@@ -196,7 +196,9 @@ tera_status check_launch(tera_ctx* ctx, const char* name, cudaStream_t s) {
 
 bool capturing(cudaStream_t s) {
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  return cudaStreamIsCapturing(s, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cs) == cudaSuccess) return cs != cudaStreamCaptureStatusNone;
+  cudaGetLastError();  // (another stream's capture forbids the question) not a launch's error
+  return true;
 }
 
 int grid_for(tera_ctx* ctx, int blocks_per_sm) { return ctx->num_sms * blocks_per_sm; }

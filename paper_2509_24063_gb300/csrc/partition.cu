@@ -267,7 +267,8 @@ __device__ __forceinline__ u64* sort_states(u64* head, u32 pass, u64 tiles, u32 
 }
 
 // Entries of a tile: kSortTile, or a single round of it while such tiles are
-// at most two per SM, so that a short list is still spread over the SMs (100
+// about two per SM of the 152 at most (a constant, as the host sizes the scratch by
+// it without a device), so that a short list is still spread over the SMs (100
 // thousand agents, 70 K entries: 103 -> 98 us per iteration.  Up to four per SM
 // 1 M agents, whose tiles then wait for one another longer, lose what they
 // gain: 306 -> 308).
@@ -328,7 +329,8 @@ __global__ void __launch_bounds__(kSortThreads)
 // other by resident blocks.  A tile counts its digits, publishes the counts,
 // and while its entries are ranked the tiles before it publish theirs; thread
 // d then walks back over digit d's counts (eight tiles' in flight) to the
-// nearest inclusive sum.  A histogram launch and a scan of three per pass did
+// nearest inclusive sum (A. Adinets and D. Merrill, "Onesweep: A Faster Least
+// Significant Digit Radix Sort for GPUs", 2022).  A histogram launch and a scan of three per pass did
 // this before: 178 + 58 us a pass at 16.6 M entries.  The tile's input
 // (keys, entry indices when given, agents) is first copied into shared memory
 // in input order by cp.async in 16-byte pieces (a ragged end, or unaligned
