@@ -1897,8 +1897,11 @@ static tera_status batched_impl(
   // this form's scratch, and outside a capture the other's if it can be had, so
   // that a call with or without a schedule may be captured after an eager call
   // of either kind
-  if ((st = tune ? ensure_batched(ctx) : ensure_tiles(ctx)) != TERA_OK) return st;
-  if (!capturing(s)) (void)(tune ? ensure_tiles(ctx) : ensure_batched(ctx));
+  if ((st = tune ? ensure_batched(ctx, s) : ensure_tiles(ctx, s)) != TERA_OK) return st;
+  if (ctx->b_both != ctx->cap_records && !capturing(s)) {
+    ctx->b_both = ctx->cap_records;  // (asked for once per capacity)
+    (void)(tune ? ensure_tiles(ctx, s) : ensure_batched(ctx, s));
+  }
   if (!ctx->pair_info) return TERA_EINVAL;  // allocated with the context
 
   EncArgs E;
@@ -1966,7 +1969,7 @@ static tera_status batched_impl(
   B.part = 0;
 
   if (PR) {
-    if ((st = ensure_pred(ctx)) != TERA_OK) return st;
+    if ((st = ensure_pred(ctx, s)) != TERA_OK) return st;
     if (enc_pred) {
       if ((enc_pred->hist_prev != nullptr) != (ref_prev != nullptr)) return TERA_EINVAL;
       fill_pred(ctx, &E.pr, enc_pred, ctx->cseg_enc);

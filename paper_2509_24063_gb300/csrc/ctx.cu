@@ -34,14 +34,6 @@ tera_status alloc_dev(T*& p, size_t count) {
   return TERA_OK;
 }
 
-// The device has done everything the host asked for.  Work on the default stream
-// (a cudaMemset, the last part of a cudaMemcpy from pageable memory) is not
-// waited for by a caller's non-blocking stream, so what clears or fills new
-// scratch ends with this.
-tera_status settled() {
-  return cudaDeviceSynchronize() == cudaSuccess ? TERA_OK : TERA_ECUDA;
-}
-
 // ---- generic exclusive scan of u32 values ----
 //
 // One launch: a block scans kScanChunk values and finds the sum before them by
@@ -249,7 +241,6 @@ tera_status ensure_agents(tera_ctx* ctx, int64_t n, cudaStream_t s) {
 }
 
 tera_status ensure_records(tera_ctx* ctx, uint64_t cap, cudaStream_t s) {
-  (void)s;
   if (cap <= ctx->cap_records && ctx->seg) return TERA_OK;
   cudaDeviceSynchronize();
   u64 c = cap < 1024 ? 1024 : cap;
@@ -267,11 +258,13 @@ tera_status ensure_records(tera_ctx* ctx, uint64_t cap, cudaStream_t s) {
   if ((st = alloc_dev(ctx->matched, c)) != TERA_OK) return st;
   if ((st = alloc_dev(ctx->slot_src, c)) != TERA_OK) return st;
   if ((st = alloc_dev(ctx->seg, 2 * c + 2 * ctx->n_pairs)) != TERA_OK) return st;
-  // epoch 0 is never current, so zeroed segments and flags are empty
-  cudaMemset(ctx->seg, 0, sizeof(U64x2) * (2 * c + 2 * ctx->n_pairs));
-  cudaMemset(ctx->matched, 0, sizeof(u32) * c);
+  // epoch 0 is never current, so zeroed segments and flags are empty.  (Here and
+  // below new scratch is cleared and filled on the caller's stream: a non-blocking
+  // one does not wait for the default stream's work.)
+  cudaMemsetAsync(ctx->seg, 0, sizeof(U64x2) * (2 * c + 2 * ctx->n_pairs), s);
+  cudaMemsetAsync(ctx->matched, 0, sizeof(u32) * c, s);
   ctx->cap_records = c;
-  return settled();
+  return TERA_OK;
 }
 
 tera_status ensure_units(tera_ctx* ctx, uint64_t cap, cudaStream_t s) {
@@ -287,7 +280,7 @@ tera_status ensure_units(tera_ctx* ctx, uint64_t cap, cudaStream_t s) {
   return TERA_OK;
 }
 
-tera_status ensure_batched(tera_ctx* ctx) {
+tera_status ensure_batched(tera_ctx* ctx, cudaStream_t s) {
   const u64 P = ctx->n_pairs;
   // work items: one per pair, plus at most (blocks + pairs) for the teams
   const u64 items = 2 * P + (u64)ctx->num_sms * 16 + 64;
@@ -308,17 +301,17 @@ tera_status ensure_batched(tera_ctx* ctx) {
     if ((st = alloc_dev(ctx->b_tbase, P)) != TERA_OK) return st;
     // block sums of the setup's first launch: 4 words per block of 1024 pairs
     if ((st = alloc_dev(ctx->b_part, 4 * (P / 1024 + 1))) != TERA_OK) return st;
-    cudaMemset(ctx->b_scalars, 0, 6 * sizeof(u64));
+    cudaMemsetAsync(ctx->b_scalars, 0, 6 * sizeof(u64), s);
   }
   if ((st = alloc_dev(ctx->b_items, items)) != TERA_OK) return st;
   if ((st = alloc_dev(ctx->b_tsum, tsum)) != TERA_OK) return st;
   ctx->b_items_cap = items;
   ctx->b_tsum_cap = tsum;
-  return settled();
+  return TERA_OK;
 }
 
 // One allocation holds every list, so that a first call pays for one.
-tera_status ensure_tiles(tera_ctx* ctx) {
+tera_status ensure_tiles(tera_ctx* ctx, cudaStream_t s) {
   if (ctx->t_cap >= ctx->cap_records && ctx->t_block) return TERA_OK;
   cudaDeviceSynchronize();
   const u64 P = ctx->n_pairs, cap = ctx->cap_records;
@@ -354,26 +347,29 @@ tera_status ensure_tiles(tera_ctx* ctx) {
   if (st != TERA_OK) return st;
   base = ctx->t_block;
   lay();
-  cudaMemset(ctx->t_part, 0, sizeof(u64) * (4 * (P / 1024 + 1) + 1));
+  cudaMemsetAsync(ctx->t_part, 0, sizeof(u64) * (4 * (P / 1024 + 1) + 1), s);
   ctx->t_cap = cap;
-  return settled();
+  return TERA_OK;
 }
 
 // The lists and the payload's place of an encode over tiles (64 bytes a record:
 // 1.06 GB for 16.6 M).  The place is only taken while it is at most an eighth of
 // the memory that is free: the launches that do without it leave a nearly full
-// device to its user.  A capacity that was refused is not asked for again on
-// every call.
-bool ensure_encode_tiles(tera_ctx* ctx) {
+// device to its user (a small place is not worth the question).  A capacity that
+// was refused is not asked for again on every call.
+constexpr u64 kPlaceUnasked = 64ull << 20;
+bool ensure_encode_tiles(tera_ctx* ctx, cudaStream_t s) {
   if (ctx->t_refused == ctx->cap_records) return false;
   ctx->t_refused = ctx->cap_records;
-  if (ensure_tiles(ctx) != TERA_OK) return false;
+  if (ensure_tiles(ctx, s) != TERA_OK) return false;
   if (!ctx->t_scratch || ctx->t_scratch_cap < ctx->cap_records) {
     const u64 bytes = (ctx->cap_records + ctx->n_pairs + 1) * (u64)kRecBytes;
-    size_t free = 0, all = 0;
-    if (cudaMemGetInfo(&free, &all) != cudaSuccess || bytes > free / 8) {
-      cudaGetLastError();
-      return false;
+    if (bytes > kPlaceUnasked) {
+      size_t free = 0, all = 0;
+      if (cudaMemGetInfo(&free, &all) != cudaSuccess || bytes > free / 8) {
+        cudaGetLastError();
+        return false;
+      }
     }
     cudaDeviceSynchronize();
     ctx->t_scratch_cap = 0;
@@ -388,7 +384,7 @@ bool encode_tiles_ready(tera_ctx* ctx, cudaStream_t s) {
   const bool have = ctx->t_block && ctx->t_cap >= ctx->cap_records && ctx->t_scratch &&
                     ctx->t_scratch_cap >= ctx->cap_records;
   if (have) return true;
-  return !capturing(s) && ensure_encode_tiles(ctx);
+  return !capturing(s) && ensure_encode_tiles(ctx, s);
 }
 
 tera_status ensure_migrate(tera_ctx* ctx, uint64_t n, uint64_t leavers) {
@@ -468,7 +464,7 @@ void cell_thresholds(double lo, double hi, double w, uint64_t n, uint64_t* T) {
 }
 
 // The predictor's cell threshold tables (once per context).
-static tera_status ensure_cell_tables(tera_ctx* ctx) {
+static tera_status ensure_cell_tables(tera_ctx* ctx, cudaStream_t s) {
   if (ctx->d_ckeys) return TERA_OK;
   uint64_t total = 0, off[3] = {0, 0, 0};
   for (int a = 0; a < 3; ++a) {
@@ -482,7 +478,8 @@ static tera_status ensure_cell_tables(tera_ctx* ctx) {
       cell_thresholds(ctx->grid.lo[a], ctx->grid.hi[a], ctx->grid.w, ctx->ncell[a], h.data() + off[a]);
   tera_status st = alloc_dev(ctx->d_ckeys, total);
   if (st != TERA_OK) return st;
-  if (cudaMemcpy(ctx->d_ckeys, h.data(), 8 * total, cudaMemcpyHostToDevice) != cudaSuccess)
+  // (from pageable memory: taken over before the call returns)
+  if (cudaMemcpyAsync(ctx->d_ckeys, h.data(), 8 * total, cudaMemcpyHostToDevice, s) != cudaSuccess)
     return TERA_ECUDA;
   for (int a = 0; a < 3; ++a) {
     ctx->ck[a] = ctx->ncell[a] <= kCellTableMax ? ctx->d_ckeys + off[a] : nullptr;
@@ -492,13 +489,13 @@ static tera_status ensure_cell_tables(tera_ctx* ctx) {
   return TERA_OK;
 }
 
-tera_status ensure_pred(tera_ctx* ctx) {
+tera_status ensure_pred(tera_ctx* ctx, cudaStream_t s) {
   const u64 cap = ctx->cap_records, P = ctx->n_pairs;
   if (ctx->cseg_enc && ctx->pred_cap >= cap && ctx->unit_res && ctx->unit_res_cap >= ctx->cap_units)
     return TERA_OK;
   cudaDeviceSynchronize();
   tera_status st;
-  if ((st = ensure_cell_tables(ctx)) != TERA_OK) return st;
+  if ((st = ensure_cell_tables(ctx, s)) != TERA_OK) return st;
   if ((st = alloc_dev(ctx->cseg_enc, 2 * (2 * cap + 2 * P))) != TERA_OK) return st;
   if ((st = alloc_dev(ctx->cseg_dec, 2 * (2 * cap + 2 * P))) != TERA_OK) return st;
   if ((st = alloc_dev(ctx->pscr, 4 * cap)) != TERA_OK) return st;
@@ -506,7 +503,7 @@ tera_status ensure_pred(tera_ctx* ctx) {
   if ((st = alloc_dev(ctx->unit_res, ctx->cap_units)) != TERA_OK) return st;
   ctx->pred_cap = cap;
   ctx->unit_res_cap = ctx->cap_units;
-  return settled();
+  return TERA_OK;
 }
 
 }  // namespace tera
@@ -826,13 +823,18 @@ tera_status tera_ctx_reserve(tera_ctx* ctx, int64_t max_agents, uint64_t max_rec
   cudaSetDevice(ctx->device);
   tera_status st = ensure_agents(ctx, max_agents, 0);
   if (st != TERA_OK) return st;
-  st = ensure_records(ctx, max_records, 0);
-  if (st != TERA_OK) return st;
-  st = ensure_units(ctx, 2 * (max_records / kCodecTile) + 4 * ctx->n_pairs + 16, 0);
-  if (st != TERA_OK) return st;
-  ctx->t_refused = 0;
-  (void)ensure_encode_tiles(ctx);  // an encode without it takes the launches that need none
-  return TERA_OK;
+  const u64 records = ctx->cap_records, listed = ctx->t_cap;
+  if ((st = ensure_records(ctx, max_records, 0)) == TERA_OK)
+    st = ensure_units(ctx, 2 * (max_records / kCodecTile) + 4 * ctx->n_pairs + 16, 0);
+  if (st == TERA_OK) {
+    ctx->t_refused = 0;
+    (void)ensure_encode_tiles(ctx, 0);  // an encode without it takes the launches that need none
+  }
+  // new scratch was cleared on the default stream, which the callers' do not wait for
+  if ((ctx->cap_records != records || ctx->t_cap != listed) &&
+      cudaDeviceSynchronize() != cudaSuccess && st == TERA_OK)
+    st = TERA_ECUDA;
+  return st;
 }
 
 tera_status tera_ctx_wait_limit(tera_ctx* ctx, int64_t limit_us) {

@@ -198,7 +198,7 @@ static tera_status decode_impl(tera_ctx* ctx, const uint8_t* wire, const uint64_
   A.st = ctx->d_status;
   const bool PR = pred != nullptr;
   if (PR) {
-    if ((st = ensure_pred(ctx)) != TERA_OK) return st;
+    if ((st = ensure_pred(ctx, s)) != TERA_OK) return st;
     if (pred->params && ((uintptr_t)pred->params & 3u)) return TERA_EINVAL;
     if (((uintptr_t)pred->hist_prev | (uintptr_t)pred->hist_next) & 15u) return TERA_EINVAL;
     if (pred->hist_prev && !ref_prev) return TERA_EINVAL;

@@ -134,6 +134,7 @@ struct tera_ctx {
   uint8_t* t_block;        // the allocation they lie in
   uint8_t* t_scratch;      // [64 * (t_scratch_cap + P)] packed payload of an encode without decode
   uint64_t t_scratch_cap;
+  uint64_t b_both;         // record capacity the scratch of both forms was asked for (0: none)
   uint64_t t_refused;      // record capacity whose encode scratch could not be had (0: none)
   tera::u64* t_pair;       // [P * 8] per-pair facts
   uint32_t* t_unit_pair;   // [t_units] pair of each tile
@@ -236,14 +237,14 @@ bool capturing(cudaStream_t s);
 // units_total[1] flags an aborted call).
 tera_status launch_unit_map(tera_ctx* ctx, u32 p0, u64 npr, cudaStream_t s);
 // Scratch of the learned predictor for the current record capacity.
-tera_status ensure_pred(tera_ctx* ctx);
+tera_status ensure_pred(tera_ctx* ctx, cudaStream_t s);
 // Scratch of the batched codec.
-tera_status ensure_batched(tera_ctx* ctx);
+tera_status ensure_batched(tera_ctx* ctx, cudaStream_t s);
 // Scratch of the batched codec over tiles.
-tera_status ensure_tiles(tera_ctx* ctx);
+tera_status ensure_tiles(tera_ctx* ctx, cudaStream_t s);
 // Scratch of an encode over tiles for the current record capacity; false when it
 // cannot be had.
-bool ensure_encode_tiles(tera_ctx* ctx);
+bool ensure_encode_tiles(tera_ctx* ctx, cudaStream_t s);
 // Whether an encode call can run over tiles: its scratch exists, or could be
 // allocated now (not inside a stream capture, and there is memory for it).
 bool encode_tiles_ready(tera_ctx* ctx, cudaStream_t s);
