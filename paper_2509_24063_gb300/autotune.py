@@ -1,5 +1,6 @@
 """Autotuner of the batched codec's schedule: no schedule (None: the codec over
-warp tiles, several launches that size themselves), or the persistent launch
+warp tiles, several launches that size themselves; the fastest at every size
+measured, 500 to 100 M agents), or the persistent launch
 with a tile/block size and resident blocks per SM (each block's shared-memory
 match table takes what its share of the SM's shared memory allows).
 

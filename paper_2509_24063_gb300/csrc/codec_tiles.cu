@@ -1,13 +1,13 @@
 // Batched codec over tiles: steps a3-a5 (paper Sec. 2.3, steps B, C and D) for
-// every pair of one iteration, as launches over tiles of kT entries that know
-// nothing of the pairs' sizes:
+// every pair of one iteration, as launches over tiles of 32 to 256 entries; only
+// the match has a block or a warp a pair, and parts the large ones:
 //
 //   setup   per-pair facts, wire slabs and the lists of tiles
 //   match   one block (a warp for a small pair) per pair: the message record of
-//           every reference slot (ids in shared memory), the matches before each tile and the list
-//           of the records no slot took; a big pair (more than kTableMax records
-//           or kBlockSlots slots) is only asked here, a tile each, whether its ids ascend, and
-//           matched by
+//           every reference slot (ids in shared memory), the matches before each
+//           tile and the list of the records no slot took; a big pair (more than
+//           kTableMax records, or kBlockSlots slots and twice a block's share) is
+//           only asked here, a tile each, whether its ids ascend, and matched by
 //   bigmatch  (tiles of such pairs; does nothing without them): by bisection
 //           over ascending ids, else in a global hash segment that its tiles
 //           index first
@@ -29,9 +29,9 @@
 // persistent launch of batched.cu, used for an explicit schedule) pays every
 // step's memory latency once per tile of every pair, one after the other, and
 // the largest pair is the launch's length.  Measured, whole codec: uniform 100
-// M agents (16.6 M records) 1.98 -> 1.43 ms, of which encode 675 us (3.65 GB,
-// 80 % of the measured copy rate), decode 465 us (2.4 GB), match 179, wire 88,
-// setup 19; 16 M agents kept box by box 0.93 -> 0.62 ms; a pair of 1.1 M
+// M agents (16.6 M records) 1.98 -> 1.45 ms, of which encode 690 us (3.58 GB,
+// 77 % of the measured copy rate), decode 467 us (2.3 GB), match 179, wire 95,
+// setup 17; 16 M agents kept box by box 0.93 -> 0.62 ms; a pair of 1.1 M
 // records among 6.5 M: 3.3 -> 0.8 ms; 6.3 K records in 12 pairs: 92 -> 60 us.
 // A look-back over the tiles in place of the second copy of the payload
 // (tiles claimed in order, sums published) left encode and decode at 1.16 ms
