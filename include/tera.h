@@ -166,9 +166,9 @@ tera_status tera_ctx_reserve(tera_ctx* ctx, int64_t max_agents, uint64_t max_rec
  * Such a wait ends by itself; one that takes longer is given up and latches
  * TERA_ETIMEOUT.  The call's outputs are then not to be used: its lists are empty,
  * its messages unwritten or without matches (training returns TERA_ETIMEOUT before
- * it trains); nothing outside them is touched.  0: any wait is given up.  Holds for the calls after this one (a captured graph
- * keeps the limit it was captured with); tera_tune.wait_limit_us is that of the
- * persistent launch. */
+ * it trains); nothing outside them is touched.  0: any wait is given up.  Holds for
+ * the calls after this one (a captured graph keeps the limit it was captured with);
+ * tera_tune.wait_limit_us is that of the persistent launch. */
 tera_status tera_ctx_wait_limit(tera_ctx* ctx, int64_t limit_us);
 
 /* Step a1 (Sec. 2.1 "Aura Update"): owner box and aura mask of every agent,
@@ -331,8 +331,8 @@ tera_status tera_mlp_train(tera_ctx* ctx, const float* samples, uint64_t n, floa
 
 /* Schedule of the batched codec's persistent launch (picked by the autotuner;
  * outputs do not depend on it; no schedule, a NULL tune, runs the codec over
- * warp tiles instead, see tera_codec_batched): threads per block = entries per tile (128, 256, 512 or
- * 1024), blocks per SM of the persistent launch (1..16, block x blocks <=
+ * warp tiles instead, see tera_codec_batched): threads per block = entries per
+ * tile (128, 256, 512 or 1024), blocks per SM of the persistent launch (1..16, block x blocks <=
  * 2048), and the largest message (records) matched in a block's shared-memory
  * hash table: 0 = as large as the shared memory left to the block allows, else
  * a power of two >= 32 (smaller when it does not fit); larger messages use the

@@ -130,8 +130,8 @@ __global__ void __launch_bounds__(kClassifyThreads)
     pack_runs_kernel(SoaPtrs soa, u64 n, const int* __restrict__ owner,
                      const u32* __restrict__ mask, const u64* __restrict__ run_base,
                      const u64* __restrict__ packable, const u32* __restrict__ ent_dest,
-                     const u64* __restrict__ pair_off, u64 P, uint8_t* __restrict__ arena, u64 arena_units, u32 class_id, DevStatus* st,
-                     u64* __restrict__ rec_ids) {
+                     const u64* __restrict__ pair_off, u64 P, uint8_t* __restrict__ arena,
+                     u64 arena_units, u32 class_id, DevStatus* st, u64* __restrict__ rec_ids) {
   chain_begin();
   const u64 E = pair_off[P];
   if (E + P > arena_units) {
