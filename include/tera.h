@@ -161,6 +161,10 @@ uint64_t tera_n_pairs(const tera_ctx* ctx);
  * an eighth of the device memory then free). */
 tera_status tera_ctx_reserve(tera_ctx* ctx, int64_t max_agents, uint64_t max_records);
 
+/* The same for tera_partition, tera_pack(_ids) and tera_codec_batched(_ids) in
+ * both its forms: no place for an encode's payload (1.06 GB for 16.6 M records). */
+tera_status tera_ctx_reserve_batched(tera_ctx* ctx, int64_t max_agents, uint64_t max_records);
+
 /* Limit, in microseconds (0 .. 60000000; 1000000 when the context is made), of a
  * wait inside one of the context's kernels for another block of the same launch.
  * Such a wait ends by itself; one that takes longer is given up and latches

@@ -72,6 +72,7 @@ SIGNATURES = {
     "tera_ctx_destroy": (C.c_int, [P]),
     "tera_n_pairs": (u64, [P]),
     "tera_ctx_reserve": (C.c_int, [P, i64, u64]),
+    "tera_ctx_reserve_batched": (C.c_int, [P, i64, u64]),
     "tera_ctx_wait_limit": (C.c_int, [P, i64]),
     "tera_partition": (C.c_int, [P, C.POINTER(Soa), C.POINTER(PartitionOut), P]),
     "tera_pack": (C.c_int, [P, C.POINTER(Soa), C.POINTER(PartitionOut), u32, u32, P, u64, P]),

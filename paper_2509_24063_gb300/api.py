@@ -200,9 +200,11 @@ class Context:
               "tera_ctx_stats")
         return {k: int(getattr(s, k)) for k, _ in s._fields_}
 
-    def reserve(self, max_agents: int, max_records: int):
-        check(self.lib.tera_ctx_reserve(self.h, int(max_agents), int(max_records)),
-              "tera_ctx_reserve")
+    def reserve(self, max_agents: int, max_records: int, batched: bool = False):
+        """Scratch for the calls of an exchange (tera_ctx_reserve; batched: of one
+        through the batched codec, tera_ctx_reserve_batched)."""
+        f = self.lib.tera_ctx_reserve_batched if batched else self.lib.tera_ctx_reserve
+        check(f(self.h, int(max_agents), int(max_records)), "tera_ctx_reserve")
 
     def wait_limit(self, limit_us: int):
         """Limit of a wait inside a kernel of the calls after this one

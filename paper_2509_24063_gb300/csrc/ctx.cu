@@ -818,23 +818,34 @@ tera_status tera_ctx_destroy(tera_ctx* c) {
   return TERA_OK;
 }
 
-tera_status tera_ctx_reserve(tera_ctx* ctx, int64_t max_agents, uint64_t max_records) {
+// Scratch of an exchange: with the encode over tiles, or with the batched codec.
+static tera_status reserve(tera_ctx* ctx, int64_t max_agents, uint64_t max_records, bool batched) {
   if (!ctx || max_agents < 0) return TERA_EINVAL;
   cudaSetDevice(ctx->device);
   tera_status st = ensure_agents(ctx, max_agents, 0);
   if (st != TERA_OK) return st;
-  const u64 records = ctx->cap_records, listed = ctx->t_cap;
+  const u64 records = ctx->cap_records, listed = ctx->t_cap, worked = ctx->b_items_cap;
   if ((st = ensure_records(ctx, max_records, 0)) == TERA_OK)
     st = ensure_units(ctx, 2 * (max_records / kCodecTile) + 4 * ctx->n_pairs + 16, 0);
-  if (st == TERA_OK) {
+  if (st == TERA_OK && batched) {
+    if ((st = ensure_tiles(ctx, 0)) == TERA_OK) st = ensure_batched(ctx, 0);
+  } else if (st == TERA_OK) {
     ctx->t_refused = 0;
     (void)ensure_encode_tiles(ctx, 0);  // an encode without it takes the launches that need none
   }
   // new scratch was cleared on the default stream, which the callers' do not wait for
-  if ((ctx->cap_records != records || ctx->t_cap != listed) &&
+  if ((ctx->cap_records != records || ctx->t_cap != listed || ctx->b_items_cap != worked) &&
       cudaDeviceSynchronize() != cudaSuccess && st == TERA_OK)
     st = TERA_ECUDA;
   return st;
+}
+
+tera_status tera_ctx_reserve(tera_ctx* ctx, int64_t max_agents, uint64_t max_records) {
+  return reserve(ctx, max_agents, max_records, false);
+}
+
+tera_status tera_ctx_reserve_batched(tera_ctx* ctx, int64_t max_agents, uint64_t max_records) {
+  return reserve(ctx, max_agents, max_records, true);
 }
 
 tera_status tera_ctx_wait_limit(tera_ctx* ctx, int64_t limit_us) {

@@ -47,7 +47,7 @@ class AuraExchange:
         self.P = P
         self.max_agents = max_agents
         self.max_records = max_records
-        ctx.reserve(max_agents, max_records)
+        ctx.reserve(max_agents, max_records, batched=self.path == "batched")
         units = max_records + P
         u8 = dict(dtype=torch.uint8, device=dev)
         i64 = dict(dtype=torch.int64, device=dev)

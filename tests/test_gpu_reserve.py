@@ -109,3 +109,22 @@ def test_capture_of_the_other_form_of_the_batched_codec(eager, captured):
     for got, want in ((ex.sender_ref()[0], res["ref_next"]), (ex.receiver_ref()[0], res["recv"])):
         assert got[:units * 64].cpu().numpy().tobytes() == want[:units * 64].tobytes()
     ctx.close()
+
+
+@pytest.mark.parametrize("tune", [None, (256, 4, 0, 0)])
+def test_batched_exchange_is_captured_without_an_eager_step(tune):
+    import paper_2509_24063_gb300 as tera
+    wl = Workload("t", 40000, (0.0,) * 3, (160.0,) * 3, (4, 4, 4), 12.0, 1, seed=15)
+    st = next(iter(Generator(wl, device="cuda").series(1)))
+    ctx = tera.Context(wl.lo, wl.hi, wl.grid, wl.w)
+    ex = tera.AuraExchange(ctx, max_agents=50000, max_records=120000, path="batched", tune=tune)
+    graph = ex.capture(st)
+    graph.replay()
+    ex.advance()
+    assert ctx.status(raise_on_error=False)[0] == tera.OK
+    res = oracle.exchange_iteration(oracle.make_grid(wl.lo, wl.hi, wl.grid, wl.w), to_numpy(st))
+    np.testing.assert_array_equal(ex.wire_len.cpu().numpy().view(np.uint64), res["wire_len"])
+    units = int(res["pair_off"][-1]) + ctx.n_pairs
+    for got, want in ((ex.sender_ref()[0], res["ref_next"]), (ex.receiver_ref()[0], res["recv"])):
+        assert got[:units * 64].cpu().numpy().tobytes() == want[:units * 64].tobytes()
+    ctx.close()
